@@ -501,34 +501,67 @@ cudaError_t launch_joint_z(const float* e, const int32_t* frame_idx, const int32
 }
 
 // =====================================================================================
-// quantize_pack: Eq. 2 on fp16/fp32 rows, eight output codes per thread.
+// quantize_pack: Eq. 2 on fp16/fp32 rows, eight output codes ("a piece") per thread.  All of it
+// is bound by reading x once and writing the codes once: 23 MB for a 64 x 10 s batch at 8 bits.
+// Rows whose pieces are 16-byte aligned (VEC: k a multiple of 8 for fp16, of 4 for fp32, aligned
+// base) are read with 128-bit loads; other rows element by element.
 // =====================================================================================
-template <bool FP16>
-__device__ __forceinline__ float ldx(const void* x, long long i) {
-  return FP16 ? __half2float(reinterpret_cast<const __half*>(x)[i]) : reinterpret_cast<const float*>(x)[i];
+struct Piece {
+  uint4 a, b;   // raw elements: eight halves in a, or eight floats in a and b; zero beyond k
+};
+template <bool FP16, bool VEC>
+__device__ __forceinline__ Piece load_piece(const void* x, long long r, int k, int kb) {
+  Piece p;
+  p.a = p.b = make_uint4(0, 0, 0, 0);
+  if (FP16) {
+    const __half* q = reinterpret_cast<const __half*>(x) + r * k + kb;
+    if (VEC) {
+      if (kb < k) p.a = *reinterpret_cast<const uint4*>(q);
+    } else {
+      uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (kb + j < k) w[j >> 1] |= (uint32_t)__half_as_ushort(q[j]) << (16 * (j & 1));
+      p.a = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+  } else {
+    const float* q = reinterpret_cast<const float*>(x) + r * k + kb;
+    if (VEC) {
+      if (kb < k) p.a = *reinterpret_cast<const uint4*>(q);
+      if (kb + 4 < k) p.b = *reinterpret_cast<const uint4*>(q + 4);
+    } else {
+      uint32_t w[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) w[j] = kb + j < k ? __float_as_uint(q[j]) : 0u;
+      p.a = make_uint4(w[0], w[1], w[2], w[3]);
+      p.b = make_uint4(w[4], w[5], w[6], w[7]);
+    }
+  }
+  return p;
 }
-
-// scale_mode 0: constants in `a`; 1: per-group scale vector (row % n_groups); 2: per-row scale.
 template <bool FP16>
-__global__ void __launch_bounds__(256) k_quantize(const void* x, long long rows, int k, int k_pad,
-                                                  q4_act a, int scale_mode, int n_groups,
-                                                  const float* scale_vec, uint8_t* out) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int per_row = k_pad >> 3;
-  if (i >= rows * per_row) return;
-  const long long r = i / per_row;
-  const int kb = (int)(i % per_row) * 8;
-  float inv = a.inv_scale;
-  if (scale_mode == 1) inv = __fdiv_rn(1.0f, scale_vec[r % n_groups]);
-  if (scale_mode == 2) inv = __fdiv_rn(1.0f, scale_vec[r]);
+__device__ __forceinline__ void piece_values(const Piece& p, float (&v)[8]) {
+  if (FP16) {
+    const uint32_t w[4] = {p.a.x, p.a.y, p.a.z, p.a.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      v[2 * j] = __half2float(__ushort_as_half((unsigned short)(w[j] & 0xFFFFu)));
+      v[2 * j + 1] = __half2float(__ushort_as_half((unsigned short)(w[j] >> 16)));
+    }
+  } else {
+    const uint32_t w[8] = {p.a.x, p.a.y, p.a.z, p.a.w, p.b.x, p.b.y, p.b.z, p.b.w};
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(w[j]);
+  }
+}
+// codes of elements kb .. kb + 7 of row r; elements beyond k get the code of the real value 0
+__device__ __forceinline__ void store_codes(const float (&v)[8], float inv, const q4_act& a, int k, int k_pad,
+                                            long long r, int kb, uint8_t* out) {
   const int lo = act_lo(a), hi = act_hi(a);
   int q[8];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const int kk = kb + j;
-    q[j] = kk < k ? quantize1(ldx<FP16>(x, r * k + kk), inv, a.zero_point, lo, hi)
-                  : (a.is_signed ? 0 : a.zero_point);
-  }
+  for (int j = 0; j < 8; ++j)
+    q[j] = kb + j < k ? quantize1(v[j], inv, a.zero_point, lo, hi) : (a.is_signed ? 0 : a.zero_point);
   if (a.bits == 4) {
     uint32_t w = 0;
 #pragma unroll
@@ -550,17 +583,158 @@ __global__ void __launch_bounds__(256) k_quantize(const void* x, long long rows,
   }
 }
 
-// largest magnitude per group (row % n_groups); non-negative floats order like their bits
-template <bool FP16>
-__global__ void __launch_bounds__(256) k_absmax(const void* x, long long rows, int k, int n_groups,
-                                                uint32_t* amax_bits) {
-  const long long r = blockIdx.x;
-  if (r >= rows) return;
-  float m = 0.0f;
-  for (int j = threadIdx.x; j < k; j += blockDim.x) m = fmaxf(m, fabsf(ldx<FP16>(x, r * k + j)));
+// scale_mode 0: constants in `a`; 1: per-group scale vector (row % n_groups); 2: per-row scale.
+template <bool FP16, bool VEC>
+__global__ void __launch_bounds__(256) k_quantize(const void* x, long long rows, int k, int k_pad,
+                                                  q4_act a, int scale_mode, int n_groups,
+                                                  const float* scale_vec, uint8_t* out) {
+  pdl_trigger();
+  pdl_wait();
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int per_row = k_pad >> 3;
+  if (i >= rows * per_row) return;
+  long long r;
+  int kb;
+  if (rows * per_row <= 0xFFFFFFFFll) {   // 32-bit division
+    const uint32_t q = (uint32_t)i / (uint32_t)per_row;
+    r = q;
+    kb = (int)((uint32_t)i - q * (uint32_t)per_row) * 8;
+  } else {
+    r = i / per_row;
+    kb = (int)(i % per_row) * 8;
+  }
+  float inv = a.inv_scale;
+  if (scale_mode == 1) inv = __fdiv_rn(1.0f, scale_vec[r % n_groups]);
+  if (scale_mode == 2) inv = __fdiv_rn(1.0f, scale_vec[r]);
+  float v[8];
+  piece_values<FP16>(load_piece<FP16, VEC>(x, r, k, kb), v);
+  store_codes(v, inv, a, k, k_pad, r, kb, out);
+}
+
+// MAX boundary (mode 1) in one launch: a cluster of QM_CLUSTER CTAs owns one group (the rows
+// r = group + n_groups i).  Every CTA reads its share of the rows once into shared memory, the
+// CTAs' maxima meet through distributed shared memory, and the codes are made from the copy in
+// shared memory: x is read once and nothing goes through global atomics.  (Before: a memset, a
+// kernel with eight global atomics per row, a conversion kernel and the quantizer: 170 us for
+// 32000 x 240 fp16 in 64 groups, of which 157 us were the atomics; now 11.3 us.)
+constexpr int QM_CLUSTER = 8;
+constexpr int QM_THREADS = 256;
+constexpr size_t QM_SMEM_MAX = 100 * 1024;   // two CTAs per SM
+
+__device__ __forceinline__ float warp_max(float m) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(amax_bits + (r % n_groups), __float_as_uint(m));
+  return m;
+}
+
+template <bool FP16, bool VEC>
+__global__ void __cluster_dims__(QM_CLUSTER, 1, 1) __launch_bounds__(QM_THREADS)
+k_quantize_max(const void* x, int rows, int k, int k_pad, q4_act a, int n_groups, uint8_t* out, float* group_scale) {
+  extern __shared__ __align__(16) uint4 qm_smem[];
+  __shared__ float red[QM_THREADS / 32];
+  __shared__ float part[QM_CLUSTER];   // every CTA's maximum, filled by the whole cluster
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int rank = blockIdx.x % QM_CLUSTER, grp = blockIdx.x / QM_CLUSTER;
+  const int in_group = (rows - grp + n_groups - 1) / n_groups;           // rows of this group
+  const int share = (in_group + QM_CLUSTER - 1) / QM_CLUSTER;
+  const int i0 = rank * share, i1 = min(in_group, i0 + share);
+  const int per_row = k_pad >> 3, n = max(i1 - i0, 0) * per_row;
+  uint4* sa = qm_smem;
+  uint4* sb = qm_smem + (FP16 ? 0 : share * per_row);
+  pdl_trigger();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");   // this CTA runs; waited for before the exchange
+  pdl_wait();
+  float m = 0.0f;
+  for (int p = tid; p < n; p += QM_THREADS) {
+    const long long r = grp + (long long)n_groups * (i0 + p / per_row);
+    const Piece q = load_piece<FP16, VEC>(x, r, k, (p % per_row) * 8);
+    sa[p] = q.a;
+    if (!FP16) sb[p] = q.b;
+    float v[8];
+    piece_values<FP16>(q, v);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) m = fmaxf(m, fabsf(v[j]));
+  }
+  m = warp_max(m);
+  if (lane == 0) red[warp] = m;
+  __syncthreads();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (warp == 0) {
+    m = warp_max(lane < QM_THREADS / 32 ? red[lane] : 0.0f);
+    if (lane < QM_CLUSTER) {   // to every CTA of the cluster
+      uint32_t addr = (uint32_t)__cvta_generic_to_shared(&part[rank]), remote;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(lane));
+      asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(m) : "memory");
+    }
+  }
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  m = 0.0f;
+#pragma unroll
+  for (int c = 0; c < QM_CLUSTER; ++c) m = fmaxf(m, part[c]);
+  if (m == 0.0f) m = 1.0f;
+  const float scale = __fdiv_rn(m, (float)((1 << (a.bits - 1)) - 1));
+  const float inv = __fdiv_rn(1.0f, scale);
+  if (rank == 0 && tid == 0) group_scale[grp] = scale;
+  for (int p = tid; p < n; p += QM_THREADS) {
+    const long long r = grp + (long long)n_groups * (i0 + p / per_row);
+    Piece q;
+    q.a = sa[p];
+    q.b = FP16 ? make_uint4(0, 0, 0, 0) : sb[p];
+    float v[8];
+    piece_values<FP16>(q, v);
+    store_codes(v, inv, a, k, k_pad, r, (p % per_row) * 8, out);
+  }
+}
+
+// One group per row (weights quantized offline with the MAX boundary): a warp per row, the row is
+// read twice, the second time from the cache.
+template <bool FP16, bool VEC>
+__global__ void __launch_bounds__(256) k_quantize_max_rows(const void* x, long long rows, int k, int k_pad, q4_act a,
+                                                           uint8_t* out, float* group_scale) {
+  const long long r = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (r >= rows) return;
+  float m = 0.0f, v[8];
+  for (int kb = 8 * lane; kb < k_pad; kb += 256) {
+    piece_values<FP16>(load_piece<FP16, VEC>(x, r, k, kb), v);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) m = fmaxf(m, fabsf(v[j]));
+  }
+  m = warp_max(m);
+  if (m == 0.0f) m = 1.0f;
+  const float scale = __fdiv_rn(m, (float)((1 << (a.bits - 1)) - 1));
+  const float inv = __fdiv_rn(1.0f, scale);
+  if (lane == 0) group_scale[r] = scale;
+  for (int kb = 8 * lane; kb < k_pad; kb += 256) {
+    piece_values<FP16>(load_piece<FP16, VEC>(x, r, k, kb), v);
+    store_codes(v, inv, a, k, k_pad, r, kb, out);
+  }
+}
+
+// Groups too large for the shared memory of a cluster: largest magnitude per group (row %
+// n_groups) through global memory; non-negative floats order like their bits.  A CTA walks rows
+// of one group (a stride of n_groups * gridDim.y rows), so that it needs one atomic.
+template <bool FP16, bool VEC>
+__global__ void __launch_bounds__(256) k_absmax(const void* x, long long rows, int k, int n_groups,
+                                                uint32_t* amax_bits) {
+  __shared__ float red[8];
+  const int grp = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float m = 0.0f, v[8];
+  for (long long r = grp + (long long)n_groups * (blockIdx.y * 8 + warp); r < rows; r += (long long)n_groups * gridDim.y * 8)
+    for (int kb = 8 * lane; kb < k; kb += 256) {
+      piece_values<FP16>(load_piece<FP16, VEC>(x, r, k, kb), v);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) m = fmaxf(m, fabsf(v[j]));
+    }
+  m = warp_max(m);
+  if (lane == 0) red[warp] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int w = 1; w < 8; ++w) m = fmaxf(m, red[w]);
+    if (m > 0.0f) atomicMax(amax_bits + grp, __float_as_uint(m));
+  }
 }
 
 __global__ void k_amax_to_scale(uint32_t* amax_bits, int n_groups, int qmax) {
@@ -571,73 +745,140 @@ __global__ void k_amax_to_scale(uint32_t* amax_bits, int n_groups, int qmax) {
   reinterpret_cast<float*>(amax_bits)[g] = __fdiv_rn(m, (float)qmax);
 }
 
-cudaError_t launch_quantize(const void* x, bool fp16, long long rows, int k, int k_pad,
-                            const q4_act& a, int mode, int n_groups, const float* scale_vec,
-                            uint8_t* out, float* group_scale_out, cudaStream_t s) {
-  if (rows <= 0) return cudaSuccess;
+template <bool FP16, bool VEC>
+static cudaError_t quantize_t(const void* x, long long rows, int k, int k_pad, const q4_act& a, int mode, int n_groups,
+                              const float* scale_vec, uint8_t* out, float* group_scale_out, cudaStream_t s) {
+  const int per_row = k_pad >> 3;
   const float* sv = scale_vec;
+  cudaError_t e = cudaSuccess;
   if (mode == 1) {
-    cudaError_t e = cudaMemsetAsync(group_scale_out, 0, sizeof(float) * n_groups, s);
+    // Groups of several rows whose eighth fits half an SM's shared memory: one launch, one cluster per
+    // group; one row per group: one launch, one warp per row; else through global memory.
+    const long long in_group = (rows + n_groups - 1) / n_groups;
+    const size_t smem = (size_t)((in_group + QM_CLUSTER - 1) / QM_CLUSTER) * per_row * (FP16 ? 16 : 32);
+    if (in_group == 1 && rows == n_groups) {
+      timing_begin(s);
+      k_quantize_max_rows<FP16, VEC><<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(x, rows, k, k_pad, a, out, group_scale_out);
+      timing_end(s);
+      ++g_launches;
+      return cudaGetLastError();
+    }
+    if (rows >= n_groups && rows <= INT32_MAX && n_groups <= 65536 && smem <= QM_SMEM_MAX) {
+      static bool configured = false;
+      if (!configured) {
+        e = cudaFuncSetAttribute(k_quantize_max<FP16, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)QM_SMEM_MAX);
+        if (e != cudaSuccess) return e;
+        configured = true;
+      }
+      timing_begin(s);
+      e = launch_ex(k_quantize_max<FP16, VEC>, dim3((unsigned)n_groups * QM_CLUSTER), dim3(QM_THREADS), smem, s, true, 1, x,
+                    (int)rows, k, k_pad, a, n_groups, out, group_scale_out);
+      timing_end(s);
+      ++g_launches;
+      return e != cudaSuccess ? e : cudaGetLastError();
+    }
+    e = cudaMemsetAsync(group_scale_out, 0, sizeof(float) * n_groups, s);
     if (e != cudaSuccess) return e;
-    if (fp16)
-      k_absmax<true><<<(unsigned)rows, 256, 0, s>>>(x, rows, k, n_groups, (uint32_t*)group_scale_out);
-    else
-      k_absmax<false><<<(unsigned)rows, 256, 0, s>>>(x, rows, k, n_groups, (uint32_t*)group_scale_out);
+    const long long splits = (in_group + 7) / 8;
+    const unsigned want = (unsigned)(4 * 148 / n_groups + 1);   // about four CTAs per SM over all groups
+    const dim3 grid((unsigned)n_groups, splits < want ? (unsigned)splits : want);
+    k_absmax<FP16, VEC><<<grid, 256, 0, s>>>(x, rows, k, n_groups, (uint32_t*)group_scale_out);
     k_amax_to_scale<<<(n_groups + 255) / 256, 256, 0, s>>>((uint32_t*)group_scale_out, n_groups,
                                                            (1 << (a.bits - 1)) - 1);
     g_launches += 2;
     sv = group_scale_out;
   }
-  const long long total = rows * (k_pad >> 3);
-  const unsigned blocks = (unsigned)((total + 255) / 256);
+  const long long total = rows * per_row;
   timing_begin(s);
-  if (fp16)
-    k_quantize<true><<<blocks, 256, 0, s>>>(x, rows, k, k_pad, a, mode, n_groups, sv, out);
-  else
-    k_quantize<false><<<blocks, 256, 0, s>>>(x, rows, k, k_pad, a, mode, n_groups, sv, out);
+  e = launch_ex(k_quantize<FP16, VEC>, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, s, true, 1, x, rows, k, k_pad,
+                a, mode, n_groups, sv, out);
   timing_end(s);
   ++g_launches;
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_quantize(const void* x, bool fp16, long long rows, int k, int k_pad,
+                            const q4_act& a, int mode, int n_groups, const float* scale_vec,
+                            uint8_t* out, float* group_scale_out, cudaStream_t s) {
+  if (rows <= 0) return cudaSuccess;
+  const bool vec = k % (fp16 ? 8 : 4) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+  if (fp16)
+    return vec ? quantize_t<true, true>(x, rows, k, k_pad, a, mode, n_groups, scale_vec, out, group_scale_out, s)
+               : quantize_t<true, false>(x, rows, k, k_pad, a, mode, n_groups, scale_vec, out, group_scale_out, s);
+  return vec ? quantize_t<false, true>(x, rows, k, k_pad, a, mode, n_groups, scale_vec, out, group_scale_out, s)
+             : quantize_t<false, false>(x, rows, k, k_pad, a, mode, n_groups, scale_vec, out, group_scale_out, s);
 }
 
 // =====================================================================================
-// Feature prologue: time differences with replicated edges, then frame stacking.
+// Feature prologue: time differences with replicated edges, then frame stacking.  A thread makes
+// both stacked frames (t, t + 1) of VEC neighbouring mel bands from six input rows and stores
+// whole runs of VEC halves; bound by the 25 MB it moves for 64 x 10 s.  (One frame and band per
+// thread with 2-byte stores: 21 us; four bands: 5.3 us = 4.7 TB/s.)
 // =====================================================================================
-__device__ __forceinline__ float mel_at(const float* m, int T, int M, int t, int j) {
-  t = max(0, min(t, T - 1));
-  return m[(long long)t * M + j];
-}
-__device__ __forceinline__ float delta_at(const float* m, int T, int M, int t, int j) {
-  t = max(0, min(t, T - 1));
-  return __fmul_rn(__fsub_rn(mel_at(m, T, M, t + 1, j), mel_at(m, T, M, t - 1, j)), 0.5f);
-}
-
-__global__ void __launch_bounds__(256) k_features(const float* mel, int B, int T100, int M,
-                                                  __half* out) {
+template <int VEC>
+__global__ void __launch_bounds__(256) k_features(const float* mel, int B, int T100, int M, __half* out) {
+  pdl_trigger();
+  pdl_wait();
+  const int per = M / VEC, S = T100 / 2;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)B * T100 * M) return;
-  const int j = (int)(i % M);
-  const int t = (int)((i / M) % T100);
-  const int b = (int)(i / ((long long)M * T100));
-  if (t >= (T100 / 2) * 2) return;
-  const float* m = mel + (long long)b * T100 * M;
-  const float x = m[(long long)t * M + j];
-  const float d = delta_at(m, T100, M, t, j);
-  const float dd = __fmul_rn(__fsub_rn(delta_at(m, T100, M, t + 1, j), delta_at(m, T100, M, t - 1, j)), 0.5f);
-  __half* o = out + (((long long)(t >> 1) * B + b) * 2 + (t & 1)) * 3 * M;
-  o[j] = __float2half_rn(x);
-  o[M + j] = __float2half_rn(d);
-  o[2 * M + j] = __float2half_rn(dd);
+  if (i >= (long long)B * S * per) return;
+  const int j = (int)(i % per) * VEC;
+  const int sb = (int)(i / per), sidx = sb % S, b = sb / S;
+  const int t = 2 * sidx;
+  const float* m = mel + (long long)b * T100 * M + j;
+  float x[6][VEC];   // rows t - 2 .. t + 3, edges replicated
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    const float* p = m + (long long)max(0, min(t - 2 + q, T100 - 1)) * M;
+    if (VEC == 4) {
+      const float4 v = *reinterpret_cast<const float4*>(p);
+      x[q][0] = v.x;
+      x[q][1] = v.y;
+      x[q][2] = v.z;
+      x[q][3] = v.w;
+    } else {
+      x[q][0] = *p;
+    }
+  }
+  float f[2][3][VEC];   // [frame][value, difference, difference of differences]
+#pragma unroll
+  for (int v = 0; v < VEC; ++v) {
+    const float d0 = __fmul_rn(__fsub_rn(x[3][v], x[1][v]), 0.5f), d1 = __fmul_rn(__fsub_rn(x[4][v], x[2][v]), 0.5f);
+    const float dm = t == 0 ? d0 : __fmul_rn(__fsub_rn(x[2][v], x[0][v]), 0.5f);             // at t - 1
+    const float dp = t + 2 > T100 - 1 ? d1 : __fmul_rn(__fsub_rn(x[5][v], x[3][v]), 0.5f);   // at t + 2
+    f[0][0][v] = x[2][v];
+    f[0][1][v] = d0;
+    f[0][2][v] = __fmul_rn(__fsub_rn(d1, dm), 0.5f);
+    f[1][0][v] = x[3][v];
+    f[1][1][v] = d1;
+    f[1][2][v] = __fmul_rn(__fsub_rn(dp, d0), 0.5f);
+  }
+  __half* o = out + ((long long)sidx * B + b) * 6 * M + j;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    if (VEC == 4) {
+      const __half2 h0 = __floats2half2_rn(f[q / 3][q % 3][0], f[q / 3][q % 3][1]);
+      const __half2 h1 = __floats2half2_rn(f[q / 3][q % 3][2], f[q / 3][q % 3][3]);
+      *reinterpret_cast<uint2*>(o + (long long)q * M) =
+          make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+    } else {
+      o[(long long)q * M] = __float2half_rn(f[q / 3][q % 3][0]);
+    }
+  }
 }
 
 cudaError_t launch_features(const float* mel, int B, int T100, int M, void* out, cudaStream_t s) {
-  const long long total = (long long)B * T100 * M;
-  if (total <= 0) return cudaSuccess;
+  if ((long long)B * T100 * M <= 0) return cudaSuccess;
+  // four bands per thread need 16-byte aligned rows of mel and 8-byte aligned runs of the output
+  const bool vec = M % 4 == 0 && (reinterpret_cast<uintptr_t>(mel) & 15) == 0 && (reinterpret_cast<uintptr_t>(out) & 7) == 0;
+  const long long total = (long long)B * (T100 / 2) * (vec ? M / 4 : M);
+  const dim3 grid((unsigned)((total + 255) / 256));
   timing_begin(s);
-  k_features<<<(unsigned)((total + 255) / 256), 256, 0, s>>>(mel, B, T100, M, (__half*)out);
+  cudaError_t e = vec ? launch_ex(k_features<4>, grid, dim3(256), 0, s, true, 1, mel, B, T100, M, (__half*)out)
+                      : launch_ex(k_features<1>, grid, dim3(256), 0, s, true, 1, mel, B, T100, M, (__half*)out);
   timing_end(s);
   ++g_launches;
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace q4

@@ -60,6 +60,22 @@ def test_max_boundary_per_utterance(Bd, bits, T, B, F):
         np.testing.assert_array_equal(codes[:, b, :], O.quantize(x[:, b, :].astype(np.float32), a))
 
 
+# one cluster per group (aligned and odd row lengths, groups of unequal size, fewer rows than a cluster's CTAs),
+# and groups too large for a cluster's shared memory
+@pytest.mark.parametrize("dtype", [np.float16, np.float32])
+@pytest.mark.parametrize("rows,k,groups", [(10, 45, 3), (2, 240, 1), (333, 340, 4), (1300, 1280, 1), (9, 1000, 8)])
+def test_max_boundary_per_group(Bd, dtype, rows, k, groups):
+    x = synth.Stream(14).normal(f"g{rows}.{k}", (rows, k)).astype(dtype)
+    base = Bd.q4_act_symmetric(1.0, 8)
+    got, scales = Bd.quantize_pack_int4(torch.from_numpy(x).cuda(), base, mode=1, n_groups=groups)
+    codes = gpu_codes(got, k, base)
+    for g in range(groups):
+        a = O.act_symmetric(O.absmax(x[g::groups].astype(np.float32)), 8)
+        assert scales[g].item() == a.scale
+        np.testing.assert_array_equal(codes[g::groups], O.quantize(x[g::groups].astype(np.float32), a))
+    assert (gpu_codes(got, Bd.pad32(k), base)[:, k:] == 0).all()
+
+
 @pytest.mark.parametrize("bits", [4, 8])
 def test_weight_mode_per_row_scale(Bd, bits):
     st = synth.Stream(5)
