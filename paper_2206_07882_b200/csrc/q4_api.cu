@@ -267,8 +267,14 @@ int q4_linear_forward(const void* xq, const q4_act* x_act, int32_t M, const q4_m
       const int Mp = (M + 127) / 128 * 128;
       TagScope tag(TAG_LINEAR);
       // the gather clears the status block and may start under the tail of whatever kernel precedes the call
-      Q4_TRY(launch_unpack_rows(xq, row_bytes(w->k_pad, x_act->bits), nullptr, *x_act, w->k_pad, M, x8, w->k_pad, 0,
-                                Mp, s, status, true));
+      UnpackJobs uj;
+      memset(&uj, 0, sizeof(uj));
+      uj.n_rows = M;
+      uj.n_rows_pad = Mp;
+      uj.zero_tail = 1;
+      uj.clear64 = status;
+      add_unpack_job(uj, xq, row_bytes(w->k_pad, x_act->bits), nullptr, *x_act, w->k_pad, x8);
+      Q4_TRY(launch_unpack_multi(uj, s, true));
       Q4_TRY(launch_mma_gemm(x8, w->k_pad, M, static_cast<const int8_t*>(prepared), w->k_pad, w->rows, w->k_pad,
                              EPI_F32, out, w->rows, nullptr, w->scale, bias, x_act->scale, nullptr, status, nullptr,
                              s, true));   // programmatic dependent of the gather before it
@@ -354,10 +360,16 @@ int qlstm_step(const void* xq, const q4_act* x_act, const int32_t* x_row_idx, co
       int8_t* h8 = x8 + align_up((size_t)Np * Kx);
       TagScope tag(TAG_PRED_LSTM);
       // every kernel of the call is a programmatic dependent of the one before (each waits for its
-      // predecessor's completion before it reads anything); the first gather clears the status block
-      Q4_TRY(launch_unpack_rows(xq, row_bytes(w_ih->k_pad, x_act->bits), x_row_idx, *x_act, (int)Kx, N, x8, (long long)Kx,
-                                0, Np, s, status, true));
-      Q4_TRY(launch_unpack_rows(hq_in, row_bytes(H, hid_act->bits), nullptr, *hid_act, H, N, h8, H, 0, Np, s, nullptr, true));
+      // predecessor's completion before it reads anything); the gather clears the status block
+      UnpackJobs uj;
+      memset(&uj, 0, sizeof(uj));
+      uj.n_rows = N;
+      uj.n_rows_pad = Np;
+      uj.zero_tail = 1;
+      uj.clear64 = status;
+      add_unpack_job(uj, xq, row_bytes(w_ih->k_pad, x_act->bits), x_row_idx, *x_act, (int)Kx, x8);
+      add_unpack_job(uj, hq_in, row_bytes(H, hid_act->bits), nullptr, *hid_act, H, h8);
+      Q4_TRY(launch_unpack_multi(uj, s, true));
       MmaLstmArgs a;
       memset(&a, 0, sizeof(a));
       a.N = N;
@@ -378,7 +390,7 @@ int qlstm_step(const void* xq, const q4_act* x_act, const int32_t* x_row_idx, co
       a.dbg_hh = dbg_acc_hh;
       a.dbg_ld = 4LL * H;
       a.status = status;
-      // programmatic dependent of the second gather (which started after the first had completed)
+      // programmatic dependent of the gather
       Q4_TRY(launch_mma_lstm(a, x8, (long long)Kx, xw8, (long long)Kx, h8, H, hw8, H, s, true));
       return Q4_OK;
     }
@@ -436,7 +448,6 @@ int qlstm_layer_forward(const void* xq, const q4_act* x_act, const float* x_scal
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   int32_t* status = reinterpret_cast<int32_t*>(ws);
   ws += 256;
-  Q4_TRY(cudaMemsetAsync(status, 0, 256, s));
   int32_t* acc_ih = reinterpret_cast<int32_t*>(ws);
   ws += align_up((size_t)dirs * TB * G * sizeof(int32_t));
   uint8_t* hbuf = ws;  // [dirs][2][B*H bytes]
@@ -458,26 +469,44 @@ int qlstm_layer_forward(const void* xq, const q4_act* x_act, const float* x_scal
 
   // time-parallel input projections for all frames
   if (use_mma) {
-    TagScope tag(TAG_QUANT);
-    Q4_TRY(launch_unpack_rows(xq, xb, nullptr, *x_act, Kx, (int)TB, x8, Kx, 0, (int)TB, s));
-    for (int d = 0; d < dirs; ++d)
-      Q4_TRY(launch_prepare_w(w_ih[d], persistent ? 1 : 0, w8 + (size_t)d * G * Kx, Kx, 0, s));
-    if (persistent) {
-      for (int d = 0; d < dirs; ++d) {
-        Q4_TRY(launch_prepare_w(w_hh[d], 1, whh8 + (size_t)d * G * H, H, 0, s));
-        Q4_TRY(launch_prepare_vec(w_ih[d].scale, G, 1, vec_ih + (size_t)d * G, s));
-        Q4_TRY(launch_prepare_vec(w_hh[d].scale, G, 1, vec_hh + (size_t)d * G, s));
-        Q4_TRY(launch_prepare_vec(bias ? bias[d] : nullptr, G, 1, vec_b + (size_t)d * G, s));
-      }
+    LayerPrep lp;
+    memset(&lp, 0, sizeof(lp));
+    lp.H = H;
+    lp.clear64 = status;
+    auto mat = [&](const void* src, int8_t* dst, long long rows, int k_pad, int bits, int is_signed, int zp, int interleave) {
+      LayerPrepMat& m = lp.mat[lp.n_mats++];
+      m.src = static_cast<const uint8_t*>(src);
+      m.dst = dst;
+      m.rows = rows;
+      m.k_pad = k_pad;
+      m.bits = bits;
+      m.is_signed = is_signed;
+      m.zp = zp;
+      m.interleave = interleave;
+    };
+    auto vec = [&](const float* src, float* dst) {
+      lp.vec_src[lp.n_vecs] = src;
+      lp.vec_dst[lp.n_vecs++] = dst;
+    };
+    mat(xq, x8, TB, Kx, x_act->bits, x_act->is_signed, x_act->zero_point, 0);
+    for (int d = 0; d < dirs; ++d) {
+      mat(w_ih[d].q, w8 + (size_t)d * G * Kx, G, Kx, w_ih[d].bits, 1, 0, persistent ? H : 0);
+      if (!persistent) continue;
+      mat(w_hh[d].q, whh8 + (size_t)d * G * H, G, H, w_hh[d].bits, 1, 0, H);
+      vec(w_ih[d].scale, vec_ih + (size_t)d * G);
+      vec(w_hh[d].scale, vec_hh + (size_t)d * G);
+      vec(bias ? bias[d] : nullptr, vec_b + (size_t)d * G);
     }
-  }
-  for (int d = 0; d < dirs; ++d) {
+    {
+      TagScope tag(TAG_QUANT);
+      Q4_TRY(launch_layer_prepare(lp, s, true));
+    }
     TagScope tag(TAG_ENC_GEMM);
-    if (use_mma) {
-      Q4_TRY(launch_mma_gemm(x8, Kx, (int)TB, w8 + (size_t)d * G * Kx, Kx, G, Kx, EPI_I32,
-                             acc_ih + (size_t)d * TB * G, G, nullptr, nullptr, nullptr, 0.0f, nullptr,
-                             status, nullptr, s));
-    } else {
+    Q4_TRY(launch_mma_gemm_i32(x8, (int)TB, w8, G, Kx, dirs, acc_ih, status, s, true));
+  } else {
+    Q4_TRY(cudaMemsetAsync(status, 0, 256, s));
+    for (int d = 0; d < dirs; ++d) {
+      TagScope tag(TAG_ENC_GEMM);
       GemmArgs g = gemm_args(xq, xb, nullptr, *x_act, (int)TB, w_ih[d], nullptr,
                              acc_ih + (size_t)d * TB * G, G, nullptr);
       Q4_TRY(launch_gemm(g, EPI_I32, s));
@@ -600,7 +629,14 @@ int qjoint_logprobs(const float* e, const int32_t* frame_idx, const void* pq, co
     int32_t* status = reinterpret_cast<int32_t*>(ws);
     int8_t* p8 = reinterpret_cast<int8_t*>(ws + 256);
     int8_t* z8 = p8 + align_up((size_t)Np * Hp);
-    Q4_TRY(launch_unpack_rows(pq, row_bytes(Hp, p_act->bits), nullptr, *p_act, Hp, N, p8, Hp, 0, Np, s, status, true));
+    UnpackJobs uj;
+    memset(&uj, 0, sizeof(uj));
+    uj.n_rows = N;
+    uj.n_rows_pad = Np;
+    uj.zero_tail = 1;
+    uj.clear64 = status;
+    add_unpack_job(uj, pq, row_bytes(Hp, p_act->bits), nullptr, *p_act, Hp, p8);
+    Q4_TRY(launch_unpack_multi(uj, s, true));
     Q4_TRY(launch_mma_gemm(p8, Hp, N, static_cast<const int8_t*>(prepared_pred), Hp, D, Hp, EPI_JOINTZ, z8, D,
                            nullptr, w_pred->scale, b_pred, p_act->scale, z_act, status, nullptr, s, true, e,
                            frame_idx));   // each kernel of the call is a programmatic dependent of the one before
@@ -969,27 +1005,14 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
     if (nets && !skinny) {
       UnpackJobs uj;
       memset(&uj, 0, sizeof(uj));
-      auto add = [&](const void* src, long long stride, const int32_t* idx, const q4_act& act, int k_pad,
-                     int8_t* dst) {
-        UnpackJob& j = uj.job[uj.n_jobs++];
-        j.src = static_cast<const uint8_t*>(src);
-        j.src_stride = stride;
-        j.idx = idx;
-        j.bits = act.bits;
-        j.is_signed = act.is_signed;
-        j.zp = act.zero_point;
-        j.k_pad = k_pad;
-        j.dst = dst;
-        j.dst_stride = k_pad;
-      };
-      add(m.pred_emb_q, row_bytes(Ep, m.pred_emb_act.bits), cst.adv_tok, m.pred_emb_act, Ep, xa8[0]);
-      add(m.src.emb_q, row_bytes(Ep, m.src.emb_act.bits), cst.adv_tok, m.src.emb_act, Ep, xa8[1]);
-      add(m.tgt.emb_q, row_bytes(Ep, m.tgt.emb_act.bits), cst.adv_tok, m.tgt.emb_act, Ep, xa8[2]);
-      add(st.pred_hq, row_bytes(Hp, m.pred_lstm.hid_act.bits), cst.adv_src, m.pred_lstm.hid_act, Hp, ha8[0]);
-      add(st.src_hq, row_bytes(Hs, m.src.lstm[0].hid_act.bits), cst.adv_src, m.src.lstm[0].hid_act, Hs, ha8[1]);
-      add(st.tgt_hq[0], row_bytes(Ht, m.tgt.lstm[0].hid_act.bits), cst.adv_src, m.tgt.lstm[0].hid_act, Ht, ha8[2]);
+      add_unpack_job(uj, m.pred_emb_q, row_bytes(Ep, m.pred_emb_act.bits), cst.adv_tok, m.pred_emb_act, Ep, xa8[0]);
+      add_unpack_job(uj, m.src.emb_q, row_bytes(Ep, m.src.emb_act.bits), cst.adv_tok, m.src.emb_act, Ep, xa8[1]);
+      add_unpack_job(uj, m.tgt.emb_q, row_bytes(Ep, m.tgt.emb_act.bits), cst.adv_tok, m.tgt.emb_act, Ep, xa8[2]);
+      add_unpack_job(uj, st.pred_hq, row_bytes(Hp, m.pred_lstm.hid_act.bits), cst.adv_src, m.pred_lstm.hid_act, Hp, ha8[0]);
+      add_unpack_job(uj, st.src_hq, row_bytes(Hs, m.src.lstm[0].hid_act.bits), cst.adv_src, m.src.lstm[0].hid_act, Hs, ha8[1]);
+      add_unpack_job(uj, st.tgt_hq[0], row_bytes(Ht, m.tgt.lstm[0].hid_act.bits), cst.adv_src, m.tgt.lstm[0].hid_act, Ht, ha8[2]);
       if (m.tgt.n_layers == 2)
-        add(st.tgt_hq[1], row_bytes(Ht, m.tgt.lstm[1].hid_act.bits), cst.adv_src, m.tgt.lstm[1].hid_act, Ht, ha8[3]);
+        add_unpack_job(uj, st.tgt_hq[1], row_bytes(Ht, m.tgt.lstm[1].hid_act.bits), cst.adv_src, m.tgt.lstm[1].hid_act, Ht, ha8[3]);
       uj.n_rows = N;
       uj.n_rows_pad = (int)Np;
       uj.zero_tail = 0;   // rows beyond the pending advances feed tiles whose results are dropped

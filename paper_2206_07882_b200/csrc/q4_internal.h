@@ -103,12 +103,6 @@ cudaError_t launch_mma_lmhead(const LmHeadArgs& a, const int8_t* h8, long long h
                               const int8_t* wo8, cudaStream_t s, bool dependent = false);
 enum { EPI_QUANT8 = 3,      // re-quantize and store (code - zero_point) as int8, one per byte
        EPI_JOINTZ = 4 };    // tanh(other factor * value), quantized, stored like EPI_QUANT8
-cudaError_t launch_unpack_rows(const void* src, long long src_stride, const int32_t* idx,
-                               const q4_act& act, int k_pad, int n_rows, int8_t* dst,
-                               long long dst_stride, int col0, int n_rows_pad, cudaStream_t s,
-                               int32_t* clear_status = nullptr, bool dependent = false);
-// clear_status: 64 status words zeroed by the kernel's first block (replaces a memset node in front of a
-// call); dependent: launched as a programmatic dependent (the kernel waits for its predecessor itself)
 struct UnpackJob {
   const uint8_t* src;       // packed code rows
   long long src_stride;
@@ -121,7 +115,10 @@ struct UnpackJobs {
   UnpackJob job[8];
   int32_t n_jobs, n_rows, n_rows_pad, zero_tail;
   const int32_t* n_active;
+  int32_t* clear64;         // 64 status words zeroed by the first block (no memset in front of a call), or null
 };
+void add_unpack_job(UnpackJobs& u, const void* src, long long src_stride, const int32_t* idx, const q4_act& act, int k_pad,
+                    int8_t* dst);
 cudaError_t launch_unpack_multi(const UnpackJobs& jobs, cudaStream_t s, bool dependent = false);
 cudaError_t launch_prepare_w(const q4_mat& w, int interleave, int8_t* dst, long long dst_stride,
                              int col0, cudaStream_t s);
@@ -134,6 +131,25 @@ cudaError_t launch_mma_gemm(const int8_t* x8, long long x_pitch, int M, const in
                             const int32_t* n_active, cudaStream_t s, bool dependent = false,
                             const float* mul_e = nullptr, const int32_t* mul_idx = nullptr);
 void test_wait_expiry_set(int skip_producer, uint32_t wait_limit);
+cudaError_t launch_mma_gemm_i32(const int8_t* x8, int M, const int8_t* w8, int J, int K, int planes, int32_t* out,
+                                int32_t* status, cudaStream_t s, bool dependent = false);
+// One launch for what a layer call prepares (k_layer_prepare).
+struct LayerPrepMat {
+  const uint8_t* src;       // packed codes [rows, k_pad]
+  int8_t* dst;              // int8 [rows, k_pad]
+  long long rows;
+  int32_t k_pad, bits, is_signed, zp;
+  int32_t interleave;       // H > 0: rows reordered from gate-major to 4*cell+gate; 0: as they are
+  int32_t blocks;           // set by the launcher
+};
+struct LayerPrep {
+  LayerPrepMat mat[5];      // input codes, then w_ih and w_hh of each direction
+  int32_t n_mats, n_vecs, H;
+  const float* vec_src[6];  // [4H] row scales and biases (null = zeros), written in 4*cell+gate order
+  float* vec_dst[6];
+  int32_t* clear64;         // 64 status words set to zero
+};
+cudaError_t launch_layer_prepare(LayerPrep a, cudaStream_t s, bool dependent);
 cudaError_t launch_mma_lstm(const MmaLstmArgs& a, const int8_t* xa, long long xa_pitch,
                             const int8_t* xw, long long xw_pitch, const int8_t* ha, long long ha_pitch,
                             const int8_t* hw, long long hw_pitch, cudaStream_t s, bool dependent = false);

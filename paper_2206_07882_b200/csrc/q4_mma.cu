@@ -1,7 +1,8 @@
 // Tensor-core path (sm_100a): TMA-fed tcgen05 kind::i8 GEMMs with int32 accumulators in
 // tensor memory.  Activations are the M operand (128 rows per tile), weight rows the N
 // operand, both K-major int8 in shared memory under the 128-byte swizzle.
-//   k_mma_gemm : D[128 x 256] tiles, epilogues: store int32 / de-quantize+bias / re-quantize.
+//   k_mma_gemm : D[128 x 32..256] tiles, epilogues: de-quantize+bias / re-quantize / joint element-wise;
+//   k_mma_gemm_persistent : the same main loop with the int32 sums stored as they are.
 //   k_mma_lstm : D_ih, D_hh[128 x 128] tiles (32 cells x 4 gates, gate-interleaved weight
 //                rows) with the whole LSTM cell update fused into the epilogue.
 // Warp roles per CTA: epilogue warps (one TMEM lane quarter each), one TMA producer thread,
@@ -16,89 +17,43 @@ namespace q4 {
 
 constexpr int BM = 128;          // activation rows per tile
 constexpr int BK = 128;          // K bytes per pipeline stage (one swizzle row)
-constexpr int GEMM_BN = 256;     // weight rows per tile, plain GEMM
-constexpr int GEMM_STAGES = 4;
+template <int BN>
+constexpr int GEMM_STAGES = BN >= 128 ? 4 : 6;   // ring depth of the plain GEMM with BN weight rows per tile
 constexpr int LSTM_BN = 128;     // weight rows per tile, LSTM (32 cells x 4 gates)
 constexpr int LSTM_STAGES = 3;
 constexpr int LSTM_EPI_WARPS = 8;
 
 // ------------------------------------------------------------------ operand preparation
-// Gather + unpack activation rows to int8: dst[n, col0 + k] = code(src[idx[n], k]) - zero_point.
-__global__ void __launch_bounds__(256) k_unpack_rows(const uint8_t* src, long long src_stride,
-                                                     const int32_t* idx, int bits, int is_signed,
-                                                     int zp, int k_pad, int n_rows, int8_t* dst,
-                                                     long long dst_stride, int col0, int n_rows_pad, int32_t* clear64) {
+__device__ __forceinline__ void unpack_piece32(const uint8_t* p, int k, int bits, bool is_signed, uint32_t zp4, uint4& o0,
+                                               uint4& o1) {   // 32 codes of a row -> int8, natural order
+  if (bits == 4) {
+    const uint4 v = *reinterpret_cast<const uint4*>(p + (k >> 1));
+    unpack8_natural(v.x, is_signed, zp4, o0.x, o0.y);
+    unpack8_natural(v.y, is_signed, zp4, o0.z, o0.w);
+    unpack8_natural(v.z, is_signed, zp4, o1.x, o1.y);
+    unpack8_natural(v.w, is_signed, zp4, o1.z, o1.w);
+  } else if (bits == 2) {
+    const uint2 v = *reinterpret_cast<const uint2*>(p + (k >> 2));
+    uint32_t a[4], b[4];
+    unpack16x2(v.x, a);
+    unpack16x2(v.y, b);
+    o0 = make_uint4(a[0], a[1], a[2], a[3]);
+    o1 = make_uint4(b[0], b[1], b[2], b[3]);
+  } else {
+    o0 = *reinterpret_cast<const uint4*>(p + k);
+    o1 = *reinterpret_cast<const uint4*>(p + k + 16);
+  }
+}
+// Gather + unpack activation rows to int8, dst[n, k] = code(src[idx[n], k]) - zero_point: several
+// jobs in one launch (blockIdx.y selects the job).  The grid is sized for the SMs, not for the
+// padded row count: each thread strides over the 32-element pieces of the rows that carry work
+// (their number may be known on the device only).
+__global__ void __launch_bounds__(256) k_unpack_multi(const __grid_constant__ UnpackJobs jobs) {
   pdl_trigger();   // a dependent successor may set itself up; it reads nothing before this grid has completed
   pdl_wait();      // launched as a programmatic dependent itself: the source rows may be the predecessor's output
-  if (clear64 && blockIdx.x == 0 && threadIdx.x < 64) clear64[threadIdx.x] = 0;   // the call's status block
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int per_row = k_pad >> 5;  // 32 elements per thread
-  if (i >= (long long)n_rows_pad * per_row) return;
-  const int n = (int)(i / per_row), k = (int)(i % per_row) * 32;
-  uint4 o0 = make_uint4(0, 0, 0, 0), o1 = o0;
-  int r = -1;
-  if (n < n_rows) r = idx ? idx[n] : n;
-  if (r >= 0) {
-    const uint8_t* p = src + (long long)r * src_stride;
-    if (bits == 4) {
-      const uint4 v = *reinterpret_cast<const uint4*>(p + (k >> 1));
-      const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-      uint32_t o[8];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        // natural element order: byte b of the output word holds element 4*word + b
-        uint32_t lo = 0, hi = 0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          int a = (w[j] >> (4 * e)) & 0xF, c = (w[j] >> (4 * (e + 4))) & 0xF;
-          if (is_signed) {
-            a = (a ^ 8) - 8;
-            c = (c ^ 8) - 8;
-          } else {
-            a -= zp;
-            c -= zp;
-          }
-          lo |= (uint32_t)(a & 0xFF) << (8 * e);
-          hi |= (uint32_t)(c & 0xFF) << (8 * e);
-        }
-        o[2 * j] = lo;
-        o[2 * j + 1] = hi;
-      }
-      o0 = make_uint4(o[0], o[1], o[2], o[3]);
-      o1 = make_uint4(o[4], o[5], o[6], o[7]);
-    } else {
-      o0 = *reinterpret_cast<const uint4*>(p + k);
-      o1 = *reinterpret_cast<const uint4*>(p + k + 16);
-    }
-  }
-  uint4* d = reinterpret_cast<uint4*>(dst + (long long)n * dst_stride + col0 + k);
-  d[0] = o0;
-  d[1] = o1;
-}
-
-cudaError_t launch_unpack_rows(const void* src, long long src_stride, const int32_t* idx,
-                               const q4_act& act, int k_pad, int n_rows, int8_t* dst,
-                               long long dst_stride, int col0, int n_rows_pad, cudaStream_t s,
-                               int32_t* clear_status, bool dependent) {
-  const long long total = (long long)n_rows_pad * (k_pad >> 5);
-  if (total <= 0) return clear_status ? cudaMemsetAsync(clear_status, 0, 256, s) : cudaSuccess;
-  timing_begin(s);
-  cudaError_t le = launch_ex(k_unpack_rows, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, s, dependent, 1,
-                             static_cast<const uint8_t*>(src), src_stride, idx, (int)act.bits, (int)act.is_signed,
-                             (int)act.zero_point, k_pad, n_rows, dst, dst_stride, col0, n_rows_pad, clear_status);
-  timing_end(s);
-  ++g_launches;
-  return le != cudaSuccess ? le : cudaGetLastError();
-}
-
-// Several gather+unpack jobs in one launch (blockIdx.y selects the job).  The grid is sized for
-// the SMs, not for the padded row count: each thread strides over the 32-element pieces of the
-// rows that carry work (their number is known on the device only).
-__global__ void __launch_bounds__(256) k_unpack_multi(const UnpackJobs jobs) {
-  pdl_trigger();
-  pdl_wait();
+  if (jobs.clear64 && (blockIdx.x | blockIdx.y) == 0 && threadIdx.x < 64) jobs.clear64[threadIdx.x] = 0;   // the call's status block
   const UnpackJob& j = jobs.job[blockIdx.y];
-  const int per_row = j.k_pad >> 5;
+  const uint32_t per_row = (uint32_t)j.k_pad >> 5;
   int rows = jobs.n_rows_pad;
   if (!jobs.zero_tail) {   // rows without work need not be cleared every time
     rows = jobs.n_rows;
@@ -106,27 +61,13 @@ __global__ void __launch_bounds__(256) k_unpack_multi(const UnpackJobs jobs) {
   }
   const int n_work = jobs.n_active ? min(jobs.n_rows, *jobs.n_active) : jobs.n_rows;
   const uint32_t zp4 = (uint32_t)j.zp * 0x01010101u;
-  const long long total = (long long)rows * per_row;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total;
-       i += (long long)gridDim.x * blockDim.x) {
-    const int n = (int)(i / per_row), k = (int)(i % per_row) * 32;
+  const uint32_t total = (uint32_t)rows * per_row;   // checked by the launcher to fit
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const int n = (int)(i / per_row), k = (int)(i - (uint32_t)n * per_row) * 32;
     uint4 o0 = make_uint4(0, 0, 0, 0), o1 = o0;
     int r = -1;
     if (n < n_work) r = j.idx ? j.idx[n] : n;
-    if (r >= 0) {
-      const uint8_t* p = j.src + (long long)r * j.src_stride;
-      if (j.bits == 4) {
-        // eight codes per word -> two words of four int8 in natural element order
-        const uint4 v = *reinterpret_cast<const uint4*>(p + (k >> 1));
-        unpack8_natural(v.x, j.is_signed != 0, zp4, o0.x, o0.y);
-        unpack8_natural(v.y, j.is_signed != 0, zp4, o0.z, o0.w);
-        unpack8_natural(v.z, j.is_signed != 0, zp4, o1.x, o1.y);
-        unpack8_natural(v.w, j.is_signed != 0, zp4, o1.z, o1.w);
-      } else {
-        o0 = *reinterpret_cast<const uint4*>(p + k);
-        o1 = *reinterpret_cast<const uint4*>(p + k + 16);
-      }
-    }
+    if (r >= 0) unpack_piece32(j.src + (long long)r * j.src_stride, k, j.bits, j.is_signed != 0, zp4, o0, o1);
     uint4* d = reinterpret_cast<uint4*>(j.dst + (long long)n * j.dst_stride + k);
     d[0] = o0;
     d[1] = o1;
@@ -138,16 +79,31 @@ cudaError_t launch_unpack_multi(const UnpackJobs& jobs, cudaStream_t s, bool dep
   int kmax = 0;
   for (int i = 0; i < jobs.n_jobs; ++i) kmax = jobs.job[i].k_pad > kmax ? jobs.job[i].k_pad : kmax;
   const long long total = (long long)jobs.n_rows_pad * (kmax >> 5);
+  if (total > INT32_MAX) return cudaErrorInvalidValue;
   long long blocks = (total + 255) / 256;
   const long long cap = (6 * 148 + jobs.n_jobs - 1) / jobs.n_jobs;   // about six CTAs per SM in all: one or two
                                                                      // pieces per thread at 1024 rows
   if (blocks > cap) blocks = cap;
+  if (blocks < 1) blocks = 1;
   dim3 grid((unsigned)blocks, jobs.n_jobs);
   timing_begin(s);
   cudaError_t e = launch_ex(k_unpack_multi, grid, dim3(256), 0, s, dependent, 1, jobs);
   timing_end(s);
   ++g_launches;
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+void add_unpack_job(UnpackJobs& u, const void* src, long long src_stride, const int32_t* idx, const q4_act& act, int k_pad,
+                    int8_t* dst) {
+  UnpackJob& j = u.job[u.n_jobs++];
+  j.src = static_cast<const uint8_t*>(src);
+  j.src_stride = src_stride;
+  j.idx = idx;
+  j.bits = act.bits;
+  j.is_signed = act.is_signed;
+  j.zp = act.zero_point;
+  j.k_pad = k_pad;
+  j.dst = dst;
+  j.dst_stride = k_pad;
 }
 
 // Weight preparation: unpack to int8; with `interleave` the 4H rows (gate-major i,f,g,o) are
@@ -218,6 +174,53 @@ cudaError_t launch_prepare_vec(const float* src, int rows, int interleave, float
   return cudaGetLastError();
 }
 
+// Everything a layer call prepares, in one launch: int8 copies of the input codes and of all
+// directions' weights (rows reordered to 4*cell+gate), row scales and biases in the same order, and
+// a cleared status block.  (As separate launches: a memset and 11 kernels of 2 us each per bidirectional layer.)  blockIdx.x walks the jobs' blocks one after the other.
+__global__ void __launch_bounds__(256) k_layer_prepare(const __grid_constant__ LayerPrep a) {
+  pdl_trigger();
+  pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x < 64 && a.clear64) a.clear64[threadIdx.x] = 0;
+  int blk = blockIdx.x, ji = 0;
+  while (ji + 1 < a.n_mats && blk >= a.mat[ji].blocks) blk -= a.mat[ji++].blocks;
+  const LayerPrepMat& m = a.mat[ji];
+  if (blk < m.blocks) {   // a matrix of codes
+    const long long i = (long long)blk * 256 + threadIdx.x;
+    const int per_row = m.k_pad >> 5;
+    if (i >= m.rows * per_row) return;
+    const long long r = i / per_row;
+    const int k = (int)(i % per_row) * 32;
+    uint4 o0, o1;
+    unpack_piece32(m.src + r * ((long long)m.k_pad * m.bits / 8), k, m.bits, m.is_signed != 0, (uint32_t)m.zp * 0x01010101u,
+                   o0, o1);
+    const int H = m.interleave;
+    const long long ro = H > 0 ? 4 * (r % H) + r / H : r;
+    uint4* d = reinterpret_cast<uint4*>(m.dst + ro * m.k_pad + k);
+    d[0] = o0;
+    d[1] = o1;
+    return;
+  }
+  // the row vectors: one block per 256 rows of each
+  blk -= m.blocks;
+  const int per = (4 * a.H + 255) / 256, v = blk / per, r = (blk % per) * 256 + threadIdx.x;
+  if (v >= a.n_vecs || r >= 4 * a.H) return;
+  a.vec_dst[v][4 * (r % a.H) + r / a.H] = a.vec_src[v] ? a.vec_src[v][r] : 0.0f;
+}
+cudaError_t launch_layer_prepare(LayerPrep a, cudaStream_t s, bool dependent) {
+  long long total = 0;
+  for (int i = 0; i < a.n_mats; ++i) {
+    const long long b = (a.mat[i].rows * (a.mat[i].k_pad >> 5) + 255) / 256;
+    a.mat[i].blocks = (int)b;
+    total += b;
+  }
+  total += (long long)a.n_vecs * ((4 * a.H + 255) / 256);
+  timing_begin(s);
+  const cudaError_t e = launch_ex(k_layer_prepare, dim3((unsigned)total), dim3(256), 0, s, dependent, 1, a);
+  timing_end(s);
+  ++g_launches;
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 // ------------------------------------------------------------------ tensor maps (host)
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
@@ -282,13 +285,15 @@ void test_wait_expiry_set(int skip_producer, uint32_t wait_limit) {
   g_wait_limit = wait_limit ? wait_limit : (1u << 22);
 }
 
+template <int GEMM_BN>
 __global__ void __launch_bounds__(192, 1)
 k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b,
            const MmaGemmArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   constexpr int A_BYTES = BM * BK, B_BYTES = GEMM_BN * BK, STAGE = A_BYTES + B_BYTES;
-  __shared__ uint64_t full[GEMM_STAGES], empty[GEMM_STAGES], acc_full;
+  constexpr int NS = GEMM_STAGES<GEMM_BN>;
+  __shared__ uint64_t full[NS], empty[NS], acc_full;
   __shared__ uint32_t tmem_base_s;
   __shared__ float s_sc[GEMM_BN], s_bi[GEMM_BN];   // de-quantization constants of this tile's columns
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -296,7 +301,7 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
   const int nk = (a.K + BK - 1) / BK;
 
   if (tid == 0) {
-    for (int s = 0; s < GEMM_STAGES; ++s) {
+    for (int s = 0; s < NS; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -321,8 +326,8 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
   } else if (warp == 4 && lane == 0) {
     bool ok = true;
     for (int i = 0; i < nk && ok && !a.skip_producer; ++i) {
-      const int s = i % GEMM_STAGES;
-      if (i >= GEMM_STAGES) ok = mbar_wait(&empty[s], ((i / GEMM_STAGES) - 1) & 1, a.wait_limit);
+      const int s = i % NS;
+      if (i >= NS) ok = mbar_wait(&empty[s], ((i / NS) - 1) & 1, a.wait_limit);
       if (!ok) break;
       mbar_expect_tx(&full[s], STAGE);
       tma_load_2d(smem + s * STAGE, &tma_a, i * BK, m0, &full[s]);
@@ -334,8 +339,8 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
     const uint32_t idesc = umma_idesc_i8(BM, GEMM_BN);
     bool ok = true;
     for (int i = 0; i < nk && ok; ++i) {
-      const int s = i % GEMM_STAGES;
-      ok = mbar_wait(&full[s], (i / GEMM_STAGES) & 1, a.wait_limit);
+      const int s = i % NS;
+      ok = mbar_wait(&full[s], (i / NS) & 1, a.wait_limit);
       if (!ok) break;
       tc_fence_after();
       const uint64_t da = umma_desc_sw128(smem_u32(smem + s * STAGE));
@@ -351,14 +356,12 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
     umma_commit(&acc_full);
     pdl_trigger();
   } else if (warp < 4) {
-    if (a.epi != EPI_I32) {   // stage scale * row scale and bias while the MMAs run
-      for (int c = tid; c < GEMM_BN; c += 128) {
-        const int j = min(n0 + c, a.J - 1);
-        s_sc[c] = __fmul_rn(a.x_scale, __ldg(a.w_scale + j));
-        s_bi[c] = a.bias ? __ldg(a.bias + j) : 0.0f;
-      }
-      asm volatile("bar.sync 1, 128;" ::: "memory");
+    for (int c = tid; c < GEMM_BN; c += 128) {   // stage scale * row scale and bias while the MMAs run
+      const int j = min(n0 + c, a.J - 1);
+      s_sc[c] = __fmul_rn(a.x_scale, __ldg(a.w_scale + j));
+      s_bi[c] = a.bias ? __ldg(a.bias + j) : 0.0f;
     }
+    asm volatile("bar.sync 1, 128;" ::: "memory");
     bool ok = mbar_wait(&acc_full, 0, a.wait_limit);
     if (ok && a.status && *reinterpret_cast<volatile int32_t*>(a.status) != 0) ok = false;   // a wait gave up somewhere
     tc_fence_after();
@@ -374,69 +377,46 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
       tmem_ld_wait();
       const int j0 = n0 + c0;
       if (!ok || m < 0 || j0 >= a.J) continue;
-      if (a.epi == EPI_I32) {
-        int32_t* o = reinterpret_cast<int32_t*>(a.out) + (long long)m * a.ldo + j0;
-        if (j0 + 32 <= a.J) {
+      float v[32];
 #pragma unroll
-          for (int i = 0; i < 32; i += 4) *reinterpret_cast<int4*>(o + i) = make_int4(r[i], r[i + 1], r[i + 2], r[i + 3]);
-        } else {
-          for (int i = 0; i < 32 && j0 + i < a.J; ++i) o[i] = r[i];
+      for (int i = 0; i < 32; ++i) v[i] = __fmaf_rn((float)r[i], s_sc[c0 + i], s_bi[c0 + i]);
+      if (a.epi == EPI_JOINTZ) {
+        // joint network: z = tanh(e * p) with p the projected value just formed; quantized below
+        const float* er = a.mul_e + (long long)a.mul_idx[mi] * a.J + j0;
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) {
+          const float4 ev = *reinterpret_cast<const float4*>(er + i);
+          v[i] = tanh_fixed(__fmul_rn(ev.x, v[i]));
+          v[i + 1] = tanh_fixed(__fmul_rn(ev.y, v[i + 1]));
+          v[i + 2] = tanh_fixed(__fmul_rn(ev.z, v[i + 2]));
+          v[i + 3] = tanh_fixed(__fmul_rn(ev.w, v[i + 3]));
         }
-      } else {
-        float v[32];
+      }
+      if (a.epi == EPI_F32) {
+        float* o = reinterpret_cast<float*>(a.out) + (long long)m * a.ldo + j0;
+        if (j0 + 32 <= a.J && (reinterpret_cast<uintptr_t>(o) & 31) == 0) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = __fmaf_rn((float)r[i], s_sc[c0 + i], s_bi[c0 + i]);
-        if (a.epi == EPI_JOINTZ) {
-          // joint network: z = tanh(e * p) with p the projected value just formed; quantized below
-          const float* er = a.mul_e + (long long)a.mul_idx[mi] * a.J + j0;
+          for (int i = 0; i < 32; i += 8)
+            st_global_v8(o + i, make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]),
+                         make_float4(v[i + 4], v[i + 5], v[i + 6], v[i + 7]));
+        } else if (j0 + 32 <= a.J && (reinterpret_cast<uintptr_t>(o) & 15) == 0) {
 #pragma unroll
-          for (int i = 0; i < 32; i += 4) {
-            const float4 ev = *reinterpret_cast<const float4*>(er + i);
-            v[i] = tanh_fixed(__fmul_rn(ev.x, v[i]));
-            v[i + 1] = tanh_fixed(__fmul_rn(ev.y, v[i + 1]));
-            v[i + 2] = tanh_fixed(__fmul_rn(ev.z, v[i + 2]));
-            v[i + 3] = tanh_fixed(__fmul_rn(ev.w, v[i + 3]));
-          }
+          for (int i = 0; i < 32; i += 4) *reinterpret_cast<float4*>(o + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+        } else {   // ragged columns, or rows that are no multiple of 16 bytes apart
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            if (j0 + i < a.J) o[i] = v[i];
         }
-        if (a.epi == EPI_F32) {
-          float* o = reinterpret_cast<float*>(a.out) + (long long)m * a.ldo + j0;
-          if (j0 + 32 <= a.J && (reinterpret_cast<uintptr_t>(o) & 31) == 0) {
+      } else {  // EPI_QUANT8 / EPI_JOINTZ (J a multiple of 32)
+        const int lo = act_lo(a.out_act), hi = act_hi(a.out_act);
+        uint8_t* o = reinterpret_cast<uint8_t*>(a.out) + (long long)m * a.ldo;
+        uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
 #pragma unroll
-            for (int i = 0; i < 32; i += 8)
-              st_global_v8(o + i, make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]),
-                           make_float4(v[i + 4], v[i + 5], v[i + 6], v[i + 7]));
-          } else if (j0 + 32 <= a.J) {
-#pragma unroll
-            for (int i = 0; i < 32; i += 4) *reinterpret_cast<float4*>(o + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-          } else {
-            for (int i = 0; i < 32 && j0 + i < a.J; ++i) o[i] = v[i];
-          }
-        } else {  // EPI_QUANT / EPI_QUANT8 (J a multiple of 32)
-          const int lo = act_lo(a.out_act), hi = act_hi(a.out_act);
-          uint8_t* o = reinterpret_cast<uint8_t*>(a.out) + (long long)m * a.ldo;
-          if (a.epi == EPI_QUANT8 || a.epi == EPI_JOINTZ) {
-            uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-              w[i >> 2] |= (uint32_t)((quantize1(v[i], a.out_act.inv_scale, a.out_act.zero_point, lo, hi) -
-                                       a.out_act.zero_point) & 0xFF) << (8 * (i & 3));
-            *reinterpret_cast<uint4*>(o + j0) = make_uint4(w[0], w[1], w[2], w[3]);
-            *reinterpret_cast<uint4*>(o + j0 + 16) = make_uint4(w[4], w[5], w[6], w[7]);
-          } else if (a.out_act.bits == 4) {
-            uint32_t w[4] = {0, 0, 0, 0};
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-              w[i >> 3] |= (uint32_t)(quantize1(v[i], a.out_act.inv_scale, a.out_act.zero_point, lo, hi) & 0xF) << (4 * (i & 7));
-            *reinterpret_cast<uint4*>(o + (j0 >> 1)) = make_uint4(w[0], w[1], w[2], w[3]);
-          } else {
-            uint32_t w[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-              w[i >> 2] |= (uint32_t)(quantize1(v[i], a.out_act.inv_scale, a.out_act.zero_point, lo, hi) & 0xFF) << (8 * (i & 3));
-            *reinterpret_cast<uint4*>(o + j0) = make_uint4(w[0], w[1], w[2], w[3]);
-            *reinterpret_cast<uint4*>(o + j0 + 16) = make_uint4(w[4], w[5], w[6], w[7]);
-          }
-        }
+        for (int i = 0; i < 32; ++i)
+          w[i >> 2] |= (uint32_t)((quantize1(v[i], a.out_act.inv_scale, a.out_act.zero_point, lo, hi) -
+                                   a.out_act.zero_point) & 0xFF) << (8 * (i & 3));
+        *reinterpret_cast<uint4*>(o + j0) = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(o + j0 + 16) = make_uint4(w[4], w[5], w[6], w[7]);
       }
     }
   } else {
@@ -454,11 +434,17 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
 // CTAs working at the same time share activation rows and all weights in L2), with two
 // accumulators in tensor memory: the epilogue warps drain one while the MMAs of the next tile
 // fill the other, and the operand ring keeps streaming across tile boundaries.
-constexpr int PG_STAGES = 4;
-
+//
+// The directions of a bidirectional layer are planes of one launch: plane p multiplies weight rows
+// [p J, (p + 1) J) of the weight map and stores at out + p * plane_out; the column tiles of all planes
+// are walked together (tiles_n per plane).
+template <int GEMM_BN>
 __global__ void __launch_bounds__(192, 1)
 k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CUtensorMap tma_b,
-                      const MmaGemmArgs a, const int tiles_m, const int tiles_n) {
+                      const MmaGemmArgs a, const int tiles_m, const int tiles_n, const int planes,
+                      const long long plane_out) {
+  constexpr int PG_STAGES = GEMM_STAGES<GEMM_BN>;
+  constexpr int TCOLS = 2 * GEMM_BN;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   constexpr int A_BYTES = BM * BK, B_BYTES = GEMM_BN * BK, STAGE = A_BYTES + B_BYTES;
@@ -466,7 +452,7 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
   __shared__ uint32_t tmem_base_s;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nk = (a.K + BK - 1) / BK;
-  const int n_tiles = tiles_m * tiles_n;
+  const int cols = tiles_n * planes, n_tiles = tiles_m * cols;
 
   if (tid == 0) {
     for (int s = 0; s < PG_STAGES; ++s) {
@@ -480,7 +466,7 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
     fence_barrier_init();
     fence_proxy_async();
   }
-  if (warp == 5) tmem_alloc(&tmem_base_s, 2 * GEMM_BN);
+  if (warp == 5) tmem_alloc(&tmem_base_s, TCOLS);
   if (warp == 4 && lane == 0) {
     prefetch_tmap(&tma_a);
     prefetch_tmap(&tma_b);
@@ -497,13 +483,14 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
     int s = 0, g = 0;
     uint32_t ph = 0;
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-      const int m0 = (t / tiles_n) * BM, n0 = (t % tiles_n) * GEMM_BN;
+      const int m0 = (t / cols) * BM, ct = t % cols;
+      const int w0 = (ct / tiles_n) * a.J + (ct % tiles_n) * GEMM_BN;   // first weight row of the tile
       for (int i = 0; i < nk; ++i, ++g) {
         if (g >= PG_STAGES) ok = mbar_wait(&empty[s], ph ^ 1);
         if (!ok) break;
         mbar_expect_tx(&full[s], STAGE);
         tma_load_2d(smem + s * STAGE, &tma_a, i * BK, m0, &full[s]);
-        tma_load_2d(smem + s * STAGE + A_BYTES, &tma_b, i * BK, n0, &full[s]);
+        tma_load_2d(smem + s * STAGE + A_BYTES, &tma_b, i * BK, w0, &full[s]);
         if (++s == PG_STAGES) {
           s = 0;
           ph ^= 1;
@@ -548,10 +535,11 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
     // ---- epilogue: warp w drains TMEM lanes [32 w, 32 w + 32) of the finished accumulator
     bool ok = true;
     int it = 0;
-    const bool wide = (reinterpret_cast<uintptr_t>(a.out) & 31) == 0 && ((a.ldo * 4) & 31) == 0;
+    const bool wide = ((reinterpret_cast<uintptr_t>(a.out) | (uintptr_t)(plane_out * 4) | (uintptr_t)(a.ldo * 4)) & 31) == 0;
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++it) {
       const int buf = it & 1, use = it >> 1;
-      const int m0 = (t / tiles_n) * BM, n0 = (t % tiles_n) * GEMM_BN;
+      const int m0 = (t / cols) * BM, ct = t % cols, n0 = (ct % tiles_n) * GEMM_BN;
+      int32_t* const plane = reinterpret_cast<int32_t*>(a.out) + (ct / tiles_n) * plane_out;
       ok = mbar_wait(&acc_full[buf], use & 1);
       if (!ok) break;
       tc_fence_after();
@@ -561,7 +549,7 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
       auto store32 = [&](const int (&r)[32], int c0) {
         const int j0 = n0 + c0;
         if (m >= a.M || j0 >= a.J) return;
-        int32_t* o = reinterpret_cast<int32_t*>(a.out) + (long long)m * a.ldo + j0;
+        int32_t* o = plane + (long long)m * a.ldo + j0;
         if (j0 + 32 <= a.J && wide) {
 #pragma unroll
           for (int i = 0; i < 32; i += 8)
@@ -601,7 +589,7 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 5) tmem_dealloc(tmem, 2 * GEMM_BN);
+  if (warp == 5) tmem_dealloc(tmem, TCOLS);
 }
 
 static int g_sm_count() {
@@ -615,6 +603,50 @@ static int g_sm_count() {
   return n;
 }
 
+template <int BN>
+static size_t gemm_smem() {
+  return (size_t)GEMM_STAGES<BN> * (BM * BK + BN * BK) + 1024;
+}
+template <int BN>
+static cudaError_t gemm_launch(const CUtensorMap& ta, const CUtensorMap& tb, const MmaGemmArgs& a, cudaStream_t s,
+                               bool dependent) {
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e = cudaFuncSetAttribute(k_mma_gemm<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem<BN>());
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  return launch_ex(k_mma_gemm<BN>, dim3((a.J + BN - 1) / BN, (a.M + BM - 1) / BM), dim3(192), gemm_smem<BN>(), s, dependent,
+                   1, ta, tb, a);
+}
+template <int BN>
+static cudaError_t gemm_persistent_launch(const CUtensorMap& ta, const CUtensorMap& tb, const MmaGemmArgs& a, int planes,
+                                          long long plane_out, cudaStream_t s, bool dependent) {
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e = cudaFuncSetAttribute(k_mma_gemm_persistent<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)gemm_smem<BN>());
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  const int tiles_m = (a.M + BM - 1) / BM, tiles_n = (a.J + BN - 1) / BN;
+  const long long tiles = (long long)tiles_m * tiles_n * planes;
+  const int ctas = tiles < g_sm_count() ? (int)tiles : g_sm_count();
+  return launch_ex(k_mma_gemm_persistent<BN>, dim3(ctas), dim3(192), gemm_smem<BN>(), s, dependent, 1, ta, tb, a, tiles_m,
+                   tiles_n, planes, plane_out);
+}
+// Weight rows per tile: the widest tile (fewest operand bytes per product) that still gives every SM
+// one.  A tile that is alone on its SM is bound by the latency of its own chain (K chunks, then
+// an epilogue proportional to its width), so narrower tiles on more SMs end sooner: the projection of 152
+// rows of 1280 codes to 256 outputs takes 14.4 us as two 256-wide tiles and 8.4 us as 16 of width 32, the
+// input projection of a bidirectional 640-cell layer over 152 rows 2 x 16.7 us as 20 tiles of width 256 per
+// direction and 9.5 us as 160 of width 64 in one launch (1903 rows: 2 x 28.9 -> 20.6 us, width 256 in both).
+static int gemm_tile_width(int M, int J, int planes, int narrowest) {
+  for (int bn = 256; bn > narrowest; bn >>= 1)
+    if ((long long)((M + BM - 1) / BM) * ((J + bn - 1) / bn) * planes >= g_sm_count()) return bn;
+  return narrowest;
+}
+
 // x8: int8 activations [M, K] (pitch x_pitch), w8: int8 weights [J, K] (pitch w_pitch).
 cudaError_t launch_mma_gemm(const int8_t* x8, long long x_pitch, int M, const int8_t* w8,
                             long long w_pitch, int J, int K, int epi, void* out, long long ldo,
@@ -624,8 +656,9 @@ cudaError_t launch_mma_gemm(const int8_t* x8, long long x_pitch, int M, const in
                             const int32_t* mul_idx) {
   if (M <= 0 || J <= 0) return cudaSuccess;
   if (epi == EPI_JOINTZ && (!mul_e || !mul_idx || J % 32 != 0)) return cudaErrorInvalidValue;
+  const int bn = gemm_tile_width(M, J, 1, 32);
   CUtensorMap ta, tb;
-  if (!make_tmap_i8(&ta, x8, K, M, x_pitch, BM) || !make_tmap_i8(&tb, w8, K, J, w_pitch, GEMM_BN))
+  if (!make_tmap_i8(&ta, x8, K, M, x_pitch, BM) || !make_tmap_i8(&tb, w8, K, J, w_pitch, bn))
     return cudaErrorInvalidValue;
   MmaGemmArgs a;
   memset(&a, 0, sizeof(a));
@@ -646,28 +679,39 @@ cudaError_t launch_mma_gemm(const int8_t* x8, long long x_pitch, int M, const in
   a.mul_idx = mul_idx;
   a.wait_limit = g_wait_limit;
   a.skip_producer = g_skip_producer;
-  const size_t smem = (size_t)GEMM_STAGES * (BM * BK + GEMM_BN * BK) + 1024;
-  const size_t smem_p = (size_t)PG_STAGES * (BM * BK + GEMM_BN * BK) + 1024;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_mma_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_mma_gemm_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_p);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
-  dim3 grid((J + GEMM_BN - 1) / GEMM_BN, (M + BM - 1) / BM);
-  if (epi == EPI_I32 && !out_idx && !n_active && (long long)grid.x * grid.y > 2 * g_sm_count()) {
-    // more than two tiles per SM: one persistent CTA per SM with overlapped epilogue
-    timing_begin(s);
-    cudaError_t le = launch_ex(k_mma_gemm_persistent, dim3(g_sm_count()), dim3(192), smem_p, s, dependent, 1, ta, tb,
-                               a, (int)grid.y, (int)grid.x);
-    timing_end(s);
-    ++g_launches;
-    return le != cudaSuccess ? le : cudaGetLastError();
-  }
   timing_begin(s);
-  cudaError_t le = launch_ex(k_mma_gemm, grid, dim3(192), smem, s, dependent, 1, ta, tb, a);
+  const cudaError_t le = bn == 256   ? gemm_launch<256>(ta, tb, a, s, dependent)
+                         : bn == 128 ? gemm_launch<128>(ta, tb, a, s, dependent)
+                         : bn == 64  ? gemm_launch<64>(ta, tb, a, s, dependent)
+                                     : gemm_launch<32>(ta, tb, a, s, dependent);
+  timing_end(s);
+  ++g_launches;
+  return le != cudaSuccess ? le : cudaGetLastError();
+}
+
+// Input projections of all directions of a layer: x8 int8 [M, K], w8 int8 [planes J, K], out int32
+// [planes][M, J]; persistent CTAs whose epilogue overlaps the next tile's MMAs.
+cudaError_t launch_mma_gemm_i32(const int8_t* x8, int M, const int8_t* w8, int J, int K, int planes, int32_t* out,
+                                int32_t* status, cudaStream_t s, bool dependent) {
+  if (M <= 0 || J <= 0) return cudaSuccess;
+  const int bn = gemm_tile_width(M, J, planes, 64);
+  CUtensorMap ta, tb;
+  if (!make_tmap_i8(&ta, x8, K, M, K, BM) || !make_tmap_i8(&tb, w8, K, (uint64_t)J * planes, K, bn))
+    return cudaErrorInvalidValue;
+  MmaGemmArgs a;
+  memset(&a, 0, sizeof(a));
+  a.M = M;
+  a.J = J;
+  a.K = K;
+  a.epi = EPI_I32;
+  a.out = out;
+  a.ldo = J;
+  a.status = status;
+  const long long plane_out = (long long)M * J;
+  timing_begin(s);
+  const cudaError_t le = bn == 256   ? gemm_persistent_launch<256>(ta, tb, a, planes, plane_out, s, dependent)
+                         : bn == 128 ? gemm_persistent_launch<128>(ta, tb, a, planes, plane_out, s, dependent)
+                                     : gemm_persistent_launch<64>(ta, tb, a, planes, plane_out, s, dependent);
   timing_end(s);
   ++g_launches;
   return le != cudaSuccess ? le : cudaGetLastError();

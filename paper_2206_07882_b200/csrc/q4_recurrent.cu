@@ -95,6 +95,7 @@ k_enc_recurrent(const EncRecArgs a) {
   }
   __syncthreads();
   cluster_barrier();   // every CTA's buffers are initialised before anyone stores into them
+  pdl_wait();          // the input accumulators are the previous kernel's output; the weights that of the one before it
 
   const int g = lane >> 2, t4 = lane & 3;   // MMA fragment coordinates
   const int ci = lane >> 3, n = lane & 7;   // this lane's item: cell ci of the warp's 4, sequence n
@@ -237,6 +238,7 @@ k_enc_recurrent(const EncRecArgs a) {
     }
     cluster_barrier();
   }
+  pdl_trigger();
   // final states
 #pragma unroll
   for (int j = 0; j < NT; ++j) {
@@ -403,6 +405,7 @@ k_enc_recurrent_w4(const EncRecArgs a) {
   fence_proxy_async();   // the zeroed buffers are later written by the bulk-copy engine
   __syncthreads();
   cluster_barrier();   // every CTA's buffers and barriers are initialised before anyone stores into them
+  pdl_wait();          // the input accumulators are the previous kernel's output; the weights that of the one before it
 
   float c_state[NU];
   bool live[NU];
@@ -572,6 +575,7 @@ k_enc_recurrent_w4(const EncRecArgs a) {
       }
     }
   }
+  pdl_trigger();
   cp_async_wait<0>();
   // the codes sent in the last step are still on their way into this CTA: wait for them (bounded), so
   // that nobody leaves while copies into its shared memory are in flight
@@ -707,6 +711,7 @@ k_enc_recurrent_w4s(const EncRecArgs a) {
   fence_proxy_async();   // the zeroed buffers are later written by the bulk-copy engine
   __syncthreads();
   cluster_barrier();   // every CTA's buffers and barriers are initialised before anyone stores into them
+  pdl_wait();          // the input accumulators are the previous kernel's output; the weights that of the one before it
 
   const int b_own = j * BG + n, b_shared = (a.groups - 1) * BG + n;
   const bool live_own = b_own < B, live_shared = host && b_shared < B;
@@ -935,6 +940,7 @@ k_enc_recurrent_w4s(const EncRecArgs a) {
       if (tid == 0) atomicAdd(flag_out, 1);
     }
   }
+  pdl_trigger();
   cp_async_wait<0>();
   // the own group's codes sent in its last step are still on their way into this CTA: wait for them
   // (bounded), so that nobody leaves while copies into its shared memory are in flight.  (The shared
@@ -967,8 +973,9 @@ static cudaError_t rec_launch(const EncRecArgs& a, size_t smem, cudaStream_t s) 
     if (e != cudaSuccess) return e;
     configured = smem;
   }
-  k_enc_recurrent<BG><<<(unsigned)(a.dirs * a.n_groups * REC_CLUSTER), REC_THREADS, smem, s>>>(a);
-  return cudaGetLastError();
+  const cudaError_t e = launch_ex(k_enc_recurrent<BG>, dim3((unsigned)(a.dirs * a.n_groups * REC_CLUSTER)), dim3(REC_THREADS),
+                                  smem, s, true, 1, a);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // How many 8-CTA clusters of this kernel can be resident at once on the current device
@@ -1078,8 +1085,9 @@ static cudaError_t rec_w4s_launch(const EncRecArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  k_enc_recurrent_w4s<KS, W8><<<(unsigned)((a.ncl[0] + a.ncl[1]) * REC_CLUSTER), REC4_THREADS, smem, s>>>(a);
-  return cudaGetLastError();
+  const cudaError_t e = launch_ex(k_enc_recurrent_w4s<KS, W8>, dim3((unsigned)((a.ncl[0] + a.ncl[1]) * REC_CLUSTER)),
+                                  dim3(REC4_THREADS), smem, s, true, 1, a);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <int NU, int KS>
@@ -1091,8 +1099,9 @@ static cudaError_t rec_w4_launch(const EncRecArgs& a, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  k_enc_recurrent_w4<NU, KS><<<(unsigned)(a.dirs * a.n_groups * REC_CLUSTER), REC4_THREADS, smem, s>>>(a);
-  return cudaGetLastError();
+  const cudaError_t e = launch_ex(k_enc_recurrent_w4<NU, KS>, dim3((unsigned)(a.dirs * a.n_groups * REC_CLUSTER)),
+                                  dim3(REC4_THREADS), smem, s, true, 1, a);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid_bits, bool hid_signed,

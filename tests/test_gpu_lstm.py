@@ -415,6 +415,23 @@ def test_step_on_the_tensor_cores_with_prepared_weights(Bd, N, K, H, xb, hb, sig
     assert Bd.launch_count() - n0 >= 3
 
 
+# every tile width of the tensor-core GEMM (32 to 256 weight rows, chosen by how many tiles there are), ragged
+# rows and columns, against exact integer sums
+@pytest.mark.parametrize("M,J,K", [(128, 32, 64), (129, 256, 1024), (300, 1000, 96), (1900, 700, 32), (1300, 2560, 160),
+                                   (9500, 510, 64)])
+def test_linear_on_the_tensor_cores_tile_widths(Bd, M, J, K):
+    w = synth._linear(synth.Stream(8), "lin", J, K)
+    lin = Bd.DeviceLinear(w).prepare()
+    act = O.act_asymmetric(-1.5, 2.0, 4)
+    xq = O.quantize(synth.Stream(9).normal("x", (M, K)).astype(np.float32), act)
+    got = Bd.q4_linear_forward(pack_codes(xq, act), to_act(act), lin)
+    assert Bd.q4_poll_status(lin.ws[:4].view(torch.int32)) == 0
+    acc = (xq.astype(np.float64) - act.zero_point) @ w.w.codes.astype(np.float64).T      # exact below 2^53
+    sc = (np.float32(act.scale) * w.w.scale).astype(np.float32)                          # one fp32 product ...
+    want = (acc * sc.astype(np.float64)[None, :] + w.bias.astype(np.float64)[None, :]).astype(np.float32)   # ... one rounding
+    np.testing.assert_array_equal(got.cpu().numpy(), want)
+
+
 def test_bounded_wait_runs_out_and_the_stream_stays_usable(Bd):
     # The consumer of the tiled tensor-core GEMM waits for operand tiles a bounded number of polls.  With
     # the test hook the producer issues nothing (so nothing asynchronous is in flight): the wait runs
