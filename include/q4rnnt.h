@@ -173,8 +173,8 @@ int q4_linear_forward(const void* xq, const q4_act* x_act, int32_t M, const q4_m
  * with z_act, passed through the output layer (w_out [V, D], b_out) and a log-softmax.
  * logp [N, V] fp32.  workspace: q4_workspace_bytes(Q4_WS_JOINT, {N, D}).
  * prepared_pred / prepared_out (nullable): buffers of q4_prepare_linear for w_pred and w_out; with
- * both, a workspace of q4_workspace_bytes(Q4_WS_JOINT, {N, D, Hp_pad}) bytes, N >= 128 and V a
- * multiple of 32 the call runs on the tensor cores in three launches (the projection's epilogue forms
+ * both, a workspace of q4_workspace_bytes(Q4_WS_JOINT, {N, D, Hp_pad}) bytes and N >= 128
+ * the call runs on the tensor cores in three launches (the projection's epilogue forms
  * tanh(e * p) and quantizes it; the output layer's epilogue takes the log-softmax).
  */
 int qjoint_logprobs(const float* e, const int32_t* frame_idx, const void* pq, const q4_act* p_act,
@@ -340,7 +340,7 @@ int q4_beam_init(q4_beam_state* state, int32_t B, int32_t W, int32_t n_iters, q4
  * T (S + 1) iterations.  History of a mode-2 call: bp_parent = slot that first proposed the entry,
  * bp_token = -1 - (call number within the frame of that proposal).
  * workspace: q4_workspace_bytes(Q4_WS_BEAM, {B, W, V, D}), or, to enable the tensor-core path
- * (needs model->prepared, LSTM widths that are multiples of 128 and V a multiple of 32),
+ * (needs model->prepared and LSTM widths that are multiples of 128),
  * q4_workspace_bytes(Q4_WS_BEAM, {B, W, V, D, E_pad, Hp, Hs, Ht}).  A bounded device wait that expires sets state->status to Q4_ERR_TIMEOUT.
  */
 int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float* e, int32_t B,

@@ -619,7 +619,7 @@ int qjoint_logprobs(const float* e, const int32_t* frame_idx, const void* pq, co
   TagScope tag(TAG_JOINT);
   ++g_quant_calls;   // tanh(e * p)
   const int32_t dims3[3] = {N, D, w_pred->k_pad};
-  if (prepared_pred && prepared_out && N >= 128 && V % 32 == 0 && z_act->is_signed && aligned16(prepared_pred) &&
+  if (prepared_pred && prepared_out && N >= 128 && z_act->is_signed && aligned16(prepared_pred) &&
       aligned16(prepared_out) && workspace_bytes >= q4_workspace_bytes(Q4_WS_JOINT, dims3, 3)) {
     // tensor cores, three launches: int8 copy of the hidden codes; projection GEMM whose epilogue forms
     // tanh(e * p) and quantizes it; output layer with the log-softmax in its epilogue (fused head kernel
@@ -956,7 +956,7 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
   const int32_t dims8[8] = {B, W, V, D, Ep, Hp, Hs, Ht};
   const bool use_mma = m.prepared != nullptr && m.src.n_layers == 1 &&
                        m.src.lstm[0].w_ih.k_pad == Ep && m.tgt.lstm[0].w_ih.k_pad == Ep &&
-                       Hp % 128 == 0 && Hs % 128 == 0 && Ht % 128 == 0 && V % 32 == 0 &&
+                       Hp % 128 == 0 && Hs % 128 == 0 && Ht % 128 == 0 &&
                        workspace_bytes >= q4_workspace_bytes(Q4_WS_BEAM, dims8, 8);
   if (use_mma) {
     const size_t Np = ((size_t)N + 127) / 128 * 128;

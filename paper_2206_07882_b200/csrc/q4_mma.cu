@@ -998,7 +998,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
         for (int i = 0; i < CPT; i += 8)   // rows of a warp's lanes are V floats apart: few, wide stores
           st_global_v8(out + i, make_float4(v[i] - lse, v[i + 1] - lse, v[i + 2] - lse, v[i + 3] - lse),
                        make_float4(v[i + 4] - lse, v[i + 5] - lse, v[i + 6] - lse, v[i + 7] - lse));
-      } else if (left >= CPT) {
+      } else if (left >= CPT && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
 #pragma unroll
         for (int i = 0; i < CPT; i += 4)
           *reinterpret_cast<float4*>(out + i) = make_float4(v[i] - lse, v[i + 1] - lse, v[i + 2] - lse, v[i + 3] - lse);

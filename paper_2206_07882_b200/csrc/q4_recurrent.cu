@@ -1122,7 +1122,7 @@ EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid
     const int lack = dirs * groups - p.max_clusters;
     const bool plain_only = w_bits == 8 || hid_bits == 8 || per_sequence_scale;
     const bool turns = g_rec_sliced && lack >= 1 && lack <= dirs && groups >= 2 && groups <= 8 && T >= 8 * groups && scratch;
-    if (turns || (lack <= 0 && plain_only && groups <= 8 && scratch)) {
+    if (turns || (lack <= 0 && plain_only && groups <= 8)) {   // the hand-over scratch is needed for turns only
       p.kernel = 2;
       p.groups_per_cluster = 1;
       for (int d = 0; d < 2; ++d) {
