@@ -296,7 +296,7 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
   __shared__ uint64_t full[NS], empty[NS], acc_full;
   __shared__ uint32_t tmem_base_s;
   __shared__ float s_sc[GEMM_BN], s_bi[GEMM_BN];   // de-quantization constants of this tile's columns
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * GEMM_BN;   // row tiles slowest: tiles with work are dispatched first
   const int nk = (a.K + BK - 1) / BK;
 
@@ -323,37 +323,52 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
 
   if (!has_work) {
     // whole tile without work
-  } else if (warp == 4 && lane == 0) {
+  } else if (warp == 4) {
     bool ok = true;
+    int s = 0;
+    uint32_t ph = 1;
     for (int i = 0; i < nk && ok && !a.skip_producer; ++i) {
-      const int s = i % NS;
-      if (i >= NS) ok = mbar_wait(&empty[s], ((i / NS) - 1) & 1, a.wait_limit);
+      ok = mbar_wait_warp(&empty[s], ph, a.wait_limit);   // passes at once for a stage that has never been filled
       if (!ok) break;
-      mbar_expect_tx(&full[s], STAGE);
-      tma_load_2d(smem + s * STAGE, &tma_a, i * BK, m0, &full[s]);
-      tma_load_2d(smem + s * STAGE + A_BYTES, &tma_b, i * BK, n0, &full[s]);
+      if (elect_one()) {
+        mbar_expect_tx(&full[s], STAGE);
+        tma_load_2d(smem + s * STAGE, &tma_a, i * BK, m0, &full[s]);
+        tma_load_2d(smem + s * STAGE + A_BYTES, &tma_b, i * BK, n0, &full[s]);
+      }
+      if (++s == NS) {
+        s = 0;
+        ph ^= 1;
+      }
     }
     pdl_trigger();
-    if (!ok) flag_timeout(a.status);
-  } else if (warp == 5 && lane == 0) {
+    if (!ok && lane == 0) flag_timeout(a.status);
+  } else if (warp == 5) {
     const uint32_t idesc = umma_idesc_i8(BM, GEMM_BN);
     bool ok = true;
+    int s = 0;
+    uint32_t ph = 0;
     for (int i = 0; i < nk && ok; ++i) {
-      const int s = i % NS;
-      ok = mbar_wait(&full[s], (i / NS) & 1, a.wait_limit);
+      ok = mbar_wait_warp(&full[s], ph, a.wait_limit);
       if (!ok) break;
       tc_fence_after();
       const uint64_t da = umma_desc_sw128(smem_u32(smem + s * STAGE));
       const uint64_t db = umma_desc_sw128(smem_u32(smem + s * STAGE + A_BYTES));
+      if (elect_one()) {
 #pragma unroll
-      for (int kk = 0; kk < BK / 32; ++kk) umma_i8(tmem, da + 2 * kk, db + 2 * kk, idesc, (i | kk) != 0);
-      umma_commit(&empty[s]);
+        for (int kk = 0; kk < BK / 32; ++kk) umma_i8(tmem, da + 2 * kk, db + 2 * kk, idesc, (i | kk) != 0);
+        umma_commit(&empty[s]);
+      }
+      if (++s == NS) {
+        s = 0;
+        ph ^= 1;
+      }
     }
     if (!ok) {   // recorded before the epilogue is released, so that it stores nothing
-      flag_timeout(a.status);
+      if (lane == 0) flag_timeout(a.status);
       __threadfence();
+      __syncwarp();
     }
-    umma_commit(&acc_full);
+    if (elect_one()) umma_commit(&acc_full);
     pdl_trigger();
   } else if (warp < 4) {
     for (int c = tid; c < GEMM_BN; c += 128) {   // stage scale * row scale and bias while the MMAs run
@@ -419,9 +434,8 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
         *reinterpret_cast<uint4*>(o + j0 + 16) = make_uint4(w[4], w[5], w[6], w[7]);
       }
     }
-  } else {
-    pdl_trigger();   // idle lanes of the producer and issuer warps
   }
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == 5) tmem_dealloc(tmem, GEMM_BN);
@@ -450,7 +464,7 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
   constexpr int A_BYTES = BM * BK, B_BYTES = GEMM_BN * BK, STAGE = A_BYTES + B_BYTES;
   __shared__ uint64_t full[PG_STAGES], empty[PG_STAGES], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_base_s;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   const int nk = (a.K + BK - 1) / BK;
   const int cols = tiles_n * planes, n_tiles = tiles_m * cols;
 
@@ -477,20 +491,22 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
   const uint32_t tmem = tmem_base_s;
   pdl_wait();
 
-  if (warp == 4 && lane == 0) {
+  if (warp == 4) {
     // ---- TMA producer: the ring position runs on across tiles
     bool ok = true;
-    int s = 0, g = 0;
-    uint32_t ph = 0;
+    int s = 0;
+    uint32_t ph = 1;
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
       const int m0 = (t / cols) * BM, ct = t % cols;
       const int w0 = (ct / tiles_n) * a.J + (ct % tiles_n) * GEMM_BN;   // first weight row of the tile
-      for (int i = 0; i < nk; ++i, ++g) {
-        if (g >= PG_STAGES) ok = mbar_wait(&empty[s], ph ^ 1);
+      for (int i = 0; i < nk; ++i) {
+        ok = mbar_wait_warp(&empty[s], ph);   // passes at once for a stage that has never been filled
         if (!ok) break;
-        mbar_expect_tx(&full[s], STAGE);
-        tma_load_2d(smem + s * STAGE, &tma_a, i * BK, m0, &full[s]);
-        tma_load_2d(smem + s * STAGE + A_BYTES, &tma_b, i * BK, w0, &full[s]);
+        if (elect_one()) {
+          mbar_expect_tx(&full[s], STAGE);
+          tma_load_2d(smem + s * STAGE, &tma_a, i * BK, m0, &full[s]);
+          tma_load_2d(smem + s * STAGE + A_BYTES, &tma_b, i * BK, w0, &full[s]);
+        }
         if (++s == PG_STAGES) {
           s = 0;
           ph ^= 1;
@@ -498,8 +514,8 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
       }
     }
     pdl_trigger();
-    if (!ok) flag_timeout(a.status);
-  } else if (warp == 5 && lane == 0) {
+    if (!ok && lane == 0) flag_timeout(a.status);
+  } else if (warp == 5) {
     // ---- MMA issuer: tile `it` of this CTA accumulates into buffer it & 1
     const uint32_t idesc = umma_idesc_i8(BM, GEMM_BN);
     bool ok = true;
@@ -508,29 +524,31 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++it) {
       const int buf = it & 1, use = it >> 1;
       if (use >= 1) {   // the epilogue must have read the previous contents of this buffer
-        ok = mbar_wait(&acc_empty[buf], (use - 1) & 1);
+        ok = mbar_wait_warp(&acc_empty[buf], (use - 1) & 1);
         if (!ok) break;
         tc_fence_after();
       }
       const uint32_t d = tmem + (uint32_t)(buf * GEMM_BN);
       for (int i = 0; i < nk; ++i) {
-        ok = mbar_wait(&full[s], ph);
+        ok = mbar_wait_warp(&full[s], ph);
         if (!ok) break;
         tc_fence_after();
         const uint64_t da = umma_desc_sw128(smem_u32(smem + s * STAGE));
         const uint64_t db = umma_desc_sw128(smem_u32(smem + s * STAGE + A_BYTES));
+        if (elect_one()) {
 #pragma unroll
-        for (int kk = 0; kk < BK / 32; ++kk) umma_i8(d, da + 2 * kk, db + 2 * kk, idesc, (i | kk) != 0);
-        umma_commit(&empty[s]);
+          for (int kk = 0; kk < BK / 32; ++kk) umma_i8(d, da + 2 * kk, db + 2 * kk, idesc, (i | kk) != 0);
+          umma_commit(&empty[s]);
+        }
         if (++s == PG_STAGES) {
           s = 0;
           ph ^= 1;
         }
       }
-      if (ok) umma_commit(&acc_full[buf]);
+      if (ok && elect_one()) umma_commit(&acc_full[buf]);
     }
     pdl_trigger();
-    if (!ok) flag_timeout(a.status);
+    if (!ok && lane == 0) flag_timeout(a.status);
   } else if (warp < 4) {
     // ---- epilogue: warp w drains TMEM lanes [32 w, 32 w + 32) of the finished accumulator
     bool ok = true;
@@ -584,9 +602,8 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
     }
     pdl_trigger();
     if (!ok && lane == 0) flag_timeout(a.status);
-  } else {
-    pdl_trigger();   // idle lanes of the producer and issuer warps
   }
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == 5) tmem_dealloc(tmem, TCOLS);
@@ -1078,7 +1095,7 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
   __shared__ uint64_t full[LSTM_STAGES], empty[LSTM_STAGES], acc_full;
   __shared__ uint32_t tmem_base_s;
   __shared__ float4 s_cst[3][LSTM_BN / 4];   // input scales, recurrent scales, bias of this tile's cells (4 gates each)
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * LSTM_BN;   // row tiles slowest: tiles with work are dispatched first
   const int nkx = a.acc_pre ? 0 : (a.Kx_pad + BK - 1) / BK;
   const int nkh = (a.H + BK - 1) / BK;
@@ -1094,6 +1111,12 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
     fence_proxy_async();
   }
   if (warp == LSTM_EPI_WARPS + 1) tmem_alloc(&tmem_base_s, TCOLS);
+  if (warp == LSTM_EPI_WARPS && lane == 0) {
+    prefetch_tmap(&tma_xa);
+    prefetch_tmap(&tma_xw);
+    prefetch_tmap(&tma_ha);
+    prefetch_tmap(&tma_hw);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -1109,31 +1132,39 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
 
   if (!has_work) {
     if (h_first) pdl_wait();   // whole tile without work; still ordered behind the previous kernel
-  } else if (warp == LSTM_EPI_WARPS && lane == 0) {
+  } else if (warp == LSTM_EPI_WARPS) {
     bool ok = true;
+    int s = 0;
+    uint32_t ph = 1;
     for (int i = 0; i < nk && ok; ++i) {
-      const int s = i % LSTM_STAGES;
-      if (i >= LSTM_STAGES) ok = mbar_wait(&empty[s], ((i / LSTM_STAGES) - 1) & 1);
+      ok = mbar_wait_warp(&empty[s], ph);   // passes at once for a stage that has never been filled
       if (!ok) break;
       const bool xpart = h_first ? i >= nkh : i < nkx;
       if (h_first && i == x_first) pdl_wait();
-      mbar_expect_tx(&full[s], STAGE);
-      if (xpart) {
-        tma_load_2d(smem + s * STAGE, &tma_xa, (i - x_first) * BK, m0, &full[s]);
-        tma_load_2d(smem + s * STAGE + A_BYTES, &tma_xw, (i - x_first) * BK, n0, &full[s]);
-      } else {
-        tma_load_2d(smem + s * STAGE, &tma_ha, (i - hh_first) * BK, m0, &full[s]);
-        tma_load_2d(smem + s * STAGE + A_BYTES, &tma_hw, (i - hh_first) * BK, n0, &full[s]);
+      if (elect_one()) {
+        mbar_expect_tx(&full[s], STAGE);
+        if (xpart) {
+          tma_load_2d(smem + s * STAGE, &tma_xa, (i - x_first) * BK, m0, &full[s]);
+          tma_load_2d(smem + s * STAGE + A_BYTES, &tma_xw, (i - x_first) * BK, n0, &full[s]);
+        } else {
+          tma_load_2d(smem + s * STAGE, &tma_ha, (i - hh_first) * BK, m0, &full[s]);
+          tma_load_2d(smem + s * STAGE + A_BYTES, &tma_hw, (i - hh_first) * BK, n0, &full[s]);
+        }
+      }
+      if (++s == LSTM_STAGES) {
+        s = 0;
+        ph ^= 1;
       }
     }
     pdl_trigger();
-    if (!ok) flag_timeout(a.status);
-  } else if (warp == LSTM_EPI_WARPS + 1 && lane == 0) {
+    if (!ok && lane == 0) flag_timeout(a.status);
+  } else if (warp == LSTM_EPI_WARPS + 1) {
     const uint32_t idesc = umma_idesc_i8(BM, LSTM_BN);
     bool ok = true;
+    int s = 0;
+    uint32_t ph = 0;
     for (int i = 0; i < nk && ok; ++i) {
-      const int s = i % LSTM_STAGES;
-      ok = mbar_wait(&full[s], (i / LSTM_STAGES) & 1);
+      ok = mbar_wait_warp(&full[s], ph);
       if (!ok) break;
       tc_fence_after();
       const uint64_t da = umma_desc_sw128(smem_u32(smem + s * STAGE));
@@ -1141,13 +1172,19 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
       const bool xpart = h_first ? i >= nkh : i < nkx;
       const uint32_t d = tmem + (xpart ? 0 : LSTM_BN);
       const int first = xpart ? x_first : hh_first;
+      if (elect_one()) {
 #pragma unroll
-      for (int kk = 0; kk < BK / 32; ++kk) umma_i8(d, da + 2 * kk, db + 2 * kk, idesc, (i != first) || kk != 0);
-      umma_commit(&empty[s]);
+        for (int kk = 0; kk < BK / 32; ++kk) umma_i8(d, da + 2 * kk, db + 2 * kk, idesc, (i != first) || kk != 0);
+        umma_commit(&empty[s]);
+      }
+      if (++s == LSTM_STAGES) {
+        s = 0;
+        ph ^= 1;
+      }
     }
-    umma_commit(&acc_full);
+    if (elect_one()) umma_commit(&acc_full);
     pdl_trigger();
-    if (!ok) flag_timeout(a.status);
+    if (!ok && lane == 0) flag_timeout(a.status);
   } else if (warp < LSTM_EPI_WARPS) {
     const int q = warp & 3, hf = warp >> 2;
     const int rt = q * 32 + lane;            // row within the tile
@@ -1320,9 +1357,8 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
         }
       }
     }
-  } else {
-    pdl_trigger();   // idle lanes of the producer and issuer warps
   }
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (warp == LSTM_EPI_WARPS + 1) tmem_dealloc(tmem, TCOLS);

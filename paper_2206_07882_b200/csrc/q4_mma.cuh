@@ -49,6 +49,25 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
   return false;
 }
 
+// One lane of a converged warp.  The loops that issue copies and MMAs are walked by a whole warp with
+// warp-uniform values, and one elected lane issues: the instructions take their operands from uniform
+// registers, and from a loop that a single lane of a divergent branch walks every operand is moved there at
+// each issue.  Measured: an int8 MMA 128 x N x 32 takes 86 clocks from a divergent branch for any N <= 128,
+// 71 (N = 32) to 77 (N = 128) this way; a K chunk (wait, four MMAs, commit) of the LM head 0.31 -> 0.22 us.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred P;\n\t.reg .b32 R;\n\t"
+      "elect.sync R|P, 0xffffffff;\n\t"
+      "selp.b32 %0, 1, 0, P;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, uint32_t limit = (1u << 22)) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit)) != 0;
+}
+
 // 2-D tiled TMA load into shared memory, completion counted on an mbarrier.  x is the
 // innermost (contiguous) coordinate and must be a multiple of 16 bytes.
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y,
