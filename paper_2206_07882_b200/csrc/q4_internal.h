@@ -98,6 +98,7 @@ struct LmHeadArgs {
   const int32_t* dst_row;     // nullptr = n, negative = skip
   const int32_t* n_active;
   int32_t* status;
+  int32_t tile_rows, n_stages;   // set by the launcher
 };
 cudaError_t launch_mma_lmhead(const LmHeadArgs& a, const int8_t* h8, long long h_pitch, const int8_t* wb8,
                               const int8_t* wo8, cudaStream_t s, bool dependent = false);

@@ -736,66 +736,89 @@ cudaError_t launch_mma_gemm_i32(const int8_t* x8, int M, const int8_t* w8, int J
 
 // ------------------------------------------------------------------ fused LM head
 // One launch per language model (and one for the joint network's output layer) and iteration.
-// A cluster of ceil(V/NB) CTAs serves one tile of 128 rows; every CTA computes the bottleneck
-// GEMM (H -> D = 256, cheap, int32 in TMEM), de-quantizes + biases + re-quantizes it
-// (asymmetric constants) straight into a swizzled shared-memory operand tile, multiplies it
-// with its own block of NB output-layer rows, and keeps its NB logits per row in registers
-// (NB/4 per thread).  Row maxima and sums of the blocks are exchanged through distributed
-// shared memory, one cluster barrier later every thread knows the row's log-sum-exp and stores
-// log-probabilities: one global write, no separate log-softmax pass.  With H = 0 there is no
-// bottleneck: the 256-wide operand rows are read from memory (joint network).
+// A cluster of 8 CTAs serves one tile of 128 rows.  Every CTA computes 32 of the 256 bottleneck columns
+// (H -> 256, int32 in TMEM), de-quantizes, adds the bias, re-quantizes (asymmetric constants) and sends its
+// codes, 32 bytes per row = the operand of one MMA, as one bulk copy to each of the 8 CTAs, counted on an
+// mbarrier of the receiver.  Then every CTA multiplies the 256 codes of the rows with its own block of NB
+// output-layer rows and keeps its NB logits per row in registers (NB / 4 per thread).  Row maxima and sums
+// of the blocks are exchanged through distributed shared memory as well; one cluster barrier later every
+// thread knows the row's log-sum-exp and stores log-probabilities: one global write, no separate log-softmax
+// pass.  With H = 0 there is no bottleneck: the 256-wide operand rows are read from memory (joint network).
+// Bound by the latency of this chain.  (With all 256 bottleneck columns in every CTA it was 5.0 us of bottleneck
+// sums + 2.8 us of re-quantization before the second MMA; codes stored to the peers 8 bytes at a time took
+// 5 us with 128 rows.  Frame-by-frame search of 5 utterances, 40 rows: 15.95 -> 14.4 ms, 64 utterances x 10 s
+// end to end 53.0 -> 51.6 ms.)
 constexpr int HEAD_D = 256;
-constexpr int HEAD_STAGES = 4;
-constexpr int HEAD_EPI_WARPS = 16;           // four warps per TMEM lane quarter, NB/4 columns each
+constexpr int HEAD_CTAS = 8;                 // = the portable cluster size
+constexpr int HEAD_BN1 = HEAD_D / HEAD_CTAS; // bottleneck columns per CTA
+constexpr int HEAD_MAX_STAGES = 8;
+constexpr int HEAD_RING = 80 * 1024;         // bytes of the operand ring; the output layer's weights, the outgoing codes, then
+                                             // the log-probabilities on their way out use the same memory
+constexpr int HEAD_EPI_WARPS = 16;           // four warps per TMEM lane quarter
 constexpr int HEAD_THREADS = 32 * (HEAD_EPI_WARPS + 2);
-constexpr int HEAD_MAX_BLOCKS = 8;           // portable cluster size: V <= 8 NB
 
 __device__ __forceinline__ void cl_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void cl_store_f32(const float* local, uint32_t rank, float v) {
-  uint32_t addr = smem_u32(local), remote;
+__device__ __forceinline__ uint32_t cl_map(uint32_t addr, uint32_t rank) {
+  uint32_t remote;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr), "r"(rank));
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(v) : "memory");
+  return remote;
+}
+__device__ __forceinline__ void cl_store_f32(const float* local, uint32_t rank, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cl_map(smem_u32(local), rank)), "f"(v) : "memory");
 }
 
 template <int NB>
-__global__ void __launch_bounds__(HEAD_THREADS, 1)
+__global__ void __cluster_dims__(HEAD_CTAS, 1, 1) __launch_bounds__(HEAD_THREADS, 1)
 k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ CUtensorMap tma_wb,
              const __grid_constant__ CUtensorMap tma_wo, const LmHeadArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  constexpr int A_BYTES = BM * BK, B_BYTES = HEAD_D * BK, STAGE = A_BYTES + B_BYTES;
+  constexpr int B1_BYTES = HEAD_BN1 * BK;
   constexpr int B2_BYTES = NB * BK;            // one K chunk of my block of output-layer rows
   constexpr int CPT = NB / 4;                  // logits per thread
-  __shared__ uint64_t full[HEAD_STAGES], empty[HEAD_STAGES], acc1_full, a2_ready, acc2_full;
+  constexpr int TCOLS = 2 * NB;                // bottleneck sums in columns 0.., logits' sums in columns NB..
+  // A stage holds the rows of this launch (a.tile_rows of the tile's 128) and the weight rows.  The MMA always
+  // reads 128 operand rows: those beyond tile_rows are whatever follows in the ring, and their sums belong to
+  // rows that are not stored.
+  const int A_BYTES = a.tile_rows * BK, STAGE = A_BYTES + B1_BYTES, NS = a.n_stages;
+  const uint32_t CODE_BYTES = (uint32_t)a.tile_rows * HEAD_BN1;   // a CTA's bottleneck codes
+  uint8_t* const ops = smem;                   // bottleneck codes [source CTA][row][32], or two chunks of operand rows
+  uint8_t* const ring = smem + 2 * BM * BK;
+  __shared__ uint64_t full[HEAD_MAX_STAGES], empty[HEAD_MAX_STAGES], acc1_full, ops_ready, w_full, acc2_full;
   __shared__ uint32_t tmem_base_s;
-  __shared__ __align__(16) float s_sc1[HEAD_D], s_b1[HEAD_D], s_sc2[NB], s_b2[NB];
-  __shared__ float red_m[4][BM], red_s[4][BM];
-  __shared__ float part_m[HEAD_MAX_BLOCKS][BM], part_s[HEAD_MAX_BLOCKS][BM];   // filled by every CTA of the cluster
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  __shared__ __align__(16) float s_sc1[HEAD_BN1], s_b1[HEAD_BN1], s_sc2[NB], s_b2[NB];
+  __shared__ float part_m[HEAD_CTAS][BM], part_s[HEAD_CTAS][BM];   // filled by every CTA of the cluster
+  const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   const int m0 = blockIdx.y * BM;
-  const int nb = blockIdx.x;                    // my block of output columns = my cluster rank
-  const int nblk = gridDim.x;
+  const int nb = blockIdx.x;                    // my blocks of columns = my cluster rank
   const int nk1 = (a.H + BK - 1) / BK;
-  const int nloads = nk1 + 2;
 
   if (tid == 0) {
-    for (int s = 0; s < HEAD_STAGES; ++s) {
+    for (int s = 0; s < NS; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
     mbar_init(&acc1_full, 1);
-    mbar_init(&a2_ready, HEAD_EPI_WARPS);
+    mbar_init(&ops_ready, 1);
+    mbar_init(&w_full, 1);
     mbar_init(&acc2_full, 1);
     fence_barrier_init();
     fence_proxy_async();
+    if (nk1 > 0) mbar_expect_tx(&ops_ready, HEAD_CTAS * CODE_BYTES);
   }
-  if (warp == HEAD_EPI_WARPS + 1) tmem_alloc(&tmem_base_s, 512);
+  if (warp == HEAD_EPI_WARPS + 1) tmem_alloc(&tmem_base_s, TCOLS);
+  if (warp == HEAD_EPI_WARPS && lane == 0) {
+    prefetch_tmap(&tma_h);
+    prefetch_tmap(&tma_wb);
+    prefetch_tmap(&tma_wo);
+  }
   if (warp < HEAD_EPI_WARPS) {   // de-quantization constants: weights only, nothing of the previous kernel
-    for (int c = tid; c < HEAD_D; c += 32 * HEAD_EPI_WARPS) {
-      s_sc1[c] = nk1 > 0 ? __fmul_rn(a.x_scale, __ldg(a.sc_bott + c)) : 0.0f;
-      s_b1[c] = (nk1 > 0 && a.b_bott) ? __ldg(a.b_bott + c) : 0.0f;
+    if (tid < HEAD_BN1 && nk1 > 0) {
+      const int c = nb * HEAD_BN1 + tid;
+      s_sc1[tid] = __fmul_rn(a.x_scale, __ldg(a.sc_bott + c));
+      s_b1[tid] = a.b_bott ? __ldg(a.b_bott + c) : 0.0f;
     }
     for (int c = tid; c < NB; c += 32 * HEAD_EPI_WARPS) {
       const int j = min(nb * NB + c, a.V - 1);
@@ -810,112 +833,112 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
   cl_barrier();   // every CTA of the cluster is running before anyone stores into a peer's shared memory
   pdl_wait();   // everything above (this barrier included) overlaps the tail of the previous kernel of the stream
   if (a.n_active && m0 >= *a.n_active) {   // whole row tile without work: the whole cluster leaves
-    if (warp == HEAD_EPI_WARPS + 1) tmem_dealloc(tmem, 512);
+    if (warp == HEAD_EPI_WARPS + 1) tmem_dealloc(tmem, TCOLS);
     return;
   }
 
-  if (warp == HEAD_EPI_WARPS && lane == 0) {
-    // ---- TMA producer: bottleneck operands, then my block of output-layer weights
+  if (warp == HEAD_EPI_WARPS) {
+    // ---- TMA producer: bottleneck operands through the ring, then my block of output-layer weights into
+    // the ring's memory, which the bottleneck's MMAs have finished reading by then
     bool ok = true;
-    for (int i = 0; i < nloads && ok; ++i) {
-      const int s = i % HEAD_STAGES;
-      if (i >= HEAD_STAGES) ok = mbar_wait(&empty[s], ((i / HEAD_STAGES) - 1) & 1);
+    int s = 0;
+    uint32_t ph = 1;
+    for (int i = 0; i < nk1 && ok; ++i) {
+      ok = mbar_wait_warp(&empty[s], ph);
       if (!ok) break;
-      if (i < nk1) {
+      if (elect_one()) {
         mbar_expect_tx(&full[s], STAGE);
-        tma_load_2d(smem + s * STAGE, &tma_h, i * BK, m0, &full[s]);
-        tma_load_2d(smem + s * STAGE + A_BYTES, &tma_wb, i * BK, 0, &full[s]);
-      } else if (nk1 > 0) {
-        // only the weight half of the stage is loaded: the activation halves of stages 0 and 1
-        // receive the re-quantized bottleneck codes from the epilogue warps
-        mbar_expect_tx(&full[s], B2_BYTES);
-        tma_load_2d(smem + s * STAGE + A_BYTES, &tma_wo, (i - nk1) * BK, nb * NB, &full[s]);
-      } else {
-        // no bottleneck: the 256-wide operand rows come from memory (stage i holds chunk i)
-        mbar_expect_tx(&full[s], A_BYTES + B2_BYTES);
-        tma_load_2d(smem + s * STAGE, &tma_h, i * BK, m0, &full[s]);
-        tma_load_2d(smem + s * STAGE + A_BYTES, &tma_wo, i * BK, nb * NB, &full[s]);
+        tma_load_2d(ring + s * STAGE, &tma_h, i * BK, m0, &full[s]);
+        tma_load_2d(ring + s * STAGE + A_BYTES, &tma_wb, i * BK, nb * HEAD_BN1, &full[s]);
+      }
+      if (++s == NS) {
+        s = 0;
+        ph ^= 1;
+      }
+    }
+    if (ok && nk1 > 0) ok = mbar_wait_warp(&acc1_full, 0);
+    if (ok && elect_one()) {
+      mbar_expect_tx(&w_full, nk1 > 0 ? 2 * B2_BYTES : 2 * (B2_BYTES + A_BYTES));
+      for (int kc = 0; kc < 2; ++kc) {
+        if (nk1 == 0) tma_load_2d(ops + kc * BM * BK, &tma_h, kc * BK, m0, &w_full);
+        tma_load_2d(ring + kc * B2_BYTES, &tma_wo, kc * BK, nb * NB, &w_full);
       }
     }
     pdl_trigger();
-    if (!ok) flag_timeout(a.status);
-  } else if (warp == HEAD_EPI_WARPS + 1 && lane == 0) {
+    if (!ok && lane == 0) flag_timeout(a.status);
+  } else if (warp == HEAD_EPI_WARPS + 1) {
     // ---- MMA issuer
-    const uint32_t idesc1 = umma_idesc_i8(BM, HEAD_D), idesc2 = umma_idesc_i8(BM, NB);
+    const uint32_t idesc1 = umma_idesc_i8(BM, HEAD_BN1), idesc2 = umma_idesc_i8(BM, NB);
     bool ok = true;
+    int s = 0;
+    uint32_t ph = 0;
     for (int i = 0; i < nk1 && ok; ++i) {
-      const int s = i % HEAD_STAGES;
-      ok = mbar_wait(&full[s], (i / HEAD_STAGES) & 1);
+      ok = mbar_wait_warp(&full[s], ph);
       if (!ok) break;
       tc_fence_after();
-      const uint64_t da = umma_desc_sw128(smem_u32(smem + s * STAGE));
-      const uint64_t db = umma_desc_sw128(smem_u32(smem + s * STAGE + A_BYTES));
+      const uint64_t da = umma_desc_sw128(smem_u32(ring + s * STAGE));
+      const uint64_t db = umma_desc_sw128(smem_u32(ring + s * STAGE + A_BYTES));
+      if (elect_one()) {
 #pragma unroll
-      for (int kk = 0; kk < BK / 32; ++kk) umma_i8(tmem, da + 2 * kk, db + 2 * kk, idesc1, (i | kk) != 0);
-      umma_commit(&empty[s]);
+        for (int kk = 0; kk < BK / 32; ++kk) umma_i8(tmem, da + 2 * kk, db + 2 * kk, idesc1, (i | kk) != 0);
+        umma_commit(&empty[s]);
+      }
+      if (++s == NS) {
+        s = 0;
+        ph ^= 1;
+      }
     }
-    umma_commit(&acc1_full);
-    if (ok && nk1 > 0) ok = mbar_wait(&a2_ready, 0);
+    if (elect_one()) umma_commit(&acc1_full);
+    if (ok) ok = mbar_wait_warp(&w_full, 0);
+    if (ok && nk1 > 0) ok = mbar_wait_warp(&ops_ready, 0);
     tc_fence_after();
-    for (int kc = 0; kc < 2 && ok; ++kc) {
-      const int i = nk1 + kc;
-      const int s = i % HEAD_STAGES;
-      ok = mbar_wait(&full[s], (i / HEAD_STAGES) & 1);
-      if (!ok) break;
-      tc_fence_after();
-      const uint64_t da = umma_desc_sw128(smem_u32(smem + kc * STAGE));      // bottleneck codes / operand rows
-      const uint64_t db = umma_desc_sw128(smem_u32(smem + s * STAGE + A_BYTES));
+    if (elect_one()) {
 #pragma unroll
-      for (int kk = 0; kk < BK / 32; ++kk) umma_i8(tmem + HEAD_D, da + 2 * kk, db + 2 * kk, idesc2, (kc | kk) != 0);
-      umma_commit(&empty[s]);
+      for (int j = 0; j < HEAD_D / 32; ++j) {
+        const uint64_t da = nk1 > 0 ? umma_desc_sw32(smem_u32(ops + j * BM * HEAD_BN1))
+                                    : umma_desc_sw128(smem_u32(ops + (j >> 2) * BM * BK)) + 2 * (j & 3);
+        const uint64_t db = umma_desc_sw128(smem_u32(ring + (j >> 2) * B2_BYTES)) + 2 * (j & 3);
+        if (ok) umma_i8(tmem + NB, da, db, idesc2, j != 0);
+      }
+      umma_commit(&acc2_full);
     }
-    umma_commit(&acc2_full);
     pdl_trigger();
-    if (!ok) flag_timeout(a.status);
-  } else if (warp < HEAD_EPI_WARPS) {
+    if (!ok && lane == 0) flag_timeout(a.status);
+  } else {
     // ---- epilogue: warp = (lane quarter q, column share cs)
     const int q = warp & 3, cs = warp >> 2;
     const int rt = q * 32 + lane;
     const int n = m0 + rt;
     int dst = -1;
     if (n < a.N && !(a.n_active && n >= *a.n_active)) dst = a.dst_row ? a.dst_row[n] : n;
+    const bool busy = __any_sync(0xffffffffu, dst >= 0);   // a warp without a row to store computes nothing
     bool ok = true;
     const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
     if (nk1 > 0) {
       const int lo = act_lo(a.bott_act), hi = act_hi(a.bott_act), zp = a.bott_act.zero_point;
       ok = mbar_wait(&acc1_full, 0);
       tc_fence_after();
-      // bottleneck codes of my row, columns [64 cs, 64 cs + 64), into the swizzled operand tiles
-#pragma unroll 1
-      for (int ch = 0; ch < 2; ++ch) {
-        const int c0 = 64 * cs + 32 * ch;
-        int r[32];
-        tmem_ld32(taddr + c0, r);
+      // codes of my row, columns 32 nb + [8 cs, 8 cs + 8): collected here, then sent as a whole
+      uint8_t* const mine = ring + HEAD_RING - BM * HEAD_BN1;   // beyond the output layer's weights
+      if (busy) {
+        int r[8];
+        tmem_ld(taddr + 8 * cs, r);
         tmem_ld_wait();
-        uint32_t w[8];
+        uint32_t w[2] = {0, 0};
 #pragma unroll
-        for (int i = 0; i < 8; ++i) w[i] = 0;
-#pragma unroll
-        for (int i = 0; i < 32; i += 4) {
-          const float4 sc = *reinterpret_cast<const float4*>(s_sc1 + c0 + i);
-          const float4 bi = *reinterpret_cast<const float4*>(s_b1 + c0 + i);
-          const float scv[4] = {sc.x, sc.y, sc.z, sc.w}, biv[4] = {bi.x, bi.y, bi.z, bi.w};
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float x = __fmaf_rn((float)r[i + e], scv[e], biv[e]);
-            const int code = quantize1(x, a.bott_act.inv_scale, zp, lo, hi) - zp;
-            w[(i + e) >> 2] |= (uint32_t)(code & 0xFF) << (8 * ((i + e) & 3));
-          }
+        for (int i = 0; i < 8; ++i) {
+          const float x = __fmaf_rn((float)r[i], s_sc1[8 * cs + i], s_b1[8 * cs + i]);
+          const int code = quantize1(x, a.bott_act.inv_scale, zp, lo, hi) - zp;
+          w[i >> 2] |= (uint32_t)(code & 0xFF) << (8 * (i & 3));
         }
-        const int kc = c0 >> 7, kb = c0 & 127;            // operand chunk and byte within its 128-byte row
-        uint8_t* tile = smem + kc * STAGE + (rt >> 3) * 1024 + (rt & 7) * 128;
-        *reinterpret_cast<uint4*>(tile + ((((kb >> 4) + 0) ^ (rt & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-        *reinterpret_cast<uint4*>(tile + ((((kb >> 4) + 1) ^ (rt & 7)) << 4)) = make_uint4(w[4], w[5], w[6], w[7]);
+        *reinterpret_cast<uint2*>(mine + rt * HEAD_BN1 + (((cs >> 1) ^ (rt >> 2 & 1)) << 4) + 8 * (cs & 1)) = make_uint2(w[0], w[1]);
       }
-      fence_proxy_async();        // generic-proxy writes -> visible to the tensor core's async proxy
+      fence_proxy_async();   // read by the copy engine
       tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&a2_ready);
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * HEAD_EPI_WARPS) : "memory");
+      if (warp == 0 && lane < HEAD_CTAS)
+        bulk_copy_to_cluster(cl_map(smem_u32(ops + nb * BM * HEAD_BN1), lane), smem_u32(mine), CODE_BYTES,
+                             cl_map(smem_u32(&ops_ready), lane));
     }
 
     // my CPT logits of this block, kept in registers until the row's log-sum-exp is known
@@ -923,33 +946,43 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
     tc_fence_after();
     pdl_trigger();   // both GEMMs are over: the next kernel may set itself up
     float v[CPT];
-    float my_m = -INFINITY;
+    float my_m = -INFINITY, my_s = 0.0f;
     const int col0 = nb * NB + CPT * cs;       // first vocabulary entry of my share
+    if (busy) {
+      constexpr int CH = CPT < 32 ? CPT : 32;
 #pragma unroll
-    for (int ch = 0; ch < CPT / 32; ++ch) {
-      const int c0 = CPT * cs + 32 * ch;
-      int r[32];
-      tmem_ld32(taddr + HEAD_D + c0, r);
-      tmem_ld_wait();
+      for (int ch = 0; ch < CPT / CH; ++ch) {
+        const int c0 = CPT * cs + CH * ch;
+        int r[CH];
+        tmem_ld(taddr + NB + c0, r);
+        tmem_ld_wait();
 #pragma unroll
-      for (int i = 0; i < 32; i += 4) {
-        const float4 sc = *reinterpret_cast<const float4*>(s_sc2 + c0 + i);
-        const float4 bi = *reinterpret_cast<const float4*>(s_b2 + c0 + i);
-        v[32 * ch + i + 0] = __fmaf_rn((float)r[i + 0], sc.x, bi.x);
-        v[32 * ch + i + 1] = __fmaf_rn((float)r[i + 1], sc.y, bi.y);
-        v[32 * ch + i + 2] = __fmaf_rn((float)r[i + 2], sc.z, bi.z);
-        v[32 * ch + i + 3] = __fmaf_rn((float)r[i + 3], sc.w, bi.w);
+        for (int i = 0; i < CH; i += 4) {
+          const float4 sc = *reinterpret_cast<const float4*>(s_sc2 + c0 + i);
+          const float4 bi = *reinterpret_cast<const float4*>(s_b2 + c0 + i);
+          v[CH * ch + i + 0] = __fmaf_rn((float)r[i + 0], sc.x, bi.x);
+          v[CH * ch + i + 1] = __fmaf_rn((float)r[i + 1], sc.y, bi.y);
+          v[CH * ch + i + 2] = __fmaf_rn((float)r[i + 2], sc.z, bi.z);
+          v[CH * ch + i + 3] = __fmaf_rn((float)r[i + 3], sc.w, bi.w);
+        }
+      }
+      // exponentials by the hardware base-2 unit: relative error near 1e-6, far inside what the
+      // log-sum-exp of a thousand terms needs
+      if (col0 + CPT <= a.V) {
+#pragma unroll
+        for (int i = 0; i < CPT; ++i) my_m = fmaxf(my_m, v[i]);
+#pragma unroll
+        for (int i = 0; i < CPT; ++i) my_s += __expf(v[i] - my_m);
+      } else {
+#pragma unroll
+        for (int i = 0; i < CPT; ++i)
+          if (col0 + i < a.V) my_m = fmaxf(my_m, v[i]);
+#pragma unroll
+        for (int i = 0; i < CPT; ++i)
+          if (col0 + i < a.V) my_s += __expf(v[i] - my_m);
       }
     }
-#pragma unroll
-    for (int i = 0; i < CPT; ++i)
-      if (col0 + i < a.V) my_m = fmaxf(my_m, v[i]);
-    // exponentials by the hardware base-2 unit: relative error near 1e-6, far inside what the
-    // log-sum-exp of a thousand terms needs
-    float my_s = 0.0f;
-#pragma unroll
-    for (int i = 0; i < CPT; ++i)
-      if (col0 + i < a.V) my_s += __expf(v[i] - my_m);
+    float (*red_m)[BM] = reinterpret_cast<float (*)[BM]>(ring), (*red_s)[BM] = red_m + 4;   // the weights have been read
     red_m[cs][rt] = my_m;
     red_s[cs][rt] = my_s;
     asm volatile("bar.sync 1, %0;" ::"n"(32 * HEAD_EPI_WARPS) : "memory");
@@ -959,41 +992,45 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (red_s[i][rt] > 0.0f) ssum += red_s[i][rt] * __expf(red_m[i][rt] - m);
-      for (int r = 0; r < nblk; ++r) {
+#pragma unroll
+      for (int r = 0; r < HEAD_CTAS; ++r) {
         cl_store_f32(&part_m[nb][rt], (uint32_t)r, m);
         cl_store_f32(&part_s[nb][rt], (uint32_t)r, ssum);
       }
     }
     cl_barrier();
-    // all partials are fetched at once (at most HEAD_MAX_BLOCKS of them), then combined in block order
-    float pm[HEAD_MAX_BLOCKS], ps[HEAD_MAX_BLOCKS];
+    // all partials are fetched at once, then combined in block order
+    float pm[HEAD_CTAS], ps[HEAD_CTAS];
 #pragma unroll
-    for (int r = 0; r < HEAD_MAX_BLOCKS; ++r) {
-      pm[r] = r < nblk ? part_m[r][rt] : -INFINITY;
-      ps[r] = r < nblk ? part_s[r][rt] : 0.0f;
+    for (int r = 0; r < HEAD_CTAS; ++r) {
+      pm[r] = part_m[r][rt];
+      ps[r] = part_s[r][rt];
     }
     float m = -INFINITY;
 #pragma unroll
-    for (int r = 0; r < HEAD_MAX_BLOCKS; ++r) m = fmaxf(m, pm[r]);
+    for (int r = 0; r < HEAD_CTAS; ++r) m = fmaxf(m, pm[r]);
     float ssum = 0.0f;
 #pragma unroll
-    for (int r = 0; r < HEAD_MAX_BLOCKS; ++r)
+    for (int r = 0; r < HEAD_CTAS; ++r)
       if (ps[r] > 0.0f) ssum += ps[r] * __expf(pm[r] - m);
     const float lse = m + logf(ssum);
-    // A thread's 32 log-probabilities belong to one row and the rows of a warp's lanes are V floats
+    // A thread's log-probabilities belong to one row and the rows of a warp's lanes are V floats
     // apart, so storing them directly touches 32 lines per instruction.  A full 128-column block goes
-    // through shared memory instead (the operand stages are free: both GEMMs are complete) and leaves
-    // as whole rows, one 512-byte row per warp-wide store.
+    // through shared memory instead (the operand ring is free: both GEMMs and the copies of the codes are
+    // complete) and leaves as whole rows, one 512-byte row per warp-wide store.
     const bool staged = NB == 128 && nb * NB + NB <= a.V && (a.V & 3) == 0 &&
                         (reinterpret_cast<uintptr_t>(a.lp) & 15) == 0;   // uniform per CTA
     if (staged) {
       constexpr int TP = NB + 4;   // row pitch in floats: rows 16-byte aligned, 32 rows spread over the banks
-      float* tile = reinterpret_cast<float*>(smem);
-      int* tdst = reinterpret_cast<int*>(smem + (size_t)BM * TP * sizeof(float));
+      static_assert(NB != 128 || (BM * TP + BM) * 4 <= HEAD_RING, "log-probabilities fit the ring");
+      float* tile = reinterpret_cast<float*>(ring);
+      int* tdst = reinterpret_cast<int*>(ring + (size_t)BM * TP * sizeof(float));
       float* trow = tile + rt * TP + CPT * cs;
+      if (busy) {
 #pragma unroll
-      for (int i = 0; i < CPT; i += 4)
-        *reinterpret_cast<float4*>(trow + i) = make_float4(v[i] - lse, v[i + 1] - lse, v[i + 2] - lse, v[i + 3] - lse);
+        for (int i = 0; i < CPT; i += 4)
+          *reinterpret_cast<float4*>(trow + i) = make_float4(v[i] - lse, v[i + 1] - lse, v[i + 2] - lse, v[i + 3] - lse);
+      }
       if (cs == 0) tdst[rt] = ok ? dst : -1;
       asm volatile("bar.sync 1, %0;" ::"n"(32 * HEAD_EPI_WARPS) : "memory");
       int d[BM / HEAD_EPI_WARPS];
@@ -1015,10 +1052,6 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
         for (int i = 0; i < CPT; i += 8)   // rows of a warp's lanes are V floats apart: few, wide stores
           st_global_v8(out + i, make_float4(v[i] - lse, v[i + 1] - lse, v[i + 2] - lse, v[i + 3] - lse),
                        make_float4(v[i + 4] - lse, v[i + 5] - lse, v[i + 6] - lse, v[i + 7] - lse));
-      } else if (left >= CPT && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
-#pragma unroll
-        for (int i = 0; i < CPT; i += 4)
-          *reinterpret_cast<float4*>(out + i) = make_float4(v[i] - lse, v[i + 1] - lse, v[i + 2] - lse, v[i + 3] - lse);
       } else {
 #pragma unroll
         for (int i = 0; i < CPT; ++i)
@@ -1034,44 +1067,53 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == HEAD_EPI_WARPS + 1) tmem_dealloc(tmem, 512);
-  // no barrier at the exit: every store into a peer's shared memory precedes the exchange barrier above
+  if (warp == HEAD_EPI_WARPS + 1) tmem_dealloc(tmem, TCOLS);
+  // no barrier at the exit: every store and copy into a peer's shared memory precedes the exchange barrier above
   // (release on arrival, acquire on the wait), after which only local memory is touched
 }
 
-cudaError_t launch_mma_lmhead(const LmHeadArgs& a, const int8_t* h8, long long h_pitch, const int8_t* wb8,
-                              const int8_t* wo8, cudaStream_t s, bool dependent) {
-  if (a.N <= 0) return cudaSuccess;
-  const int rows_pad = (a.N + BM - 1) / BM * BM;
-  const int NB = a.V <= 128 * HEAD_MAX_BLOCKS ? 128 : 256;   // the narrower block spreads a row over more CTAs
-  const int nblk = (a.V + NB - 1) / NB;
-  if (nblk > HEAD_MAX_BLOCKS) return cudaErrorInvalidValue;
-  CUtensorMap th, tb, to;
-  const int Ka = a.H > 0 ? a.H : HEAD_D;
-  if (!make_tmap_i8(&th, h8, Ka, rows_pad, h_pitch, BM) || !make_tmap_i8(&to, wo8, HEAD_D, a.V, HEAD_D, NB))
-    return cudaErrorInvalidValue;
-  if (a.H > 0) {
-    if (!make_tmap_i8(&tb, wb8, a.H, HEAD_D, a.H, HEAD_D)) return cudaErrorInvalidValue;
-  } else {
-    tb = to;   // unused without a bottleneck
-  }
-  const size_t smem = (size_t)HEAD_STAGES * (BM * BK + HEAD_D * BK) + 1024;
+template <int NB>
+static cudaError_t lmhead_launch(const CUtensorMap& th, const CUtensorMap& tb, const CUtensorMap& to, const LmHeadArgs& a,
+                                 cudaStream_t s, bool dependent) {
+  static_assert(2 * NB * BK + BM * HEAD_BN1 <= HEAD_RING, "output-layer weights and outgoing codes share the ring's memory");
+  const size_t smem = 2 * BM * BK + (size_t)HEAD_RING + 1024;
   static bool configured = false;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_mma_lmhead<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_mma_lmhead<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_mma_lmhead<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     configured = true;
   }
+  return launch_ex(k_mma_lmhead<NB>, dim3(HEAD_CTAS, (a.N + BM - 1) / BM), dim3(HEAD_THREADS), smem, s, dependent, 1, th, tb,
+                   to, a);
+}
+
+cudaError_t launch_mma_lmhead(const LmHeadArgs& args, const int8_t* h8, long long h_pitch, const int8_t* wb8,
+                              const int8_t* wo8, cudaStream_t s, bool dependent) {
+  if (args.N <= 0) return cudaSuccess;
+  LmHeadArgs a = args;
+  const int rows_pad = (a.N + BM - 1) / BM * BM;
+  int nbw = 32;   // output-layer rows per CTA: the narrowest block that covers the vocabulary with 8 CTAs
+  while (nbw < 256 && nbw * HEAD_CTAS < a.V) nbw *= 2;
+  if (nbw * HEAD_CTAS < a.V) return cudaErrorInvalidValue;
+  a.tile_rows = a.N < BM ? (a.N + 7) / 8 * 8 : BM;
+  const int stage = (a.tile_rows + HEAD_BN1) * BK;
+  a.n_stages = (HEAD_RING - BM * BK) / stage + 1;   // the MMA reads 128 rows from the last stage's start
+  if (a.n_stages * stage > HEAD_RING) --a.n_stages;
+  if (a.n_stages > HEAD_MAX_STAGES) a.n_stages = HEAD_MAX_STAGES;
+  CUtensorMap th, tb, to;
+  const int Ka = a.H > 0 ? a.H : HEAD_D;
+  if (!make_tmap_i8(&th, h8, Ka, rows_pad, h_pitch, a.tile_rows) || !make_tmap_i8(&to, wo8, HEAD_D, a.V, HEAD_D, nbw))
+    return cudaErrorInvalidValue;
+  if (a.H > 0) {
+    if (!make_tmap_i8(&tb, wb8, a.H, HEAD_D, a.H, HEAD_BN1)) return cudaErrorInvalidValue;
+  } else {
+    tb = to;   // unused without a bottleneck
+  }
   timing_begin(s);
-  cudaError_t e;
-  if (NB == 128)
-    e = launch_ex(k_mma_lmhead<128>, dim3(nblk, rows_pad / BM), dim3(HEAD_THREADS), smem, s, dependent,
-                  (unsigned)nblk, th, tb, to, a);
-  else
-    e = launch_ex(k_mma_lmhead<256>, dim3(nblk, rows_pad / BM), dim3(HEAD_THREADS), smem, s, dependent,
-                  (unsigned)nblk, th, tb, to, a);
+  const cudaError_t e = nbw == 32    ? lmhead_launch<32>(th, tb, to, a, s, dependent)
+                        : nbw == 64  ? lmhead_launch<64>(th, tb, to, a, s, dependent)
+                        : nbw == 128 ? lmhead_launch<128>(th, tb, to, a, s, dependent)
+                                     : lmhead_launch<256>(th, tb, to, a, s, dependent);
   timing_end(s);
   ++g_launches;
   return e != cudaSuccess ? e : cudaGetLastError();

@@ -77,6 +77,15 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
       ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y)
       : "memory");
 }
+// `bytes` (a multiple of 16) from this CTA's shared memory into the shared memory of a CTA of the cluster by
+// the bulk-copy engine; counted on the mbarrier at `mbar_addr`, an address in the receiver's window.  No
+// multicast: one destination per copy.
+__device__ __forceinline__ void bulk_copy_to_cluster(uint32_t dst_addr, uint32_t src_addr, uint32_t bytes,
+                                                     uint32_t mbar_addr) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst_addr), "r"(src_addr), "r"(bytes), "r"(mbar_addr)
+               : "memory");
+}
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
@@ -107,6 +116,16 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t smem_addr) {
   d |= (uint64_t)(1024u >> 4) << 32;                    // stride byte offset between 8-row groups
   d |= (uint64_t)1 << 46;                               // descriptor version for sm_100
   d |= (uint64_t)2 << 61;                               // layout: 128-byte swizzle
+  return d;
+}
+// The same for a tile whose rows are 32 bytes (one MMA's worth of K) under the 32-byte swizzle: groups of 8
+// rows 256 bytes apart, the 16-byte halves of rows 4..7 of a group exchanged.
+__device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t smem_addr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)(256u >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)6 << 61;                               // layout: 32-byte swizzle
   return d;
 }
 // Instruction descriptor: signed 8-bit A and B, both K-major, int32 accumulate, M x N tile.
@@ -150,6 +169,15 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, int (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, int (&r)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, int (&r)[16]) { tmem_ld16(taddr, r); }
+__device__ __forceinline__ void tmem_ld(uint32_t taddr, int (&r)[32]) { tmem_ld32(taddr, r); }
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }

@@ -290,15 +290,6 @@ k_enc_recurrent(const EncRecArgs a) {
 // CTAs still meet at the closing cluster barrier (the others' waits expire in turn).
 // The input accumulators of the next step are fetched into shared memory by cp.async one step
 // ahead.  The layer output codes leave through a staging buffer as 8-byte stores.
-// `bytes` (a multiple of 16) from this CTA's shared memory into the shared memory of a CTA of the
-// cluster by the bulk-copy engine; their arrival is counted on the mbarrier at `mbar_addr`, an
-// address in the receiving CTA's window.  No multicast: one destination per copy.
-__device__ __forceinline__ void bulk_copy_to_cluster(uint32_t dst_addr, uint32_t src_addr, uint32_t bytes,
-                                                     uint32_t mbar_addr) {
-  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst_addr), "r"(src_addr), "r"(bytes), "r"(mbar_addr)
-               : "memory");
-}
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
