@@ -33,28 +33,206 @@ __device__ __forceinline__ float key_score(uint64_t key) {
   return __uint_as_float(b);
 }
 __device__ __forceinline__ uint64_t u64max(uint64_t a, uint64_t b) { return a > b ? a : b; }
-__device__ __forceinline__ uint64_t warp_max_u64(uint64_t v) {
+// A selection is a chain of short phases on 16 warps of one SM per utterance, each bound by a memory or barrier
+// latency: rows of the three tables 3.0 us (196 KB into one SM), state 1.3 to 2.2, list 1.2, ranking 1, merge
+// .5 to 1, bookkeeping 1.2 (64 utterances, label iteration: 9.9 us after its wait; 12.6 before).  Every
+// instruction runs a few times at most and other kernels have used the instruction caches in between, so
+// code size counts: 41 KB instead of 108 KB with every pass over the proposals in registers and unrolled loops.
+// ---- proposals of one slot, by one warp.  A label's score is (float)(S + rho + inc) in double, where inc =
+// log P(k) + lambda_t log P_tgt(k) - lambda_s log P_src(k) in fp32 (magnitude of tens) and S is the slot's
+// running score: within a slot the score grows with inc, so proposals are compared by inc and only the few
+// that matter are scored (conversions to and from double run at an eighth of the fp32 rate: scoring all
+// 16 x 1024 proposals cost 1 us of the selection).
+// MODE 2: V <= 1024, a multiple of 4, 16-byte aligned rows: element i of a lane is k = 128 (i / 4) + 4 lane +
+// i % 4; MODE 1: V <= 1024: k = lane + 32 i; the 32 values of a lane stay in registers.  MODE 0: any V, by loops
+// over shared memory.
+template <int MODE>
+__device__ __forceinline__ int slot_elem(int i, int lane) {
+  return MODE == 2 ? 128 * (i >> 2) + 4 * lane + (i & 3) : lane + 32 * i;
+}
+template <int MODE, int N>
+__device__ __forceinline__ void load_elems(const float* p, int i0, int V, int lane, float beyond, float (&v)[N]) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = u64max(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
+  for (int i = 0; i < N; i += MODE == 2 ? 4 : 1) {
+    const int k = slot_elem<MODE>(i0 + i, lane);
+    if (MODE == 2) {
+      const float4 q = k < V ? *reinterpret_cast<const float4*>(p + k) : make_float4(beyond, beyond, beyond, beyond);
+      v[i] = q.x;
+      v[i + 1] = q.y;
+      v[i + 2] = q.z;
+      v[i + 3] = q.w;
+    } else {
+      v[i] = k < V ? p[k] : beyond;
+    }
+  }
+}
+// log(sum(exp)) of a row of logits in memory, by a warp
+__device__ __forceinline__ float row_lse(const float* x, int V, int lane) {
+  float m = -INFINITY;
+#pragma unroll 8
+  for (int k = lane; k < V; k += 32) m = fmaxf(m, x[k]);
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  float sum = 0.0f;
+#pragma unroll 4
+  for (int k = lane; k < V; k += 32) sum += expf(x[k] - m);
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  return m + logf(sum);
+}
+__device__ __forceinline__ float label_inc(const BeamSelArgs& a, float lp, float s, float t) {
+  return __fmaf_rn(a.lambda_t, t, __fmaf_rn(-a.lambda_s, s, lp));
+}
+// The increments of a slot's labels, from the joint's row (v: loaded already in MODE 1 and 2), into inc[]
+// (shared memory) and v; returns the lane's best one, elements with a bit in `skip` left out.
+template <int MODE>
+__device__ __forceinline__ float slot_increments(const BeamSelArgs& a, float (&v)[32], const float* x, const float* ls,
+                                                 const float* lt, float lse, uint32_t skip, float* inc, int lane) {
+  const int V = a.V;
+  float best = -INFINITY;
+  if (MODE == 0) {
+#pragma unroll 4
+    for (int k = lane; k < V; k += 32) {
+      const float w = label_inc(a, x[k] - lse, ls[k], lt[k]);
+      inc[k] = w;
+      if (k > 0) best = fmaxf(best, w);   // (no bound is taken from it)
+    }
+  } else {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {   // two round trips to memory
+      float sv[16], tv[16];
+      load_elems<MODE>(ls, 16 * h, V, lane, 0.0f, sv);
+      load_elems<MODE>(lt, 16 * h, V, lane, 0.0f, tv);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[16 * h + i] = label_inc(a, v[16 * h + i] - lse, sv[i], tv[i]);
+    }
+#pragma unroll
+    for (int i = 0; i < 32; i += MODE == 2 ? 4 : 1) {
+      const int k = slot_elem<MODE>(i, lane);
+      if (k < V) {
+        if (MODE == 2)
+          *reinterpret_cast<float4*>(inc + k) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+        else
+          inc[k] = v[i];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      if (!((skip >> i) & 1u)) best = fmaxf(best, v[i]);   // -inf beyond the row
+  }
+  return best;
+}
+__device__ __forceinline__ float label_score(double s_rho, float inc) { return (float)(s_rho + (double)inc); }
+
+// A lower bound of the W-th best label proposal: the proposals are split into 16 disjoint groups (by lane
+// modulo 16); each group's best is a distinct proposal, so at least 16 >= W proposals reach the smallest of
+// the 16 group maxima.  An empty group gives -inf: everything valid passes.
+__device__ __forceinline__ float label_bound(const float (*gmax)[16], int W, int lane) {
+  float g = -INFINITY;
+  (void)W;   // rows of slots that are not there hold -inf
+#pragma unroll
+  for (int w = 0; w < SEL_NT / 32; w += 2) g = fmaxf(g, gmax[w + (lane >> 4)][lane & 15]);
+  g = fmaxf(g, __shfl_xor_sync(0xffffffffu, g, 16));
+#pragma unroll 1
+  for (int o = 8; o > 0; o >>= 1) g = fminf(g, __shfl_xor_sync(0xffffffffu, g, o));
+  return g;
+}
+__device__ __forceinline__ void list_add(uint64_t* list, int* list_n, int cap, float score, uint32_t idx) {
+  const int p = atomicAdd(list_n, 1);
+  if (p < cap) list[p] = make_key(score, idx);
+}
+// The labels of a slot with a score of at least `bound` go to the list (entries beyond `cap` are only counted).
+template <int MODE>
+__device__ __forceinline__ void collect_labels(const float (&v)[32], uint32_t skip, const float* inc, double s_rho, float bound,
+                                               uint32_t off, uint64_t* list, int* list_n, int cap, int lane) {
+  // (float)(s_rho + inc) >= bound implies inc >= bound - s_rho - (half a rounding step of bound)
+  const float thr = __double2float_rd((double)bound - s_rho - 2.4e-7 * fabs((double)bound) - 1e-30);
+  uint32_t hit = 0;
+#pragma unroll
+  for (int i = 0; i < 32; ++i)
+    if (v[i] >= thr) hit |= 1u << i;
+  hit &= ~skip;
+#pragma unroll 1
+  while (hit) {
+    const int i = __ffs(hit) - 1;
+    hit &= hit - 1;
+    const int k = slot_elem<MODE>(i, lane);
+    const float sc = label_score(s_rho, inc[k]);
+    if (sc >= bound && sc > -INFINITY) list_add(list, list_n, cap, sc, off + (uint32_t)k);
+  }
 }
 
-// Largest key of this lane's strided share of a shared array, and warp-wide arg-max helpers.
-__device__ __forceinline__ uint64_t strided_max(const uint64_t* arr, int n, int lane) {
-  uint64_t m = 0;
-  for (int i = lane; i < n; i += 32) m = u64max(m, arr[i]);
-  return m;
+// The list by the exact threshold: (1) every thread's best proposal ("head") among its strided share of its
+// slots; (2) the W-th best head, found bit by bit with block-wide counts, is a lower bound of the W-th
+// best proposal, and only the threads owning the W best heads can hold anything at or above it; (3) those
+// go to the list.  blank: the slots' blank scores (null: blanks are no proposals here).
+__device__ __forceinline__ void collect_exact(const float* cand, const int* s_row, const int* s_lab, const float* s_score, float rho,
+                                              const float* blank, int W, int V, uint64_t* list, int* list_n, int cap, int warp,
+                                              int lane) {
+  uint64_t head = 0, th = 0;
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    if (pass == 0 || (head != 0ull && head >= th)) {
+#pragma unroll 1
+      for (int w = warp; w < W; w += SEL_NT / 32) {
+        if (s_row[w] < 0) continue;
+        const double s_rho = (double)s_score[w] + (double)rho;
+#pragma unroll 2
+        for (int k = lane; k < (s_lab[w] ? V : 1); k += 32) {
+          if (k == 0 && !blank) continue;
+          const float x = k == 0 ? blank[w] : label_score(s_rho, cand[(size_t)w * V + k]);
+          if (!(x > -INFINITY)) continue;
+          const uint64_t key = make_key(x, (uint32_t)w * (uint32_t)V + (uint32_t)k);
+          if (pass == 0) {
+            head = u64max(head, key);
+          } else if (key >= th) {
+            const int p = atomicAdd(list_n, 1);
+            if (p < cap) list[p] = key;
+          }
+        }
+      }
+    }
+    if (pass == 1) break;
+    // score bits first (32 counts); the index bits matter only if equal scores straddle the bound
+#pragma unroll 1
+    for (int bit = 63; bit >= 0; --bit) {
+      if (bit == 31 && __syncthreads_count(head >= th) <= W) break;
+      const uint64_t c = th | (1ull << bit);
+      if (__syncthreads_count(head >= c) >= W) th = c;
+    }
+    // th = the W-th best head (0 if there are fewer than W heads: then everything valid passes)
+  }
+  __syncthreads();
 }
 
-__global__ void __launch_bounds__(SEL_NT) k_beam_select(const __grid_constant__ BeamSelArgs a) {
+// rank of every list entry by counting; the W best are the winners
+__device__ __forceinline__ void rank_list(const uint64_t* list, int ln, int W, int* win_idx, float* win_score, int tid) {
+#pragma unroll 1
+  for (int i = tid; i < ln; i += SEL_NT) {
+    const uint64_t mine = list[i];
+    int rank = 0;
+#pragma unroll 8
+    for (int j = 0; j < ln; ++j) rank += list[j] > mine;
+    if (rank < W) {
+      win_idx[rank] = (int)(~(uint32_t)mine);
+      win_score[rank] = key_score(mine);
+    }
+  }
+}
+// entries of the short list; smaller vocabularies have as many proposals near the bound as large ones
+__host__ __device__ constexpr int sel_list_cap(int V) { return 16 * ((V + 31) / 32) > 512 ? 16 * ((V + 31) / 32) : 512; }
+
+template <int MODE>
+__global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant__ BeamSelArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int W = a.W, V = a.V;
-  float* cand = reinterpret_cast<float*>(smem_raw);                         // [W * V]
-  uint64_t* list = reinterpret_cast<uint64_t*>(cand + (size_t)W * V);       // survivors of the filter
+  float* cand = reinterpret_cast<float*>(smem_raw);                         // [W * V] increments of the labels
+  uint64_t* list = reinterpret_cast<uint64_t*>(smem_raw + ((size_t)W * V * sizeof(float) + 15) / 16 * 16);       // survivors of the filter
   __shared__ float s_score[MAXW];
   __shared__ int s_t[MAXW], s_u[MAXW], s_row[MAXW], s_last[MAXW];
   __shared__ uint64_t s_hash[MAXW], s_prev[MAXW];
-  __shared__ int list_n;
+  __shared__ int list_n, s_lab[MAXW];   // s_lab: the slot proposes labels
+  __shared__ float s_blank[MAXW];       // scores of the blank proposals
   __shared__ int win_idx[MAXW];
   __shared__ float win_score[MAXW];
   __shared__ float s_gmax[SEL_NT / 32][16];   // per warp: best label proposal of lanes g and g + 16
@@ -65,28 +243,32 @@ __global__ void __launch_bounds__(SEL_NT) k_beam_select(const __grid_constant__ 
   const q4_beam_state& st = a.st;
   const float NEG = -INFINITY;
   const int N = a.B * W;
-  const bool fast = V <= 1024 && W <= SEL_NT / 32 && !a.exact_only;   // one warp per slot, row in registers
+  const bool normalized = a.normalized != 0;   // `logits` holds log-probabilities already
 
   pdl_wait();
-  // the joint logits of slot `warp` do not depend on the beam state: request them first
+  // what the proposals of slot `warp` read does not wait for the block: the joint's row at once, the language
+  // models' rows as soon as the slot's state row is known
+  const float* const x = a.logits + (size_t)(base + warp) * V;
   float v[32];
-  if (fast && warp < W) {
-    const float* x = a.logits + (size_t)(base + warp) * V;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const int k = lane + 32 * i;
-      v[i] = k < V ? x[k] : NEG;
-    }
+  int my_row = -1, my_u = 0;
+  float my_score = 0.0f;
+  if (warp < W) {
+    my_row = st.row[base + warp];
+    my_u = st.u[base + warp];
+    my_score = st.score[base + warp];
+    if (MODE > 0) load_elems<MODE>(x, 0, V, lane, NEG, v);
   }
   if (tid < W) {
     const int o = base + tid;
-    s_row[tid] = st.row[o];
+    const int row = st.row[o], u = st.u[o];
     s_score[tid] = st.score[o];
     s_t[tid] = st.t[o];
-    s_u[tid] = st.u[o];
     s_last[tid] = st.last_tok[o];
     s_hash[tid] = st.hash[o];
     s_prev[tid] = st.prev_hash[o];
+    s_row[tid] = row;
+    s_u[tid] = u;
+    s_lab[tid] = row >= 0 && u < a.u_max;
   }
   if (tid == 0) {
     list_n = 0;
@@ -94,22 +276,20 @@ __global__ void __launch_bounds__(SEL_NT) k_beam_select(const __grid_constant__ 
     if (b == 0) st.pend_n[a.iter & 1] = 0;
   }
   if (lane < 16) s_gmax[warp][lane] = NEG;
-  __syncthreads();
+  const bool any_labels = __syncthreads_or(my_row >= 0 && my_u < a.u_max) != 0;
 
   // ---- no slot of this utterance may emit a label (all at their label budget, or empty): the only
   // proposals are the blanks of the live slots, at most W of them, no two of which can describe the
   // same string.  One warp, lane = slot: the same score arithmetic, the same finished list and the
   // same order (score descending, then slot) as the general path below, without its passes over V.
-  const int cap = 16 * ((V + 31) / 32);
-  bool any_labels = false;
-  for (int w = 0; w < W; ++w) any_labels |= s_row[w] >= 0 && s_u[w] < a.u_max;
-  const bool blank_only = fast && a.normalized != 0 && !any_labels;
+  const int cap = sel_list_cap(V);
+  const bool blank_only = !a.exact_only && normalized && !any_labels;
   if (blank_only) {
     if (warp == 0) {
       const int w = lane;
       const bool alive = w < W && s_row[w] >= 0;
       float sc = NEG;
-      if (alive) sc = (float)((double)s_score[w] + (double)(a.logits[(size_t)(base + w) * V] - 0.0f));
+      if (alive) sc = (float)((double)s_score[w] + (double)a.logits[(size_t)(base + w) * V]);
       const bool fin = alive && s_t[w] + 1 == a.T;   // consumed the last frame: goes to the finished list
       if (__any_sync(0xffffffffu, fin)) {
         if (w < W) win_score[w] = sc;                // staging only; overwritten by the ranking below
@@ -119,13 +299,16 @@ __global__ void __launch_bounds__(SEL_NT) k_beam_select(const __grid_constant__ 
           int* fi = st.fin_iter + base;
           int* fl = st.fin_slot + base;
           int n = st.fin_n[b];
+#pragma unroll 1
           for (int x = 0; x < W; ++x) {
             if (s_row[x] < 0 || s_t[x] + 1 != a.T) continue;
             const float S = win_score[x];
             int pos = n;
+#pragma unroll 1
             while (pos > 0 && fs[pos - 1] < S) --pos;
             if (pos >= W) continue;
             const int last = min(n, W - 1);
+#pragma unroll 1
             for (int i = last; i > pos; --i) {
               fs[i] = fs[i - 1];
               fi[i] = fi[i - 1];
@@ -143,6 +326,7 @@ __global__ void __launch_bounds__(SEL_NT) k_beam_select(const __grid_constant__ 
       const bool cnd = alive && !fin && sc > NEG;
       const uint64_t key = cnd ? make_key(sc, (uint32_t)w * (uint32_t)V) : 0ull;
       int rank = 0;
+#pragma unroll 1
       for (int x = 0; x < W; ++x) rank += __shfl_sync(0xffffffffu, key, x) > key;
       if (cnd) {
         win_idx[rank] = w * V;
@@ -153,141 +337,33 @@ __global__ void __launch_bounds__(SEL_NT) k_beam_select(const __grid_constant__ 
     }
     __syncthreads();
   } else {
-  // ---- proposals
-  uint32_t skip = 0;   // fast path: bit i = element lane + 32 i is not a label proposal that can win
-  if (fast) {
-    if (warp < W) {
-      const int w = warp;
-      float* cw = cand + (size_t)w * V;
-      const int row = s_row[w];
-      const bool labels = row >= 0 && s_u[w] < a.u_max;
-      if (row < 0) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int k = lane + 32 * i;
-          if (k < V) cw[k] = NEG;
+  // ---- proposals: one warp per slot
+  const bool fast = MODE > 0 && !a.exact_only;   // a lower bound of the W-th best from group maxima
+  const bool my_labels = my_row >= 0 && my_u < a.u_max;
+  const double s_rho = (double)my_score + (double)a.rho;
+  // elements that do not count for the bound and are not collected: element 0 (blank), and labels that the merge
+  // below folds into another slot's blank (lane w1 tests slot w1, the few hits are handed round the warp)
+  uint32_t skip = lane == 0 ? 1u : 0u;
+  if (my_row >= 0) {
+    const float lse = normalized ? 0.0f : row_lse(x, V, lane);
+    if (lane == 0) s_blank[warp] = (float)((double)my_score + (double)((MODE > 0 ? v[0] : x[0]) - lse));
+    if (my_labels) {
+      if (MODE > 0) {
+        const bool hit = lane < W && s_row[lane] >= 0 && s_u[lane] == my_u + 1 && s_prev[lane] == s_hash[warp];
+        const int tok = hit ? s_last[lane] : 0;
+        unsigned hits = __ballot_sync(0xffffffffu, hit);
+#pragma unroll 1
+        while (hits) {
+          const int src = __ffs(hits) - 1;
+          hits &= hits - 1;
+          const int t = __shfl_sync(0xffffffffu, tok, src);
+          if (MODE == 2 ? (t >> 2 & 31) == lane : (t & 31) == lane) skip |= 1u << (MODE == 2 ? (t >> 7) * 4 + (t & 3) : t >> 5);
         }
-        skip = 0xFFFFFFFFu;
-      } else {
-        // one round trip to memory for both LM rows
-        float ltv[32], lsv[32];
-        const float* lt = a.tgt_lp + (size_t)row * V;
-        const float* ls = a.src_lp + (size_t)row * V;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int k = lane + 32 * i;
-          ltv[i] = (k < V && labels) ? lt[k] : 0.0f;
-          lsv[i] = (k < V && labels) ? ls[k] : 0.0f;
-        }
-        const double S = (double)s_score[w];
-        const double S_rho = S + (double)a.rho;
-        float lse = 0.0f;       // the joint kernel may already have normalised its rows
-        if (!a.normalized) {
-          float m = NEG;
-#pragma unroll
-          for (int i = 0; i < 32; ++i) m = fmaxf(m, v[i]);
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-          float sum = 0.0f;
-#pragma unroll
-          for (int i = 0; i < 32; ++i) sum += expf(v[i] - m);   // exp(-inf) = 0 for the padding
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-          lse = m + logf(sum);
-        }
-        // label proposals of this slot that the merge below folds into another slot's blank: lane w1
-        // tests slot w1 (all W tests at once), the few hits are then handed round the warp
-        {
-          const bool hit = lane < W && labels && s_row[lane] >= 0 && s_u[lane] == s_u[w] + 1 && s_prev[lane] == s_hash[w];
-          const int tok = hit ? s_last[lane] : 0;
-          unsigned hits = __ballot_sync(0xffffffffu, hit);
-          while (hits) {
-            const int src = __ffs(hits) - 1;
-            hits &= hits - 1;
-            const int t = __shfl_sync(0xffffffffu, tok, src);
-            if ((t & 31) == lane) skip |= 1u << (t >> 5);
-          }
-        }
-        float best = NEG;
-        const float blank = (float)(S + (double)(v[0] - lse));   // element 0 of lane 0 is the blank proposal
-        if (labels) {   // uniform per warp: a slot at its label budget skips the double-precision adds
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const int k = lane + 32 * i;
-            const float lp = v[i] - lse;
-            float sc;
-            if (k >= V) {
-              sc = NEG;
-              skip |= 1u << i;
-            } else if (k == 0) {
-              sc = blank;
-              skip |= 1u << i;          // the blank proposal is read back after merge and finished list
-            } else {
-              // label increment in fp32 (magnitude of tens), one double add onto the running score
-              const float inc = __fmaf_rn(a.lambda_t, ltv[i], __fmaf_rn(-a.lambda_s, lsv[i], lp));
-              sc = (float)(S_rho + (double)inc);
-            }
-            v[i] = sc;
-            if (k < V) cw[k] = sc;
-            if (!((skip >> i) & 1u)) best = fmaxf(best, sc);
-          }
-        } else {
-          skip = 0xFFFFFFFFu;       // no label proposals: only the blank, read back from shared memory
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const int k = lane + 32 * i;
-            const float sc = k == 0 ? blank : NEG;
-            v[i] = sc;
-            if (k < V) cw[k] = sc;
-          }
-        }
-        best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, 16));
-        if (lane < 16) s_gmax[w][lane] = best;
       }
-    } else {
-      skip = 0xFFFFFFFFu;
-    }
-  } else {
-    for (int w = warp; w < W; w += SEL_NT / 32) {
-      float* cw = cand + (size_t)w * V;
-      const int row = s_row[w];
-      if (row < 0) {
-        for (int k = lane; k < V; k += 32) cw[k] = NEG;
-        continue;
-      }
-      const float* x = a.logits + (size_t)(base + w) * V;
-      const float* lt = a.tgt_lp + (size_t)row * V;
-      const float* ls = a.src_lp + (size_t)row * V;
-      const double S = (double)s_score[w];
-      const double S_rho = S + (double)a.rho;
-      const bool labels = s_u[w] < a.u_max;
-      // general vocabulary size: three passes over the row
-      float lse = 0.0f;
-      if (!a.normalized) {
-        float m = NEG;
-        for (int k = lane; k < V; k += 32) m = fmaxf(m, x[k]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-        float sum = 0.0f;
-        for (int k = lane; k < V; k += 32) sum += expf(x[k] - m);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        lse = m + logf(sum);
-      }
-      for (int k = lane; k < V; k += 32) {
-        const float lp = x[k] - lse;
-        float sc;
-        if (k == 0) {
-          sc = (float)(S + (double)lp);
-        } else if (labels) {
-          // label increment in fp32 (magnitude of tens), one double add onto the running score
-          const float inc = __fmaf_rn(a.lambda_t, lt[k], __fmaf_rn(-a.lambda_s, ls[k], lp));
-          sc = (float)(S_rho + (double)inc);
-        } else {
-          sc = NEG;
-        }
-        cw[k] = sc;
-      }
+      float best = slot_increments<MODE>(a, v, x, a.src_lp + (size_t)my_row * V, a.tgt_lp + (size_t)my_row * V, lse, skip,
+                                         cand + (size_t)warp * V, lane);
+      best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, 16));
+      if (lane < 16) s_gmax[warp][lane] = label_score(s_rho, best);
     }
   }
   __syncthreads();
@@ -295,48 +371,36 @@ __global__ void __launch_bounds__(SEL_NT) k_beam_select(const __grid_constant__ 
   // ---- merge: label proposal (w2, k) describing the same string as the blank proposal of w
   if (tid < W * W) {
     const int w = tid / W, w2 = tid % W;
-    if (s_row[w] >= 0 && s_row[w2] >= 0 && s_u[w] == s_u[w2] + 1 && s_prev[w] == s_hash[w2] &&
-        s_u[w2] < a.u_max) {
+    if (s_row[w] >= 0 && s_lab[w2] && s_u[w] == s_u[w2] + 1 && s_prev[w] == s_hash[w2]) {
       const int k = s_last[w];
-      const double x = (double)cand[(size_t)w * V], y = (double)cand[(size_t)w2 * V + k];
-      const double mx = fmax(x, y);
-      cand[(size_t)w * V] = (float)(mx + log1p(exp(-fabs(x - y))));
+      const double p = (double)s_blank[w];
+      const double q = (double)label_score((double)s_score[w2] + (double)a.rho, cand[(size_t)w2 * V + k]);
+      s_blank[w] = (float)(fmax(p, q) + log1p(exp(-fabs(p - q))));
       cand[(size_t)w2 * V + k] = NEG;
     }
   }
-  // fast path: a lower bound of the W-th best proposal.  The label proposals are split into 16
-  // disjoint groups (by lane modulo 16); each group's best is a distinct proposal, so at least
-  // 16 >= W proposals reach the smallest of the 16 group maxima.  An empty group (no slot may
-  // emit labels) gives -inf: then only the at most W blank proposals exist and all pass.
-  float bound = NEG;
-  if (fast) {
-    float g = NEG;
-    if (lane < 16)
-      for (int w = 0; w < W; ++w) g = fmaxf(g, s_gmax[w][lane]);
-    g = __shfl_sync(0xffffffffu, g, lane & 15);
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) g = fminf(g, __shfl_xor_sync(0xffffffffu, g, o));
-    bound = g;
-  }
+  const float bound = fast ? label_bound(s_gmax, W, lane) : NEG;
   __syncthreads();
 
   // ---- finished hypotheses: blank proposals that consume the last frame
-  if (tid == 0) {
-    bool any = false;
-    for (int w = 0; w < W; ++w) any |= s_row[w] >= 0 && s_t[w] + 1 == a.T;
-    if (any) {
+  const bool any_fin = __any_sync(0xffffffffu, lane < W && s_row[lane] >= 0 && s_t[lane] + 1 == a.T);
+  if (any_fin) {   // uniform for the block
+    if (tid == 0) {
       float* fs = st.fin_score + base;
       int* fi = st.fin_iter + base;
       int* fl = st.fin_slot + base;
       int n = st.fin_n[b];
+#pragma unroll 1
       for (int w = 0; w < W; ++w) {
         if (s_row[w] < 0 || s_t[w] + 1 != a.T) continue;
-        const float S = cand[(size_t)w * V];
-        cand[(size_t)w * V] = NEG;
+        const float S = s_blank[w];
+        s_blank[w] = NEG;
         int pos = n;
+#pragma unroll 1
         while (pos > 0 && fs[pos - 1] < S) --pos;
         if (pos >= W) continue;
         const int last = min(n, W - 1);
+#pragma unroll 1
         for (int i = last; i > pos; --i) {
           fs[i] = fs[i - 1];
           fi[i] = fi[i - 1];
@@ -349,113 +413,27 @@ __global__ void __launch_bounds__(SEL_NT) k_beam_select(const __grid_constant__ 
       }
       st.fin_n[b] = n;
     }
+    __syncthreads();
   }
-  __syncthreads();
 
   // ---- the W best remaining proposals
   bool exact = !fast;
   if (fast) {
-    // everything at or above the bound goes to the short list (label proposals from registers,
-    // the blank proposal from shared memory, where merge and finished list have updated it)
-    if (warp < W && s_row[warp] >= 0) {   // uniform per warp: one list reservation per warp
+    if (my_row >= 0) {
       const uint32_t off = (uint32_t)warp * (uint32_t)V;
-      uint32_t hit = 0;
-#pragma unroll
-      for (int i = 0; i < 32; ++i)
-        if (!((skip >> i) & 1u) && v[i] >= bound) hit |= 1u << i;
-      float vb = NEG;
-      if (lane == 0) {
-        vb = cand[(size_t)warp * V];
-        if (!(vb >= bound)) vb = NEG;
-      }
-      const int mine = __popc(hit) + (vb > NEG ? 1 : 0);
-      int incl = mine;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      const int total = __shfl_sync(0xffffffffu, incl, 31);
-      int p0 = 0;
-      if (lane == 31 && total > 0) p0 = atomicAdd(&list_n, total);
-      p0 = __shfl_sync(0xffffffffu, p0, 31) + incl - mine;
-      if (vb > NEG) {
-        if (p0 < cap) list[p0] = make_key(vb, off);
-        ++p0;
-      }
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {   // static register indices
-        if ((hit >> i) & 1u) {
-          if (p0 < cap) list[p0] = make_key(v[i], off + (uint32_t)(lane + 32 * i));
-          ++p0;
-        }
-      }
+      if (lane == 0 && s_blank[warp] >= bound && s_blank[warp] > NEG) list_add(list, &list_n, cap, s_blank[warp], off);
+      if (my_labels) collect_labels<MODE>(v, skip, cand + (size_t)warp * V, s_rho, bound, off, list, &list_n, cap, lane);
     }
     __syncthreads();
     exact = list_n > cap;     // the bound was too loose for the list: take the exact threshold instead
-    __syncthreads();
-    if (exact && tid == 0) list_n = 0;
-    if (exact) __syncthreads();
+    if (exact) {
+      __syncthreads();
+      if (tid == 0) list_n = 0;
+      __syncthreads();
+    }
   }
-  if (exact) {
-    // Threshold filter.  (1) every thread's best proposal ("head") among its strided share of
-    // its slot; (2) the W-th best head, found bit by bit with block-wide counts, is a lower bound
-    // of the W-th best proposal, and only the threads owning the W best heads can hold anything
-    // at or above it; (3) those go to the short list.
-    uint64_t head = 0;
-    for (int w = warp; w < W; w += SEL_NT / 32) {
-      if (s_row[w] < 0) continue;
-      const float* cw = cand + (size_t)w * V;
-      const uint32_t off = (uint32_t)w * (uint32_t)V;
-      for (int k = lane; k < V; k += 32) {
-        const float x = cw[k];
-        if (x > NEG) head = u64max(head, make_key(x, off + (uint32_t)k));
-      }
-    }
-    // score bits first (32 counts); the index bits matter only if equal scores straddle the bound
-    uint64_t th = 0;
-    for (int bit = 63; bit >= 32; --bit) {
-      const uint64_t c = th | (1ull << bit);
-      if (__syncthreads_count(head >= c) >= W) th = c;
-    }
-    if (__syncthreads_count(head >= th) > W) {
-      for (int bit = 31; bit >= 0; --bit) {
-        const uint64_t c = th | (1ull << bit);
-        if (__syncthreads_count(head >= c) >= W) th = c;
-      }
-    }
-    // th = the W-th best head (0 if there are fewer than W heads: then everything valid passes)
-    if (head != 0ull && head >= th) {
-      for (int w = warp; w < W; w += SEL_NT / 32) {
-        if (s_row[w] < 0) continue;
-        const float* cw = cand + (size_t)w * V;
-        const uint32_t off = (uint32_t)w * (uint32_t)V;
-        for (int k = lane; k < V; k += 32) {
-          const float x = cw[k];
-          if (!(x > NEG)) continue;
-          const uint64_t key = make_key(x, off + (uint32_t)k);
-          if (key >= th) {
-            const int p = atomicAdd(&list_n, 1);
-            if (p < cap) list[p] = key;
-          }
-        }
-      }
-    }
-    __syncthreads();
-  }
-  }
-  // each list entry's rank is counted in parallel
-  if (!blank_only) {
-    const int ln = min(list_n, cap);
-    for (int i = tid; i < ln; i += SEL_NT) {
-      const uint64_t mine = list[i];
-      int rank = 0;
-      for (int j = 0; j < ln; ++j) rank += list[j] > mine;
-      if (rank < W) {
-        win_idx[rank] = (int)(~(uint32_t)mine);
-        win_score[rank] = key_score(mine);
-      }
-    }
+  if (exact) collect_exact(cand, s_row, s_lab, s_score, a.rho, s_blank, W, V, list, &list_n, cap, warp, lane);
+  rank_list(list, min(list_n, cap), W, win_idx, win_score, tid);
   }
   __syncthreads();
   pdl_trigger();   // only the bookkeeping is left: the next kernel of the stream may set itself up
@@ -466,9 +444,7 @@ __global__ void __launch_bounds__(SEL_NT) k_beam_select(const __grid_constant__ 
     // ---- next beam, state rows, back-pointers, pending advances: lane s writes slot s
     const int nw = n_win;
     const int row0 = b * (st.rows_per_utt > 0 ? st.rows_per_utt : 2 * W);
-    uint32_t used = 0;
-    for (int w = 0; w < W; ++w)
-      if (s_row[w] >= 0) used |= 1u << (s_row[w] - row0);
+    const uint32_t used = __reduce_or_sync(0xffffffffu, lane < W && s_row[lane] >= 0 ? 1u << (s_row[lane] - row0) : 0u);
     const uint32_t free_mask = ~used & (W >= 16 ? 0xFFFFFFFFu : ((1u << (2 * W)) - 1u));
     const int s = lane;
     int idx = 0, w = 0, k = 0;
@@ -504,7 +480,10 @@ __global__ void __launch_bounds__(SEL_NT) k_beam_select(const __grid_constant__ 
           // the j-th label extension (in slot order) takes the j-th state row not used by the
           // beam that is being replaced
           const int j = __popc(lab & ((1u << s) - 1u));
-          const int f = (int)__fns(free_mask, 0, j + 1);
+          uint32_t rest = free_mask;
+#pragma unroll 1
+          for (int i = 0; i < j; ++i) rest &= rest - 1;
+          const int f = __ffs(rest) - 1;
           st.t[o] = s_t[w];
           st.u[o] = s_u[w] + 1;
           st.hash[o] = hash_mix(s_hash[w], (uint32_t)k);
@@ -534,17 +513,33 @@ __global__ void __launch_bounds__(SEL_NT) k_beam_select(const __grid_constant__ 
   }
 }
 
-cudaError_t launch_beam_select(const BeamSelArgs& a, cudaStream_t s, bool dependent) {
-  const size_t smem = (size_t)a.W * a.V * sizeof(float) + (size_t)16 * ((a.V + 31) / 32) * sizeof(uint64_t);
+// rows of the three log-probability tables can be read 16 bytes at a time
+static int sel_mode(const BeamSelArgs& a) {
+  if (a.V > 1024) return 0;
+  const bool wide = a.V % 4 == 0 && ((reinterpret_cast<uintptr_t>(a.logits) | reinterpret_cast<uintptr_t>(a.src_lp) |
+                                      reinterpret_cast<uintptr_t>(a.tgt_lp)) & 15) == 0;
+  return wide ? 2 : 1;
+}
+static size_t sel_smem(const BeamSelArgs& a) {
+  return ((size_t)a.W * a.V * sizeof(float) + 15) / 16 * 16 + (size_t)sel_list_cap(a.V) * sizeof(uint64_t);
+}
+template <int MODE>
+static cudaError_t beam_select_launch(const BeamSelArgs& a, cudaStream_t s, bool dependent) {
+  const size_t smem = sel_smem(a);
   static size_t configured = 0;
   if (smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_beam_select, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_beam_select<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     configured = smem;
   }
+  return launch_ex(k_beam_select<MODE>, dim3(a.B), dim3(SEL_NT), smem, s, dependent, 1, a);
+}
+cudaError_t launch_beam_select(const BeamSelArgs& a, cudaStream_t s, bool dependent) {
+  const int mode = sel_mode(a);
   timing_begin(s);
-  cudaError_t le = launch_ex(k_beam_select, dim3(a.B), dim3(SEL_NT), smem, s, dependent, 1, a);
+  const cudaError_t le = mode == 2   ? beam_select_launch<2>(a, s, dependent)
+                         : mode == 1 ? beam_select_launch<1>(a, s, dependent)
+                                     : beam_select_launch<0>(a, s, dependent);
   timing_end(s);
   ++g_launches;
   return le != cudaSuccess ? le : cudaGetLastError();
@@ -560,15 +555,16 @@ cudaError_t launch_beam_select(const BeamSelArgs& a, cudaStream_t s, bool depend
 // extensions of the alignment-length synchronous search.  In the frame-closing call (mode 2) no
 // label is proposed and the W best candidates (score, insertion order) open frame t + 1.
 constexpr int TSD_MAXC = 64;
-__global__ void __launch_bounds__(SEL_NT) k_tsd_select(const __grid_constant__ BeamSelArgs a) {
+template <int MODE>
+__global__ void __launch_bounds__(SEL_NT, 1) k_tsd_select(const __grid_constant__ BeamSelArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int W = a.W, V = a.V;
-  float* cand = reinterpret_cast<float*>(smem_raw);                         // [W * V] label proposals
-  uint64_t* list = reinterpret_cast<uint64_t*>(cand + (size_t)W * V);
+  float* cand = reinterpret_cast<float*>(smem_raw);                         // [W * V] increments of the labels
+  uint64_t* list = reinterpret_cast<uint64_t*>(smem_raw + ((size_t)W * V * sizeof(float) + 15) / 16 * 16);
   __shared__ float s_score[MAXW], s_blank[MAXW];
   __shared__ int s_u[MAXW], s_row[MAXW], s_last[MAXW];
   __shared__ uint64_t s_hash[MAXW], s_prev[MAXW];
-  __shared__ int list_n;
+  __shared__ int list_n, s_lab[MAXW];
   __shared__ int win_idx[MAXW];
   __shared__ float win_score[MAXW];
   __shared__ float c_score[TSD_MAXC];
@@ -587,11 +583,19 @@ __global__ void __launch_bounds__(SEL_NT) k_tsd_select(const __grid_constant__ B
   const int step = a.iter % (S + 1), frame = a.iter / (S + 1);
   const bool inner = a.mode == 1;
   const int RW = st.rows_per_utt;
-  // inner calls with a vocabulary of at most 1024: one warp per slot keeps its proposals in registers
-  // and the W best are found from a lower bound, as in k_beam_select
-  const bool fast = inner && V <= 1024 && W <= SEL_NT / 32 && !a.exact_only;
+  const bool fast = inner && MODE > 0 && !a.exact_only;   // as in k_beam_select
 
   pdl_wait();
+  const float* const x = a.logits + (size_t)(base + warp) * V;
+  float v[32];
+  int my_row = -1, my_u = 0;
+  float my_score = 0.0f;
+  if (warp < W) {
+    my_row = st.row[base + warp];
+    my_u = st.u[base + warp];
+    my_score = st.score[base + warp];
+    if (MODE > 0 && inner) load_elems<MODE>(x, 0, V, lane, NEG, v);
+  }
   if (tid < W) {
     const int o = base + tid;
     s_row[tid] = st.row[o];
@@ -600,8 +604,10 @@ __global__ void __launch_bounds__(SEL_NT) k_tsd_select(const __grid_constant__ B
     s_last[tid] = st.last_tok[o];
     s_hash[tid] = st.hash[o];
     s_prev[tid] = st.prev_hash[o];
+    s_lab[tid] = inner && s_row[tid] >= 0 && s_u[tid] < a.u_max;   // a frame close proposes blanks only
   }
   const int cn0 = st.nb_n[b];
+#pragma unroll 1
   for (int j = tid; j < cn0; j += SEL_NT) {
     const size_t o = (size_t)b * CB + j;
     c_score[j] = st.nb_score[o];
@@ -620,128 +626,32 @@ __global__ void __launch_bounds__(SEL_NT) k_tsd_select(const __grid_constant__ B
   if (lane < 16) s_gmax[warp][lane] = NEG;
   __syncthreads();
 
-  // ---- proposals
-  float v[32];
-  uint32_t skip = 0xFFFFFFFFu;   // fast path: bit i = element lane + 32 i is not a label proposal
-  if (!inner && a.normalized) {
-    // a frame close proposes blanks only, and the joint kernel has normalised its rows
-    if (tid < W)
-      s_blank[tid] = s_row[tid] >= 0
-                         ? (float)((double)s_score[tid] + (double)a.logits[(size_t)(base + tid) * V])
-                         : NEG;
-  } else if (fast) {
-    if (warp < W) {
-      const int w = warp;
-      float* cw = cand + (size_t)w * V;
-      const int row = s_row[w];
-      if (row < 0) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int k = lane + 32 * i;
-          if (k < V) cw[k] = NEG;
-        }
-        if (lane == 0) s_blank[w] = NEG;
-      } else {
-        const bool labels = s_u[w] < a.u_max;
-        const float* x = a.logits + (size_t)(base + w) * V;
-        const float* lt = a.tgt_lp + (size_t)row * V;
-        const float* ls = a.src_lp + (size_t)row * V;
-        float ltv[32], lsv[32];
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int k = lane + 32 * i;
-          v[i] = k < V ? x[k] : NEG;
-          ltv[i] = (k < V && labels) ? lt[k] : 0.0f;
-          lsv[i] = (k < V && labels) ? ls[k] : 0.0f;
-        }
-        const double S_rho = (double)s_score[w] + (double)a.rho;
-        float lse = 0.0f;
-        if (!a.normalized) {
-          float m = NEG;
-#pragma unroll
-          for (int i = 0; i < 32; ++i) m = fmaxf(m, v[i]);
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-          float sum = 0.0f;
-#pragma unroll
-          for (int i = 0; i < 32; ++i) sum += expf(v[i] - m);
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-          lse = m + logf(sum);
-        }
-        skip = 0;
-        float best = NEG;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int k = lane + 32 * i;
-          const float lp = v[i] - lse;
-          float sc = NEG;
-          if (k >= V) {
-            skip |= 1u << i;
-          } else if (k == 0) {
-            s_blank[w] = (float)((double)s_score[w] + (double)lp);
-            skip |= 1u << i;
-          } else if (labels) {
-            const float inc = __fmaf_rn(a.lambda_t, ltv[i], __fmaf_rn(-a.lambda_s, lsv[i], lp));
-            sc = (float)(S_rho + (double)inc);
-            best = fmaxf(best, sc);
-          } else {
-            skip |= 1u << i;
-          }
-          v[i] = sc;
-          if (k < V) cw[k] = sc;
-        }
-        best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, 16));
-        if (lane < 16) s_gmax[w][lane] = best;
-      }
-    }
-  } else
-  for (int w = warp; w < W; w += SEL_NT / 32) {
-    float* cw = cand + (size_t)w * V;
-    const int row = s_row[w];
-    if (row < 0) {
-      for (int k = lane; k < V; k += 32) cw[k] = NEG;
-      if (lane == 0) s_blank[w] = NEG;
-      continue;
-    }
-    const float* x = a.logits + (size_t)(base + w) * V;
-    const float* lt = a.tgt_lp + (size_t)row * V;
-    const float* ls = a.src_lp + (size_t)row * V;
-    const double S_rho = (double)s_score[w] + (double)a.rho;
-    const bool labels = inner && s_u[w] < a.u_max;
-    float lse = 0.0f;
-    if (!a.normalized) {
-      float m = NEG;
-      for (int k = lane; k < V; k += 32) m = fmaxf(m, x[k]);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      float sum = 0.0f;
-      for (int k = lane; k < V; k += 32) sum += expf(x[k] - m);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-      lse = m + logf(sum);
-    }
-    for (int k = lane; k < V; k += 32) {
-      const float lp = x[k] - lse;
-      float sc = NEG;
-      if (k == 0) {
-        s_blank[w] = (float)((double)s_score[w] + (double)lp);
-      } else if (labels) {
-        const float inc = __fmaf_rn(a.lambda_t, lt[k], __fmaf_rn(-a.lambda_s, ls[k], lp));
-        sc = (float)(S_rho + (double)inc);
-      }
-      cw[k] = sc;
+  // ---- proposals: one warp per slot
+  const bool my_labels = inner && my_row >= 0 && my_u < a.u_max;
+  const double s_rho = (double)my_score + (double)a.rho;
+  const uint32_t skip = lane == 0 ? 1u : 0u;   // element 0 is the blank
+  if (warp < W && my_row < 0 && lane == 0) s_blank[warp] = NEG;
+  if (my_row >= 0) {
+    const float lse = a.normalized ? 0.0f : row_lse(x, V, lane);
+    if (lane == 0) s_blank[warp] = (float)((double)my_score + (double)(x[0] - lse));
+    if (my_labels) {
+      float best = slot_increments<MODE>(a, v, x, a.src_lp + (size_t)my_row * V, a.tgt_lp + (size_t)my_row * V, lse, skip,
+                                         cand + (size_t)warp * V, lane);
+      best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, 16));
+      if (lane < 16) s_gmax[warp][lane] = label_score(s_rho, best);
     }
   }
   __syncthreads();
 
   // ---- blanks join the candidate set, in slot order (warp 0; lanes search, lane 0 updates)
   if (warp == 0) {
+#pragma unroll 1
     for (int w = 0; w < W; ++w) {
       if (s_row[w] < 0) continue;             // uniform
       const int n = c_n;
       const uint64_t h = s_hash[w];
       int found = -1;
+#pragma unroll 1
       for (int j0 = 0; j0 < n; j0 += 32) {
         const int j = j0 + lane;
         const unsigned m = __ballot_sync(0xffffffffu, j < n && c_hash[j] == h);
@@ -768,107 +678,25 @@ __global__ void __launch_bounds__(SEL_NT) k_tsd_select(const __grid_constant__ B
       __syncwarp();
     }
   }
-  // lower bound of the W-th best label proposal: the smallest of the 16 group maxima (k_beam_select)
-  float bound = NEG;
-  if (fast) {
-    float g = NEG;
-    if (lane < 16)
-      for (int w = 0; w < W; ++w) g = fmaxf(g, s_gmax[w][lane]);
-    g = __shfl_sync(0xffffffffu, g, lane & 15);
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) g = fminf(g, __shfl_xor_sync(0xffffffffu, g, o));
-    bound = g;
-  }
+  const float bound = fast ? label_bound(s_gmax, W, lane) : NEG;
   __syncthreads();
 
   if (inner) {
-    const int cap = 16 * ((V + 31) / 32);
+    const int cap = sel_list_cap(V);
     bool exact = !fast;
     if (fast) {
-      if (warp < W && s_row[warp] >= 0) {   // uniform per warp: one list reservation per warp
-        const uint32_t off = (uint32_t)warp * (uint32_t)V;
-        uint32_t hit = 0;
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-          if (!((skip >> i) & 1u) && v[i] >= bound) hit |= 1u << i;
-        const int mine = __popc(hit);
-        int incl = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int t = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += t;
-        }
-        const int total = __shfl_sync(0xffffffffu, incl, 31);
-        int p0 = 0;
-        if (lane == 31 && total > 0) p0 = atomicAdd(&list_n, total);
-        p0 = __shfl_sync(0xffffffffu, p0, 31) + incl - mine;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {   // static register indices
-          if ((hit >> i) & 1u) {
-            if (p0 < cap) list[p0] = make_key(v[i], off + (uint32_t)(lane + 32 * i));
-            ++p0;
-          }
-        }
-      }
+      if (my_labels)
+        collect_labels<MODE>(v, skip, cand + (size_t)warp * V, s_rho, bound, (uint32_t)warp * (uint32_t)V, list, &list_n, cap, lane);
       __syncthreads();
-      exact = list_n > cap;     // the bound was too loose for the list: take the exact threshold instead
-      __syncthreads();
-      if (exact && tid == 0) list_n = 0;
-      if (exact) __syncthreads();
-    }
-    // ---- otherwise the exact threshold search (see k_beam_select)
-    uint64_t head = 0;
-    if (exact) {
-    for (int w = warp; w < W; w += SEL_NT / 32) {
-      if (s_row[w] < 0) continue;
-      const float* cw = cand + (size_t)w * V;
-      const uint32_t off = (uint32_t)w * (uint32_t)V;
-      for (int k = lane; k < V; k += 32) {
-        const float x = cw[k];
-        if (x > NEG) head = u64max(head, make_key(x, off + (uint32_t)k));
+      exact = list_n > cap;
+      if (exact) {
+        __syncthreads();
+        if (tid == 0) list_n = 0;
+        __syncthreads();
       }
     }
-    uint64_t th = 0;
-    for (int bit = 63; bit >= 32; --bit) {
-      const uint64_t c = th | (1ull << bit);
-      if (__syncthreads_count(head >= c) >= W) th = c;
-    }
-    if (__syncthreads_count(head >= th) > W) {
-      for (int bit = 31; bit >= 0; --bit) {
-        const uint64_t c = th | (1ull << bit);
-        if (__syncthreads_count(head >= c) >= W) th = c;
-      }
-    }
-    if (head != 0ull && head >= th) {
-      for (int w = warp; w < W; w += SEL_NT / 32) {
-        if (s_row[w] < 0) continue;
-        const float* cw = cand + (size_t)w * V;
-        const uint32_t off = (uint32_t)w * (uint32_t)V;
-        for (int k = lane; k < V; k += 32) {
-          const float x = cw[k];
-          if (!(x > NEG)) continue;
-          const uint64_t key = make_key(x, off + (uint32_t)k);
-          if (key >= th) {
-            const int p = atomicAdd(&list_n, 1);
-            if (p < cap) list[p] = key;
-          }
-        }
-      }
-    }
-    __syncthreads();
-    }   // exact
-    {
-      const int ln = min(list_n, cap);
-      for (int i = tid; i < ln; i += SEL_NT) {
-        const uint64_t mine = list[i];
-        int rank = 0;
-        for (int j = 0; j < ln; ++j) rank += list[j] > mine;
-        if (rank < W) {
-          win_idx[rank] = (int)(~(uint32_t)mine);
-          win_score[rank] = key_score(mine);
-        }
-      }
-    }
+    if (exact) collect_exact(cand, s_row, s_lab, s_score, a.rho, nullptr, W, V, list, &list_n, cap, warp, lane);
+    rank_list(list, min(list_n, cap), W, win_idx, win_score, tid);
     __syncthreads();
     pdl_trigger();
     if (warp == 0) {
@@ -876,8 +704,10 @@ __global__ void __launch_bounds__(SEL_NT) k_tsd_select(const __grid_constant__ B
       const int row0 = b * RW;
       // rows in use: those of the current set and those the candidates refer to
       uint64_t used = 0;
+#pragma unroll 1
       for (int w = 0; w < W; ++w)
         if (s_row[w] >= 0) used |= 1ull << (s_row[w] - row0);
+#pragma unroll 1
       for (int j = 0; j < c_n; ++j) used |= 1ull << (c_row[j] - row0);
       const uint64_t all = RW >= 64 ? ~0ull : ((1ull << RW) - 1ull);
       uint64_t free_mask = ~used & all;
@@ -886,6 +716,7 @@ __global__ void __launch_bounds__(SEL_NT) k_tsd_select(const __grid_constant__ B
       int f = -1;
       {
         uint64_t m = free_mask;
+#pragma unroll 1
         for (int j = 0; j <= s && j < nw; ++j) {
           f = m ? __ffsll((long long)m) - 1 : -1;
           m &= m - 1;
@@ -929,6 +760,7 @@ __global__ void __launch_bounds__(SEL_NT) k_tsd_select(const __grid_constant__ B
       }
     }
     // the candidate set goes back to memory
+#pragma unroll 1
     for (int j = tid; j < c_n; j += SEL_NT) {
       const size_t o = (size_t)b * CB + j;
       st.nb_score[o] = c_score[j];
@@ -948,6 +780,7 @@ __global__ void __launch_bounds__(SEL_NT) k_tsd_select(const __grid_constant__ B
     if (tid < n) {
       const float mine = c_score[tid];
       int rank = 0;
+#pragma unroll 1
       for (int j = 0; j < n; ++j) rank += (c_score[j] > mine) || (c_score[j] == mine && j < tid);
       if (rank < W) {
         const int o = base + rank;
@@ -990,16 +823,23 @@ __global__ void __launch_bounds__(SEL_NT) k_tsd_select(const __grid_constant__ B
   }
 }
 
-cudaError_t launch_tsd_select(const BeamSelArgs& a, cudaStream_t s, bool dependent) {
-  const size_t smem = (size_t)a.W * a.V * sizeof(float) + (size_t)16 * ((a.V + 31) / 32) * sizeof(uint64_t);
+template <int MODE>
+static cudaError_t tsd_select_launch(const BeamSelArgs& a, cudaStream_t s, bool dependent) {
+  const size_t smem = sel_smem(a);
   static size_t configured = 0;
   if (smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_tsd_select, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(k_tsd_select<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     configured = smem;
   }
+  return launch_ex(k_tsd_select<MODE>, dim3(a.B), dim3(SEL_NT), smem, s, dependent, 1, a);
+}
+cudaError_t launch_tsd_select(const BeamSelArgs& a, cudaStream_t s, bool dependent) {
+  const int mode = sel_mode(a);
   timing_begin(s);
-  cudaError_t le = launch_ex(k_tsd_select, dim3(a.B), dim3(SEL_NT), smem, s, dependent, 1, a);
+  const cudaError_t le = mode == 2   ? tsd_select_launch<2>(a, s, dependent)
+                         : mode == 1 ? tsd_select_launch<1>(a, s, dependent)
+                                     : tsd_select_launch<0>(a, s, dependent);
   timing_end(s);
   ++g_launches;
   return le != cudaSuccess ? le : cudaGetLastError();

@@ -256,10 +256,11 @@ def test_fused_lm_head_small_search(Bd):
             np.testing.assert_allclose(np.exp(lp.astype(np.float64)).sum(1), 1.0, atol=1e-5)
 
 
-@pytest.mark.parametrize("V,D", [(46, 256), (37, 64)])
+@pytest.mark.parametrize("V,D", [(46, 256), (37, 64), (300, 256), (1100, 256)])
 def test_tensor_core_search_odd_vocabulary(Bd, V, D):
-    # the paper's 46 characters and 10-wide embedding (rows of 46 floats are 8-byte aligned only), and an odd count
-    # without the fused head; 3 utterances x 16 slots, every beam of every iteration
+    # the paper's 46 characters and 10-wide embedding (rows of 46 floats are 8-byte aligned only), an odd count
+    # without the fused head, and the head's and the selection's other widths (64 columns per CTA; 256, and more
+    # labels than a warp holds); 3 utterances x 16 slots, every beam of every iteration
     dw = synth.decoder(seed=63, V=V, E=10, Hp=128, D=D, Hs=128, Ht=256, tgt_layers=2, U_max=6, W=16, out_bits=8)
     e = synth.Stream(18).normal("e", (10, 3, D)).astype(np.float32)
     dd, tokens, lens, scores, ref = run_search(Bd, dw, e)
