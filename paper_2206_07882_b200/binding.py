@@ -467,8 +467,9 @@ class Encoder:
         self.in_act = q4_act_symmetric(1.0 if enc.in_max else enc.in_clip, enc.in_bits)
         self.out_acts = []
         for l, dirs in enumerate(enc.layers):
-            nxt = enc.layers[l + 1][0].w_ih.bits if l + 1 < len(enc.layers) else (
-                enc.proj.w.bits if enc.proj is not None else dirs[0].hid_bits)
+            # codes as wide as the next layer's weights; 2-bit weights take 4-bit codes
+            nxt = max(4, enc.layers[l + 1][0].w_ih.bits) if l + 1 < len(enc.layers) else (
+                max(4, enc.proj.w.bits) if enc.proj is not None else dirs[0].hid_bits)
             self.out_acts.append(q4_act_symmetric(dirs[0].hid_alpha, nxt))
         self.ws = None
 

@@ -144,7 +144,7 @@ __device__ __forceinline__ void list_add(uint64_t* list, int* list_n, int cap, f
 // The labels of a slot with a score of at least `bound` go to the list (entries beyond `cap` are only counted).
 template <int MODE>
 __device__ __forceinline__ void collect_labels(const float (&v)[32], uint32_t skip, const float* inc, double s_rho, float bound,
-                                               uint32_t off, uint64_t* list, int* list_n, int cap, int lane) {
+                                               int V, uint32_t off, uint64_t* list, int* list_n, int cap, int lane) {
   // (float)(s_rho + inc) >= bound implies inc >= bound - s_rho - (half a rounding step of bound)
   const float thr = __double2float_rd((double)bound - s_rho - 2.4e-7 * fabs((double)bound) - 1e-30);
   uint32_t hit = 0;
@@ -157,6 +157,7 @@ __device__ __forceinline__ void collect_labels(const float (&v)[32], uint32_t sk
     const int i = __ffs(hit) - 1;
     hit &= hit - 1;
     const int k = slot_elem<MODE>(i, lane);
+    if (k >= V) continue;   // without a bound (a group is empty) -inf passes the comparison
     const float sc = label_score(s_rho, inc[k]);
     if (sc >= bound && sc > -INFINITY) list_add(list, list_n, cap, sc, off + (uint32_t)k);
   }
@@ -422,7 +423,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
     if (my_row >= 0) {
       const uint32_t off = (uint32_t)warp * (uint32_t)V;
       if (lane == 0 && s_blank[warp] >= bound && s_blank[warp] > NEG) list_add(list, &list_n, cap, s_blank[warp], off);
-      if (my_labels) collect_labels<MODE>(v, skip, cand + (size_t)warp * V, s_rho, bound, off, list, &list_n, cap, lane);
+      if (my_labels) collect_labels<MODE>(v, skip, cand + (size_t)warp * V, s_rho, bound, V, off, list, &list_n, cap, lane);
     }
     __syncthreads();
     exact = list_n > cap;     // the bound was too loose for the list: take the exact threshold instead
@@ -686,7 +687,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_tsd_select(const __grid_constant_
     bool exact = !fast;
     if (fast) {
       if (my_labels)
-        collect_labels<MODE>(v, skip, cand + (size_t)warp * V, s_rho, bound, (uint32_t)warp * (uint32_t)V, list, &list_n, cap, lane);
+        collect_labels<MODE>(v, skip, cand + (size_t)warp * V, s_rho, bound, V, (uint32_t)warp * (uint32_t)V, list, &list_n, cap, lane);
       __syncthreads();
       exact = list_n > cap;
       if (exact) {

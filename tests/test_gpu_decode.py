@@ -268,6 +268,18 @@ def test_tensor_core_search_odd_vocabulary(Bd, V, D):
     assert tr == 1.0
 
 
+@pytest.mark.parametrize("V", [20, 46])
+@pytest.mark.parametrize("tensor_cores", [True, False])
+def test_search_label_budget_of_one(Bd, V, tensor_cores):
+    # with a budget of one label the only slot that proposes labels is the empty string, and nearly all of its
+    # proposals merge into the blanks of the other slots: too few are left to bound the selection from below
+    dw = synth.decoder(seed=65, V=V, E=32, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=1, W=16)
+    e = synth.Stream(19).normal("e", (12, 6, 256)).astype(np.float32)
+    dd, tokens, lens, scores, ref = run_search(Bd, dw, e, tensor_cores=tensor_cores)
+    frac, tr = compare_search(dd, tokens, lens, scores, ref, list(range(6)), 12, 1, 16, min_same=1.0)
+    assert tr == 1.0
+
+
 def test_selection_paths_and_launch_modes_agree(Bd):
     # the bounded fast filter against the exact threshold search, and programmatic dependent
     # launches against plain stream order: bit-identical beams and scores
