@@ -1129,8 +1129,11 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
       TagScope tag(TAG_JOINT);
       Q4_TRY(launch_joint_z(e, nullptr, st.t, B, W, st.pred_p, st.row, N, D, m.z_act, nullptr, z8, live, sp, true));
     }
-    joint_normalized = fused_head ? 1 : 0;
-    if (fused_head) {
+    // small vocabularies: logits, which the selection normalises in passing (one short kernel instead of a cluster's
+    // exchange, and the order of sums of the kernels for few rows)
+    const bool joint_head = fused_head && V > 256;
+    joint_normalized = joint_head ? 1 : 0;
+    if (joint_head) {
       // output layer of the joint network with the log-softmax over the vocabulary in its epilogue
       TagScope tag(TAG_JOINT);
       LmHeadArgs ja;

@@ -82,6 +82,7 @@ struct MmaLstmArgs {
   int32_t h_first;          // 1: only the input operand comes from the previous kernel of the stream, so
                             // the recurrent half of the K loop runs before waiting for that kernel
   int32_t trigger_early;    // 1: let the next kernel of the stream start beside this one
+  int32_t tile_rows, n_stages;   // set by the launcher
   int32_t premultiplied;    // 1: sc_ih = x_scale * row scale and sc_hh = hidden scale * row scale already
 };
 struct LmHeadArgs {

@@ -19,8 +19,9 @@ constexpr int BM = 128;          // activation rows per tile
 constexpr int BK = 128;          // K bytes per pipeline stage (one swizzle row)
 template <int BN>
 constexpr int GEMM_STAGES = BN >= 128 ? 4 : 6;   // ring depth of the plain GEMM with BN weight rows per tile
-constexpr int LSTM_BN = 128;     // weight rows per tile, LSTM (32 cells x 4 gates)
-constexpr int LSTM_STAGES = 3;
+constexpr int LSTM_MAX_STAGES = 8;
+constexpr int LSTM_RING = 96 * 1024;   // bytes of operand ring per CTA of the LSTM kernel: two CTAs per SM
+constexpr int LSTM_SMEM_MAX = LSTM_RING + 10 * 1024;
 constexpr int LSTM_EPI_WARPS = 8;
 
 // ------------------------------------------------------------------ operand preparation
@@ -946,7 +947,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
     tc_fence_after();
     pdl_trigger();   // both GEMMs are over: the next kernel may set itself up
     float v[CPT];
-    float my_m = -INFINITY, my_s = 0.0f;
+    float my_m = -INFINITY, lse;
     const int col0 = nb * NB + CPT * cs;       // first vocabulary entry of my share
     if (busy) {
       constexpr int CH = CPT < 32 ? CPT : 32;
@@ -966,54 +967,89 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
           v[CH * ch + i + 3] = __fmaf_rn((float)r[i + 3], sc.w, bi.w);
         }
       }
+    }
+    // the block's maximum of every row, over the four column shares
+    float (*red_m)[BM] = reinterpret_cast<float (*)[BM]>(ring), (*red_s)[BM] = red_m + 4;   // the weights have been read
+#pragma unroll
+    for (int i = 0; i < CPT; ++i)
+      if (busy && col0 + i < a.V) my_m = fmaxf(my_m, v[i]);
+    if (NB == 32) {
+      // Vocabularies of at most 256: the sums in the order of k_logsoftmax (one thread per entry, pairwise over
+      // lanes, then over warps), so that the kernels for few rows and the tensor-core path give the same bits.
+      float (*ex)[33] = reinterpret_cast<float (*)[33]>(ring + 8 * BM * sizeof(float));
+      red_m[cs][rt] = my_m;
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * HEAD_EPI_WARPS) : "memory");
+      if (cs == 0) {
+        const float m = fmaxf(fmaxf(red_m[0][rt], red_m[1][rt]), fmaxf(red_m[2][rt], red_m[3][rt]));
+#pragma unroll
+        for (int r = 0; r < HEAD_CTAS; ++r) cl_store_f32(&part_m[nb][rt], (uint32_t)r, m);
+      }
+      cl_barrier();
+      float m = -INFINITY;
+#pragma unroll
+      for (int r = 0; r < HEAD_CTAS; ++r) m = fmaxf(m, part_m[r][rt]);
+#pragma unroll
+      for (int i = 0; i < CPT; ++i) ex[rt][CPT * cs + i] = busy && col0 + i < a.V ? expf(v[i] - m) : 0.0f;
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * HEAD_EPI_WARPS) : "memory");
+      if (cs == 0) {
+        float t[16];
+#pragma unroll
+        for (int l = 0; l < 16; ++l) t[l] = ex[rt][l] + ex[rt][l + 16];
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+          for (int l = 0; l < o; ++l) t[l] += t[l + o];
+#pragma unroll
+        for (int r = 0; r < HEAD_CTAS; ++r) cl_store_f32(&part_s[nb][rt], (uint32_t)r, t[0]);
+      }
+      cl_barrier();
+      float t[HEAD_CTAS];
+#pragma unroll
+      for (int r = 0; r < HEAD_CTAS; ++r) t[r] = part_s[r][rt];
+#pragma unroll
+      for (int o = HEAD_CTAS / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int r = 0; r < o; ++r) t[r] += t[r + o];
+      lse = m + logf(t[0]);
+    } else {
       // exponentials by the hardware base-2 unit: relative error near 1e-6, far inside what the
       // log-sum-exp of a thousand terms needs
-      if (col0 + CPT <= a.V) {
+      float my_s = 0.0f;
 #pragma unroll
-        for (int i = 0; i < CPT; ++i) my_m = fmaxf(my_m, v[i]);
+      for (int i = 0; i < CPT; ++i)
+        if (busy && col0 + i < a.V) my_s += __expf(v[i] - my_m);
+      red_m[cs][rt] = my_m;
+      red_s[cs][rt] = my_s;
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * HEAD_EPI_WARPS) : "memory");
+      if (cs == 0) {   // this CTA's (max, sum) of the row goes to every CTA of the cluster
+        const float m = fmaxf(fmaxf(red_m[0][rt], red_m[1][rt]), fmaxf(red_m[2][rt], red_m[3][rt]));
+        float ssum = 0.0f;
 #pragma unroll
-        for (int i = 0; i < CPT; ++i) my_s += __expf(v[i] - my_m);
-      } else {
+        for (int i = 0; i < 4; ++i)
+          if (red_s[i][rt] > 0.0f) ssum += red_s[i][rt] * __expf(red_m[i][rt] - m);
 #pragma unroll
-        for (int i = 0; i < CPT; ++i)
-          if (col0 + i < a.V) my_m = fmaxf(my_m, v[i]);
-#pragma unroll
-        for (int i = 0; i < CPT; ++i)
-          if (col0 + i < a.V) my_s += __expf(v[i] - my_m);
+        for (int r = 0; r < HEAD_CTAS; ++r) {
+          cl_store_f32(&part_m[nb][rt], (uint32_t)r, m);
+          cl_store_f32(&part_s[nb][rt], (uint32_t)r, ssum);
+        }
       }
-    }
-    float (*red_m)[BM] = reinterpret_cast<float (*)[BM]>(ring), (*red_s)[BM] = red_m + 4;   // the weights have been read
-    red_m[cs][rt] = my_m;
-    red_s[cs][rt] = my_s;
-    asm volatile("bar.sync 1, %0;" ::"n"(32 * HEAD_EPI_WARPS) : "memory");
-    if (cs == 0) {   // this CTA's (max, sum) of the row goes to every CTA of the cluster
-      const float m = fmaxf(fmaxf(red_m[0][rt], red_m[1][rt]), fmaxf(red_m[2][rt], red_m[3][rt]));
-      float ssum = 0.0f;
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        if (red_s[i][rt] > 0.0f) ssum += red_s[i][rt] * __expf(red_m[i][rt] - m);
+      cl_barrier();
+      // all partials are fetched at once, then combined in block order
+      float pm[HEAD_CTAS], ps[HEAD_CTAS];
 #pragma unroll
       for (int r = 0; r < HEAD_CTAS; ++r) {
-        cl_store_f32(&part_m[nb][rt], (uint32_t)r, m);
-        cl_store_f32(&part_s[nb][rt], (uint32_t)r, ssum);
+        pm[r] = part_m[r][rt];
+        ps[r] = part_s[r][rt];
       }
+      float m = -INFINITY;
+#pragma unroll
+      for (int r = 0; r < HEAD_CTAS; ++r) m = fmaxf(m, pm[r]);
+      float ssum = 0.0f;
+#pragma unroll
+      for (int r = 0; r < HEAD_CTAS; ++r)
+        if (ps[r] > 0.0f) ssum += ps[r] * __expf(pm[r] - m);
+      lse = m + logf(ssum);
     }
-    cl_barrier();
-    // all partials are fetched at once, then combined in block order
-    float pm[HEAD_CTAS], ps[HEAD_CTAS];
-#pragma unroll
-    for (int r = 0; r < HEAD_CTAS; ++r) {
-      pm[r] = part_m[r][rt];
-      ps[r] = part_s[r][rt];
-    }
-    float m = -INFINITY;
-#pragma unroll
-    for (int r = 0; r < HEAD_CTAS; ++r) m = fmaxf(m, pm[r]);
-    float ssum = 0.0f;
-#pragma unroll
-    for (int r = 0; r < HEAD_CTAS; ++r)
-      if (ps[r] > 0.0f) ssum += ps[r] * __expf(pm[r] - m);
-    const float lse = m + logf(ssum);
     // A thread's log-probabilities belong to one row and the rows of a warp's lanes are V floats
     // apart, so storing them directly touches 32 lines per instruction.  A full 128-column block goes
     // through shared memory instead (the operand ring is free: both GEMMs and the copies of the codes are
@@ -1064,6 +1100,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
   if (warp >= HEAD_EPI_WARPS) {   // the producer and issuer warps join the cluster barrier too
     pdl_trigger();
     cl_barrier();
+    if (NB == 32) cl_barrier();
   }
   tc_fence_before();
   __syncthreads();
@@ -1125,16 +1162,19 @@ cudaError_t launch_mma_lmhead(const LmHeadArgs& args, const int8_t* h8, long lon
 // of a thread are scheduled as one block.
 // PREMUL = true: sc_ih / sc_hh already hold (input scale * row scale) and (hidden scale * row
 // scale), the products the de-quantization needs (same fp32 multiplication, done once).
-template <bool EXTRAS, bool PREMUL>
+// LSTM_BN = weight rows per tile (4 gates of LSTM_BN / 4 cells), see lstm_tile_width.
+template <bool EXTRAS, bool PREMUL, int LSTM_BN>
 __global__ void __launch_bounds__(32 * (LSTM_EPI_WARPS + 2), 2)
 k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ CUtensorMap tma_xw,
            const __grid_constant__ CUtensorMap tma_ha, const __grid_constant__ CUtensorMap tma_hw,
            const MmaLstmArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  constexpr int A_BYTES = BM * BK, B_BYTES = LSTM_BN * BK, STAGE = A_BYTES + B_BYTES;
+  // a stage holds the launch's rows of the tile only; the MMA reads 128 (see k_mma_lmhead)
+  constexpr int B_BYTES = LSTM_BN * BK;
+  const int A_BYTES = a.tile_rows * BK, STAGE = A_BYTES + B_BYTES, NS = a.n_stages;
   constexpr int TCOLS = 2 * LSTM_BN;
-  __shared__ uint64_t full[LSTM_STAGES], empty[LSTM_STAGES], acc_full;
+  __shared__ uint64_t full[LSTM_MAX_STAGES], empty[LSTM_MAX_STAGES], acc_full;
   __shared__ uint32_t tmem_base_s;
   __shared__ float4 s_cst[3][LSTM_BN / 4];   // input scales, recurrent scales, bias of this tile's cells (4 gates each)
   const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
@@ -1144,7 +1184,7 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
   const int nk = nkx + nkh;
 
   if (tid == 0) {
-    for (int s = 0; s < LSTM_STAGES; ++s) {
+    for (int s = 0; s < NS; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -1193,7 +1233,7 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
           tma_load_2d(smem + s * STAGE + A_BYTES, &tma_hw, (i - hh_first) * BK, n0, &full[s]);
         }
       }
-      if (++s == LSTM_STAGES) {
+      if (++s == NS) {
         s = 0;
         ph ^= 1;
       }
@@ -1219,7 +1259,7 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
         for (int kk = 0; kk < BK / 32; ++kk) umma_i8(d, da + 2 * kk, db + 2 * kk, idesc, (i != first) || kk != 0);
         umma_commit(&empty[s]);
       }
-      if (++s == LSTM_STAGES) {
+      if (++s == NS) {
         s = 0;
         ph ^= 1;
       }
@@ -1239,7 +1279,7 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
     // previous cell states of all my cells: requested before the main loop ends (they belong to
     // rows no kernel of this iteration writes), so that their trip to memory costs the epilogue nothing
     float4 cprev_all[LSTM_BN / 32];
-    // 16 cells = 64 contiguous bytes per row: two 256-bit accesses when the layout allows it
+    // 8 or 16 contiguous cells per row: 256-bit accesses when the layout allows it
     const bool wide = (n0 >> 2) + hf * (LSTM_BN / 8) + LSTM_BN / 8 <= a.H && (a.H & 7) == 0 &&
                       ((reinterpret_cast<uintptr_t>(a.c_in) | reinterpret_cast<uintptr_t>(a.c_out)) & 31) == 0;
 #pragma unroll
@@ -1247,8 +1287,8 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
     if (wide) {
       if (dst >= 0 && src >= 0) {
         const float* cp0 = a.c_in + (long long)src * a.H + (n0 >> 2) + hf * (LSTM_BN / 8);
-        ld_global_v8(cp0, cprev_all[0], cprev_all[1]);
-        ld_global_v8(cp0 + 8, cprev_all[2], cprev_all[3]);
+#pragma unroll
+        for (int ch = 0; ch < LSTM_BN / 32; ch += 2) ld_global_v8(cp0 + 4 * ch, cprev_all[ch], cprev_all[ch + 1]);
       }
     } else {
 #pragma unroll
@@ -1279,7 +1319,7 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
     const float sh = a.hid_act.scale;
     const int hlo = act_lo(a.hid_act), hhi = act_hi(a.hid_act);
     const int ylo = act_lo(a.out_act), yhi = act_hi(a.out_act);
-    constexpr int CELLS_PER_HALF = LSTM_BN / 4 / 2;   // 16
+    constexpr int CELLS_PER_HALF = LSTM_BN / 4 / 2;   // 16 or 8
     // Without the extras the codes of all 16 cells of a thread are kept and stored once: the rows
     // of a warp's lanes lie far apart, so every store instruction touches 32 lines, and four small
     // stores per output cost the load/store unit four times as much as one wide one.
@@ -1382,20 +1422,32 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
       }
     }
     if (combine && live) {
-      static_assert(CELLS_PER_HALF == 16, "one uint4 of int8 codes per thread");
-      if (a.h8_out)
-        *reinterpret_cast<uint4*>(a.h8_out + (long long)n * a.h8_ld + cell_first) = make_uint4(w8[0], w8[1], w8[2], w8[3]);
+      constexpr int NW = CELLS_PER_HALF / 4;   // words of int8 codes per thread
+      static_assert(NW == 4 || NW == 2, "16 or 8 cells");
+      auto put8 = [&](uint8_t* o) {
+        if (NW == 4)
+          *reinterpret_cast<uint4*>(o) = make_uint4(w8[0], w8[1], w8[NW - 2], w8[NW - 1]);
+        else
+          *reinterpret_cast<uint2*>(o) = make_uint2(w8[0], w8[1]);
+      };
+      if (a.h8_out) put8(reinterpret_cast<uint8_t*>(a.h8_out) + (long long)n * a.h8_ld + cell_first);
       if (a.hq_out) {
         if (a.hid_act.bits == 4) {
-          uint32_t lo = 0, hi = 0;   // 16 nibbles, cell order
+          uint32_t q[NW / 2];   // nibbles, cell order
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            lo |= ((w8[0] >> (8 * c)) & 0xFu) << (4 * c) | ((w8[1] >> (8 * c)) & 0xFu) << (16 + 4 * c);
-            hi |= ((w8[2] >> (8 * c)) & 0xFu) << (4 * c) | ((w8[3] >> (8 * c)) & 0xFu) << (16 + 4 * c);
+          for (int j = 0; j < NW / 2; ++j) {
+            q[j] = 0;
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              q[j] |= ((w8[2 * j] >> (8 * c)) & 0xFu) << (4 * c) | ((w8[2 * j + 1] >> (8 * c)) & 0xFu) << (16 + 4 * c);
           }
-          *reinterpret_cast<uint2*>(a.hq_out + (long long)dst * a.hq_ld + (cell_first >> 1)) = make_uint2(lo, hi);
+          uint8_t* o = a.hq_out + (long long)dst * a.hq_ld + (cell_first >> 1);
+          if (NW == 4)
+            *reinterpret_cast<uint2*>(o) = make_uint2(q[0], q[NW / 2 - 1]);
+          else
+            *reinterpret_cast<uint32_t*>(o) = q[0];
         } else {
-          *reinterpret_cast<uint4*>(a.hq_out + (long long)dst * a.hq_ld + cell_first) = make_uint4(w8[0], w8[1], w8[2], w8[3]);
+          put8(a.hq_out + (long long)dst * a.hq_ld + cell_first);
         }
       }
     }
@@ -1406,6 +1458,36 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
   if (warp == LSTM_EPI_WARPS + 1) tmem_dealloc(tmem, TCOLS);
 }
 
+template <int BN>
+static cudaError_t lstm_launch(const MmaLstmArgs& a, const CUtensorMap& txa, const CUtensorMap& txw, const CUtensorMap& tha,
+                               const CUtensorMap& thw, size_t smem, cudaStream_t s, bool dependent) {
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e = cudaFuncSetAttribute(k_mma_lstm<true, false, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, LSTM_SMEM_MAX);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_mma_lstm<false, false, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, LSTM_SMEM_MAX);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_mma_lstm<false, true, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, LSTM_SMEM_MAX);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  const dim3 grid((4 * a.H + BN - 1) / BN, (a.N + BM - 1) / BM), block(32 * (LSTM_EPI_WARPS + 2));
+  if (a.yq_out || a.h_f32 || a.dbg_ih)
+    return launch_ex(k_mma_lstm<true, false, BN>, grid, block, smem, s, dependent, 1, txa, txw, tha, thw, a);
+  if (a.premultiplied)
+    return launch_ex(k_mma_lstm<false, true, BN>, grid, block, smem, s, dependent, 1, txa, txw, tha, thw, a);
+  return launch_ex(k_mma_lstm<false, false, BN>, grid, block, smem, s, dependent, 1, txa, txw, tha, thw, a);
+}
+// Weight rows per tile.  An int8 MMA of 128 operand rows takes 77 clocks with 128 weight rows and 73 with 64
+// (the operand rows' way into the tensor core bounds it), so narrower tiles cost nearly twice the tensor time
+// in all; they pay only where every tile has an SM of its own, by a deeper ring and half the cell updates
+// per CTA: frame-by-frame search of 5 utterances (40 rows) 13.7 -> 12.9 ms, forced scoring of 256 rows 2.36 ->
+// 2.25 ms; with 32-wide tiles, and with 64 at two tiles per SM, the target LM's layers waited for the tiles of the
+// other networks instead (search of 16 utterances, label iteration 65 -> 70 us).
+static int lstm_tile_width(int row_tiles, int H) {
+  return row_tiles * ((4 * H + 63) / 64) <= 148 ? 64 : 128;
+}
+
 // Operands: xa int8 [rows_pad, Kx_pad] (ignored with acc_pre), xw int8 [4H, Kx_pad] interleaved,
 // ha int8 [rows_pad, H], hw int8 [4H, H] interleaved.  rows_pad = N rounded up to 128.
 cudaError_t launch_mma_lstm(const MmaLstmArgs& a, const int8_t* xa, long long xa_pitch,
@@ -1413,39 +1495,29 @@ cudaError_t launch_mma_lstm(const MmaLstmArgs& a, const int8_t* xa, long long xa
                             const int8_t* hw, long long hw_pitch, cudaStream_t s, bool dependent) {
   if (a.N <= 0) return cudaSuccess;
   const int rows_pad = (a.N + BM - 1) / BM * BM;
+  const int bn = lstm_tile_width(rows_pad / BM, a.H);
+  MmaLstmArgs b = a;
+  b.tile_rows = a.N < BM ? (a.N + 7) / 8 * 8 : BM;   // a single row tile fetches no rows beyond the launch's
+  const int stage = (b.tile_rows + bn) * BK;
+  b.n_stages = LSTM_RING / stage < LSTM_MAX_STAGES ? LSTM_RING / stage : LSTM_MAX_STAGES;
   CUtensorMap txa, txw, tha, thw;
-  if (!make_tmap_i8(&tha, ha, a.H, rows_pad, ha_pitch, BM) || !make_tmap_i8(&thw, hw, a.H, 4 * a.H, hw_pitch, LSTM_BN))
+  if (!make_tmap_i8(&tha, ha, a.H, rows_pad, ha_pitch, b.tile_rows) || !make_tmap_i8(&thw, hw, a.H, 4 * a.H, hw_pitch, bn))
     return cudaErrorInvalidValue;
   if (a.acc_pre) {
     txa = tha;
     txw = thw;
-  } else if (!make_tmap_i8(&txa, xa, a.Kx_pad, rows_pad, xa_pitch, BM) ||
-             !make_tmap_i8(&txw, xw, a.Kx_pad, 4 * a.H, xw_pitch, LSTM_BN)) {
+  } else if (!make_tmap_i8(&txa, xa, a.Kx_pad, rows_pad, xa_pitch, b.tile_rows) ||
+             !make_tmap_i8(&txw, xw, a.Kx_pad, 4 * a.H, xw_pitch, bn)) {
     return cudaErrorInvalidValue;
   }
-  const size_t smem = (size_t)LSTM_STAGES * (BM * BK + LSTM_BN * BK) + 1024;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_mma_lstm<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_mma_lstm<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_mma_lstm<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
-  dim3 grid((4 * a.H + LSTM_BN - 1) / LSTM_BN, rows_pad / BM);
-  const bool extras = a.yq_out || a.h_f32 || a.dbg_ih;
-  if (a.premultiplied && (extras || a.x_scale_vec)) return cudaErrorInvalidValue;
-  const dim3 block(32 * (LSTM_EPI_WARPS + 2));
+  if (a.premultiplied && (a.yq_out || a.h_f32 || a.dbg_ih || a.x_scale_vec)) return cudaErrorInvalidValue;
+  // the MMA reads 128 operand rows from the start of every stage, of the last one too
+  const int ring = b.n_stages * stage, last = (b.n_stages - 1) * stage + BM * BK;
+  const size_t smem = (size_t)(ring > last ? ring : last) + 1024;
+  if (smem > (size_t)LSTM_SMEM_MAX) return cudaErrorInvalidValue;
   timing_begin(s);
-  cudaError_t le;
-  if (extras)
-    le = launch_ex(k_mma_lstm<true, false>, grid, block, smem, s, dependent, 1, txa, txw, tha, thw, a);
-  else if (a.premultiplied)
-    le = launch_ex(k_mma_lstm<false, true>, grid, block, smem, s, dependent, 1, txa, txw, tha, thw, a);
-  else
-    le = launch_ex(k_mma_lstm<false, false>, grid, block, smem, s, dependent, 1, txa, txw, tha, thw, a);
+  const cudaError_t le = bn == 128 ? lstm_launch<128>(b, txa, txw, tha, thw, smem, s, dependent)
+                                   : lstm_launch<64>(b, txa, txw, tha, thw, smem, s, dependent);
   timing_end(s);
   ++g_launches;
   return le != cudaSuccess ? le : cudaGetLastError();
