@@ -3,7 +3,7 @@
  *
  * C ABI of the CUDA library.  All tensor pointers are DEVICE pointers owned by
  * the caller unless a parameter says "host"; they must be 16-byte aligned.  No
- * entry point allocates, frees, or keeps a copy of anything; work is enqueued
+ * entry point (but q4_search_plan_create) allocates, frees, or keeps a copy of anything; work is enqueued
  * on the stream passed last and the call returns without synchronising (except
  * q4_poll_status).  Every function returns 0 on success or a negative Q4_ERR_*;
  * argument errors are detected on the host before anything is launched.
@@ -347,6 +347,24 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
                         int32_t T, int32_t W, int32_t iter, int32_t u_max, float lambda_t,
                         float lambda_s, float rho, int32_t mode, void* workspace,
                         size_t workspace_bytes, q4_stream stream);
+
+/*
+ * q4_beam_search — all steps of a search on the stream, after q4_beam_init: T + u_max steps of mode 0, or
+ * with time_synchronous != 0 the T (S + 1) steps of modes 1 and 2 (S = state->tsd_smax).  Arguments and
+ * results as dr_fusion_beam_step; same workspace.  `plan` (nullable): an object of q4_search_plan_create, in which
+ * the call keeps a number of steps as a CUDA graph.  The graph belongs to the model, state, weights of Eq. 1
+ * and workspace it was built for and is rebuilt when one of them changes; frames, T and u_max may change from
+ * call to call.  One plan serves one search at a time.  Without a plan, in a stream capture and while launches
+ * are timed, the steps are enqueued one by one (same results).
+ * q4_search_plan_create / _destroy are the only entry points that allocate: a host object, a stream and the
+ * graph.  Destroy a plan before the memory that its last search used is given to anything else.
+ */
+typedef void* q4_search_plan;
+int q4_search_plan_create(q4_search_plan* out);
+int q4_search_plan_destroy(q4_search_plan plan);
+int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, int32_t B, int32_t T, int32_t W,
+                   int32_t u_max, float lambda_t, float lambda_s, float rho, int32_t time_synchronous,
+                   void* workspace, size_t workspace_bytes, q4_search_plan plan, q4_stream stream);
 
 /* Label strings of the best finished hypothesis per utterance (the best live one if none
  * finished): tokens [B, u_max], lens [B], scores [B] (device). */

@@ -79,7 +79,7 @@ class BeamStateS(C.Structure):
 
 EXPORTS = ["q4_act_symmetric", "q4_act_asymmetric", "quantize_pack_int4", "qlstm_layer_forward",
            "qlstm_step", "q4_linear_forward", "qjoint_logprobs", "q4_beam_init",
-           "dr_fusion_beam_step", "q4_traceback", "q4_feature_prologue", "q4_workspace_bytes",
+           "dr_fusion_beam_step", "q4_beam_search", "q4_search_plan_create", "q4_search_plan_destroy", "q4_traceback", "q4_feature_prologue", "q4_workspace_bytes",
            "q4_poll_status", "q4_version", "q4_launch_count", "q4_dependent_launch_set", "q4_beam_select_exact_set", "q4_timing_set", "q4_timing_count", "q4_prepared_bytes", "q4_prepare_model", "qjoint_logprobs_static", "q4_quantizer_calls", "q4_prepared_lstm_bytes", "q4_prepare_lstm",
            "q4_prepared_linear_bytes", "q4_prepare_linear", "q4_test_wait_expiry_set", "q4_encoder_time_slicing_set", "q4_encoder_recurrence_plan"]
 
@@ -529,6 +529,19 @@ class DeviceLm:
         return self.emb_q.numel() + sum(l.nbytes() for l in self.lstm) + self.bott.nbytes() + self.out.nbytes()
 
 
+class _SearchPlan:
+    """Owner of a library search plan."""
+
+    def __init__(self, handle):
+        self.handle = handle
+
+    def __del__(self):
+        try:
+            lib().q4_search_plan_destroy(self.handle)
+        except Exception:       # interpreter shutdown
+            pass
+
+
 class Decoder:
     """Device copy of prediction network, joint network and both fusion LMs, the search
     state, and the iteration loop (one library call per search iteration)."""
@@ -540,6 +553,7 @@ class Decoder:
         self.concurrent = concurrent and tensor_cores
         self.state = None
         self.S_max = None
+        self._plan = None
         if share_from is not None:
             # a second search state over the same device weights (read-only, prepared operands included)
             for name in ("V", "E", "D", "pred_emb_act", "pred_emb_q", "pred_lstm", "pred_proj", "z_act", "joint_out",
@@ -657,6 +671,20 @@ class Decoder:
                                        _p(self.ws), C.c_size_t(self.ws.numel()), _stream()),
              "dr_fusion_beam_step")
 
+    def q4_beam_search(self, e: torch.Tensor, T: int, u_max: int, time_synchronous: bool = False):
+        """All steps of a search (after q4_beam_init) in one library call.  The decoder keeps a plan for it, in
+        which the library replays groups of steps as a CUDA graph (only with the streams of a concurrent state)."""
+        if self._plan is None and self.state.aux_stream[0]:
+            plan = C.c_void_p()
+            _chk(lib().q4_search_plan_create(C.byref(plan)), "q4_search_plan_create")
+            self._plan = _SearchPlan(plan)
+        plan = self._plan.handle if self._plan is not None and self.state.aux_stream[0] else None
+        dw = self.dw
+        _chk(lib().q4_beam_search(C.byref(self.model), C.byref(self.state), _p(e), C.c_int32(self.B), C.c_int32(T),
+                                  C.c_int32(self.W), C.c_int32(u_max), C.c_float(dw.lambda_t), C.c_float(dw.lambda_s),
+                                  C.c_float(dw.rho), C.c_int32(1 if time_synchronous else 0), _p(self.ws),
+                                  C.c_size_t(self.ws.numel()), plan, _stream()), "q4_beam_search")
+
     def q4_traceback(self, n_iters: int, u_max: int):
         dev = self.device
         tokens = torch.zeros((self.B, max(u_max, 1)), dtype=torch.int32, device=dev)
@@ -677,8 +705,7 @@ class Decoder:
         if self.state is None or (self.B, self.W) != (B, W) or self.n_iters < n_iters or self.S_max is not None:
             self.alloc_state(B, W, n_iters)
         self.q4_beam_init()
-        for it in range(n_iters):
-            self.dr_fusion_beam_step(e, T, it, u_max)
+        self.q4_beam_search(e, T, u_max)
         return self.q4_traceback(n_iters, u_max)
 
     def decode_time_synchronous(self, e: torch.Tensor, S_max: int, u_max: Optional[int] = None,
@@ -693,8 +720,7 @@ class Decoder:
                 self.S_max != S_max):
             self.alloc_state(B, W, n_iters, S_max)
         self.q4_beam_init()
-        for it in range(n_iters):
-            self.dr_fusion_beam_step(e, T, it, u_max, mode=2 if it % (S_max + 1) == S_max else 1)
+        self.q4_beam_search(e, T, u_max, time_synchronous=True)
         return self.q4_traceback(n_iters, u_max)
 
 

@@ -247,6 +247,13 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
   const bool normalized = a.normalized != 0;   // `logits` holds log-probabilities already
 
   pdl_wait();
+  // a replayed search: its length, budget and iteration are in memory
+  int T = a.T, u_max = a.u_max, iter = a.iter;
+  if (a.call) {
+    T = a.call->T;
+    u_max = a.call->u_max;
+    iter += a.call->iter;
+  }
   // what the proposals of slot `warp` read does not wait for the block: the joint's row at once, the language
   // models' rows as soon as the slot's state row is known
   const float* const x = a.logits + (size_t)(base + warp) * V;
@@ -269,15 +276,15 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
     s_prev[tid] = st.prev_hash[o];
     s_row[tid] = row;
     s_u[tid] = u;
-    s_lab[tid] = row >= 0 && u < a.u_max;
+    s_lab[tid] = row >= 0 && u < u_max;
   }
   if (tid == 0) {
     list_n = 0;
     // the list of pending advances consumed by this iteration is free again
-    if (b == 0) st.pend_n[a.iter & 1] = 0;
+    if (b == 0) st.pend_n[iter & 1] = 0;
   }
   if (lane < 16) s_gmax[warp][lane] = NEG;
-  const bool any_labels = __syncthreads_or(my_row >= 0 && my_u < a.u_max) != 0;
+  const bool any_labels = __syncthreads_or(my_row >= 0 && my_u < u_max) != 0;
 
   // ---- no slot of this utterance may emit a label (all at their label budget, or empty): the only
   // proposals are the blanks of the live slots, at most W of them, no two of which can describe the
@@ -291,7 +298,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
       const bool alive = w < W && s_row[w] >= 0;
       float sc = NEG;
       if (alive) sc = (float)((double)s_score[w] + (double)a.logits[(size_t)(base + w) * V]);
-      const bool fin = alive && s_t[w] + 1 == a.T;   // consumed the last frame: goes to the finished list
+      const bool fin = alive && s_t[w] + 1 == T;   // consumed the last frame: goes to the finished list
       if (__any_sync(0xffffffffu, fin)) {
         if (w < W) win_score[w] = sc;                // staging only; overwritten by the ranking below
         __syncwarp();
@@ -302,7 +309,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
           int n = st.fin_n[b];
 #pragma unroll 1
           for (int x = 0; x < W; ++x) {
-            if (s_row[x] < 0 || s_t[x] + 1 != a.T) continue;
+            if (s_row[x] < 0 || s_t[x] + 1 != T) continue;
             const float S = win_score[x];
             int pos = n;
 #pragma unroll 1
@@ -316,7 +323,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
               fl[i] = fl[i - 1];
             }
             fs[pos] = S;
-            fi[pos] = a.iter;
+            fi[pos] = iter;
             fl[pos] = x;
             n = min(n + 1, W);
           }
@@ -340,7 +347,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
   } else {
   // ---- proposals: one warp per slot
   const bool fast = MODE > 0 && !a.exact_only;   // a lower bound of the W-th best from group maxima
-  const bool my_labels = my_row >= 0 && my_u < a.u_max;
+  const bool my_labels = my_row >= 0 && my_u < u_max;
   const double s_rho = (double)my_score + (double)a.rho;
   // elements that do not count for the bound and are not collected: element 0 (blank), and labels that the merge
   // below folds into another slot's blank (lane w1 tests slot w1, the few hits are handed round the warp)
@@ -384,7 +391,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
   __syncthreads();
 
   // ---- finished hypotheses: blank proposals that consume the last frame
-  const bool any_fin = __any_sync(0xffffffffu, lane < W && s_row[lane] >= 0 && s_t[lane] + 1 == a.T);
+  const bool any_fin = __any_sync(0xffffffffu, lane < W && s_row[lane] >= 0 && s_t[lane] + 1 == T);
   if (any_fin) {   // uniform for the block
     if (tid == 0) {
       float* fs = st.fin_score + base;
@@ -393,7 +400,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
       int n = st.fin_n[b];
 #pragma unroll 1
       for (int w = 0; w < W; ++w) {
-        if (s_row[w] < 0 || s_t[w] + 1 != a.T) continue;
+        if (s_row[w] < 0 || s_t[w] + 1 != T) continue;
         const float S = s_blank[w];
         s_blank[w] = NEG;
         int pos = n;
@@ -408,7 +415,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
           fl[i] = fl[i - 1];
         }
         fs[pos] = S;
-        fi[pos] = a.iter;
+        fi[pos] = iter;
         fl[pos] = w;
         n = min(n + 1, W);
       }
@@ -459,12 +466,12 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
     const unsigned lab = __ballot_sync(0xffffffffu, is_label);
     // reserve a range of the next iteration's pending list for this utterance's label extensions
     int pbase = 0;
-    if (lane == 0 && lab != 0u) pbase = atomicAdd(st.pend_n + ((a.iter + 1) & 1), __popc(lab));
+    if (lane == 0 && lab != 0u) pbase = atomicAdd(st.pend_n + ((iter + 1) & 1), __popc(lab));
     pbase = __shfl_sync(0xffffffffu, pbase, 0);
-    const size_t poff = (size_t)((a.iter + 1) & 1) * N;
+    const size_t poff = (size_t)((iter + 1) & 1) * N;
     if (s < W) {
       const int o = base + s;
-      const size_t hist = ((size_t)a.iter * a.B + b) * W + s;
+      const size_t hist = ((size_t)iter * a.B + b) * W + s;
       if (s < nw) {
         st.score[o] = win_score[s];
         if (!is_label) {
@@ -581,12 +588,19 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_tsd_select(const __grid_constant_
   const int N = a.B * W;
   const int S = st.tsd_smax;
   const int CB = W * (S + 1);
-  const int step = a.iter % (S + 1), frame = a.iter / (S + 1);
   const bool inner = a.mode == 1;
   const int RW = st.rows_per_utt;
   const bool fast = inner && MODE > 0 && !a.exact_only;   // as in k_beam_select
 
   pdl_wait();
+  // a replayed search: its length, budget and iteration are in memory
+  int T = a.T, u_max = a.u_max, iter = a.iter;
+  if (a.call) {
+    T = a.call->T;
+    u_max = a.call->u_max;
+    iter += a.call->iter;
+  }
+  const int step = iter % (S + 1), frame = iter / (S + 1);
   const float* const x = a.logits + (size_t)(base + warp) * V;
   float v[32];
   int my_row = -1, my_u = 0;
@@ -605,7 +619,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_tsd_select(const __grid_constant_
     s_last[tid] = st.last_tok[o];
     s_hash[tid] = st.hash[o];
     s_prev[tid] = st.prev_hash[o];
-    s_lab[tid] = inner && s_row[tid] >= 0 && s_u[tid] < a.u_max;   // a frame close proposes blanks only
+    s_lab[tid] = inner && s_row[tid] >= 0 && s_u[tid] < u_max;   // a frame close proposes blanks only
   }
   const int cn0 = st.nb_n[b];
 #pragma unroll 1
@@ -622,13 +636,13 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_tsd_select(const __grid_constant_
   if (tid == 0) {
     list_n = 0;
     c_n = cn0;
-    if (b == 0) st.pend_n[a.iter & 1] = 0;   // the list consumed by this call is free again
+    if (b == 0) st.pend_n[iter & 1] = 0;   // the list consumed by this call is free again
   }
   if (lane < 16) s_gmax[warp][lane] = NEG;
   __syncthreads();
 
   // ---- proposals: one warp per slot
-  const bool my_labels = inner && my_row >= 0 && my_u < a.u_max;
+  const bool my_labels = inner && my_row >= 0 && my_u < u_max;
   const double s_rho = (double)my_score + (double)a.rho;
   const uint32_t skip = lane == 0 ? 1u : 0u;   // element 0 is the blank
   if (warp < W && my_row < 0 && lane == 0) s_blank[warp] = NEG;
@@ -724,12 +738,12 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_tsd_select(const __grid_constant_
         }
       }
       int pbase = 0;
-      if (lane == 0 && nw > 0) pbase = atomicAdd(st.pend_n + ((a.iter + 1) & 1), nw);
+      if (lane == 0 && nw > 0) pbase = atomicAdd(st.pend_n + ((iter + 1) & 1), nw);
       pbase = __shfl_sync(0xffffffffu, pbase, 0);
-      const size_t poff = (size_t)((a.iter + 1) & 1) * N;
+      const size_t poff = (size_t)((iter + 1) & 1) * N;
       if (s < W) {
         const int o = base + s;
-        const size_t hist = ((size_t)a.iter * a.B + b) * W + s;
+        const size_t hist = ((size_t)iter * a.B + b) * W + s;
         if (s < nw && f >= 0) {
           const int idx = win_idx[s];
           const int w = idx / V, k = idx % V;
@@ -785,7 +799,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_tsd_select(const __grid_constant_
       for (int j = 0; j < n; ++j) rank += (c_score[j] > mine) || (c_score[j] == mine && j < tid);
       if (rank < W) {
         const int o = base + rank;
-        const size_t hist = ((size_t)a.iter * a.B + b) * W + rank;
+        const size_t hist = ((size_t)iter * a.B + b) * W + rank;
         st.score[o] = mine;
         st.t[o] = frame + 1;
         st.u[o] = c_u[tid];
@@ -799,16 +813,16 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_tsd_select(const __grid_constant_
         st.bp_parent[hist] = c_org[tid] & 0xFF;
         st.bp_token[hist] = -1 - (c_org[tid] >> 8);
         st.bp_score[hist] = mine;
-        if (frame + 1 == a.T) {
+        if (frame + 1 == T) {
           st.fin_score[base + rank] = mine;
-          st.fin_iter[base + rank] = a.iter + 1;
+          st.fin_iter[base + rank] = iter + 1;
           st.fin_slot[base + rank] = rank;
         }
       }
     }
     if (tid >= nw && tid < W) {
       const int o = base + tid;
-      const size_t hist = ((size_t)a.iter * a.B + b) * W + tid;
+      const size_t hist = ((size_t)iter * a.B + b) * W + tid;
       st.row[o] = -1;
       st.adv_src[o] = -1;
       st.adv_dst[o] = -1;
@@ -819,7 +833,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_tsd_select(const __grid_constant_
     }
     if (tid == 0) {
       st.nb_n[b] = 0;
-      if (frame + 1 == a.T) st.fin_n[b] = nw;
+      if (frame + 1 == T) st.fin_n[b] = nw;
     }
   }
 }
@@ -919,6 +933,24 @@ __global__ void k_beam_init(q4_beam_state st, int B, int W) {
     st.pend_n[0] = B;
     st.pend_n[1] = 0;
   }
+}
+
+__global__ void k_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter) {
+  call->e = e;
+  call->T = T;
+  call->u_max = u_max;
+  call->iter = iter;
+}
+__global__ void k_search_advance(SearchCall* call, int iters) { call->iter += iters; }
+cudaError_t launch_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter, cudaStream_t s) {
+  k_search_begin<<<1, 1, 0, s>>>(call, e, T, u_max, iter);
+  ++g_launches;
+  return cudaGetLastError();
+}
+cudaError_t launch_search_advance(SearchCall* call, int iters, cudaStream_t s) {
+  k_search_advance<<<1, 1, 0, s>>>(call, iters);
+  ++g_launches;
+  return cudaGetLastError();
 }
 
 cudaError_t launch_beam_init(const q4_beam_state& st, int B, int W, int n_iters, cudaStream_t s) {

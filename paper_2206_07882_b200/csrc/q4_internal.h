@@ -12,13 +12,23 @@ cudaError_t launch_logsoftmax(const float* in, float* out, int rows, int V, long
 cudaError_t launch_joint_z(const float* e, const int32_t* frame_idx, const int32_t* t_arr, int B,
                            int W, const float* p, const int32_t* p_idx, int N, int D,
                            const q4_act& za, uint8_t* zq, int8_t* z8, int32_t* live_out,
-                           cudaStream_t s, bool dependent = false);
+                           cudaStream_t s, bool dependent = false, const struct SearchCall* call = nullptr);
 cudaError_t launch_quantize(const void* x, bool fp16, long long rows, int k, int k_pad,
                             const q4_act& a, int mode, int n_groups, const float* scale_vec,
                             uint8_t* out, float* group_scale_out, cudaStream_t s);
 cudaError_t launch_features(const float* mel, int B, int T100, int M, void* out, cudaStream_t s);
 
+// What changes from one search to the next, in device memory: the steps of a replayed search read it there
+// (null pointer: the launch's own arguments count).
+struct SearchCall {
+  const float* e;           // projected encoder frames
+  int32_t T, u_max;
+  int32_t iter;             // added to the launch's iteration number
+};
+cudaError_t launch_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter, cudaStream_t s);
+cudaError_t launch_search_advance(SearchCall* call, int iters, cudaStream_t s);
 struct BeamSelArgs {
+  const SearchCall* call;
   const float* logits;      // [B*W, V] joint logits (bias included), rows of empty slots ignored
   const float* src_lp;      // [R, V]
   const float* tgt_lp;      // [R, V]
@@ -50,6 +60,7 @@ void timing_begin(cudaStream_t s);
 void timing_end(cudaStream_t s);
 void timing_set(uint32_t mask, cudaEvent_t* start, cudaEvent_t* stop, int32_t* tags, int cap);
 int timing_count();
+bool timing_active();
 
 // ---- tensor-core path (q4_mma.cu)
 struct MmaLstmArgs {

@@ -47,6 +47,7 @@ void timing_set(uint32_t mask, cudaEvent_t* start, cudaEvent_t* stop, int32_t* t
   g_timing.open = false;
 }
 int timing_count() { return g_timing.n; }
+bool timing_active() { return g_timing.mask != 0; }
 
 // =====================================================================================
 // Integer tile GEMM: acc[m, j] = sum_k W[j,k] * (x[m,k] - z).  64 x 64 outputs per CTA,
@@ -458,9 +459,10 @@ cudaError_t launch_logsoftmax(const float* in, float* out, int rows, int V, long
 __global__ void __launch_bounds__(256) k_joint_z(const float* e, const int32_t* frame_idx,
                                                  const int32_t* t_arr, int B, int W, const float* p,
                                                  const int32_t* p_idx, int N, int D, q4_act za,
-                                                 uint8_t* zq, int8_t* z8, int32_t* live_out) {
+                                                 uint8_t* zq, int8_t* z8, int32_t* live_out, const SearchCall* call) {
   pdl_trigger();
   pdl_wait();
+  if (call) e = call->e;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int half = D >> 1;
   if (i >= (long long)N * half) return;
@@ -489,12 +491,12 @@ __global__ void __launch_bounds__(256) k_joint_z(const float* e, const int32_t* 
 cudaError_t launch_joint_z(const float* e, const int32_t* frame_idx, const int32_t* t_arr, int B,
                            int W, const float* p, const int32_t* p_idx, int N, int D,
                            const q4_act& za, uint8_t* zq, int8_t* z8, int32_t* live_out,
-                           cudaStream_t s, bool dependent) {
+                           cudaStream_t s, bool dependent, const SearchCall* call) {
   if (N <= 0) return cudaSuccess;
   const long long total = (long long)N * (D / 2);
   timing_begin(s);
   cudaError_t le = launch_ex(k_joint_z, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, s, dependent, 1, e,
-                             frame_idx, t_arr, B, W, p, p_idx, N, D, za, zq, z8, live_out);
+                             frame_idx, t_arr, B, W, p, p_idx, N, D, za, zq, z8, live_out, call);
   timing_end(s);
   ++g_launches;
   return le != cudaSuccess ? le : cudaGetLastError();

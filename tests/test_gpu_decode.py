@@ -409,6 +409,28 @@ def test_time_synchronous_search_small(Bd, S_max, W):
     assert compare_tsd(dd, tokens, lens, scores, ref, list(range(6)), 10, S_max, W) == 1.0
 
 
+@pytest.mark.parametrize("S", [None, 0, 1, 2, 3])
+def test_replayed_search_equals_its_steps(Bd, S):
+    # searches on one state, long, short, long with other frames (the same graph serves them), then another batch
+    # size (built anew): bit-identical to the steps called one by one
+    dw = synth.decoder(seed=67, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=9, W=6)
+    a, b = Bd.Decoder(dw), Bd.Decoder(dw)
+    for B, T, U in ((3, 111, 9), (3, 97, 5), (3, 111, 9), (5, 98, 0)):
+        e = torch.from_numpy(synth.Stream(T + B + U).normal("e", (T, B, 256)).astype(np.float32)).cuda()
+        n = T + U if S is None else T * (S + 1)
+        got = a.decode(e, U) if S is None else a.decode_time_synchronous(e, S, U)
+        b.alloc_state(B, 6, n, S)
+        b.q4_beam_init()
+        for it in range(n):
+            b.dr_fusion_beam_step(e, T, it, U, mode=0 if S is None else 2 if it % (S + 1) == S else 1)
+        want = b.q4_traceback(n, U)
+        for x, y in zip(got, want):
+            assert torch.equal(x, y)
+        assert a.tensors["status"].item() == 0 and torch.equal(a.tensors["fin_n"], b.tensors["fin_n"])
+        for k in ("bp_parent", "bp_token", "bp_score"):
+            assert torch.equal(a.tensors[k][:n], b.tensors[k]), k
+
+
 def test_time_synchronous_search_tensor_core_path(Bd):
     # 8 utterances x 16 slots = 128 rows and a 256-wide bottleneck: tensor-core LSTMs and cluster heads
     dw = synth.decoder(seed=83, V=128, E=32, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=9, W=16)
