@@ -424,7 +424,7 @@ int q4_encoder_time_slicing_set(int32_t enabled);
 /* How qlstm_layer_forward lays a layer's recurrence on thread-block clusters (host logic only, no
  * launch; for tests and diagnostics; with no device present the cluster capacity defaults to 15).
  * out[17]: [0] kernel (0 general, 1 packed 4-bit weights in registers, 2 the kernel whose clusters
- * may take turns), [1] groups of 8 sequences per cluster, [2..3] clusters per direction, [4..5]
+ * may take turns, 3 few groups on clusters of up to 16 CTAs), [1] groups of 8 sequences per cluster, [2..3] clusters per direction, [4..5]
  * whether the direction's clusters take turns at its last group, [6] groups per direction, [7]
  * clusters that can be resident, [8..16] step bounds of the turns: cluster j of such a direction
  * advances the shared group over steps [out[8+j], out[9+j]).  Assumes a signed hidden quantizer,

@@ -233,7 +233,8 @@ int enc_recurrent_sliced_set(int enabled);   // returns the previous setting
 // Which recurrence kernel a layer takes and how its groups of sequences are laid on clusters (host only).
 struct EncRecPlan {
   int32_t kernel;           // 0: general kernel (int8 weights in shared memory), 1: packed weights in registers,
-                            // groups_per_cluster groups per cluster, 2: kernel whose clusters may take turns
+                            // groups_per_cluster groups per cluster, 2: kernel whose clusters may take turns,
+                            // 3: few groups, int8 fragments in registers, clusters of up to 16 CTAs
   int32_t groups_per_cluster;
   int32_t ncl[2], sliced[2], groups, max_clusters;
   int32_t win[9];

@@ -949,6 +949,219 @@ k_enc_recurrent_w4s(const EncRecArgs a) {
   if (live_shared && w1 == T && D.c_n) D.c_n[(size_t)b_shared * H + cell] = c_shared;
 }
 
+// ---------------------------------------------------------------------------------------------
+// The recurrence of few groups of sequences, one group of 8 per cluster, spread as wide as a cluster goes.
+//
+// A step of k_enc_recurrent_w4 (8 CTAs of 640 threads) spends 3900 cycles: 1330 multiplying and 1040 in the cell update,
+// both bound by issue slots (5 warps on every scheduler), 200 staging, 1330 until the other CTAs' codes are here.
+// With 16 CTAs a cluster each SM has half of the first two; while all clusters find their SMs, that is the better
+// split: one step of 640 cells 1.87 -> 1.42 us (1 utterance, 152 frames x 6 layers: 1.71 -> 1.30 ms; 11 utterances, 173
+// frames: 2.14 -> 1.50 ms; 8-bit weights 2.06 -> 1.30 ms).  From the eighth group on two clusters would share SMs, and
+// the kernels with 8 CTAs a cluster take over.  Layers of at most 128 cells need no cluster at all: 1.72 -> 1.43
+// us a step (128 cells).  (Codes sent as 16-byte st.async by all threads instead of one bulk copy per CTA: 1.44, and
+// 1.55 instead of 1.44 with two groups per direction.)
+//
+// A CTA owns cpc = H / CL cells, a warp 4 of them: its 16 weight rows stay in registers as the int8 A fragments
+// they are (4 registers per 32 columns), whatever the stored width.  Hidden codes lie in units of 8 cells,
+// [unit][sequence][8 codes], so that a lane's B fragment of a 32-column step is one 8-byte word, the 32 lanes' words
+// are 256 consecutive bytes, and a CTA's new codes are one block of every receiver's buffer.  Which column an
+// operand register stands for is immaterial to the sums: lane t4's are the 8 columns of its unit.  Tile rows
+// and items as in k_enc_recurrent_w4; a lane's item is fixed, so its de-quantization products (with a scale
+// per sequence or one for all) stay in registers.  CL = 1: the codes go straight into the next buffer and a block
+// barrier ends the step.
+template <int KS, int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(8 * 32 * KS / CL, 1)
+k_enc_recurrent_few(const EncRecArgs a) {
+  extern __shared__ __align__(16) uint8_t rec_smem[];
+  constexpr int BG = REC_BG, H = 32 * KS, G = 4 * H;
+  constexpr int cpc = H / CL;               // cells per CTA
+  constexpr int NTHR = 8 * cpc, CW = NTHR / 32;
+  constexpr int UB = BG * H, MB = BG * cpc; // bytes of the group's hidden codes, of this CTA's part
+  static_assert(cpc % 8 == 0 && NTHR <= 1024, "units of 8 cells, one item per thread");
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = CL == 1 ? 0u : cluster_rank();
+  const int cid = blockIdx.x / CL;
+  const int d = cid / a.n_groups, grp = cid % a.n_groups;
+  const EncRecDir& D = a.d[d];
+  const int T = a.T, B = a.B;
+  int8_t* hb = reinterpret_cast<int8_t*>(rec_smem);      // [2][H / 8][BG][8] h_{t-1}
+  int8_t* stage = hb + 2 * UB;                           // [2][cpc / 8][BG][8] new recurrent codes
+  int8_t* stage_y = stage + 2 * MB;                      // [2][cpc / 8][BG][8] new output codes
+  uint64_t* full = reinterpret_cast<uint64_t*>(stage_y + 2 * MB);
+  volatile int* dead = reinterpret_cast<volatile int*>(full + 2);
+
+  const int g = lane >> 2, t4 = lane & 3;   // MMA fragment coordinates
+  const int e = g & 1, ci = g >> 1;         // this lane's item: cell ci of the warp's 4 ...
+  const int n = 2 * t4 + e;                 // ... and sequence n of the group's 8
+  const int cl = warp * 4 + ci;             // cell within the CTA
+  const int cell = (int)rank * cpc + cl;    // cell within the layer
+  const int b = grp * BG + n;
+  const bool live = b < B;
+
+  // tile row g = gate e of cell ci, tile row g + 8 = gate 2 + e (weight rows are stored in 4*cell+gate order)
+  uint32_t w[4 * KS];
+  {
+    const int8_t* r0 = D.w_hh + (size_t)(4 * cell + e) * H + 8 * t4;
+    const int8_t* r1 = r0 + (size_t)2 * H;
+#pragma unroll
+    for (int s = 0; s < KS; ++s) {
+      const uint2 p = *reinterpret_cast<const uint2*>(r0 + 32 * s), q = *reinterpret_cast<const uint2*>(r1 + 32 * s);
+      w[4 * s] = p.x;
+      w[4 * s + 1] = q.x;
+      w[4 * s + 2] = p.y;
+      w[4 * s + 3] = q.y;
+    }
+  }
+  float4 s_ih = reinterpret_cast<const float4*>(D.sc_ih)[cell], s_hh = reinterpret_cast<const float4*>(D.sc_hh)[cell];
+  const float4 bb = reinterpret_cast<const float4*>(D.bias)[cell];
+  {
+    const float sx = a.x_scale_b && live ? a.x_scale_b[b] : a.x_scale, sh = a.hid_act.scale;
+    s_ih = make_float4(__fmul_rn(sx, s_ih.x), __fmul_rn(sx, s_ih.y), __fmul_rn(sx, s_ih.z), __fmul_rn(sx, s_ih.w));
+    s_hh = make_float4(__fmul_rn(sh, s_hh.x), __fmul_rn(sh, s_hh.y), __fmul_rn(sh, s_hh.z), __fmul_rn(sh, s_hh.w));
+  }
+  for (int i = tid; i < 2 * UB / 16; i += NTHR) reinterpret_cast<uint4*>(hb)[i] = make_uint4(0, 0, 0, 0);   // h_0 = 0
+  if (CL > 1 && tid == 0) {
+    *dead = 0;
+    for (int i = 0; i < 2; ++i) mbar_init(&full[i], 1);
+    fence_barrier_init();
+    for (int i = 0; i < 2; ++i) mbar_expect_tx(&full[i], (uint32_t)UB);   // the first fill of either buffer
+  }
+  fence_proxy_async();   // the zeroed buffers are later written by the bulk-copy engine
+  __syncthreads();
+  if (CL > 1) cluster_barrier();   // every CTA's buffers and barriers are initialised before anyone stores into them
+  pdl_wait();            // the input accumulators are the previous kernel's output; the weights that of the one before it
+
+  const uint32_t hb_addr = smem_u32(hb), full_addr = smem_u32(full);
+  const int hlo = act_lo(a.hid_act), hhi = act_hi(a.hid_act);
+  const int ylo = act_lo(a.out_act), yhi = act_hi(a.out_act);
+  const bool y4 = a.out_act.bits == 4;
+  const int at = (cl >> 3) * 64 + n * 8 + (cl & 7);      // my code within the CTA's part
+  float c_state = 0.0f;
+  int q = 0;
+  // input accumulators of my item, fetched one step ahead
+  const long long pstep = (d == 0 ? 1LL : -1LL) * B * G;
+  const int32_t* pre_p = D.acc_pre + ((size_t)(d == 0 ? 0 : T - 1) * B + (live ? b : 0)) * G + 4 * cell;
+  int4 pre_next = make_int4(0, 0, 0, 0);
+  if (live && T > 0) pre_next = *reinterpret_cast<const int4*>(pre_p);
+  bool ok = true;
+  for (int step = 0; step < T; ++step) {
+    const int t = d == 0 ? step : T - 1 - step;
+    const int cur = step & 1, nxt = cur ^ 1;
+    const int4 pre = pre_next;
+    pre_p += pstep;
+    if (live && step + 1 < T) pre_next = *reinterpret_cast<const int4*>(pre_p);
+    // h_{t-1} is complete here once every CTA's copy has landed; waits, their limit and the order of buffers as in
+    // k_enc_recurrent_w4
+    if (CL > 1 && step > 0 && ok) {
+      uint64_t* bar = &full[cur];
+      const uint32_t parity = (uint32_t)(((step - 1) >> 1) & 1);
+      bool got = false;
+      for (uint32_t i = 0; i < (1u << 22); ++i) {
+        if (mbar_try_wait(bar, parity)) {
+          got = true;
+          break;
+        }
+        if ((i & 255u) == 255u && *dead) break;
+      }
+      if (!got) {
+        ok = false;
+        *dead = 1;
+        if (a.status) atomicExch(a.status, Q4_ERR_TIMEOUT);
+      }
+      if (tid == 0 && got) mbar_expect_tx(bar, (uint32_t)UB);   // armed for the next fill of this buffer
+    }
+    int acc[2][4];
+#pragma unroll
+    for (int c = 0; c < 2; ++c)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) acc[c][r] = 0;
+    const int8_t* hrow = hb + cur * UB + t4 * 64 + g * 8;
+#pragma unroll
+    for (int s = 0; s < KS; ++s) {
+      const uint2 v = *reinterpret_cast<const uint2*>(hrow + 256 * s);
+      mma_s8(acc[s & 1], w[4 * s], w[4 * s + 1], w[4 * s + 2], w[4 * s + 3], v.x, v.y);
+    }
+    // the four gates of my item: two of them come from lane ^ 4
+    int hh[4];
+    {
+      const int v0 = acc[0][0] + acc[1][0], v1 = acc[0][1] + acc[1][1];
+      const int v2 = acc[0][2] + acc[1][2], v3 = acc[0][3] + acc[1][3];
+      const int r0 = __shfl_xor_sync(0xffffffffu, e ? v0 : v1, 4);
+      const int r1 = __shfl_xor_sync(0xffffffffu, e ? v2 : v3, 4);
+      const int m0 = e ? v1 : v0, m1 = e ? v3 : v2;
+      hh[0] = e ? r0 : m0;
+      hh[1] = e ? m0 : r0;
+      hh[2] = e ? r1 : m1;
+      hh[3] = e ? m1 : r1;
+    }
+    int q2 = 0;
+    if (live) {
+      const float pi = __fmaf_rn((float)hh[0], s_hh.x, __fmaf_rn((float)pre.x, s_ih.x, bb.x));
+      const float pf = __fmaf_rn((float)hh[1], s_hh.y, __fmaf_rn((float)pre.y, s_ih.y, bb.y));
+      const float pg = __fmaf_rn((float)hh[2], s_hh.z, __fmaf_rn((float)pre.z, s_ih.z, bb.z));
+      const float po = __fmaf_rn((float)hh[3], s_hh.w, __fmaf_rn((float)pre.w, s_ih.w, bb.w));
+      float hval;
+      cell_fixed_p(pi, pf, pg, po, c_state, c_state, hval);
+      q = quantize1(hval, a.hid_act.inv_scale, a.hid_act.zero_point, hlo, hhi);
+      q2 = quantize1(hval, a.out_act.inv_scale, a.out_act.zero_point, ylo, yhi);
+    }
+    (CL == 1 ? hb + nxt * UB : stage + cur * MB)[at] = (int8_t)q;
+    stage_y[cur * MB + at] = (int8_t)q2;
+    if (CL > 1) fence_proxy_async();   // the staged codes are read by the bulk-copy engine
+    // One warp, a different one every step, waits until all threads have stored their codes, sends them to every CTA and
+    // writes this CTA's share of the layer output
+    const bool mine = warp == step % CW;
+    if (CL == 1) {
+      __syncthreads();
+    } else if (!mine) {
+      named_bar_arrive(1 + cur, NTHR);
+    } else {
+      named_bar_sync(1 + cur, NTHR);
+      if (lane < CL)
+        bulk_copy_to_cluster(map_to_rank(hb_addr + (uint32_t)(nxt * UB + (int)rank * MB), (uint32_t)lane),
+                             smem_u32(stage + cur * MB), (uint32_t)MB, map_to_rank(full_addr + (uint32_t)(nxt * 8), (uint32_t)lane));
+    }
+    if (mine) {
+      for (int i = lane; i < MB / 8; i += 32) {
+        const int bl = i & 7, by = grp * BG + bl, c0 = (int)rank * cpc + (i & ~7);
+        if (by >= B) continue;
+        const uint2 v = *reinterpret_cast<const uint2*>(stage_y + cur * MB + i * 8);
+        uint8_t* y = D.yq + ((size_t)t * B + by) * a.yq_ld;
+        if (y4) {
+          auto pk = [](uint32_t x) -> uint32_t {   // bytes (c, c+1) -> one byte: low nibble c, high nibble c+1
+            const uint32_t m = (x & 0x000F000Fu) | ((x >> 4) & 0x00F000F0u);
+            return (m & 0xFFu) | ((m >> 8) & 0xFF00u);
+          };
+          *reinterpret_cast<uint32_t*>(y + (c0 >> 1)) = pk(v.x) | (pk(v.y) << 16);
+        } else {
+          *reinterpret_cast<uint2*>(y + c0) = v;
+        }
+      }
+    }
+  }
+  pdl_trigger();
+  // the codes sent in the last step are still on their way: nobody leaves before they have landed (bounded)
+  if (CL > 1) {
+    if (T > 0) {
+      const uint32_t parity = (uint32_t)(((T - 1) >> 1) & 1);
+      for (uint32_t i = 0; i < (1u << 22); ++i) {
+        if (mbar_try_wait(&full[T & 1], parity)) break;
+        if ((i & 255u) == 255u && *dead) break;
+      }
+    }
+    __syncthreads();
+    cluster_barrier();
+  }
+  // final states
+  if (D.hq_n) {
+    const int qn = __shfl_down_sync(0xffffffffu, q, 8);   // the next cell, same sequence
+    if (live && a.hid_act.bits == 8) D.hq_n[(size_t)b * H + cell] = (uint8_t)(q & 0xFF);
+    if (live && a.hid_act.bits == 4 && (cl & 1) == 0)
+      D.hq_n[(size_t)b * (H >> 1) + (cell >> 1)] = (uint8_t)((q & 0xF) | ((qn & 0xF) << 4));
+  }
+  if (live && D.c_n) D.c_n[(size_t)b * H + cell] = c_state;
+}
+
 constexpr size_t REC_SMEM_MAX = 232448 - 128;   // 227 KB per CTA on sm_100, minus a margin
 
 size_t enc_recurrent_smem(int H, int BG) {
@@ -1095,6 +1308,26 @@ static cudaError_t rec_w4_launch(const EncRecArgs& a, cudaStream_t s) {
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// A CTA of the kernel for few groups has an SM to itself: with 16 CTAs a cluster that makes 7 clusters (of the 8 GPCs
+// one has fewer than 16 SMs to spare).
+constexpr size_t REC_FEW_SMEM = 120 * 1024;
+constexpr int REC_FEW_CLUSTERS = 7;
+
+template <int KS, int CL>
+static cudaError_t rec_few_launch(const EncRecArgs& a, cudaStream_t s) {
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e = cudaFuncSetAttribute(k_enc_recurrent_few<KS, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)REC_FEW_SMEM);
+    if (e == cudaSuccess && CL > 8)
+      e = cudaFuncSetAttribute(k_enc_recurrent_few<KS, CL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  const cudaError_t e = launch_ex(k_enc_recurrent_few<KS, CL>, dim3((unsigned)(a.dirs * a.n_groups * CL)), dim3(8 * 32 * KS / CL),
+                                  REC_FEW_SMEM, s, true, 1, a);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid_bits, bool hid_signed,
                               bool per_sequence_scale, bool dump, bool scratch) {
   EncRecPlan p;
@@ -1103,6 +1336,14 @@ EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid
   p.groups = groups;
   p.max_clusters = rec_max_clusters(H);
   if (H == 640) p.max_clusters = p.max_clusters < rec_turns_max_clusters() ? p.max_clusters : rec_turns_max_clusters();
+  const bool few_h = H == 64 || H == 128 || H == 256 || H == 320 || H == 512 || H == 640;
+  if (few_h && hid_signed && !dump && (hid_bits == 4 || hid_bits == 8) && dirs * groups <= REC_FEW_CLUSTERS) {
+    p.kernel = 3;
+    p.groups_per_cluster = 1;
+    p.ncl[0] = groups;
+    p.ncl[1] = dirs == 2 ? groups : 0;
+    return p;
+  }
   // 640 cells, no accumulator dump: the kernels that keep (most of) a CTA's recurrent weights in
   // registers; the general kernel otherwise
   const bool regs_ok = hid_signed && H == 640 && !dump && (w_bits == 4 || w_bits == 8) && (hid_bits == 4 || hid_bits == 8);
@@ -1145,6 +1386,22 @@ cudaError_t launch_enc_recurrent(EncRecArgs a, cudaStream_t s) {
   const EncRecPlan p = enc_recurrent_plan(a.T, a.B, a.dirs, a.H, a.w_bits, a.hid_act.bits, a.hid_act.is_signed != 0,
                                           a.x_scale_b != nullptr, a.d[0].dbg_ih != nullptr,
                                           a.flags && a.hand_h[0] && a.hand_c[0]);
+  if (p.kernel == 3) {
+    a.n_groups = p.groups;
+    timing_begin(s);
+    cudaError_t e = cudaErrorInvalidValue;
+    switch (a.H) {
+      case 64: e = rec_few_launch<2, 1>(a, s); break;
+      case 128: e = rec_few_launch<4, 1>(a, s); break;
+      case 256: e = rec_few_launch<8, 8>(a, s); break;
+      case 320: e = rec_few_launch<10, 8>(a, s); break;
+      case 512: e = rec_few_launch<16, 16>(a, s); break;
+      case 640: e = rec_few_launch<20, 16>(a, s); break;
+    }
+    timing_end(s);
+    ++g_launches;
+    return e;
+  }
   if (p.kernel == 2) {
     a.groups = p.groups;
     for (int d = 0; d < 2; ++d) {

@@ -155,6 +155,16 @@ def test_layer_shapes_directions_precisions(Bd, T, B, K, H, dirs, xb, hb, ob):
     layer_case(Bd, T, B, K, H, dirs, xb, hb, ob, seed=11)
 
 
+@pytest.mark.parametrize("T,B,K,H,dirs,xb,hb,ob", [(40, 5, 32, 64, 2, 4, 4, 4), (130, 1, 64, 128, 1, 4, 4, 8),
+                                                   (16, 9, 32, 128, 2, 8, 8, 4), (17, 9, 32, 256, 2, 8, 8, 4),
+                                                   (20, 9, 32, 320, 1, 4, 4, 4), (44, 3, 32, 512, 2, 8, 8, 8),
+                                                   (7, 24, 32, 640, 2, 4, 4, 8), (6, 50, 32, 640, 1, 8, 8, 4)])
+def test_layer_few_groups(Bd, T, B, K, H, dirs, xb, hb, ob):
+    # every width the kernel for few groups is built for; ragged and full groups, all 7 clusters, odd and even T
+    assert Bd.encoder_recurrence_plan(T, B, dirs, H, w_bits=hb, hid_bits=hb)["kernel"] == 3
+    layer_case(Bd, T, B, K, H, dirs, xb, hb, ob, seed=29)
+
+
 def test_layer_clusters_taking_turns_at_a_surplus_group(Bd):
     # 57 sequences x 2 directions of 640 cells = 16 groups of 8 for the 15 clusters that fit: the seven
     # clusters of one direction take turns at its eighth group (9 of 64 steps each, one more on the
@@ -193,7 +203,7 @@ def test_layer_time_slicing_equals_two_groups_per_cluster(Bd):
 @pytest.mark.parametrize("T,B,K,H", [(8, 5, 64, 32),
                                      # 640 cells: int8 weights mostly in registers; 20 sequences = one group per
                                      # cluster, 57 over 64 steps = the clusters of one direction take turns
-                                     (8, 20, 64, 640), (64, 57, 64, 640)])
+                                     (8, 20, 64, 640), (64, 57, 64, 640), (9, 30, 64, 640), (70, 2, 64, 128)])
 def test_layer_per_sequence_input_scale(Bd, T, B, K, H):
     w = synth.single_layer(seed=5, T=T, B=B, K=K, H=H, bits=8, dirs=2)
     base = O.act_symmetric(1.0, 8)
