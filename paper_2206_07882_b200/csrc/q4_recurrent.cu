@@ -949,17 +949,25 @@ k_enc_recurrent_w4s(const EncRecArgs a) {
   if (live_shared && w1 == T && D.c_n) D.c_n[(size_t)b_shared * H + cell] = c_shared;
 }
 
+// 16 bytes into another CTA's shared memory, counted on that CTA's mbarrier
+__device__ __forceinline__ void st_async_v4(uint32_t addr, uint4 v, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(addr), "r"(v.x),
+               "r"(v.y), "r"(v.z), "r"(v.w), "r"(bar)
+               : "memory");
+}
+
 // ---------------------------------------------------------------------------------------------
 // The recurrence of few groups of sequences, one group of 8 per cluster, spread as wide as a cluster goes.
 //
 // A step of k_enc_recurrent_w4 (8 CTAs of 640 threads) spends 3900 cycles: 1330 multiplying and 1040 in the cell update,
 // both bound by issue slots (5 warps on every scheduler), 200 staging, 1330 until the other CTAs' codes are here.
-// With 16 CTAs a cluster each SM has half of the first two; while all clusters find their SMs, that is the better
-// split: one step of 640 cells 1.87 -> 1.42 us (1 utterance, 152 frames x 6 layers: 1.71 -> 1.30 ms; 11 utterances, 173
-// frames: 2.14 -> 1.50 ms; 8-bit weights 2.06 -> 1.30 ms).  From the eighth group on two clusters would share SMs, and
-// the kernels with 8 CTAs a cluster take over.  Layers of at most 128 cells need no cluster at all: 1.72 -> 1.43
-// us a step (128 cells).  (Codes sent as 16-byte st.async by all threads instead of one bulk copy per CTA: 1.44, and
-// 1.55 instead of 1.44 with two groups per direction.)
+// With 16 CTAs a cluster each SM has half of the first two, with 10 four fifths; while all clusters find their SMs (7 of
+// 16, 11 of 10) that is the better split.  Narrower layers take clusters of 32 or 40 cells per CTA.  The codes travel as
+// 16-byte st.async stores, a destination's on consecutive lanes: an exchange alone takes 840 cycles among 16 CTAs, against
+// 1270 as one bulk copy per destination (the engine takes them one by one) and 1300 with a lane's destinations
+// interleaved.  Whole encoders of 6 layers: 11 utterances x 173 frames 2.27 -> 1.50 ms (16 CTAs; 1.62 with bulk
+// copies), 32 x 500 6.65 -> 6.06 ms (10 CTAs); one layer of 128 cells, 50 steps with its projection: 92 -> 44 us (4 CTAs; 76
+// on one CTA without any exchange, whose 32 warps are bound by issue slots).
 //
 // A CTA owns cpc = H / CL cells, a warp 4 of them: its 16 weight rows stay in registers as the int8 A fragments
 // they are (4 registers per 32 columns), whatever the stored width.  Hidden codes lie in units of 8 cells,
@@ -967,8 +975,7 @@ k_enc_recurrent_w4s(const EncRecArgs a) {
 // are 256 consecutive bytes, and a CTA's new codes are one block of every receiver's buffer.  Which column an
 // operand register stands for is immaterial to the sums: lane t4's are the 8 columns of its unit.  Tile rows
 // and items as in k_enc_recurrent_w4; a lane's item is fixed, so its de-quantization products (with a scale
-// per sequence or one for all) stay in registers.  CL = 1: the codes go straight into the next buffer and a block
-// barrier ends the step.
+// per sequence or one for all) stay in registers.
 template <int KS, int CL>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(8 * 32 * KS / CL, 1)
 k_enc_recurrent_few(const EncRecArgs a) {
@@ -977,9 +984,10 @@ k_enc_recurrent_few(const EncRecArgs a) {
   constexpr int cpc = H / CL;               // cells per CTA
   constexpr int NTHR = 8 * cpc, CW = NTHR / 32;
   constexpr int UB = BG * H, MB = BG * cpc; // bytes of the group's hidden codes, of this CTA's part
-  static_assert(cpc % 8 == 0 && NTHR <= 1024, "units of 8 cells, one item per thread");
+  constexpr int PIECES = MB / 16;           // of this CTA's codes
+  static_assert(cpc % 8 == 0 && PIECES * CL <= NTHR, "units of 8 cells; a thread sends at most one piece");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t rank = CL == 1 ? 0u : cluster_rank();
+  const uint32_t rank = cluster_rank();
   const int cid = blockIdx.x / CL;
   const int d = cid / a.n_groups, grp = cid % a.n_groups;
   const EncRecDir& D = a.d[d];
@@ -1020,16 +1028,16 @@ k_enc_recurrent_few(const EncRecArgs a) {
     s_hh = make_float4(__fmul_rn(sh, s_hh.x), __fmul_rn(sh, s_hh.y), __fmul_rn(sh, s_hh.z), __fmul_rn(sh, s_hh.w));
   }
   for (int i = tid; i < 2 * UB / 16; i += NTHR) reinterpret_cast<uint4*>(hb)[i] = make_uint4(0, 0, 0, 0);   // h_0 = 0
-  if (CL > 1 && tid == 0) {
+  if (tid == 0) {
     *dead = 0;
     for (int i = 0; i < 2; ++i) mbar_init(&full[i], 1);
     fence_barrier_init();
     for (int i = 0; i < 2; ++i) mbar_expect_tx(&full[i], (uint32_t)UB);   // the first fill of either buffer
   }
-  fence_proxy_async();   // the zeroed buffers are later written by the bulk-copy engine
+  fence_proxy_async();   // the zeroed buffers are later written by asynchronous stores
   __syncthreads();
-  if (CL > 1) cluster_barrier();   // every CTA's buffers and barriers are initialised before anyone stores into them
-  pdl_wait();            // the input accumulators are the previous kernel's output; the weights that of the one before it
+  cluster_barrier();   // every CTA's buffers and barriers are initialised before anyone stores into them
+  pdl_wait();          // the input accumulators are the previous kernel's output; the weights that of the one before it
 
   const uint32_t hb_addr = smem_u32(hb), full_addr = smem_u32(full);
   const int hlo = act_lo(a.hid_act), hhi = act_hi(a.hid_act);
@@ -1050,9 +1058,9 @@ k_enc_recurrent_few(const EncRecArgs a) {
     const int4 pre = pre_next;
     pre_p += pstep;
     if (live && step + 1 < T) pre_next = *reinterpret_cast<const int4*>(pre_p);
-    // h_{t-1} is complete here once every CTA's copy has landed; waits, their limit and the order of buffers as in
+    // h_{t-1} is complete here once every CTA's part has landed; waits, their limit and the order of buffers as in
     // k_enc_recurrent_w4
-    if (CL > 1 && step > 0 && ok) {
+    if (step > 0 && ok) {
       uint64_t* bar = &full[cur];
       const uint32_t parity = (uint32_t)(((step - 1) >> 1) & 1);
       bool got = false;
@@ -1105,23 +1113,19 @@ k_enc_recurrent_few(const EncRecArgs a) {
       q = quantize1(hval, a.hid_act.inv_scale, a.hid_act.zero_point, hlo, hhi);
       q2 = quantize1(hval, a.out_act.inv_scale, a.out_act.zero_point, ylo, yhi);
     }
-    (CL == 1 ? hb + nxt * UB : stage + cur * MB)[at] = (int8_t)q;
+    // staged by step parity; every thread then sends one 16-byte piece of this CTA's codes to one CTA.  The pieces of a
+    // destination belong to consecutive lanes: their stores travel together.
+    stage[cur * MB + at] = (int8_t)q;
     stage_y[cur * MB + at] = (int8_t)q2;
-    if (CL > 1) fence_proxy_async();   // the staged codes are read by the bulk-copy engine
-    // One warp, a different one every step, waits until all threads have stored their codes, sends them to every CTA and
-    // writes this CTA's share of the layer output
-    const bool mine = warp == step % CW;
-    if (CL == 1) {
-      __syncthreads();
-    } else if (!mine) {
-      named_bar_arrive(1 + cur, NTHR);
-    } else {
-      named_bar_sync(1 + cur, NTHR);
-      if (lane < CL)
-        bulk_copy_to_cluster(map_to_rank(hb_addr + (uint32_t)(nxt * UB + (int)rank * MB), (uint32_t)lane),
-                             smem_u32(stage + cur * MB), (uint32_t)MB, map_to_rank(full_addr + (uint32_t)(nxt * 8), (uint32_t)lane));
+    __syncthreads();
+    if (tid < PIECES * CL) {
+      const uint32_t r = (uint32_t)(tid / PIECES);
+      const int ch = tid % PIECES;
+      st_async_v4(map_to_rank(hb_addr + (uint32_t)(nxt * UB + (int)rank * MB + ch * 16), r),
+                  *reinterpret_cast<const uint4*>(stage + cur * MB + ch * 16), map_to_rank(full_addr + (uint32_t)(nxt * 8), r));
     }
-    if (mine) {
+    // one warp, a different one every step, writes this CTA's share of the layer output
+    if (warp == step % CW) {
       for (int i = lane; i < MB / 8; i += 32) {
         const int bl = i & 7, by = grp * BG + bl, c0 = (int)rank * cpc + (i & ~7);
         if (by >= B) continue;
@@ -1141,17 +1145,15 @@ k_enc_recurrent_few(const EncRecArgs a) {
   }
   pdl_trigger();
   // the codes sent in the last step are still on their way: nobody leaves before they have landed (bounded)
-  if (CL > 1) {
-    if (T > 0) {
-      const uint32_t parity = (uint32_t)(((T - 1) >> 1) & 1);
-      for (uint32_t i = 0; i < (1u << 22); ++i) {
-        if (mbar_try_wait(&full[T & 1], parity)) break;
-        if ((i & 255u) == 255u && *dead) break;
-      }
+  if (T > 0) {
+    const uint32_t parity = (uint32_t)(((T - 1) >> 1) & 1);
+    for (uint32_t i = 0; i < (1u << 22); ++i) {
+      if (mbar_try_wait(&full[T & 1], parity)) break;
+      if ((i & 255u) == 255u && *dead) break;
     }
-    __syncthreads();
-    cluster_barrier();
   }
+  __syncthreads();
+  cluster_barrier();
   // final states
   if (D.hq_n) {
     const int qn = __shfl_down_sync(0xffffffffu, q, 8);   // the next cell, same sequence
@@ -1308,10 +1310,9 @@ static cudaError_t rec_w4_launch(const EncRecArgs& a, cudaStream_t s) {
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// A CTA of the kernel for few groups has an SM to itself: with 16 CTAs a cluster that makes 7 clusters (of the 8 GPCs
-// one has fewer than 16 SMs to spare).
+// A CTA of the kernel for few groups has an SM to itself.  Resident clusters: 7 of 16 CTAs, 11 of 10, 15 of 8 (a cluster
+// stays within a GPC, whose SMs are not a multiple of these).
 constexpr size_t REC_FEW_SMEM = 120 * 1024;
-constexpr int REC_FEW_CLUSTERS = 7;
 
 template <int KS, int CL>
 static cudaError_t rec_few_launch(const EncRecArgs& a, cudaStream_t s) {
@@ -1337,7 +1338,7 @@ EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid
   p.max_clusters = rec_max_clusters(H);
   if (H == 640) p.max_clusters = p.max_clusters < rec_turns_max_clusters() ? p.max_clusters : rec_turns_max_clusters();
   const bool few_h = H == 64 || H == 128 || H == 256 || H == 320 || H == 512 || H == 640;
-  if (few_h && hid_signed && !dump && (hid_bits == 4 || hid_bits == 8) && dirs * groups <= REC_FEW_CLUSTERS) {
+  if (few_h && hid_signed && !dump && (hid_bits == 4 || hid_bits == 8) && dirs * groups <= (H <= 256 ? 15 : 7)) {
     p.kernel = 3;
     p.groups_per_cluster = 1;
     p.ncl[0] = groups;
@@ -1356,6 +1357,7 @@ EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid
     const bool turns = g_rec_sliced && lack >= 1 && lack <= dirs && groups >= 2 && groups <= 8 && T >= 8 * groups && scratch;
     if (turns || (lack <= 0 && plain_only && groups <= 8)) {   // the hand-over scratch is needed for turns only
       p.kernel = 2;
+      p.ctas = !turns && dirs * groups <= 11 ? 10 : REC_CLUSTER;
       p.groups_per_cluster = 1;
       for (int d = 0; d < 2; ++d) {
         p.sliced[d] = turns && d < dirs && d < lack ? 1 : 0;
@@ -1372,6 +1374,7 @@ EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid
     while (nu <= 4 && dirs * ((groups + nu - 1) / nu) > p.max_clusters) ++nu;
     if (nu <= 4) {
       p.kernel = 1;
+      p.ctas = nu == 1 && dirs * groups <= 11 ? 10 : REC_CLUSTER;
       p.groups_per_cluster = nu;
       p.ncl[0] = (groups + nu - 1) / nu;
       p.ncl[1] = dirs == 2 ? p.ncl[0] : 0;
@@ -1386,13 +1389,14 @@ cudaError_t launch_enc_recurrent(EncRecArgs a, cudaStream_t s) {
   const EncRecPlan p = enc_recurrent_plan(a.T, a.B, a.dirs, a.H, a.w_bits, a.hid_act.bits, a.hid_act.is_signed != 0,
                                           a.x_scale_b != nullptr, a.d[0].dbg_ih != nullptr,
                                           a.flags && a.hand_h[0] && a.hand_c[0]);
-  if (p.kernel == 3) {
+  if (p.kernel == 3 || p.ctas == 10) {
     a.n_groups = p.groups;
     timing_begin(s);
     cudaError_t e = cudaErrorInvalidValue;
-    switch (a.H) {
-      case 64: e = rec_few_launch<2, 1>(a, s); break;
-      case 128: e = rec_few_launch<4, 1>(a, s); break;
+    switch (p.ctas == 10 ? 0 : a.H) {
+      case 0: e = rec_few_launch<20, 10>(a, s); break;
+      case 64: e = rec_few_launch<2, 2>(a, s); break;
+      case 128: e = rec_few_launch<4, 4>(a, s); break;
       case 256: e = rec_few_launch<8, 8>(a, s); break;
       case 320: e = rec_few_launch<10, 8>(a, s); break;
       case 512: e = rec_few_launch<16, 16>(a, s); break;

@@ -165,6 +165,12 @@ def test_layer_few_groups(Bd, T, B, K, H, dirs, xb, hb, ob):
     layer_case(Bd, T, B, K, H, dirs, xb, hb, ob, seed=29)
 
 
+@pytest.mark.parametrize("T,B,dirs,xb,hb,ob", [(7, 30, 2, 4, 4, 4), (6, 88, 1, 8, 8, 4), (6, 81, 1, 4, 4, 8)])
+def test_layer_clusters_of_ten(Bd, T, B, dirs, xb, hb, ob):
+    # 8 to 11 groups of 640 cells: clusters of 10 CTAs
+    layer_case(Bd, T, B, 32, 640, dirs, xb, hb, ob, seed=31)
+
+
 def test_layer_clusters_taking_turns_at_a_surplus_group(Bd):
     # 57 sequences x 2 directions of 640 cells = 16 groups of 8 for the 15 clusters that fit: the seven
     # clusters of one direction take turns at its eighth group (9 of 64 steps each, one more on the
