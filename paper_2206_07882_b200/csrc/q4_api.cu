@@ -1022,22 +1022,20 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
       Q4_TRY(launch_unpack_multi(uj, s, true));
     }
     // the three networks are independent until the selection: with two lent streams they run side
-    // by side.  The call's own stream carries the chain that is critical: with many hypothesis rows
-    // the target LM (two wide layers; the fork and the join would add to its path), with few rows
-    // the prediction/joint chain, the only one with work in every iteration, which then runs
-    // gather -> ... -> joint -> selection as programmatic dependents without an event in between
-    // (measured: 16 utterances 18.8 -> 18.5 ms, one utterance 11.5 -> 11.2 ms; 64 utterances the other
-    // way round, 49.7 -> 50.5 ms)
-    const bool joint_on_call_stream = N <= 256;
+    // by side.  The call's own stream carries the longest chain, the target LM's (gather -> two layers -> head ->
+    // selection as programmatic dependents without an event in between; a fork costs 2 to 4 us, a join 1 to 4).
+    // Against the prediction/joint chain there, 150 iterations with labels in most: 16 slots 4.62 -> 4.38 ms, 16 x 16
+    // slots 6.64 -> 6.36, time-synchronous 4 x 8 slots 12.8 -> 12.1; with labels in a third: 3.61 -> 3.59, 5.15 ->
+    // 5.22, 12.9 -> 12.1
     cudaStream_t sp = s, ss = s, stt = s;
     const bool forked = nets && st.aux_stream[0] && st.aux_stream[1] && st.aux_event[0] && st.aux_event[1] &&
                         st.aux_event[2];
     if (forked) {
-      (joint_on_call_stream ? stt : sp) = reinterpret_cast<cudaStream_t>(st.aux_stream[0]);
+      sp = reinterpret_cast<cudaStream_t>(st.aux_stream[0]);
       ss = reinterpret_cast<cudaStream_t>(st.aux_stream[1]);
       cudaEvent_t fork = reinterpret_cast<cudaEvent_t>(st.aux_event[0]);
       Q4_TRY(cudaEventRecord(fork, s));
-      Q4_TRY(cudaStreamWaitEvent(joint_on_call_stream ? stt : sp, fork, 0));
+      Q4_TRY(cudaStreamWaitEvent(sp, fork, 0));
       Q4_TRY(cudaStreamWaitEvent(ss, fork, 0));
     }
     // one LSTM layer of one network for every pending slot
@@ -1121,7 +1119,7 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
     const bool fused_head = D == 256 && V <= 2048;   // the fused head kernel: 256-wide bottleneck, one cluster per row tile
     // 1a. prediction network, then the joint network for every live slot (stream sp)
     if (nets) {
-      Q4_CHECK(lstm_mma(sp, !forked || joint_on_call_stream, TAG_PRED_LSTM, 0, m.pred_lstm, m.pred_emb_act, xa8[0], ha8[0], st.pred_hq,
+      Q4_CHECK(lstm_mma(sp, !forked, TAG_PRED_LSTM, 0, m.pred_lstm, m.pred_emb_act, xa8[0], ha8[0], st.pred_hq,
                         st.pred_c, pred_h8));
       Q4_CHECK(linear_mma(sp, true, TAG_PRED_PROJ, 0, m.pred_proj, pred_h8, m.pred_lstm.hid_act.scale, EPI_F32,
                           st.pred_p, D, cst.adv_dst, nullptr, n_active));
@@ -1162,7 +1160,7 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
       float* c0 = which == 0 ? st.src_c : st.tgt_c[0];
       int8_t* h8_0 = which == 0 ? src_h8 : tgt_h8[0];
       float* lp = which == 0 ? st.src_lp : st.tgt_lp;
-      Q4_CHECK(lstm_mma(sl, (which == 1 && !joint_on_call_stream) || !forked, which == 0 ? TAG_SRC_LSTM : TAG_TGT_L1, which == 0 ? 1 : 2, L0, lm.emb_act,
+      Q4_CHECK(lstm_mma(sl, which == 1 || !forked, which == 0 ? TAG_SRC_LSTM : TAG_TGT_L1, which == 0 ? 1 : 2, L0, lm.emb_act,
                         xa8[which + 1], ha8[which + 1], hq0, c0, h8_0, 0, lm.n_layers == 2 ? 1 : 0));
       const int8_t* top8 = h8_0;
       const q4_lstm* last = &L0;
@@ -1207,7 +1205,7 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
     if (forked) {   // join: the call's stream waits for both side chains
       cudaEvent_t j0 = reinterpret_cast<cudaEvent_t>(st.aux_event[1]);
       cudaEvent_t j1 = reinterpret_cast<cudaEvent_t>(st.aux_event[2]);
-      Q4_TRY(cudaEventRecord(j0, joint_on_call_stream ? stt : sp));
+      Q4_TRY(cudaEventRecord(j0, sp));
       Q4_TRY(cudaEventRecord(j1, ss));
       Q4_TRY(cudaStreamWaitEvent(s, j0, 0));
       Q4_TRY(cudaStreamWaitEvent(s, j1, 0));
