@@ -135,9 +135,9 @@ int qlstm_layer_forward(const void* xq, const q4_act* x_act, const float* x_scal
  *   placement of Section 3.4, where every cell quantizes its two inputs on entry instead
  *   (quantize_pack_int4 on x_t and on the previous real-valued cell output, then this call).
  *   prepared / workspace (all nullable): with the buffer filled by q4_prepare_lstm for these weights
- *   and a workspace of q4_workspace_bytes(Q4_WS_LSTM_STEP, {N, kx_pad, H}) bytes, calls with N >= 128
- *   and H a multiple of 128 run on the tensor cores (same results, bit for bit); otherwise, and
- *   always without them, the DP4A kernel reads the packed weights directly.
+ *   and a workspace of q4_workspace_bytes(Q4_WS_LSTM_STEP, {N, kx_pad, H}) bytes, calls with H a
+ *   multiple of 128 run on the tensor cores (same results, bit for bit).  Otherwise, and for at most 32 rows of
+ *   4-bit codes, kernels that read the packed weights directly.
  */
 int qlstm_step(const void* xq, const q4_act* x_act, const int32_t* x_row_idx, const void* hq_in,
                const float* c_in, int32_t N, const q4_mat* w_ih, const q4_mat* w_hh,
@@ -173,7 +173,7 @@ int q4_linear_forward(const void* xq, const q4_act* x_act, int32_t M, const q4_m
  * with z_act, passed through the output layer (w_out [V, D], b_out) and a log-softmax.
  * logp [N, V] fp32.  workspace: q4_workspace_bytes(Q4_WS_JOINT, {N, D}).
  * prepared_pred / prepared_out (nullable): buffers of q4_prepare_linear for w_pred and w_out; with
- * both, a workspace of q4_workspace_bytes(Q4_WS_JOINT, {N, D, Hp_pad}) bytes and N >= 128
+ * both, a workspace of q4_workspace_bytes(Q4_WS_JOINT, {N, D, Hp_pad}) bytes
  * the call runs on the tensor cores in three launches (the projection's epilogue forms
  * tanh(e * p) and quantizes it; the output layer's epilogue takes the log-softmax).
  */

@@ -8,6 +8,7 @@ missing, or CUDA is unavailable, the first call raises.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 from typing import List, Optional, Sequence
 
@@ -103,9 +104,15 @@ def lib() -> C.CDLL:
     return _lib
 
 
+_cuda_seen = False
+
+
 def _need_cuda():
-    if not torch.cuda.is_available():
-        raise RuntimeError("q4rnnt needs a CUDA device; there is no CPU path")
+    global _cuda_seen
+    if not _cuda_seen:       # a device does not go away; asking for it takes longer than a launch
+        if not torch.cuda.is_available():
+            raise RuntimeError("q4rnnt needs a CUDA device; there is no CPU path")
+        _cuda_seen = True
 
 
 def _p(t: Optional[torch.Tensor]):
@@ -113,7 +120,7 @@ def _p(t: Optional[torch.Tensor]):
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def _chk(code: int, where: str):
@@ -168,6 +175,11 @@ def beam_select_exact_set(enabled: bool) -> bool:
 
 
 def workspace_bytes(call_id: int, dims: Sequence[int]) -> int:
+    return _workspace_bytes(call_id, tuple(dims))
+
+
+@functools.lru_cache(maxsize=256)
+def _workspace_bytes(call_id: int, dims: tuple) -> int:
     arr = (C.c_int32 * len(dims))(*dims)
     return int(lib().q4_workspace_bytes(C.c_int32(call_id), arr, C.c_int32(len(dims))))
 
@@ -352,7 +364,7 @@ def qlstm_step(xq: torch.Tensor, x_act: Act, hq_in: torch.Tensor, c_in: torch.Te
         r["acc_hh"] = torch.empty((N, 4 * H), dtype=torch.int32, device=dev)
     wih, whh = layer.w_ih.c(), layer.w_hh.c()
     ws = None
-    if layer.prepared is not None:      # tensor-core path (taken by the library from 128 rows on)
+    if layer.prepared is not None:      # tensor-core path
         need = workspace_bytes(WS_LSTM_STEP, [N, layer.w_ih.k_pad, H])
         if layer.ws is None or layer.ws.numel() < need:
             layer.ws = torch.empty(need, dtype=torch.uint8, device=dev)

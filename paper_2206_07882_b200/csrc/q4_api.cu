@@ -339,12 +339,42 @@ int qlstm_step(const void* xq, const q4_act* x_act, const int32_t* x_row_idx, co
   if (!aligned16(xq) || !aligned16(hq_in) || !aligned16(hq_out)) return Q4_ERR_ALIGN;
   if (N == 0) return Q4_OK;
   if (hq_out) ++g_quant_calls;   // the one quantizer call at the cell output (Outer placement)
+  if (!dbg_acc_ih && !dbg_acc_hh && skinny_lstm_supported(N, H, w_ih->k_pad, w_ih->bits, w_hh->bits, *x_act, *hid_act)) {
+    // at most 32 rows of 4-bit codes: the kernel that reads the packed weights once (1024 cells, 16 rows:
+    // 4.6 us of device time; two launches on the tensor cores 8.2, the DP4A kernel 24)
+    SkinnyLstmArgs k;
+    memset(&k, 0, sizeof(k));
+    k.N = N;
+    k.H = H;
+    k.Kx = w_ih->k_pad;
+    k.w_ih = static_cast<const uint8_t*>(w_ih->q);
+    k.w_hh = static_cast<const uint8_t*>(w_hh->q);
+    k.s_wih = w_ih->scale;
+    k.s_whh = w_hh->scale;
+    k.bias = bias;
+    k.x = static_cast<const uint8_t*>(xq);
+    k.x_stride = row_bytes(w_ih->k_pad, 4);
+    k.x_idx = x_row_idx;
+    k.x_signed = x_act->is_signed;
+    k.x_zp = x_act->zero_point;
+    k.x_scale = x_act->scale;
+    k.hid_act = *hid_act;
+    k.hq_in = static_cast<const uint8_t*>(hq_in);
+    k.c_in = c_in;
+    k.hq_out = static_cast<uint8_t*>(hq_out);
+    k.c_out = c_out;
+    k.h_f32 = h_f32_out;
+    TagScope tag(TAG_PRED_LSTM);
+    Q4_TRY(launch_skinny_lstm(k, S(stream), true));
+    return Q4_OK;
+  }
   {
     const int32_t wd[3] = {N, w_ih->k_pad, H};
-    if (prepared && workspace && hq_out && N >= 128 && H % 128 == 0 && aligned16(workspace) && aligned16(prepared) &&
+    if (prepared && workspace && hq_out && H % 128 == 0 && aligned16(workspace) && aligned16(prepared) &&
         (dbg_acc_ih == nullptr) == (dbg_acc_hh == nullptr) && c_out != nullptr &&
         workspace_bytes >= q4_workspace_bytes(Q4_WS_LSTM_STEP, wd, 3)) {
-      // tensor cores: int8 copies of the x rows (gathered) and h rows, then the fused LSTM kernel on the
+      // tensor cores, any number of rows (33: 8.4 us of device time, 24.7 on the DP4A kernel): int8 copies of
+      // the x rows (gathered) and h rows, then the fused LSTM kernel on the
       // prepared int8 weights (rows 4*cell+gate, scales and bias in the same order)
       cudaStream_t s = S(stream);
       const size_t G = 4 * (size_t)H, Kx = w_ih->k_pad;
@@ -620,9 +650,10 @@ int qjoint_logprobs(const float* e, const int32_t* frame_idx, const void* pq, co
   TagScope tag(TAG_JOINT);
   ++g_quant_calls;   // tanh(e * p)
   const int32_t dims3[3] = {N, D, w_pred->k_pad};
-  if (prepared_pred && prepared_out && N >= 128 && z_act->is_signed && aligned16(prepared_pred) &&
+  if (prepared_pred && prepared_out && z_act->is_signed && aligned16(prepared_pred) &&
       aligned16(prepared_out) && workspace_bytes >= q4_workspace_bytes(Q4_WS_JOINT, dims3, 3)) {
-    // tensor cores, three launches: int8 copy of the hidden codes; projection GEMM whose epilogue forms
+    // tensor cores for any number of rows (a 128-row tile of mostly empty rows included: 16 rows 15.7 us of device time in
+    // three launches, 26.9 in the four of the kernels for unprepared weights): int8 copy of the hidden codes; projection GEMM whose epilogue forms
     // tanh(e * p) and quantizes it; output layer with the log-softmax in its epilogue (fused head kernel
     // when D = 256, else GEMM + row log-softmax)
     const int Hp = w_pred->k_pad, Np = (N + 127) / 128 * 128;

@@ -189,6 +189,7 @@ struct SkinnyLstmArgs {
   float* c_out;
   int8_t* h8_out;           // int8 codes at launch row n (nullable)
   long long h8_ld;
+  float* h_f32;             // [N, H] unquantized cell output (nullable)
   const int32_t* n_active;  // optional device count: rows >= *n_active carry no work
 };
 bool skinny_lstm_supported(int N, int H, int Kx, int w_bits_ih, int w_bits_hh, const q4_act& x_act,

@@ -120,6 +120,7 @@ __global__ void __launch_bounds__(SK_THREADS, NT == 4 ? 2 : SK_CTAS_PER_SM) k_sk
 #pragma unroll
       for (int r = 0; r < 4; ++r) acc[p][j][r] = 0;
 
+  const uint32_t x_null = x_unsigned ? 0x11111111u * (uint32_t)a.x_zp : 0u;   // the codes of an input row of zeros
   // chunk q of this warp: weight pieces of two rows and activation pieces of NT rows, 16 bytes each
   auto fetch = [&](int q, uint4& wa, uint4& wb, uint4 (&xb)[NT]) {
     wa = wb = make_uint4(0, 0, 0, 0);
@@ -127,6 +128,7 @@ __global__ void __launch_bounds__(SK_THREADS, NT == 4 ? 2 : SK_CTAS_PER_SM) k_sk
     for (int j = 0; j < NT; ++j) xb[j] = make_uint4(0, 0, 0, 0);
     if (q >= nxc + nhc) return;
     const bool is_x = q < nxc;
+    const uint32_t null_word = is_x ? x_null : 0u;
     const int kb = ((is_x ? q : q - nxc) << 6) + 16 * t4;   // byte offset of this lane's 32 codes in a row
     const uint8_t* wbase = is_x ? a.w_ih : a.w_hh;
     const long long wpitch = is_x ? (a.Kx >> 1) : (H >> 1);
@@ -135,6 +137,7 @@ __global__ void __launch_bounds__(SK_THREADS, NT == 4 ? 2 : SK_CTAS_PER_SM) k_sk
 #pragma unroll
     for (int j = 0; j < NT; ++j) {
       const int r = is_x ? xrow[j] : hrow[j];
+      xb[j] = make_uint4(null_word, null_word, null_word, null_word);
       if (r >= 0)
         xb[j] = *reinterpret_cast<const uint4*>((is_x ? a.x + (long long)r * a.x_stride : a.hq_in + (long long)r * (H >> 1)) + kb);
     }
@@ -216,6 +219,7 @@ __global__ void __launch_bounds__(SK_THREADS, NT == 4 ? 2 : SK_CTAS_PER_SM) k_sk
     cell_fixed(pre[0], pre[1], pre[2], pre[3], e_cprev, cn, hn);
     a.c_out[(long long)dst * H + cell] = cn;
     q = quantize1(hn, a.hid_act.inv_scale, a.hid_act.zero_point, act_lo(a.hid_act), act_hi(a.hid_act));
+    if (a.h_f32) a.h_f32[(long long)n * H + cell] = hn;
     if (a.h8_out) a.h8_out[(long long)n * a.h8_ld + cell] = (int8_t)q;
   }
   // two cells per byte: the even cell's thread writes

@@ -25,7 +25,9 @@ def Bd():
                                                   # tensor-core path: fused head (D = 256), ragged last row tile;
                                                   # GEMM + row log-softmax (D = 64); 8-bit output layer
                                                   (200, 1024, 256, 1024, 4, True), (130, 96, 64, 128, 4, True),
-                                                  (257, 992, 256, 256, 8, True)])
+                                                  (257, 992, 256, 256, 8, True),
+                                                  # one row tile, mostly empty
+                                                  (1, 1024, 256, 256, 4, True), (70, 96, 64, 128, 8, True)])
 def test_joint_logprobs(Bd, N, V, D, Hp, zb, prep):
     dw = synth.decoder(seed=5, V=V, E=32, Hp=Hp, D=D, Hs=32, Ht=32, out_bits=zb)
     dec = O.Decoder(dw)

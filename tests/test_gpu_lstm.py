@@ -410,8 +410,34 @@ def test_outer_and_inner_quantizer_placement_counted_on_the_device(Bd):
     np.testing.assert_array_equal(x.cpu().numpy(), O.encoder_forward_inner(E, enc["features"]))
 
 
+@pytest.mark.parametrize("N", [1, 8, 9, 16, 17, 32])
+@pytest.mark.parametrize("signed", [True, False])
+def test_step_few_rows(Bd, N, signed):
+    # the weight-streaming kernel (edges of its 8-row tiles), with a gathered row of zeros and without, against
+    # the oracle: the float stages are one fp32 operation sequence, bit-exact
+    st = synth.Stream(200 + N)
+    lw = synth._lstm(st, "l", 128, 256, 4, bias_std=0.2, hid_alpha=0.95, hid_bits=4)
+    x_act = O.act_symmetric(3.0, 4) if signed else O.act_asymmetric(-1.7, 1.4, 4)
+    hid = O.act_symmetric(0.95, 4)
+    table = st.integers("x", (40, 128), x_act.lo(), x_act.hi()).astype(np.int16)
+    idx = st.integers("i", (N,), 0, 39).astype(np.int32)
+    idx[N // 2] = -1
+    hq = st.integers("h", (N, 256), -7, 7).astype(np.int16)
+    c = st.normal("c", (N, 256)).astype(np.float32)
+    zero = 0 if signed else x_act.zero_point
+    xq = np.where(idx[:, None] >= 0, table[idx], np.int16(zero))
+    want = O.lstm_step(O.Lstm([lw]), xq, x_act, hq, c, hid)
+    dl = Bd.DeviceLstm(lw)
+    got = Bd.qlstm_step(pack_codes(table, x_act, dl.w_ih.k_pad), to_act(x_act), pack_codes(hq, hid),
+                        torch.from_numpy(c).cuda(), dl, x_row_idx=torch.from_numpy(idx).cuda())
+    np.testing.assert_array_equal(got["c"].cpu().numpy(), want["c"])
+    np.testing.assert_array_equal(got["h"].cpu().numpy(), want["h"])
+    np.testing.assert_array_equal(gpu_codes(got["hq"], 256, hid), want["hq"])
+
+
 @pytest.mark.parametrize("N,K,H,xb,hb,signed", [(130, 256, 128, 4, 4, True), (300, 96, 256, 4, 4, False),
-                                                 (128, 240, 128, 8, 8, True), (257, 64, 384, 4, 8, True)])
+                                                 (128, 240, 128, 8, 8, True), (257, 64, 384, 4, 8, True),
+                                                 (1, 64, 128, 8, 8, True), (33, 96, 256, 4, 4, False)])
 def test_step_on_the_tensor_cores_with_prepared_weights(Bd, N, K, H, xb, hb, signed):
     # qlstm_step with the one-time int8 operands: tcgen05 kernel, same integers and floats as the oracle
     st = synth.Stream(400 + N)
