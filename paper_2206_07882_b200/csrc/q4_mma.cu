@@ -50,8 +50,11 @@ __device__ __forceinline__ void unpack_piece32(const uint8_t* p, int k, int bits
 // padded row count: each thread strides over the 32-element pieces of the rows that carry work
 // (their number may be known on the device only).
 __global__ void __launch_bounds__(256) k_unpack_multi(const __grid_constant__ UnpackJobs jobs) {
-  pdl_trigger();   // a dependent successor may set itself up; it reads nothing before this grid has completed
+  // A dependent successor may set itself up; it reads nothing before this grid has completed but, in a search, the count
+  // of rows with work (see count_visible), so there the trigger has to follow the wait.
+  if (!jobs.n_active) pdl_trigger();
   pdl_wait();      // launched as a programmatic dependent itself: the source rows may be the predecessor's output
+  if (jobs.n_active) pdl_trigger();
   if (jobs.clear64 && (blockIdx.x | blockIdx.y) == 0 && threadIdx.x < 64) jobs.clear64[threadIdx.x] = 0;   // the call's status block
   const UnpackJob& j = jobs.job[blockIdx.y];
   const uint32_t per_row = (uint32_t)j.k_pad >> 5;
@@ -260,6 +263,14 @@ __device__ __forceinline__ void flag_timeout(int32_t* status) {
   if (status) atomicExch(status, Q4_ERR_TIMEOUT);
 }
 
+// Row counts of the search (n_active of the kernels below), count_visible: the count is written by the selection, and
+// the first kernel of a step's chains (the gather, or a kernel behind an event) waits for that before it
+// triggers its successor.  So every later kernel of the step may read the count as its first act, and a tile
+// without work leaves before it has set anything up or occupied an SM for long: in an iteration without labels
+// (two of three in speech) that is every tile of seven kernels.  Against tiles that
+// found out after their set-up, 150 iterations: few labels 1 x 16 slots 3.59 -> 3.43 ms, 4 x 8 slots of the paper's model
+// 3.36 -> 3.10; labels in most 4.38 -> 4.35 and 5.26 -> 4.99.
+
 // ------------------------------------------------------------------ plain GEMM
 struct MmaGemmArgs {
   int M, J, K, epi;
@@ -300,6 +311,7 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
   const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * GEMM_BN;   // row tiles slowest: tiles with work are dispatched first
   const int nk = (a.K + BK - 1) / BK;
+  if (a.n_active && m0 >= *a.n_active) return;   // whole tile without work (count_visible)
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -320,11 +332,7 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
   pdl_wait();   // everything above overlaps the tail of the previous kernel of the stream
-  const bool has_work = !(a.n_active && m0 >= *a.n_active);   // uniform per CTA
-
-  if (!has_work) {
-    // whole tile without work
-  } else if (warp == 4) {
+  if (warp == 4) {
     bool ok = true;
     int s = 0;
     uint32_t ph = 1;
@@ -795,6 +803,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
   const int m0 = blockIdx.y * BM;
   const int nb = blockIdx.x;                    // my blocks of columns = my cluster rank
   const int nk1 = (a.H + BK - 1) / BK;
+  if (a.n_active && m0 >= *a.n_active) return;   // row tile without work: the whole cluster leaves (count_visible)
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -833,10 +842,6 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
   const uint32_t tmem = tmem_base_s;
   cl_barrier();   // every CTA of the cluster is running before anyone stores into a peer's shared memory
   pdl_wait();   // everything above (this barrier included) overlaps the tail of the previous kernel of the stream
-  if (a.n_active && m0 >= *a.n_active) {   // whole row tile without work: the whole cluster leaves
-    if (warp == HEAD_EPI_WARPS + 1) tmem_dealloc(tmem, TCOLS);
-    return;
-  }
 
   if (warp == HEAD_EPI_WARPS) {
     // ---- TMA producer: bottleneck operands through the ring, then my block of output-layer weights into
@@ -1182,6 +1187,7 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
   const int nkx = a.acc_pre ? 0 : (a.Kx_pad + BK - 1) / BK;
   const int nkh = (a.H + BK - 1) / BK;
   const int nk = nkx + nkh;
+  if (a.n_active && m0 >= *a.n_active) return;   // whole tile without work (count_visible)
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -1208,13 +1214,10 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
   // kernels further back, all complete) runs before the wait, the input half after it.
   const bool h_first = a.h_first != 0 && nkx > 0;
   if (!h_first) pdl_wait();
-  const bool has_work = !(a.n_active && m0 >= *a.n_active);   // uniform per CTA
   if (a.trigger_early) pdl_trigger();   // the successor has a half it can run beside this kernel
   const int x_first = h_first ? nkh : 0, hh_first = h_first ? 0 : nkx;   // first chunk of each part
 
-  if (!has_work) {
-    if (h_first) pdl_wait();   // whole tile without work; still ordered behind the previous kernel
-  } else if (warp == LSTM_EPI_WARPS) {
+  if (warp == LSTM_EPI_WARPS) {
     bool ok = true;
     int s = 0;
     uint32_t ph = 1;
