@@ -686,7 +686,7 @@ class Decoder:
     def q4_beam_search(self, e: torch.Tensor, T: int, u_max: int, time_synchronous: bool = False):
         """All steps of a search (after q4_beam_init) in one library call.  The decoder keeps a plan for it, in
         which the library replays groups of steps as a CUDA graph (only with the streams of a concurrent state)."""
-        if self._plan is None and self.state.aux_stream[0]:
+        if self._plan is None and self.state.aux_stream[0] and not torch.cuda.is_current_stream_capturing():
             plan = C.c_void_p()
             _chk(lib().q4_search_plan_create(C.byref(plan)), "q4_search_plan_create")
             self._plan = _SearchPlan(plan)
