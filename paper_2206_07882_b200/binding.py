@@ -123,6 +123,27 @@ def _stream():
     return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
+_SCRATCH_STREAMS = 16
+
+
+def _scratch(owner, need: int, device) -> torch.Tensor:
+    """Workspace of a prepared layer's call, one per stream: calls on one stream are ordered, calls on different
+    streams must not share one.  It is allocated on the stream that uses it, so a buffer that is replaced or dropped
+    is handed on in that stream's order.  A capture gets a buffer of its own from the graph's memory, which lives as
+    long as the graph, whatever happens to the layer meanwhile."""
+    if torch.cuda.is_current_stream_capturing():
+        return torch.empty(need, dtype=torch.uint8, device=device)
+    per = owner.stream_ws
+    key = torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    ws = per.get(key)
+    if ws is None or ws.numel() < need:
+        if ws is None and len(per) >= _SCRATCH_STREAMS:
+            del per[next(iter(per))]
+        ws = per[key] = torch.empty(need, dtype=torch.uint8, device=device)
+    owner.ws = ws
+    return ws
+
+
 def _chk(code: int, where: str):
     if code != 0:
         raise Q4Error(code, where)
@@ -273,7 +294,8 @@ class DeviceLstm:
         self.hid_act = q4_act_symmetric(lw.hid_alpha, lw.hid_bits)
         self.H = self.w_hh.k
         self.prepared = None
-        self.ws = None
+        self.ws = None            # the workspace of the last call (its first word is the call's status)
+        self.stream_ws = {}
 
     def prepare(self):
         """One-time int8 operands for the tensor-core path of qlstm_step (q4_prepare_lstm)."""
@@ -297,7 +319,8 @@ class DeviceLinear:
         self.w = DeviceMat.from_codes(lw.w.codes, lw.w.scale, lw.w.bits, device)
         self.bias = _dev_f32(lw.bias, device)
         self.prepared = None
-        self.ws = None
+        self.ws = None            # the workspace of the last call (its first word is the call's status)
+        self.stream_ws = {}
 
     def prepare(self):
         """One-time int8 operand for the tensor-core paths (q4_prepare_linear)."""
@@ -366,9 +389,7 @@ def qlstm_step(xq: torch.Tensor, x_act: Act, hq_in: torch.Tensor, c_in: torch.Te
     ws = None
     if layer.prepared is not None:      # tensor-core path
         need = workspace_bytes(WS_LSTM_STEP, [N, layer.w_ih.k_pad, H])
-        if layer.ws is None or layer.ws.numel() < need:
-            layer.ws = torch.empty(need, dtype=torch.uint8, device=dev)
-        ws = layer.ws
+        ws = _scratch(layer, need, dev)
     _chk(lib().qlstm_step(_p(xq), C.byref(x_act), _p(x_row_idx), _p(hq_in), _p(c_in), C.c_int32(N),
                           C.byref(wih), C.byref(whh), _p(layer.bias), C.byref(layer.hid_act),
                           _p(r.get("hq")), _p(r["c"]), _p(r.get("h")), _p(r.get("acc_ih")),
@@ -414,9 +435,7 @@ def q4_linear_forward(xq: torch.Tensor, x_act: Act, lin: DeviceLinear, want_acc:
     ws = None
     if getattr(lin, "prepared", None) is not None and not want_acc:
         need = workspace_bytes(WS_LINEAR, [M, lin.w.k_pad])
-        if lin.ws is None or lin.ws.numel() < need:
-            lin.ws = torch.empty(need, dtype=torch.uint8, device=xq.device)
-        ws = lin.ws
+        ws = _scratch(lin, need, xq.device)
     _chk(lib().q4_linear_forward(_p(xq), C.byref(x_act), C.c_int32(M), C.byref(w), _p(lin.bias),
                                  _p(out), _p(acc), _p(getattr(lin, "prepared", None)), _p(ws),
                                  C.c_size_t(ws.numel() if ws is not None else 0), _stream()), "q4_linear_forward")

@@ -457,6 +457,67 @@ def test_step_on_the_tensor_cores_with_prepared_weights(Bd, N, K, H, xb, hb, sig
     assert Bd.launch_count() - n0 >= 3
 
 
+def wide_step_operands(seed, N, K, H):
+    """One 8-bit layer (the same for every seed) and a set of operands of a step"""
+    st, wt = synth.Stream(seed), synth.Stream(1)
+    x_act, hid = O.act_symmetric(3.0, 8), O.act_symmetric(0.95, 8)
+    lw = synth._lstm(wt, "l", K, H, 4, bias_std=0.2, hid_alpha=0.95, hid_bits=8)
+    lw.w_ih, lw.w_hh = synth._qmat(wt, "w8", 4 * H, K, 8), synth._qmat(wt, "h8", 4 * H, H, 8)
+    xq = pack_codes(st.integers("xq", (N, K), x_act.lo(), x_act.hi()).astype(np.int16), x_act)
+    hq = pack_codes(st.integers("hq", (N, H), -127, 127).astype(np.int16), hid)
+    return lw, to_act(x_act), xq, hq, torch.from_numpy(st.normal("c", (N, H)).astype(np.float32)).cuda()
+
+
+def test_streams_that_step_one_layer(Bd):
+    # 40 rows of 8-bit codes gather their operands into the call's workspace: two streams have two of them
+    lw, x_act, *first = wide_step_operands(1, 40, 128, 256)
+    _, _, *second = wide_step_operands(2, 40, 128, 256)
+    layer = Bd.DeviceLstm(lw).prepare()
+
+    def chain(x, h, c):
+        for _ in range(100):
+            r = Bd.qlstm_step(x, x_act, h, c, layer)
+            h, c = r["hq"], r["c"]
+        return h, c
+
+    want = [chain(*first), chain(*second)]
+    for _ in range(3):
+        got = []
+        torch.cuda._sleep(100_000_000)          # both chains are enqueued before either runs
+        gate = torch.cuda.Event()
+        gate.record()
+        for stream, operands in zip((torch.cuda.Stream(), torch.cuda.Stream()), (first, second)):
+            with torch.cuda.stream(stream):
+                stream.wait_event(gate)
+                got.append(chain(*operands))
+        torch.cuda.synchronize()
+        for g, w in zip(got, want):
+            assert torch.equal(g[0], w[0]) and torch.equal(g[1], w[1])
+    for _ in range(40):                         # more streams than workspaces are kept for
+        with torch.cuda.stream(torch.cuda.Stream()):
+            Bd.qlstm_step(first[0], x_act, first[1], first[2], layer)
+    assert len(layer.stream_ws) <= 16
+
+
+def test_captured_step_outlives_a_larger_one(Bd):
+    # a graph of a step keeps its workspace when a later call with more rows needs a larger one
+    lw, x_act, x, h, c = wide_step_operands(1, 40, 128, 256)
+    layer = Bd.DeviceLstm(lw).prepare()
+    want = Bd.qlstm_step(x, x_act, h, c, layer)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        r = Bd.qlstm_step(x, x_act, h, c, layer)
+    _, _, *more = wide_step_operands(3, 300, 128, 256)
+    Bd.qlstm_step(more[0], x_act, more[1], more[2], layer)
+    torch.cuda.synchronize()
+    need = Bd.workspace_bytes(Bd.WS_LSTM_STEP, [40, 128, 256])
+    blocks = [torch.full((need,), 0x5A, dtype=torch.uint8, device="cuda") for _ in range(64)]
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(r["hq"], want["hq"]) and torch.equal(r["c"], want["c"])
+    assert all(bool((b == 0x5A).all()) for b in blocks)
+
+
 # every tile width of the tensor-core GEMM (32 to 256 weight rows, chosen by how many tiles there are), ragged
 # rows and columns, against exact integer sums
 @pytest.mark.parametrize("M,J,K", [(128, 32, 64), (129, 256, 1024), (300, 1000, 96), (1900, 700, 32), (1300, 2560, 160),
