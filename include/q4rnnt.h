@@ -170,7 +170,8 @@ int q4_linear_forward(const void* xq, const q4_act* x_act, int32_t M, const q4_m
  * qjoint_logprobs — joint network (Section 2): the prediction-network cell output codes pq
  * [N, Hp] (p_act) are projected to D dims (w_pred, b_pred), combined multiplicatively with
  * the projected encoder frame e[frame_idx[n]] ([*, D] fp32), z = tanh(e * p), z is quantized
- * with z_act, passed through the output layer (w_out [V, D], b_out) and a log-softmax.
+ * with z_act, passed through the output layer (w_out [V, D], b_out) and a log-softmax.  A negative
+ * frame index means no frame: z = 0.
  * logp [N, V] fp32.  workspace: q4_workspace_bytes(Q4_WS_JOINT, {N, D}).
  * prepared_pred / prepared_out (nullable): buffers of q4_prepare_linear for w_pred and w_out; with
  * both, a workspace of q4_workspace_bytes(Q4_WS_JOINT, {N, D, Hp_pad}) bytes

@@ -405,10 +405,16 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
 #pragma unroll
       for (int i = 0; i < 32; ++i) v[i] = __fmaf_rn((float)r[i], s_sc[c0 + i], s_bi[c0 + i]);
       if (a.epi == EPI_JOINTZ) {
-        // joint network: z = tanh(e * p) with p the projected value just formed; quantized below
-        const float* er = a.mul_e + (long long)a.mul_idx[mi] * a.J + j0;
+        // joint network: z = tanh(e * p) with p the projected value just formed; quantized below.  A row without a
+        // frame (negative index) has z = 0, as in k_joint_z
+        const int er_idx = a.mul_idx[mi];
+        const float* er = a.mul_e + (long long)er_idx * a.J + j0;
 #pragma unroll
         for (int i = 0; i < 32; i += 4) {
+          if (er_idx < 0) {
+            v[i] = v[i + 1] = v[i + 2] = v[i + 3] = 0.0f;
+            continue;
+          }
           const float4 ev = *reinterpret_cast<const float4*>(er + i);
           v[i] = tanh_fixed(__fmul_rn(ev.x, v[i]));
           v[i + 1] = tanh_fixed(__fmul_rn(ev.y, v[i + 1]));

@@ -51,6 +51,28 @@ def test_joint_logprobs(Bd, N, V, D, Hp, zb, prep):
     np.testing.assert_allclose(np.exp(got.astype(np.float64)).sum(1), 1.0, atol=1e-5)
 
 
+@pytest.mark.parametrize("N,D", [(3, 256), (40, 64), (130, 256)])
+def test_joint_rows_without_a_frame(Bd, N, D):
+    # a negative frame index stands for a frame of zeros, with prepared weights as without
+    dw = synth.decoder(seed=7, V=64, E=32, Hp=128, D=D, Hs=32, Ht=32)
+    st = synth.Stream(11)
+    e = st.normal("e", (9, D)).astype(np.float32)
+    fi = st.integers("fi", (N,), 0, 8).astype(np.int32)
+    fi[[0, N // 2, N - 1]] = -1
+    hid = O.act_symmetric(1.0, 4)
+    pq = st.integers("pq", (N, 128), -7, 7).astype(np.int16)
+    frames = np.where(fi[:, None] >= 0, e[fi], np.float32(0))
+    want = O.joint(O.Decoder(dw), frames, O.linear(O.Linear(dw.pred.proj), pq, hid))
+    dd = Bd.Decoder(dw)
+    for prepare in (False, True):
+        if prepare:
+            dd.pred_proj.prepare()
+            dd.joint_out.prepare()
+        got = Bd.qjoint_logprobs(torch.from_numpy(e).cuda(), torch.from_numpy(fi).cuda(), pack_codes(pq, hid), to_act(hid),
+                                 dd.pred_proj, dd.z_act, dd.joint_out).cpu().numpy()
+        assert np.abs(got - want).max() <= LP_ATOL
+
+
 def pred_joint_gpu(Bd, dd, e_dev, frame_idx, tokens):
     """Teacher-forced prediction network + joint on the GPU: logp [N,S,V], hq codes [N,S,Hp]."""
     N, S = tokens.shape
