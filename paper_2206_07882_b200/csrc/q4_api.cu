@@ -371,7 +371,8 @@ int qlstm_step(const void* xq, const q4_act* x_act, const int32_t* x_row_idx, co
   {
     const int32_t wd[3] = {N, w_ih->k_pad, H};
     if (prepared && workspace && hq_out && H % 128 == 0 && aligned16(workspace) && aligned16(prepared) &&
-        (dbg_acc_ih == nullptr) == (dbg_acc_hh == nullptr) && c_out != nullptr &&
+        (dbg_acc_ih == nullptr) == (dbg_acc_hh == nullptr) &&
+        aligned16(c_in) && aligned16(c_out) && aligned16(h_f32_out) &&   // moved 16 bytes and more at a time
         workspace_bytes >= q4_workspace_bytes(Q4_WS_LSTM_STEP, wd, 3)) {
       // tensor cores, any number of rows (33: 8.4 us of device time, 24.7 on the DP4A kernel): int8 copies of
       // the x rows (gathered) and h rows, then the fused LSTM kernel on the
@@ -989,6 +990,7 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
   const bool use_mma = m.prepared != nullptr && m.src.n_layers == 1 &&
                        m.src.lstm[0].w_ih.k_pad == Ep && m.tgt.lstm[0].w_ih.k_pad == Ep &&
                        Hp % 128 == 0 && Hs % 128 == 0 && Ht % 128 == 0 &&
+                       aligned16(st.pred_c) && aligned16(st.src_c) && aligned16(st.tgt_c[0]) && aligned16(st.tgt_c[1]) &&
                        workspace_bytes >= q4_workspace_bytes(Q4_WS_BEAM, dims8, 8);
   if (use_mma) {
     const size_t Np = ((size_t)N + 127) / 128 * 128;

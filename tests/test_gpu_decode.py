@@ -292,6 +292,28 @@ def test_tensor_core_search_odd_vocabulary(Bd, V, D):
     assert tr == 1.0
 
 
+def test_search_with_cell_states_at_odd_addresses(Bd):
+    # cell states that start at no 16-byte boundary: the kernels for unprepared weights take such a search
+    dw = synth.decoder(seed=64, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=5, W=8)
+    e = synth.Stream(18).normal("e", (12, 3, 256)).astype(np.float32)
+    dd = Bd.Decoder(dw)
+    dd.alloc_state(3, 8, 17)
+    keep = []
+
+    def odd(name):
+        n = dd.tensors[name].numel()
+        keep.append(torch.zeros(n + 1, device="cuda"))
+        return keep[-1][1:].data_ptr()
+
+    dd.state.pred_c, dd.state.src_c = odd("pred_c"), odd("src_c")
+    dd.state.tgt_c[0], dd.state.tgt_c[1] = odd("tgt_c0"), odd("tgt_c1")
+    tokens, lens, scores = (t.cpu().numpy() for t in dd.decode(torch.from_numpy(e).cuda()))
+    assert dd.tensors["status"].item() == 0
+    ref = O.alsd(O.Decoder(dw), e)
+    frac, tr = compare_search(dd, tokens, lens, scores, ref, list(range(3)), 12, 5, 8, min_same=1.0)
+    assert tr == 1.0
+
+
 @pytest.mark.parametrize("V", [20, 46])
 @pytest.mark.parametrize("tensor_cores", [True, False])
 def test_search_label_budget_of_one(Bd, V, tensor_cores):

@@ -457,6 +457,30 @@ def test_step_on_the_tensor_cores_with_prepared_weights(Bd, N, K, H, xb, hb, sig
     assert Bd.launch_count() - n0 >= 3
 
 
+@pytest.mark.parametrize("N", [20, 40, 130])
+def test_step_with_cell_states_at_odd_addresses(Bd, N):
+    # cell states and the real-valued output that start at no 16-byte boundary: the general kernel takes them
+    st = synth.Stream(600 + N)
+    lw = synth._lstm(st, "l", 64, 128, 4, bias_std=0.2, hid_alpha=0.95, hid_bits=4)
+    x_act, hid = O.act_symmetric(3.0, 4), O.act_symmetric(0.95, 4)
+    xq = st.integers("xq", (N, 64), -7, 7).astype(np.int16)
+    hq = st.integers("hq", (N, 128), -7, 7).astype(np.int16)
+    c = st.normal("c", (N, 128)).astype(np.float32)
+    want = O.lstm_step(O.Lstm([lw]), xq, x_act, hq, c, hid)
+    dl = Bd.DeviceLstm(lw).prepare()
+    odd = lambda: torch.zeros(N * 128 + 1, device="cuda")[1:].view(N, 128)
+    for which in ("c_in", "c", "h", "all"):
+        c_in = odd() if which in ("c_in", "all") else torch.empty((N, 128), device="cuda")
+        c_in.copy_(torch.from_numpy(c))
+        out = {"hq": torch.empty((N, 64), dtype=torch.uint8, device="cuda")}
+        out["c"] = odd() if which in ("c", "all") else torch.empty((N, 128), device="cuda")
+        out["h"] = odd() if which in ("h", "all") else torch.empty((N, 128), device="cuda")
+        got = Bd.qlstm_step(pack_codes(xq, x_act, dl.w_ih.k_pad), to_act(x_act), pack_codes(hq, hid), c_in, dl, out=out)
+        np.testing.assert_array_equal(got["c"].cpu().numpy(), want["c"])
+        np.testing.assert_array_equal(got["h"].cpu().numpy(), want["h"])
+        np.testing.assert_array_equal(gpu_codes(got["hq"], 128, hid), want["hq"])
+
+
 def wide_step_operands(seed, N, K, H):
     """One 8-bit layer (the same for every seed) and a set of operands of a step"""
     st, wt = synth.Stream(seed), synth.Stream(1)
