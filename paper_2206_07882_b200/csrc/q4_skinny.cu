@@ -67,22 +67,8 @@ __global__ void __launch_bounds__(SK_THREADS, NT == 4 ? 2 : SK_CTAS_PER_SM) k_sk
   const uint32_t M = 0xF0F0F0F0u;
   const bool x_unsigned = a.x_signed == 0;
 
-  // the de-quantization constants of the thread's item of the closing stage (cell ec of the CTA's 4,
-  // row en) do not depend on the previous kernel of the stream: they are sent on their way to shared
-  // memory first (row scales and bias of the item's four gate rows; no registers are held for them)
-  const int ec = tid & 3, en = tid >> 2;
-  float* ecst = reinterpret_cast<float*>(sk_smem + SK_WARPS * 2 * 16 * 8 * NT + SK_WARPS * 16);   // [12][32 NT]
-  if (tid < 32 * NT) {
-#pragma unroll
-    for (int gate = 0; gate < 4; ++gate) {
-      const long long row = (long long)gate * H + cell0 + ec;
-      cp_async4(ecst + (gate * 3 + 0) * 32 * NT + tid, a.s_wih + row);
-      cp_async4(ecst + (gate * 3 + 1) * 32 * NT + tid, a.s_whh + row);
-      if (a.bias) cp_async4(ecst + (gate * 3 + 2) * 32 * NT + tid, a.bias + row);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  }
-  pdl_wait();   // nothing produced by an earlier kernel is read before this
+  pdl_wait();   // nothing is read before this: an earlier kernel of the stream may be writing the weights' scales
+  const int ec = tid & 3, en = tid >> 2;   // the thread's item of the closing stage: cell ec of the CTA's 4, row en
   // row bookkeeping: every index is requested at once (the arrays hold an entry for each of the N launch
   // rows), the count of rows with work only masks them afterwards
   int n_act = a.N;
@@ -102,6 +88,19 @@ __global__ void __launch_bounds__(SK_THREADS, NT == 4 ? 2 : SK_CTAS_PER_SM) k_sk
   }
   if (a.n_active) n_act = min(n_act, *a.n_active);
   if (n_act <= 0) return;
+  // the item's de-quantization constants (row scales and bias of its four gate rows) are sent on their way to
+  // shared memory: no registers are held for them
+  float* ecst = reinterpret_cast<float*>(sk_smem + SK_WARPS * 2 * 16 * 8 * NT + SK_WARPS * 16);   // [12][32 NT]
+  if (tid < 32 * NT) {
+#pragma unroll
+    for (int gate = 0; gate < 4; ++gate) {
+      const long long row = (long long)gate * H + cell0 + ec;
+      cp_async4(ecst + (gate * 3 + 0) * 32 * NT + tid, a.s_wih + row);
+      cp_async4(ecst + (gate * 3 + 1) * 32 * NT + tid, a.s_whh + row);
+      if (a.bias) cp_async4(ecst + (gate * 3 + 2) * 32 * NT + tid, a.bias + row);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
 #pragma unroll
   for (int j = 0; j < NT; ++j)
     if (8 * j + g >= n_act || drow[j] < 0) xrow[j] = hrow[j] = -1;

@@ -1,4 +1,6 @@
 """Helpers shared by the GPU parity tests (comparison rules, code unpacking)."""
+import ctypes as C
+
 import numpy as np
 import torch
 
@@ -68,3 +70,20 @@ def to_act(a):
     """oracle Act -> library Act (same five constants)."""
     from paper_2206_07882_b200 import binding as Bd
     return Bd.Act(a.scale, a.inv_scale, a.zero_point, a.bits, a.is_signed)
+
+
+def written_late(Bd, scales: torch.Tensor):
+    """A function that has the first of `scales` (row scales of a weight matrix) rewritten by a quantizer on the
+    current stream, which lets its successor start at once and takes some microseconds; the value is the same
+    every time and is zero until then.  What is enqueued next is on the stream before the quantizer runs."""
+    x = torch.linspace(-0.03, 0.03, 384 * 512, device="cuda").reshape(384, 512)
+    codes = torch.empty((384, 256), dtype=torch.uint8, device="cuda")
+    act = Bd.q4_act_symmetric(1.0, 4)
+
+    def write():
+        scales[:1].zero_()
+        torch.cuda._sleep(2_000_000)
+        assert Bd.lib().quantize_pack_int4(Bd._p(x), C.c_int32(0), C.c_int64(384), C.c_int32(512), C.c_int32(512),
+                                           C.byref(act), C.c_int32(1), C.c_int32(1), None, Bd._p(codes), Bd._p(scales),
+                                           Bd._stream()) == 0
+    return write

@@ -6,7 +6,7 @@ import torch
 
 from oracle import oracle as O
 from paper_2206_07882_b200 import synth
-from _parity import assert_close, assert_codes_match, gpu_codes, near_tie, pack_codes, to_act
+from _parity import assert_close, assert_codes_match, gpu_codes, near_tie, pack_codes, to_act, written_late
 
 pytestmark = pytest.mark.gpu
 
@@ -479,6 +479,28 @@ def test_step_with_cell_states_at_odd_addresses(Bd, N):
         np.testing.assert_array_equal(got["c"].cpu().numpy(), want["c"])
         np.testing.assert_array_equal(got["h"].cpu().numpy(), want["h"])
         np.testing.assert_array_equal(gpu_codes(got["hq"], 128, hid), want["hq"])
+
+
+@pytest.mark.parametrize("N,bits", [(8, 4), (20, 4), (40, 4), (8, 8)])
+def test_step_after_a_kernel_that_writes_its_scales(Bd, N, bits):
+    # the kernel before the step on the stream, which lets its successor start early, writes one of the row scales
+    st = synth.Stream(700 + N)
+    x_act, hid = O.act_symmetric(3.0, bits), O.act_symmetric(0.95, bits)
+    lw = synth._lstm(st, "l", 128, 128, 4, bias_std=0.2, hid_alpha=0.95, hid_bits=bits)
+    xq = pack_codes(st.integers("xq", (N, 128), -7, 7).astype(np.int16), x_act)
+    hq = pack_codes(st.integers("hq", (N, 128), -7, 7).astype(np.int16), hid)
+    c = torch.from_numpy(st.normal("c", (N, 128)).astype(np.float32)).cuda()
+    dl = Bd.DeviceLstm(lw)
+    for scales in (dl.w_ih.scale, dl.w_hh.scale):
+        write = written_late(Bd, scales)
+        write()
+        torch.cuda.synchronize()
+        want = Bd.qlstm_step(xq, to_act(x_act), hq, c, dl)
+        for _ in range(3):
+            write()
+            got = Bd.qlstm_step(xq, to_act(x_act), hq, c, dl)
+            for k in ("c", "h", "hq"):
+                assert torch.equal(got[k], want[k])
 
 
 def wide_step_operands(seed, N, K, H):
