@@ -830,18 +830,6 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
     prefetch_tmap(&tma_wb);
     prefetch_tmap(&tma_wo);
   }
-  if (warp < HEAD_EPI_WARPS) {   // de-quantization constants: weights only, nothing of the previous kernel
-    if (tid < HEAD_BN1 && nk1 > 0) {
-      const int c = nb * HEAD_BN1 + tid;
-      s_sc1[tid] = __fmul_rn(a.x_scale, __ldg(a.sc_bott + c));
-      s_b1[tid] = a.b_bott ? __ldg(a.b_bott + c) : 0.0f;
-    }
-    for (int c = tid; c < NB; c += 32 * HEAD_EPI_WARPS) {
-      const int j = min(nb * NB + c, a.V - 1);
-      s_sc2[c] = __fmul_rn(a.q_scale, __ldg(a.sc_out + j));
-      s_b2[c] = a.b_out ? __ldg(a.b_out + j) : 0.0f;
-    }
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -926,6 +914,18 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
     const bool busy = __any_sync(0xffffffffu, dst >= 0);   // a warp without a row to store computes nothing
     bool ok = true;
     const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16);
+    // de-quantization constants, in the shadow of the operands' way; like all else after the wait
+    if (tid < HEAD_BN1 && nk1 > 0) {
+      const int c = nb * HEAD_BN1 + tid;
+      s_sc1[tid] = __fmul_rn(a.x_scale, __ldg(a.sc_bott + c));
+      s_b1[tid] = a.b_bott ? __ldg(a.b_bott + c) : 0.0f;
+    }
+    for (int c = tid; c < NB; c += 32 * HEAD_EPI_WARPS) {
+      const int j = min(nb * NB + c, a.V - 1);
+      s_sc2[c] = __fmul_rn(a.q_scale, __ldg(a.sc_out + j));
+      s_b2[c] = a.b_out ? __ldg(a.b_out + j) : 0.0f;
+    }
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * HEAD_EPI_WARPS) : "memory");
     if (nk1 > 0) {
       const int lo = act_lo(a.bott_act), hi = act_hi(a.bott_act), zp = a.bott_act.zero_point;
       ok = mbar_wait(&acc1_full, 0);

@@ -6,7 +6,7 @@ import torch
 
 from oracle import oracle as O
 from paper_2206_07882_b200 import synth
-from _parity import gpu_codes, pack_codes, to_act
+from _parity import gpu_codes, pack_codes, to_act, written_late
 
 pytestmark = pytest.mark.gpu
 
@@ -475,6 +475,31 @@ def test_replayed_search_equals_its_steps(Bd, S):
         assert a.tensors["status"].item() == 0 and torch.equal(a.tensors["fin_n"], b.tensors["fin_n"])
         for k in ("bp_parent", "bp_token", "bp_score"):
             assert torch.equal(a.tensors[k][:n], b.tensors[k]), k
+
+
+def test_step_after_a_kernel_that_writes_the_output_scales(Bd):
+    # the first call of a frame runs the joint network only; the kernel before it, which lets its successor start
+    # early, writes the blank's row scale of the output layer
+    dw = synth.decoder(seed=69, V=300, E=32, Hp=128, D=256, Hs=128, Ht=128, U_max=4, W=4)
+    e = torch.from_numpy(synth.Stream(21).normal("e", (3, 2, 256)).astype(np.float32)).cuda()
+    dd = Bd.Decoder(dw)
+    write = written_late(Bd, dd.joint_out.w.scale)
+
+    def scores(late):
+        dd.alloc_state(2, 4, 6, 1)
+        write()
+        torch.cuda.synchronize()
+        dd.q4_beam_init()
+        for it in range(3):
+            if late and it == 2:
+                write()
+            dd.dr_fusion_beam_step(e, 3, it, 4, mode=1 + it % 2)
+        torch.cuda.synchronize()
+        return torch.cat([dd.tensors["bp_score"][:3].flatten(), dd.tensors["nb_score"].flatten()])
+
+    want = scores(False)
+    for _ in range(3):
+        assert torch.equal(scores(True), want)
 
 
 def test_time_synchronous_search_tensor_core_path(Bd):
