@@ -51,7 +51,7 @@ __device__ __forceinline__ void unpack_piece32(const uint8_t* p, int k, int bits
 // (their number may be known on the device only).
 __global__ void __launch_bounds__(256) k_unpack_multi(const __grid_constant__ UnpackJobs jobs) {
   // A dependent successor may set itself up; it reads nothing before this grid has completed but, in a search, the count
-  // of rows with work (see count_visible), so there the trigger has to follow the wait.
+  // of rows with work (see tile_without_work), so there the trigger has to follow the wait.
   if (!jobs.n_active) pdl_trigger();
   pdl_wait();      // launched as a programmatic dependent itself: the source rows may be the predecessor's output
   if (jobs.n_active) pdl_trigger();
@@ -263,13 +263,27 @@ __device__ __forceinline__ void flag_timeout(int32_t* status) {
   if (status) atomicExch(status, Q4_ERR_TIMEOUT);
 }
 
-// Row counts of the search (n_active of the kernels below), count_visible: the count is written by the selection, and
-// the first kernel of a step's chains (the gather, or a kernel behind an event) waits for that before it
-// triggers its successor.  So every later kernel of the step may read the count as its first act, and a tile
-// without work leaves before it has set anything up or occupied an SM for long: in an iteration without labels
-// (two of three in speech) that is every tile of seven kernels.  Against tiles that
-// found out after their set-up, 150 iterations: few labels 1 x 16 slots 3.59 -> 3.43 ms, 4 x 8 slots of the paper's model
-// 3.36 -> 3.10; labels in most 4.38 -> 4.35 and 5.26 -> 4.99.
+// Row tiles without work (n_active: the device's count of rows with work in a search step).  A tile beyond the count
+// leaves as its first act, before it has set anything up or waited: in an iteration without labels (two of three in
+// speech) that is every tile of seven kernels, and tiles that found out after their set-up cost 150 iterations with few
+// labels 1 x 16 slots 3.59 against 3.43 ms, 4 x 8 slots of the paper's model 3.36 against 3.10.
+//   The count is the one thing that is read before the kernel's wait.  The selection writes it; the first kernel of
+// a step's chains (the gather, the weight-streaming step or a kernel behind an event) triggers its successor only after its own wait
+// for the selection, and every later kernel of a chain starts after that.  So the count is in memory when any of these
+// kernels starts, and a load that acquires at the scope of the device cannot meet an older copy of it.
+//   A grid whose tiles all leave must not complete before its predecessor does, because its successor waits for this
+// grid only: one CTA of the first row tile, which leaves only if all do, waits before it leaves.
+__device__ __forceinline__ bool tile_without_work(const int32_t* n_active, int m0) {
+  if (!n_active) return false;
+  int32_t n;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(n) : "l"(n_active) : "memory");
+  if (m0 < n) return false;
+  if (m0 == 0 && blockIdx.x == 0) {
+    pdl_trigger();
+    pdl_wait();
+  }
+  return true;
+}
 
 // ------------------------------------------------------------------ plain GEMM
 struct MmaGemmArgs {
@@ -311,7 +325,7 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
   const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * GEMM_BN;   // row tiles slowest: tiles with work are dispatched first
   const int nk = (a.K + BK - 1) / BK;
-  if (a.n_active && m0 >= *a.n_active) return;   // whole tile without work (count_visible)
+  if (tile_without_work(a.n_active, m0)) return;
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -809,7 +823,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
   const int m0 = blockIdx.y * BM;
   const int nb = blockIdx.x;                    // my blocks of columns = my cluster rank
   const int nk1 = (a.H + BK - 1) / BK;
-  if (a.n_active && m0 >= *a.n_active) return;   // row tile without work: the whole cluster leaves (count_visible)
+  if (tile_without_work(a.n_active, m0)) return;   // the whole cluster leaves
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -1193,7 +1207,7 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
   const int nkx = a.acc_pre ? 0 : (a.Kx_pad + BK - 1) / BK;
   const int nkh = (a.H + BK - 1) / BK;
   const int nk = nkx + nkh;
-  if (a.n_active && m0 >= *a.n_active) return;   // whole tile without work (count_visible)
+  if (tile_without_work(a.n_active, m0)) return;
 
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
@@ -1216,8 +1230,9 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
   // Everything above overlaps the tail of the previous kernel of the stream.  With h_first only
-  // the input operand is that kernel's output: the recurrent half of the K loop (operands from
-  // kernels further back, all complete) runs before the wait, the input half after it.
+  // the input operand is that kernel's output: the recurrent half of the K loop runs before the wait, the input half
+  // after it.  Its operands are weights and rows that the gather wrote; the kernel between waited for the gather
+  // before it triggered, and the tile copies read them from the L2.
   const bool h_first = a.h_first != 0 && nkx > 0;
   if (!h_first) pdl_wait();
   if (a.trigger_early) pdl_trigger();   // the successor has a half it can run beside this kernel
@@ -1277,6 +1292,7 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
     pdl_trigger();
     if (!ok && lane == 0) flag_timeout(a.status);
   } else if (warp < LSTM_EPI_WARPS) {
+    if (h_first) pdl_wait();   // the row lists and cell states below are read after it, beside the input half
     const int q = warp & 3, hf = warp >> 2;
     const int rt = q * 32 + lane;            // row within the tile
     const int n = m0 + rt;                   // row of this launch
@@ -1318,7 +1334,6 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
     asm volatile("bar.sync 1, %0;" ::"n"(32 * LSTM_EPI_WARPS) : "memory");
     const bool ok = mbar_wait(&acc_full, 0);
     tc_fence_after();
-    if (h_first) pdl_wait();   // before the first global write of this thread
     pdl_trigger();   // the main loop is over: the next kernel may set itself up
     if (!ok && lane == 0) flag_timeout(a.status);
     const bool live = ok && dst >= 0;

@@ -351,6 +351,29 @@ def test_selection_paths_and_launch_modes_agree(Bd):
         np.testing.assert_array_equal(base[3], other[3])
 
 
+@pytest.mark.parametrize("V,act_bits", [(1024, 4), (46, 8)])
+def test_search_on_one_stream_without_labels(Bd, V, act_bits):
+    # 64 rows without side streams; the label budgets are spent early, so that in most iterations every tile of the
+    # networks' kernels leaves at once, between the joint network and the selection: the same beams as in plain
+    # stream order
+    dw = synth.decoder(seed=66, V=V, E=32, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=5, W=16, all_bits=act_bits)
+    dw.joint.out.bias[0] -= np.float32(10.0)
+    e = torch.from_numpy(synth.Stream(22).normal("e", (60, 4, 256)).astype(np.float32)).cuda()
+    dd = Bd.Decoder(dw, concurrent=False)
+    keys = ("bp_parent", "bp_token", "bp_score", "fin_score", "fin_iter", "fin_slot")
+    prev = Bd.dependent_launch_set(False)
+    try:
+        dd.decode(e)
+        want = {k: dd.tensors[k].clone() for k in keys}
+    finally:
+        Bd.dependent_launch_set(prev)
+    assert int(((want["bp_token"] > 0).flatten(1).sum(1) == 0).sum()) > 40
+    for _ in range(5):
+        dd.decode(e)
+        for k in keys:
+            assert torch.equal(dd.tensors[k], want[k]), k
+
+
 def check_search_invariants(dd, tokens, lens, scores, T, B, W, U, V=1024):
     """Properties of an alignment-length synchronous search that hold at any size."""
     assert dd.tensors["status"].item() == 0
