@@ -48,10 +48,11 @@ extern "C" {
 
 typedef void* q4_stream; /* a cudaStream_t, passed as an opaque handle (NULL = default stream) */
 /* All work of a call is enqueued on its stream, in stream order with whatever the caller enqueued before.
- * Kernels of the tensor-core paths are launched with programmatic stream serialization: one may be
- * scheduled while its predecessor in the stream is draining, but every kernel waits for the completion of
- * its predecessor (and the visibility of its writes) before it reads anything, so results never depend on
- * it. */
+ * Kernels of the tensor-core paths are launched with programmatic stream serialization: one may
+ * be scheduled while its predecessor in the stream is draining, but it waits for the completion of its predecessor
+ * (and the visibility of its writes) before it reads anything that work before the call may be writing:
+ * inputs, weights, scales and states.  Before that it reads at most what an earlier kernel of the same call wrote and
+ * has completed (prepared operands of a layer, the count of rows with work).  Results never depend on it. */
 
 /* Integer weight matrix [rows, k_pad] with per-row scales (device pointers). */
 typedef struct {
@@ -403,9 +404,8 @@ int64_t q4_launch_count(void);
  * sequences counts once).  reset != 0 sets the counter back to zero after reading it. */
 int64_t q4_quantizer_calls(int32_t reset);
 
-/* dr_fusion_beam_step launches consecutive kernels of one stream as programmatic dependents
- * (each kernel sets itself up while its predecessor drains and waits for the predecessor's
- * completion before it reads anything).  enabled = 0 switches this off (plain stream order),
+/* Consecutive kernels of one stream are launched as programmatic dependents (each sets itself up
+ * while its predecessor drains and waits for the predecessor's completion, see above).  enabled = 0 switches this off (plain stream order),
  * non-zero switches it on (the default).  Returns the previous setting.  Results do not depend
  * on it.  Not an operation of the paper. */
 int q4_dependent_launch_set(int32_t enabled);

@@ -13,10 +13,49 @@ namespace q4 {
 // start while its predecessor in the stream is still running; pdl_wait() returns once that
 // predecessor has completed and its writes are visible (at once when the launch carries no such
 // attribute), pdl_trigger() lets the successor's CTAs be scheduled once every CTA of this grid
-// has called it or exited.  Nothing produced by an earlier kernel is read before pdl_wait().
+// has called it or exited.
+//
+// What a kernel may read before pdl_wait(): nothing that any kernel before it on the stream may be writing, the
+// caller's own kernels included.  Two exceptions read what a kernel of the same call further back wrote, in
+// chains whose every kernel between triggers only after its own wait, so that the writer has completed and its
+// writes are in the L2 when the reader starts:
+//   the count of rows with work (tile_without_work in q4_mma.cu);
+//   a layer's recurrence its prepared weights, constants and input scales (written before the input projection),
+//   and a second LSTM layer the operand tiles of its recurrent half (weights, and rows that the gather wrote).
+// They are read by the loads below, or by tile copies, which do not look into the L1.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
+__device__ __forceinline__ int32_t ld_acquire(const int32_t* p) {
+  int32_t v;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+// loads that are coherent at device scope
+__device__ __forceinline__ uint32_t ld_coherent(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ld_coherent(const float* p) {
+  float v;
+  asm volatile("ld.relaxed.gpu.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint2 ld_coherent(const uint2* p) {
+  uint2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint4 ld_coherent(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.relaxed.gpu.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_coherent(const float4* p) {
+  float4 v;
+  asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
 
 constexpr int TILE = 64;        // rows of each operand per CTA tile
 constexpr int KC = 128;         // K elements staged per chunk

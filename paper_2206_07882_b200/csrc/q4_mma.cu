@@ -275,9 +275,7 @@ __device__ __forceinline__ void flag_timeout(int32_t* status) {
 // grid only: one CTA of the first row tile, which leaves only if all do, waits before it leaves.
 __device__ __forceinline__ bool tile_without_work(const int32_t* n_active, int m0) {
   if (!n_active) return false;
-  int32_t n;
-  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(n) : "l"(n_active) : "memory");
-  if (m0 < n) return false;
+  if (m0 < ld_acquire(n_active)) return false;
   if (m0 == 0 && blockIdx.x == 0) {
     pdl_trigger();
     pdl_wait();

@@ -88,14 +88,14 @@ k_enc_recurrent(const EncRecArgs a) {
     for (int i = tid; i < rows * per_row; i += REC_THREADS) {
       const int r = i / per_row, c = i % per_row;
       *reinterpret_cast<uint4*>(Ws + (size_t)r * pitch + c * 16) =
-          *reinterpret_cast<const uint4*>(src + (size_t)r * H + c * 16);
+          ld_coherent(reinterpret_cast<const uint4*>(src + (size_t)r * H + c * 16));
     }
     for (int i = tid; i < 2 * BG * pitch / 16; i += REC_THREADS)
       reinterpret_cast<uint4*>(hb)[i] = make_uint4(0, 0, 0, 0);   // h_0 = 0
   }
   __syncthreads();
   cluster_barrier();   // every CTA's buffers are initialised before anyone stores into them
-  pdl_wait();          // the input accumulators are the previous kernel's output; the weights that of the one before it
+  pdl_wait();          // the input accumulators are the previous kernel's output; what was read above is older
 
   const int g = lane >> 2, t4 = lane & 3;   // MMA fragment coordinates
   const int ci = lane >> 3, n = lane & 7;   // this lane's item: cell ci of the warp's 4, sequence n
@@ -361,10 +361,10 @@ k_enc_recurrent_w4(const EncRecArgs a) {
     const int8_t* r1 = r0 + (size_t)2 * H;
 #pragma unroll
     for (int s = 0; s < KS; ++s) {
-      const uint32_t q0 = *reinterpret_cast<const uint32_t*>(r0 + 32 * s);
-      const uint32_t p0 = *reinterpret_cast<const uint32_t*>(r1 + 32 * s);
-      const uint32_t q1 = *reinterpret_cast<const uint32_t*>(r0 + 32 * s + 16);
-      const uint32_t p1 = *reinterpret_cast<const uint32_t*>(r1 + 32 * s + 16);
+      const uint32_t q0 = ld_coherent(reinterpret_cast<const uint32_t*>(r0 + 32 * s));
+      const uint32_t p0 = ld_coherent(reinterpret_cast<const uint32_t*>(r1 + 32 * s));
+      const uint32_t q1 = ld_coherent(reinterpret_cast<const uint32_t*>(r0 + 32 * s + 16));
+      const uint32_t p1 = ld_coherent(reinterpret_cast<const uint32_t*>(r1 + 32 * s + 16));
       const uint32_t w0 = (q0 & 0x0F0F0F0Fu) | ((p0 << 4) & 0xF0F0F0F0u);
       const uint32_t w1 = (q1 & 0x0F0F0F0Fu) | ((p1 << 4) & 0xF0F0F0F0u);
       if (s < KR) {
@@ -380,11 +380,11 @@ k_enc_recurrent_w4(const EncRecArgs a) {
   for (int i = tid; i < cpc; i += REC4_THREADS) {
     // de-quantization products per gate row: input scale * row scale, hidden scale * row scale; bias
     const int c = (int)rank * cpc + i;
-    const float4 w = reinterpret_cast<const float4*>(D.sc_hh)[c], v = reinterpret_cast<const float4*>(D.sc_ih)[c];
+    const float4 w = ld_coherent(reinterpret_cast<const float4*>(D.sc_hh) + c), v = ld_coherent(reinterpret_cast<const float4*>(D.sc_ih) + c);
     const float sxs = a.x_scale;
     cst[i] = make_float4(__fmul_rn(sxs, v.x), __fmul_rn(sxs, v.y), __fmul_rn(sxs, v.z), __fmul_rn(sxs, v.w));
     cst[cpc + i] = make_float4(__fmul_rn(sh, w.x), __fmul_rn(sh, w.y), __fmul_rn(sh, w.z), __fmul_rn(sh, w.w));
-    cst[2 * cpc + i] = reinterpret_cast<const float4*>(D.bias)[c];
+    cst[2 * cpc + i] = ld_coherent(reinterpret_cast<const float4*>(D.bias) + c);
   }
   if (tid == 0) {
     *dead = 0;
@@ -396,7 +396,7 @@ k_enc_recurrent_w4(const EncRecArgs a) {
   fence_proxy_async();   // the zeroed buffers are later written by the bulk-copy engine
   __syncthreads();
   cluster_barrier();   // every CTA's buffers and barriers are initialised before anyone stores into them
-  pdl_wait();          // the input accumulators are the previous kernel's output; the weights that of the one before it
+  pdl_wait();          // the input accumulators are the previous kernel's output; what was read above is older
 
   float c_state[NU];
   bool live[NU];
@@ -659,10 +659,10 @@ k_enc_recurrent_w4s(const EncRecArgs a) {
     const int8_t* r1 = r0 + (size_t)2 * H;
 #pragma unroll
     for (int s = 0; s < KS; ++s) {
-      const uint32_t q0 = *reinterpret_cast<const uint32_t*>(r0 + 32 * s);
-      const uint32_t p0 = *reinterpret_cast<const uint32_t*>(r1 + 32 * s);
-      const uint32_t q1 = *reinterpret_cast<const uint32_t*>(r0 + 32 * s + 16);
-      const uint32_t p1 = *reinterpret_cast<const uint32_t*>(r1 + 32 * s + 16);
+      const uint32_t q0 = ld_coherent(reinterpret_cast<const uint32_t*>(r0 + 32 * s));
+      const uint32_t p0 = ld_coherent(reinterpret_cast<const uint32_t*>(r1 + 32 * s));
+      const uint32_t q1 = ld_coherent(reinterpret_cast<const uint32_t*>(r0 + 32 * s + 16));
+      const uint32_t p1 = ld_coherent(reinterpret_cast<const uint32_t*>(r1 + 32 * s + 16));
       if (W8) {   // one code per byte: the MMA fragment as it is
         if (s < KR) {
           wreg[WPK * s] = q0;
@@ -688,10 +688,10 @@ k_enc_recurrent_w4s(const EncRecArgs a) {
     reinterpret_cast<uint4*>(hb)[i] = make_uint4(0, 0, 0, 0);   // h_0 = 0
   for (int i = tid; i < cpc; i += REC4_THREADS) {
     const int c = (int)rank * cpc + i;
-    const float4 w = reinterpret_cast<const float4*>(D.sc_hh)[c], v = reinterpret_cast<const float4*>(D.sc_ih)[c];
+    const float4 w = ld_coherent(reinterpret_cast<const float4*>(D.sc_hh) + c), v = ld_coherent(reinterpret_cast<const float4*>(D.sc_ih) + c);
     cst[i] = v;   // multiplied with the sequence's input scale at every use (the same fp32 product)
     cst[cpc + i] = make_float4(__fmul_rn(sh, w.x), __fmul_rn(sh, w.y), __fmul_rn(sh, w.z), __fmul_rn(sh, w.w));
-    cst[2 * cpc + i] = reinterpret_cast<const float4*>(D.bias)[c];
+    cst[2 * cpc + i] = ld_coherent(reinterpret_cast<const float4*>(D.bias) + c);
   }
   if (tid == 0) {
     *dead = 0;
@@ -702,7 +702,7 @@ k_enc_recurrent_w4s(const EncRecArgs a) {
   fence_proxy_async();   // the zeroed buffers are later written by the bulk-copy engine
   __syncthreads();
   cluster_barrier();   // every CTA's buffers and barriers are initialised before anyone stores into them
-  pdl_wait();          // the input accumulators are the previous kernel's output; the weights that of the one before it
+  pdl_wait();          // the input accumulators are the previous kernel's output; what was read above is older
 
   const int b_own = j * BG + n, b_shared = (a.groups - 1) * BG + n;
   const bool live_own = b_own < B, live_shared = host && b_shared < B;
@@ -1013,17 +1013,17 @@ k_enc_recurrent_few(const EncRecArgs a) {
     const int8_t* r1 = r0 + (size_t)2 * H;
 #pragma unroll
     for (int s = 0; s < KS; ++s) {
-      const uint2 p = *reinterpret_cast<const uint2*>(r0 + 32 * s), q = *reinterpret_cast<const uint2*>(r1 + 32 * s);
+      const uint2 p = ld_coherent(reinterpret_cast<const uint2*>(r0 + 32 * s)), q = ld_coherent(reinterpret_cast<const uint2*>(r1 + 32 * s));
       w[4 * s] = p.x;
       w[4 * s + 1] = q.x;
       w[4 * s + 2] = p.y;
       w[4 * s + 3] = q.y;
     }
   }
-  float4 s_ih = reinterpret_cast<const float4*>(D.sc_ih)[cell], s_hh = reinterpret_cast<const float4*>(D.sc_hh)[cell];
-  const float4 bb = reinterpret_cast<const float4*>(D.bias)[cell];
+  float4 s_ih = ld_coherent(reinterpret_cast<const float4*>(D.sc_ih) + cell), s_hh = ld_coherent(reinterpret_cast<const float4*>(D.sc_hh) + cell);
+  const float4 bb = ld_coherent(reinterpret_cast<const float4*>(D.bias) + cell);
   {
-    const float sx = a.x_scale_b && live ? a.x_scale_b[b] : a.x_scale, sh = a.hid_act.scale;
+    const float sx = a.x_scale_b && live ? ld_coherent(a.x_scale_b + b) : a.x_scale, sh = a.hid_act.scale;
     s_ih = make_float4(__fmul_rn(sx, s_ih.x), __fmul_rn(sx, s_ih.y), __fmul_rn(sx, s_ih.z), __fmul_rn(sx, s_ih.w));
     s_hh = make_float4(__fmul_rn(sh, s_hh.x), __fmul_rn(sh, s_hh.y), __fmul_rn(sh, s_hh.z), __fmul_rn(sh, s_hh.w));
   }
@@ -1037,7 +1037,7 @@ k_enc_recurrent_few(const EncRecArgs a) {
   fence_proxy_async();   // the zeroed buffers are later written by asynchronous stores
   __syncthreads();
   cluster_barrier();   // every CTA's buffers and barriers are initialised before anyone stores into them
-  pdl_wait();          // the input accumulators are the previous kernel's output; the weights that of the one before it
+  pdl_wait();          // the input accumulators are the previous kernel's output; what was read above is older
 
   const uint32_t hb_addr = smem_u32(hb), full_addr = smem_u32(full);
   const int hlo = act_lo(a.hid_act), hhi = act_hi(a.hid_act);
