@@ -353,7 +353,7 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
 /*
  * q4_beam_search — all steps of a search on the stream, after q4_beam_init: T + u_max steps of mode 0, or
  * with time_synchronous != 0 the T (S + 1) steps of modes 1 and 2 (S = state->tsd_smax).  Arguments and
- * results as dr_fusion_beam_step; same workspace.  `plan` (nullable): an object of q4_search_plan_create, in which
+ * results as dr_fusion_beam_step; same workspace; no steps (no frames and no label budget) is no error.  `plan` (nullable): an object of q4_search_plan_create, in which
  * the call keeps a number of steps as a CUDA graph.  The graph belongs to the model, state, weights of Eq. 1
  * and workspace it was built for and is rebuilt when one of them changes; frames, T and u_max may change from
  * call to call.  One plan serves one search at a time.  Without a plan, in a stream capture and while launches

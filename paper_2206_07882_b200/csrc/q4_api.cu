@@ -1424,7 +1424,10 @@ static int plan_build(SearchPlan* p, const SearchKey& key) {
 int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, int32_t B, int32_t T, int32_t W, int32_t u_max,
                    float lambda_t, float lambda_s, float rho, int32_t time_synchronous, void* workspace,
                    size_t workspace_bytes, q4_search_plan plan, q4_stream stream) {
-  if (!model || !state || !e || !workspace) return Q4_ERR_NULL;
+  if (!model || !state || !workspace) return Q4_ERR_NULL;
+  const int S1 = time_synchronous ? state->tsd_smax + 1 : 1, n_iters = time_synchronous ? T * S1 : T + u_max;
+  if (n_iters == 0) return Q4_OK;   // no steps: the state stays as q4_beam_init left it
+  if (!e) return Q4_ERR_NULL;
   if (T <= 0 || u_max < 0) return Q4_ERR_DIM;
   if (time_synchronous && (state->tsd_smax < 0 || state->tsd_smax > 3)) return Q4_ERR_DIM;
   SearchKey key;
@@ -1441,7 +1444,6 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
   key.lambda_t = lambda_t;
   key.lambda_s = lambda_s;
   key.rho = rho;
-  const int S1 = key.tsd ? state->tsd_smax + 1 : 1, n_iters = key.tsd ? T * S1 : T + u_max;
   cudaStream_t s = S(stream);
   // step by step: in a stream that is being captured, while launches are timed, and in a short search
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;

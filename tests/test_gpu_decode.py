@@ -292,6 +292,18 @@ def test_tensor_core_search_odd_vocabulary(Bd, V, D):
     assert tr == 1.0
 
 
+def test_search_without_frames(Bd):
+    # no frames and, in the alignment-length search, no label budget: no steps, every utterance's string is empty
+    dw = synth.decoder(seed=64, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=5, W=8)
+    dd = Bd.Decoder(dw)
+    e = torch.empty((0, 3, 256), device="cuda")
+    for result in (dd.decode(e, u_max=0), dd.decode_time_synchronous(e, 2), dd.decode_time_synchronous(e, 0, u_max=0)):
+        tokens, lens, scores = result
+        assert lens.tolist() == [0, 0, 0] and scores.tolist() == [0.0, 0.0, 0.0] and not tokens.any()
+    with pytest.raises(Bd.Q4Error):
+        dd.decode(e, u_max=1)          # a label needs a frame
+
+
 def test_search_with_cell_states_at_odd_addresses(Bd):
     # cell states that start at no 16-byte boundary: the kernels for unprepared weights take such a search
     dw = synth.decoder(seed=64, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=5, W=8)
