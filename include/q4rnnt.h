@@ -364,6 +364,9 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
 typedef void* q4_search_plan;
 int q4_search_plan_create(q4_search_plan* out);
 int q4_search_plan_destroy(q4_search_plan plan);
+/* What a plan has done so far (host counters, for tests and diagnostics): out[0] graphs built, out[1] replays
+ * enqueued, out[2] attempts to build a graph that failed (the search then enqueued its steps one by one). */
+int q4_search_plan_info(q4_search_plan plan, int64_t* out);
 int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, int32_t B, int32_t T, int32_t W,
                    int32_t u_max, float lambda_t, float lambda_s, float rho, int32_t time_synchronous,
                    void* workspace, size_t workspace_bytes, q4_search_plan plan, q4_stream stream);

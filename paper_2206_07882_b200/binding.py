@@ -80,7 +80,7 @@ class BeamStateS(C.Structure):
 
 EXPORTS = ["q4_act_symmetric", "q4_act_asymmetric", "quantize_pack_int4", "qlstm_layer_forward",
            "qlstm_step", "q4_linear_forward", "qjoint_logprobs", "q4_beam_init",
-           "dr_fusion_beam_step", "q4_beam_search", "q4_search_plan_create", "q4_search_plan_destroy", "q4_traceback", "q4_feature_prologue", "q4_workspace_bytes",
+           "dr_fusion_beam_step", "q4_beam_search", "q4_search_plan_create", "q4_search_plan_destroy", "q4_search_plan_info", "q4_traceback", "q4_feature_prologue", "q4_workspace_bytes",
            "q4_poll_status", "q4_version", "q4_launch_count", "q4_dependent_launch_set", "q4_beam_select_exact_set", "q4_timing_set", "q4_timing_count", "q4_prepared_bytes", "q4_prepare_model", "qjoint_logprobs_static", "q4_quantizer_calls", "q4_prepared_lstm_bytes", "q4_prepare_lstm",
            "q4_prepared_linear_bytes", "q4_prepare_linear", "q4_test_wait_expiry_set", "q4_encoder_time_slicing_set", "q4_encoder_recurrence_plan"]
 
@@ -718,6 +718,13 @@ class Decoder:
                                   C.c_int32(self.W), C.c_int32(u_max), C.c_float(dw.lambda_t), C.c_float(dw.lambda_s),
                                   C.c_float(dw.rho), C.c_int32(1 if time_synchronous else 0), _p(self.ws),
                                   C.c_size_t(self.ws.numel()), plan, _stream()), "q4_beam_search")
+
+    def search_plan_info(self) -> dict:
+        """Graphs built, replays enqueued and failed builds of the decoder's search plan."""
+        out = (C.c_int64 * 3)()
+        if self._plan is not None:
+            _chk(lib().q4_search_plan_info(self._plan.handle, out), "q4_search_plan_info")
+        return dict(zip(("built", "replays", "failed"), out))
 
     def q4_traceback(self, n_iters: int, u_max: int):
         dev = self.device

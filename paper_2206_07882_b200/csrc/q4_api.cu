@@ -1357,6 +1357,7 @@ struct SearchKey {                   // everything the graph was built from
 struct SearchPlan {
   SearchKey key;
   int64_t launches, quant_calls;     // of the graph
+  int64_t built, replays, failed;    // graphs made, replays enqueued, attempts to make a graph that failed
   cudaStream_t stream;               // captured on
   cudaEvent_t done;                  // of the last replay
   cudaGraphExec_t exec;
@@ -1402,7 +1403,10 @@ static int plan_build(SearchPlan* p, const SearchKey& key) {
   p->key = key;
   SearchCall* call = static_cast<SearchCall*>(key.workspace);
   const int64_t l0 = g_launches, q0 = g_quant_calls;
-  if (cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return Q4_ERR_CUDA;
+  if (cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+    ++p->failed;
+    return Q4_ERR_CUDA;
+  }
   int r = Q4_OK;
   // T and u_max (and the frames) only have to pass the argument checks here; the first frame's steps are never in the graph
   for (int it = PLAN_ITERS; it < 2 * PLAN_ITERS && r == Q4_OK; ++it)
@@ -1418,7 +1422,17 @@ static int plan_build(SearchPlan* p, const SearchKey& key) {
   p->quant_calls = g_quant_calls - q0;
   g_launches = l0;
   g_quant_calls = q0;
+  ++(r == Q4_OK ? p->built : p->failed);
   return r;
+}
+
+int q4_search_plan_info(q4_search_plan plan, int64_t* out) {
+  if (!plan || !out) return Q4_ERR_NULL;
+  const SearchPlan* p = static_cast<const SearchPlan*>(plan);
+  out[0] = p->built;
+  out[1] = p->replays;
+  out[2] = p->failed;
+  return Q4_OK;
 }
 
 int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, int32_t B, int32_t T, int32_t W, int32_t u_max,
@@ -1466,6 +1480,7 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
       Q4_TRY(cudaGraphLaunch(p->exec, s));
       g_launches += p->launches;
       g_quant_calls += p->quant_calls;
+      ++p->replays;
       it += PLAN_ITERS;
       if (it + PLAN_ITERS > n_iters) Q4_TRY(cudaEventRecord(p->done, s));
       continue;

@@ -537,6 +537,30 @@ def test_step_after_a_kernel_that_writes_the_output_scales(Bd):
         assert torch.equal(scores(True), want)
 
 
+def test_search_plan_builds_and_replays(Bd):
+    # groups of 12 steps after the first two frames' steps; one graph serves the searches on a state, another batch
+    # size takes another; none below 96 steps, in a capture, or without side streams
+    dw = synth.decoder(seed=67, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=9, W=6)
+    frames = lambda T, B: torch.from_numpy(synth.Stream(T + B).normal("e", (T, B, 256)).astype(np.float32)).cuda()
+    dd = Bd.Decoder(dw)
+    dd.decode(frames(80, 3), 15)
+    assert dd.search_plan_info() == dict(built=0, replays=0, failed=0)     # 95 steps
+    dd.alloc_state(3, 6, 120)
+    replays = 0
+    for T, U in ((81, 15), (111, 9), (97, 5)):
+        dd.decode(frames(T, 3), U)
+        replays += (T + U - 2) // 12
+        assert dd.search_plan_info() == dict(built=1, replays=replays, failed=0)
+    dd.decode(frames(111, 5), 9)
+    assert dd.search_plan_info() == dict(built=2, replays=replays + 9, failed=0)
+    captured = Bd.GraphedStep(lambda e=frames(111, 5): dd.decode(e, 9))
+    captured()                                                             # one eager pass, one captured
+    assert dd.search_plan_info() == dict(built=2, replays=replays + 18, failed=0)
+    plain = Bd.Decoder(dw, concurrent=False)
+    plain.decode(frames(111, 5), 9)
+    assert plain.search_plan_info() == dict(built=0, replays=0, failed=0)
+
+
 def test_time_synchronous_search_tensor_core_path(Bd):
     # 8 utterances x 16 slots = 128 rows and a 256-wide bottleneck: tensor-core LSTMs and cluster heads
     dw = synth.decoder(seed=83, V=128, E=32, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=9, W=16)
