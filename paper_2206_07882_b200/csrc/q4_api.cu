@@ -1358,7 +1358,8 @@ struct SearchPlan {
   SearchKey key;
   int64_t launches, quant_calls;     // of the graph
   int64_t built, replays, failed;    // graphs made, replays enqueued, attempts to make a graph that failed
-  cudaStream_t stream;               // captured on
+  cudaStream_t stream, side[2];      // captured on: the graph's chains, none of the caller's streams
+  cudaEvent_t side_event[3];
   cudaEvent_t done;                  // of the last replay
   cudaGraphExec_t exec;
 };
@@ -1379,9 +1380,11 @@ int q4_search_plan_create(q4_search_plan* out) {
   SearchPlan* p = static_cast<SearchPlan*>(calloc(1, sizeof(SearchPlan)));
   if (!p) return Q4_ERR_CUDA;
   *out = p;
-  if (cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking) == cudaSuccess &&
-      cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming) == cudaSuccess)
-    return Q4_OK;
+  bool ok = cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking) == cudaSuccess &&
+            cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming) == cudaSuccess;
+  for (int i = 0; i < 2 && ok; ++i) ok = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking) == cudaSuccess;
+  for (int i = 0; i < 3 && ok; ++i) ok = cudaEventCreateWithFlags(&p->side_event[i], cudaEventDisableTiming) == cudaSuccess;
+  if (ok) return Q4_OK;
   q4_search_plan_destroy(p);
   *out = nullptr;
   return Q4_ERR_CUDA;
@@ -1392,6 +1395,10 @@ int q4_search_plan_destroy(q4_search_plan plan) {
   plan_clear(p);
   if (p->done) cudaEventDestroy(p->done);
   if (p->stream) cudaStreamDestroy(p->stream);
+  for (int i = 0; i < 2; ++i)
+    if (p->side[i]) cudaStreamDestroy(p->side[i]);
+  for (int i = 0; i < 3; ++i)
+    if (p->side_event[i]) cudaEventDestroy(p->side_event[i]);
   free(p);
   return Q4_OK;
 }
@@ -1459,9 +1466,15 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
   key.lambda_s = lambda_s;
   key.rho = rho;
   cudaStream_t s = S(stream);
+  // The graph's side chains are captured on the plan's own streams: a stream lent by the caller may be in use for other
+  // work meanwhile, which would be captured with them.
+  SearchPlan* p = static_cast<SearchPlan*>(plan);
+  const q4_beam_state& st = key.state;
+  const bool lent = st.aux_stream[0] && st.aux_stream[1] && st.aux_event[0] && st.aux_event[1] && st.aux_event[2];
+  for (int i = 0; i < 2; ++i) key.state.aux_stream[i] = p && lent ? p->side[i] : nullptr;
+  for (int i = 0; i < 3; ++i) key.state.aux_event[i] = p && lent ? p->side_event[i] : nullptr;
   // step by step: in a stream that is being captured, while launches are timed, and in a short search
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  SearchPlan* p = static_cast<SearchPlan*>(plan);
   if (p && (n_iters < PLAN_MIN_ITERS || timing_active() || cudaStreamIsCapturing(s, &cap) != cudaSuccess ||
             cap != cudaStreamCaptureStatusNone))
     p = nullptr;

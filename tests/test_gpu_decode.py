@@ -561,6 +561,24 @@ def test_search_plan_builds_and_replays(Bd):
     assert plain.search_plan_info() == dict(built=0, replays=0, failed=0)
 
 
+def test_search_plan_captures_no_stream_of_the_caller(Bd):
+    # the side streams lent with the state are not part of the graph: with others in their place it still serves
+    dw = synth.decoder(seed=67, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=9, W=6)
+    e = torch.from_numpy(synth.Stream(23).normal("e", (111, 3, 256)).astype(np.float32)).cuda()
+    dd = Bd.Decoder(dw)
+    want = [t.clone() for t in dd.decode(e)]
+    lent = [torch.cuda.Stream() for _ in range(2)], [torch.cuda.Event() for _ in range(3)]
+    for ev in lent[1]:
+        ev.record()
+    for i in range(2):
+        dd.state.aux_stream[i] = lent[0][i].cuda_stream
+    for i in range(3):
+        dd.state.aux_event[i] = lent[1][i].cuda_event
+    for x, y in zip(dd.decode(e), want):
+        assert torch.equal(x, y)
+    assert dd.search_plan_info() == dict(built=1, replays=18, failed=0)
+
+
 def test_time_synchronous_search_tensor_core_path(Bd):
     # 8 utterances x 16 slots = 128 rows and a 256-wide bottleneck: tensor-core LSTMs and cluster heads
     dw = synth.decoder(seed=83, V=128, E=32, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=9, W=16)
