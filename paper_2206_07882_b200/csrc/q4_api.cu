@@ -1363,6 +1363,14 @@ struct SearchPlan {
   cudaEvent_t done;                  // of the last replay
   cudaGraphExec_t exec;
 };
+// While one of these lives, calls of this thread that a capture elsewhere in the process would take for unsafe (streams
+// and events made or destroyed, a graph instantiated, an event asked) leave that capture alone: none of them
+// concerns it.  A plan may be made, used or dropped while another thread captures.
+struct BesideCaptures {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
 void plan_clear(SearchPlan* p) {
   if (!p->exec) return;
   cudaEventSynchronize(p->done);
@@ -1377,6 +1385,7 @@ int step_mode(const SearchKey& k, int iter) {
 
 int q4_search_plan_create(q4_search_plan* out) {
   if (!out) return Q4_ERR_NULL;
+  const BesideCaptures guard;
   SearchPlan* p = static_cast<SearchPlan*>(calloc(1, sizeof(SearchPlan)));
   if (!p) return Q4_ERR_CUDA;
   *out = p;
@@ -1391,6 +1400,7 @@ int q4_search_plan_create(q4_search_plan* out) {
 }
 int q4_search_plan_destroy(q4_search_plan plan) {
   if (!plan) return Q4_OK;
+  const BesideCaptures guard;
   SearchPlan* p = static_cast<SearchPlan*>(plan);
   plan_clear(p);
   if (p->done) cudaEventDestroy(p->done);
@@ -1406,6 +1416,7 @@ int q4_search_plan_destroy(q4_search_plan plan) {
 // The graph of the present arguments, rebuilt when any of them has changed.
 static int plan_build(SearchPlan* p, const SearchKey& key) {
   if (p->exec && memcmp(&p->key, &key, sizeof(key)) == 0) return Q4_OK;
+  const BesideCaptures guard;
   plan_clear(p);
   p->key = key;
   SearchCall* call = static_cast<SearchCall*>(key.workspace);

@@ -579,6 +579,45 @@ def test_search_plan_captures_no_stream_of_the_caller(Bd):
     assert dd.search_plan_info() == dict(built=1, replays=18, failed=0)
 
 
+def test_search_beside_a_capture_of_another_thread(Bd):
+    # a search that creates its plan and builds its graph on one thread leaves a capture that another thread has open
+    # (in the strictest mode, torch's default) as it is
+    import threading
+    dw = synth.decoder(seed=67, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=9, W=6)
+    e = torch.from_numpy(synth.Stream(23).normal("e", (111, 3, 256)).astype(np.float32)).cuda()
+    first = Bd.Decoder(dw)
+    first.decode(e)                          # kernels are loaded
+    dd = Bd.Decoder(dw, share_from=first)
+    dd.alloc_state(3, 6, 120)
+    x = torch.zeros(8, device="cuda")
+    side, failure = torch.cuda.Stream(), []
+
+    def search():
+        try:
+            for lam in (dw.lambda_t, 0.25):                  # the second search builds another graph
+                dd.dw.lambda_t = lam
+                with torch.cuda.stream(side):
+                    dd.q4_beam_init()
+                    dd.q4_beam_search(e, 111, 9)
+        except Exception as error:
+            failure.append(error)
+
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        x.add_(1.0)
+        worker = threading.Thread(target=search)
+        worker.start()
+        worker.join()
+        x.add_(2.0)
+    assert not failure, failure
+    x.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert x.tolist() == [3.0] * 8
+    assert dd.search_plan_info() == dict(built=2, replays=18, failed=0)
+
+
 def test_time_synchronous_search_tensor_core_path(Bd):
     # 8 utterances x 16 slots = 128 rows and a 256-wide bottleneck: tensor-core LSTMs and cluster heads
     dw = synth.decoder(seed=83, V=128, E=32, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=9, W=16)
