@@ -3,9 +3,9 @@
  *
  * C ABI of the CUDA library.  All tensor pointers are DEVICE pointers owned by
  * the caller unless a parameter says "host"; they must be 16-byte aligned.  No
- * entry point (but q4_search_plan_create) allocates, frees, or keeps a copy of anything; work is enqueued
+ * entry point allocates, frees, or keeps a copy of anything but a search plan (q4_beam_search); work is enqueued
  * on the stream passed last and the call returns without synchronising (except
- * q4_poll_status).  Every function returns 0 on success or a negative Q4_ERR_*;
+ * q4_poll_status and q4_search_plan_destroy).  Every function returns 0 on success or a negative Q4_ERR_*;
  * argument errors are detected on the host before anything is launched.
  *
  * Number formats
@@ -353,13 +353,16 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
 /*
  * q4_beam_search — all steps of a search on the stream, after q4_beam_init: T + u_max steps of mode 0, or
  * with time_synchronous != 0 the T (S + 1) steps of modes 1 and 2 (S = state->tsd_smax).  Arguments and
- * results as dr_fusion_beam_step; same workspace; no steps (no frames and no label budget) is no error.  `plan` (nullable): an object of q4_search_plan_create, in which
- * the call keeps a number of steps as a CUDA graph.  The graph belongs to the model, state, weights of Eq. 1
- * and workspace it was built for and is rebuilt when one of them changes; frames, T and u_max may change from
- * call to call.  One plan serves one search at a time.  Without a plan, in a stream capture and while launches
- * are timed, the steps are enqueued one by one (same results).
- * q4_search_plan_create / _destroy are the only entry points that allocate: a host object, a stream and the
- * graph.  Destroy a plan before the memory that its last search used is given to anything else.
+ * results as dr_fusion_beam_step; same workspace; no steps (no frames and no label budget) is no error.  `plan`
+ * (nullable): an object of q4_search_plan_create, in which the library keeps a number of steps of up to four searches as
+ * CUDA graphs.  A graph belongs to the model, state, weights of Eq. 1 and workspace it was built for; frames, T and
+ * u_max may change from call to call.  A call that finds no graph of its own builds one (host time of about a
+ * millisecond; memory for the graph) in place of one whose replays have ended, and enqueues its steps one by one if
+ * there is none: it waits for nothing.  One plan serves one search at a time.  Without a plan, in a stream capture and
+ * while launches are timed, the steps are enqueued one by one (same results).
+ * Graphs, and what they are captured on, are the plan's own: the streams lent with the state are used by single
+ * steps only, and a plan may be made, used or destroyed while another thread captures a stream.  A plan uses the memory
+ * of a search only in a search on it.  q4_search_plan_destroy waits for the replays on their way.
  */
 typedef void* q4_search_plan;
 int q4_search_plan_create(q4_search_plan* out);

@@ -1,5 +1,6 @@
 // C ABI of the library (see include/q4rnnt.h): argument checking on the host, argument
-// blocks for the kernels, launch sequencing.  Nothing here allocates or synchronises.
+// blocks for the kernels, launch sequencing.  Nothing here waits for the device but q4_poll_status and
+// q4_search_plan_destroy, and nothing allocates but a search plan.
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -1345,7 +1346,7 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
 // 5 utterances x 8 slots, 360 time-synchronous calls: 12.9 -> 11.9 ms.
 namespace {
 constexpr int PLAN_ITERS = 12;       // even (the pending lists alternate) and a multiple of the 1, 2, 3 or 4 calls per frame
-constexpr int PLAN_MIN_ITERS = 96;   // below, building the graph (1.0 ms of host time, once per state) outweighs it
+constexpr int PLAN_MIN_ITERS = 96;   // below, building the graph (1.0 ms of host time, once per kind of search and state) outweighs it
 struct SearchKey {                   // everything the graph was built from
   q4_model model;
   q4_beam_state state;
@@ -1354,14 +1355,22 @@ struct SearchKey {                   // everything the graph was built from
   int32_t B, W, tsd, dependent, exact;
   float lambda_t, lambda_s, rho;
 };
-struct SearchPlan {
+// One graph and the search it was built for.  PLAN_GRAPHS of them: a decoder that alternates between a few batch sizes,
+// beams or kinds of search, whose states come and go at the same addresses, builds one for each.
+constexpr int PLAN_GRAPHS = 4;
+struct SearchGraph {
   SearchKey key;
   int64_t launches, quant_calls;     // of the graph
-  int64_t built, replays, failed;    // graphs made, replays enqueued, attempts to make a graph that failed
-  cudaStream_t stream, side[2];      // captured on: the graph's chains, none of the caller's streams
-  cudaEvent_t side_event[3];
+  int64_t last_use;
   cudaEvent_t done;                  // of the last replay
   cudaGraphExec_t exec;
+};
+struct SearchPlan {
+  SearchGraph graph[PLAN_GRAPHS];
+  int64_t built, replays, failed;    // graphs made, replays enqueued, attempts to make a graph that failed
+  int64_t uses;
+  cudaStream_t stream, side[2];      // captured on: the graphs' chains, none of the caller's streams
+  cudaEvent_t side_event[3];
 };
 // While one of these lives, calls of this thread that a capture elsewhere in the process would take for unsafe (streams
 // and events made or destroyed, a graph instantiated, an event asked) leave that capture alone: none of them
@@ -1371,12 +1380,6 @@ struct BesideCaptures {
   BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
   ~BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
 };
-void plan_clear(SearchPlan* p) {
-  if (!p->exec) return;
-  cudaEventSynchronize(p->done);
-  cudaGraphExecDestroy(p->exec);
-  p->exec = nullptr;
-}
 int step_mode(const SearchKey& k, int iter) {
   const int S1 = k.state.tsd_smax + 1;
   return !k.tsd ? 0 : iter % S1 == S1 - 1 ? 2 : 1;
@@ -1389,8 +1392,9 @@ int q4_search_plan_create(q4_search_plan* out) {
   SearchPlan* p = static_cast<SearchPlan*>(calloc(1, sizeof(SearchPlan)));
   if (!p) return Q4_ERR_CUDA;
   *out = p;
-  bool ok = cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking) == cudaSuccess &&
-            cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming) == cudaSuccess;
+  bool ok = cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking) == cudaSuccess;
+  for (int i = 0; i < PLAN_GRAPHS && ok; ++i)
+    ok = cudaEventCreateWithFlags(&p->graph[i].done, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; i < 2 && ok; ++i) ok = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking) == cudaSuccess;
   for (int i = 0; i < 3 && ok; ++i) ok = cudaEventCreateWithFlags(&p->side_event[i], cudaEventDisableTiming) == cudaSuccess;
   if (ok) return Q4_OK;
@@ -1402,8 +1406,13 @@ int q4_search_plan_destroy(q4_search_plan plan) {
   if (!plan) return Q4_OK;
   const BesideCaptures guard;
   SearchPlan* p = static_cast<SearchPlan*>(plan);
-  plan_clear(p);
-  if (p->done) cudaEventDestroy(p->done);
+  for (SearchGraph& g : p->graph) {
+    if (g.exec) {
+      cudaEventSynchronize(g.done);   // a replay of a search may be on its way
+      cudaGraphExecDestroy(g.exec);
+    }
+    if (g.done) cudaEventDestroy(g.done);
+  }
   if (p->stream) cudaStreamDestroy(p->stream);
   for (int i = 0; i < 2; ++i)
     if (p->side[i]) cudaStreamDestroy(p->side[i]);
@@ -1413,35 +1422,51 @@ int q4_search_plan_destroy(q4_search_plan plan) {
   return Q4_OK;
 }
 
-// The graph of the present arguments, rebuilt when any of them has changed.
-static int plan_build(SearchPlan* p, const SearchKey& key) {
-  if (p->exec && memcmp(&p->key, &key, sizeof(key)) == 0) return Q4_OK;
+// The graph of a search: the one that was built for the same arguments, else a new one in a free place or in
+// place of the one used longest ago whose last replay has ended.  Null (the search then enqueues its steps one by one)
+// if there is no such place, for the host does not wait for a replay here, or if the graph cannot be built.
+static SearchGraph* plan_graph(SearchPlan* p, const SearchKey& key) {
+  SearchGraph* place = nullptr;
+  for (SearchGraph& g : p->graph)
+    if (g.exec && memcmp(&g.key, &key, sizeof(key)) == 0) {
+      g.last_use = ++p->uses;
+      return &g;
+    }
   const BesideCaptures guard;
-  plan_clear(p);
-  p->key = key;
+  for (SearchGraph& g : p->graph)
+    if ((!g.exec || cudaEventQuery(g.done) == cudaSuccess) && (!place || g.last_use < place->last_use)) place = &g;
+  if (cudaPeekAtLastError() == cudaErrorNotReady) cudaGetLastError();   // an event that is not ready is no error
+  if (!place) return nullptr;
+  if (place->exec) cudaGraphExecDestroy(place->exec);
+  place->exec = nullptr;
+  place->last_use = 0;
+  memcpy(&place->key, &key, sizeof(key));   // padding included: keys are compared as bytes
   SearchCall* call = static_cast<SearchCall*>(key.workspace);
   const int64_t l0 = g_launches, q0 = g_quant_calls;
-  if (cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
-    ++p->failed;
-    return Q4_ERR_CUDA;
+  int r = cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeRelaxed) == cudaSuccess ? Q4_OK : Q4_ERR_CUDA;
+  if (r == Q4_OK) {
+    // T and u_max (and the frames) only have to pass the argument checks here; the first frame's steps are never in the graph
+    for (int it = PLAN_ITERS; it < 2 * PLAN_ITERS && r == Q4_OK; ++it)
+      r = beam_step(&key.model, &place->key.state, static_cast<const float*>(key.workspace), key.B, 1 << 24, key.W, it, 0,
+                    key.lambda_t, key.lambda_s, key.rho, step_mode(key, it), key.workspace, key.workspace_bytes, p->stream, call);
+    if (r == Q4_OK && launch_search_advance(call, PLAN_ITERS, p->stream) != cudaSuccess) r = Q4_ERR_CUDA;
+    cudaGraph_t g = nullptr;
+    if (cudaStreamEndCapture(p->stream, &g) != cudaSuccess && r == Q4_OK) r = Q4_ERR_CUDA;
+    if (r == Q4_OK && cudaGraphInstantiate(&place->exec, g, 0) != cudaSuccess) r = Q4_ERR_CUDA;
+    if (g) cudaGraphDestroy(g);
   }
-  int r = Q4_OK;
-  // T and u_max (and the frames) only have to pass the argument checks here; the first frame's steps are never in the graph
-  for (int it = PLAN_ITERS; it < 2 * PLAN_ITERS && r == Q4_OK; ++it)
-    r = beam_step(&key.model, &p->key.state, static_cast<const float*>(key.workspace), key.B, 1 << 24, key.W, it, 0,
-                  key.lambda_t, key.lambda_s, key.rho, step_mode(key, it), key.workspace, key.workspace_bytes, p->stream, call);
-  if (r == Q4_OK && launch_search_advance(call, PLAN_ITERS, p->stream) != cudaSuccess) r = Q4_ERR_CUDA;
-  cudaGraph_t g = nullptr;
-  if (cudaStreamEndCapture(p->stream, &g) != cudaSuccess && r == Q4_OK) r = Q4_ERR_CUDA;
-  if (r == Q4_OK && cudaGraphInstantiate(&p->exec, g, 0) != cudaSuccess) r = Q4_ERR_CUDA;
-  if (r != Q4_OK) p->exec = nullptr;
-  if (g) cudaGraphDestroy(g);
-  p->launches = g_launches - l0;
-  p->quant_calls = g_quant_calls - q0;
+  place->launches = g_launches - l0;
+  place->quant_calls = g_quant_calls - q0;
   g_launches = l0;
   g_quant_calls = q0;
   ++(r == Q4_OK ? p->built : p->failed);
-  return r;
+  if (r != Q4_OK) {
+    place->exec = nullptr;
+    cudaGetLastError();
+    return nullptr;
+  }
+  place->last_use = ++p->uses;
+  return place;
 }
 
 int q4_search_plan_info(q4_search_plan plan, int64_t* out) {
@@ -1492,22 +1517,25 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
   for (int it = 0; it < n_iters;) {
     // the first two frames' steps always: the first step's networks start from the reset state, and the kernels set their
     // attributes at their first launch
-    if (p && it >= 2 * S1 && it + PLAN_ITERS <= n_iters) {
-      if (it == 2 * S1) {
-        if (plan_build(p, key) != Q4_OK) {
-          cudaGetLastError();
-          p = nullptr;
-          continue;
-        }
+    if (p && it == 2 * S1) {
+      SearchGraph* g = plan_graph(p, key);
+      const int first = it;
+      if (g) {
         Q4_TRY(launch_search_begin(static_cast<SearchCall*>(workspace), e, T, u_max, it - PLAN_ITERS, s));
+        for (; it + PLAN_ITERS <= n_iters; it += PLAN_ITERS) {
+          const cudaError_t le = cudaGraphLaunch(g->exec, s);
+          if (le != cudaSuccess) {
+            cudaEventRecord(g->done, s);   // of the replays before it
+            return Q4_ERR_CUDA;
+          }
+          g_launches += g->launches;
+          g_quant_calls += g->quant_calls;
+          ++p->replays;
+        }
+        Q4_TRY(cudaEventRecord(g->done, s));
       }
-      Q4_TRY(cudaGraphLaunch(p->exec, s));
-      g_launches += p->launches;
-      g_quant_calls += p->quant_calls;
-      ++p->replays;
-      it += PLAN_ITERS;
-      if (it + PLAN_ITERS > n_iters) Q4_TRY(cudaEventRecord(p->done, s));
-      continue;
+      p = nullptr;                         // the rest step by step
+      if (it != first) continue;
     }
     Q4_CHECK(beam_step(model, state, e, B, T, W, it, u_max, lambda_t, lambda_s, rho, step_mode(key, it), workspace,
                        workspace_bytes, stream, nullptr));

@@ -579,6 +579,45 @@ def test_search_plan_captures_no_stream_of_the_caller(Bd):
     assert dd.search_plan_info() == dict(built=1, replays=18, failed=0)
 
 
+def test_search_plan_keeps_graphs_of_several_searches(Bd):
+    # searches with other fusion weights, in turn on one state: a graph each, up to four, without waiting for the device;
+    # with more, the one used longest ago gives way once it has run
+    import time
+    dw = synth.decoder(seed=67, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=9, W=6)
+    e = torch.from_numpy(synth.Stream(24).normal("e", (111, 3, 256)).astype(np.float32)).cuda()
+    dd = Bd.Decoder(dw)
+
+    def decode(lam):
+        dw.lambda_t = lam
+        return [t.clone() for t in dd.decode(e)] + [dd.tensors["bp_score"].clone()]
+
+    lams = (0.5, 0.4, 0.3, 0.2, 0.1)
+    want = {}
+    for lam in lams:
+        want[lam] = decode(lam)
+        torch.cuda.synchronize()
+    assert dd.search_plan_info() == dict(built=5, replays=45, failed=0)
+    for _ in range(2):
+        for lam in lams[1:]:                     # 0.5 has given way
+            for x, y in zip(decode(lam), want[lam]):
+                assert torch.equal(x, y)
+    assert dd.search_plan_info() == dict(built=5, replays=45 + 72, failed=0)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(1_000_000_000)             # about half a second
+    start = time.perf_counter()
+    got = [decode(lam) for lam in (0.1, 0.2, 0.3, 0.4, 0.5)]
+    enqueued = time.perf_counter() - start
+    torch.cuda.synchronize()
+    assert enqueued < 0.5 * (time.perf_counter() - start)
+    for g, lam in zip(got, (0.1, 0.2, 0.3, 0.4, 0.5)):
+        for x, y in zip(g, want[lam]):
+            assert torch.equal(x, y)
+    assert dd.search_plan_info()["built"] == 5   # every place was in use: the last search went step by step
+    torch.cuda.synchronize()
+    decode(0.5)
+    assert dd.search_plan_info()["built"] == 6
+
+
 def test_search_beside_a_capture_of_another_thread(Bd):
     # a search that creates its plan and builds its graph on one thread leaves a capture that another thread has open
     # (in the strictest mode, torch's default) as it is
