@@ -358,8 +358,8 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
  * CUDA graphs.  A graph belongs to the model, state, weights of Eq. 1 and workspace it was built for; frames, T and
  * u_max may change from call to call.  A call that finds no graph of its own builds one (host time of about a
  * millisecond; memory for the graph) in place of one whose replays have ended, and enqueues its steps one by one if
- * there is none: it waits for nothing.  One plan serves one search at a time.  Without a plan, in a stream capture and
- * while launches are timed, the steps are enqueued one by one (same results).
+ * there is none: it waits for nothing.  One plan serves one search at a time.  Without a plan, in a stream capture,
+ * while launches are timed and under q4_test_wait_expiry_set, the steps are enqueued one by one (same results).
  * Graphs, and what they are captured on, are the plan's own: the streams lent with the state are used by single
  * steps only, and a plan may be made, used or destroyed while another thread captures a stream.  A plan uses the memory
  * of a search only in a search on it.  q4_search_plan_destroy waits for the replays on their way.

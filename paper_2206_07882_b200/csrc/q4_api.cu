@@ -1509,9 +1509,10 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
   const bool lent = st.aux_stream[0] && st.aux_stream[1] && st.aux_event[0] && st.aux_event[1] && st.aux_event[2];
   for (int i = 0; i < 2; ++i) key.state.aux_stream[i] = p && lent ? p->side[i] : nullptr;
   for (int i = 0; i < 3; ++i) key.state.aux_event[i] = p && lent ? p->side_event[i] : nullptr;
-  // step by step: in a stream that is being captured, while launches are timed, and in a short search
+  // step by step: in a stream that is being captured, while launches are timed or waits are made to run out (a graph
+  // would keep that), and in a short search
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (p && (n_iters < PLAN_MIN_ITERS || timing_active() || cudaStreamIsCapturing(s, &cap) != cudaSuccess ||
+  if (p && (n_iters < PLAN_MIN_ITERS || timing_active() || test_wait_expiry_active() || cudaStreamIsCapturing(s, &cap) != cudaSuccess ||
             cap != cudaStreamCaptureStatusNone))
     p = nullptr;
   for (int it = 0; it < n_iters;) {

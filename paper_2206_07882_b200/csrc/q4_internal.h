@@ -144,6 +144,7 @@ cudaError_t launch_mma_gemm(const int8_t* x8, long long x_pitch, int M, const in
                             const int32_t* n_active, cudaStream_t s, bool dependent = false,
                             const float* mul_e = nullptr, const int32_t* mul_idx = nullptr);
 void test_wait_expiry_set(int skip_producer, uint32_t wait_limit);
+bool test_wait_expiry_active();
 cudaError_t launch_mma_gemm_i32(const int8_t* x8, int M, const int8_t* w8, int J, int K, int planes, int32_t* out,
                                 int32_t* status, cudaStream_t s, bool dependent = false);
 // One launch for what a layer call prepares (k_layer_prepare).

@@ -308,6 +308,7 @@ void test_wait_expiry_set(int skip_producer, uint32_t wait_limit) {
   g_skip_producer = skip_producer;
   g_wait_limit = wait_limit ? wait_limit : (1u << 22);
 }
+bool test_wait_expiry_active() { return g_skip_producer != 0 || g_wait_limit != (1u << 22); }
 
 template <int GEMM_BN>
 __global__ void __launch_bounds__(192, 1)

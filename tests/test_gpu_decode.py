@@ -618,6 +618,25 @@ def test_search_plan_keeps_graphs_of_several_searches(Bd):
     assert dd.search_plan_info()["built"] == 6
 
 
+def test_search_plan_keeps_no_test_hook(Bd):
+    # a search while waits of the tiled GEMM are made to run out reports it, and leaves nothing of it in a graph
+    import ctypes as C
+    dw = synth.decoder(seed=67, V=300, E=32, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=9, W=6)
+    e = torch.from_numpy(synth.Stream(25).normal("e", (111, 3, 256)).astype(np.float32)).cuda()
+    want = [t.clone() for t in Bd.Decoder(dw).decode(e)]
+    dd = Bd.Decoder(dw)
+    assert Bd.lib().q4_test_wait_expiry_set(C.c_int32(1), C.c_uint32(1 << 12)) == 0
+    try:
+        dd.decode(e)
+        assert dd.tensors["status"].item() == -8                      # Q4_ERR_TIMEOUT
+    finally:
+        Bd.lib().q4_test_wait_expiry_set(C.c_int32(0), C.c_uint32(0))
+    assert dd.search_plan_info()["replays"] == 0
+    for x, y in zip(dd.decode(e), want):
+        assert torch.equal(x, y)
+    assert dd.tensors["status"].item() == 0
+
+
 def test_search_beside_a_capture_of_another_thread(Bd):
     # a search that creates its plan and builds its graph on one thread leaves a capture that another thread has open
     # (in the strictest mode, torch's default) as it is
