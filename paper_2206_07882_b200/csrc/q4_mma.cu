@@ -852,6 +852,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
   const uint32_t tmem = tmem_base_s;
   cl_barrier();   // every CTA of the cluster is running before anyone stores into a peer's shared memory
   pdl_wait();   // everything above (this barrier included) overlaps the tail of the previous kernel of the stream
+  bool codes_due = false;   // a wait has run out: the peers' codes may still be on their way here
 
   if (warp == HEAD_EPI_WARPS) {
     // ---- TMA producer: bottleneck operands through the ring, then my block of output-layer weights into
@@ -907,6 +908,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
     if (elect_one()) umma_commit(&acc1_full);
     if (ok) ok = mbar_wait_warp(&w_full, 0);
     if (ok && nk1 > 0) ok = mbar_wait_warp(&ops_ready, 0);
+    codes_due = !ok && nk1 > 0;
     tc_fence_after();
     if (elect_one()) {
 #pragma unroll
@@ -1128,12 +1130,13 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
     pdl_trigger();
     cl_barrier();
     if (NB == 32) cl_barrier();
+    if (codes_due) mbar_wait_warp(&ops_ready, 0);   // all have been sent by now: nobody leaves while they arrive (bounded)
   }
   tc_fence_before();
   __syncthreads();
   if (warp == HEAD_EPI_WARPS + 1) tmem_dealloc(tmem, TCOLS);
-  // no barrier at the exit: every store and copy into a peer's shared memory precedes the exchange barrier above
-  // (release on arrival, acquire on the wait), after which only local memory is touched
+  // no barrier at the exit: every store and copy into a peer's shared memory is issued before the exchange barrier
+  // above; stores have arrived with it (release on arrival, acquire on the wait), copies once ops_ready has been waited for
 }
 
 template <int NB>
