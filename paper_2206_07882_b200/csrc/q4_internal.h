@@ -238,7 +238,7 @@ struct EncRecPlan {
                             // groups_per_cluster groups per cluster, 2: kernel whose clusters may take turns,
                             // 3: few groups, int8 fragments in registers, clusters of up to 16 CTAs
   int32_t groups_per_cluster;
-  int32_t ctas;             // CTAs per cluster; 10: kernels 1 and 2 run as kernel 3
+  int32_t ctas;             // CTAs per cluster
   int32_t ncl[2], sliced[2], groups, max_clusters;
   int32_t win[9];
 };

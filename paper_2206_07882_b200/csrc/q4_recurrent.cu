@@ -1340,6 +1340,7 @@ EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid
   const bool few_h = H == 64 || H == 128 || H == 256 || H == 320 || H == 512 || H == 640;
   if (few_h && hid_signed && !dump && (hid_bits == 4 || hid_bits == 8) && dirs * groups <= (H <= 256 ? 15 : 7)) {
     p.kernel = 3;
+    p.ctas = H / 32 <= 8 ? H / 32 : H == 320 ? 8 : 16;
     p.groups_per_cluster = 1;
     p.ncl[0] = groups;
     p.ncl[1] = dirs == 2 ? groups : 0;
@@ -1354,10 +1355,19 @@ EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid
     // weights, 8-bit hidden codes, an input scale per sequence.
     const int lack = dirs * groups - p.max_clusters;
     const bool plain_only = w_bits == 8 || hid_bits == 8 || per_sequence_scale;
+    // few enough groups for clusters of 10 CTAs of the kernel above (of what needs int8 fragments up to 8 a direction)
+    if (dirs * groups <= 11 && (!plain_only || groups <= 8)) {
+      p.kernel = 3;
+      p.ctas = 10;
+      p.groups_per_cluster = 1;
+      p.ncl[0] = groups;
+      p.ncl[1] = dirs == 2 ? groups : 0;
+      return p;
+    }
     const bool turns = g_rec_sliced && lack >= 1 && lack <= dirs && groups >= 2 && groups <= 8 && T >= 8 * groups && scratch;
     if (turns || (lack <= 0 && plain_only && groups <= 8)) {   // the hand-over scratch is needed for turns only
       p.kernel = 2;
-      p.ctas = !turns && dirs * groups <= 11 ? 10 : REC_CLUSTER;
+      p.ctas = REC_CLUSTER;
       p.groups_per_cluster = 1;
       for (int d = 0; d < 2; ++d) {
         p.sliced[d] = turns && d < dirs && d < lack ? 1 : 0;
@@ -1374,7 +1384,7 @@ EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid
     while (nu <= 4 && dirs * ((groups + nu - 1) / nu) > p.max_clusters) ++nu;
     if (nu <= 4) {
       p.kernel = 1;
-      p.ctas = nu == 1 && dirs * groups <= 11 ? 10 : REC_CLUSTER;
+      p.ctas = REC_CLUSTER;
       p.groups_per_cluster = nu;
       p.ncl[0] = (groups + nu - 1) / nu;
       p.ncl[1] = dirs == 2 ? p.ncl[0] : 0;
@@ -1389,7 +1399,7 @@ cudaError_t launch_enc_recurrent(EncRecArgs a, cudaStream_t s) {
   const EncRecPlan p = enc_recurrent_plan(a.T, a.B, a.dirs, a.H, a.w_bits, a.hid_act.bits, a.hid_act.is_signed != 0,
                                           a.x_scale_b != nullptr, a.d[0].dbg_ih != nullptr,
                                           a.flags && a.hand_h[0] && a.hand_c[0]);
-  if (p.kernel == 3 || p.ctas == 10) {
+  if (p.kernel == 3) {
     a.n_groups = p.groups;
     timing_begin(s);
     cudaError_t e = cudaErrorInvalidValue;

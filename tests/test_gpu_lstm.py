@@ -165,9 +165,11 @@ def test_layer_few_groups(Bd, T, B, K, H, dirs, xb, hb, ob):
     layer_case(Bd, T, B, K, H, dirs, xb, hb, ob, seed=29)
 
 
-@pytest.mark.parametrize("T,B,dirs,xb,hb,ob", [(7, 30, 2, 4, 4, 4), (6, 88, 1, 8, 8, 4), (6, 81, 1, 4, 4, 8)])
+@pytest.mark.parametrize("T,B,dirs,xb,hb,ob", [(7, 30, 2, 4, 4, 4), (6, 88, 1, 8, 8, 4), (6, 81, 1, 4, 4, 8), (6, 62, 1, 8, 8, 4)])
 def test_layer_clusters_of_ten(Bd, T, B, dirs, xb, hb, ob):
-    # 8 to 11 groups of 640 cells: clusters of 10 CTAs
+    # 8 to 11 groups of 640 cells: clusters of 10 CTAs; of 8-bit layers up to 8 groups a direction (11 of them take the
+    # general kernel)
+    assert Bd.encoder_recurrence_plan(T, B, dirs, 640, w_bits=hb, hid_bits=hb)["kernel"] == (0 if hb == 8 and B > 64 else 3)
     layer_case(Bd, T, B, 32, 640, dirs, xb, hb, ob, seed=31)
 
 

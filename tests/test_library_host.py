@@ -117,9 +117,14 @@ def test_encoder_recurrence_plan_lays_groups_on_clusters():
     # host logic of qlstm_layer_forward's recurrence: which kernel, how many clusters, whose turn when
     from paper_2206_07882_b200 import binding as Bd
     plan = Bd.encoder_recurrence_plan
-    p = plan(500, 32, 2, 640)                      # 4 groups x 2 directions: one group per cluster
+    # one group per cluster: up to 7 groups in all clusters of 16 CTAs, up to 11 clusters of 10, then clusters of 8 of
+    # the kernel with packed weights
+    for B, dirs, kernel in ((1, 1, 3), (24, 2, 3), (56, 1, 3), (32, 2, 3), (40, 2, 3), (88, 1, 3), (48, 2, 1), (96, 1, 1)):
+        p = plan(500, B, dirs, 640)
+        n = (B + 7) // 8
+        assert p["kernel"] == kernel and p["groups_per_cluster"] == 1 and p["clusters"] == [n, n if dirs == 2 else 0]
     cap = p["max_clusters"]
-    assert cap >= 8 and p["kernel"] == 1 and p["groups_per_cluster"] == 1 and p["clusters"] == [4, 4]
+    assert cap >= 12
     for T, B in ((500, 64), (64, 57), (152, 60)):   # 8 groups x 2 directions
         p = plan(T, B, 2, 640)
         lack = 16 - cap
@@ -136,8 +141,14 @@ def test_encoder_recurrence_plan_lays_groups_on_clusters():
     assert p["kernel"] == 1 and sum(p["clusters"]) <= cap and p["groups_per_cluster"] * p["clusters"][0] >= 16
     # 8-bit weights or codes, or an input scale per sequence: the kernel with int8 fragments / per-sequence
     # scales while one group per cluster fits, the general kernel beyond
-    assert plan(500, 32, 2, 640, w_bits=8, hid_bits=8)["kernel"] == 2
-    assert plan(500, 32, 2, 640, per_sequence_scale=True)["kernel"] == 2
+    assert plan(500, 32, 2, 640, w_bits=8, hid_bits=8)["kernel"] == 3
+    assert plan(500, 32, 2, 640, per_sequence_scale=True)["kernel"] == 3
+    assert plan(500, 48, 2, 640, w_bits=8, hid_bits=8)["kernel"] == 2
+    assert plan(500, 48, 2, 640, per_sequence_scale=True)["kernel"] == 2
+    assert plan(500, 88, 1, 640, w_bits=8, hid_bits=8)["kernel"] == 0
+    # the widths and numbers of clusters of the kernel for few groups
+    for H, most in ((64, 15), (128, 15), (256, 15), (320, 7), (512, 7)):
+        assert plan(9, 8 * most, 1, H)["kernel"] == 3 and plan(9, 8 * most + 1, 1, H)["kernel"] == 0
     assert plan(500, 64, 2, 640, w_bits=8, hid_bits=8)["kernel"] == (2 if 1 <= 16 - cap <= 2 else 0)
     assert plan(500, 128, 2, 640, w_bits=8, hid_bits=8)["kernel"] == 0
     assert plan(500, 32, 2, 320)["kernel"] == 0     # other widths: general kernel
