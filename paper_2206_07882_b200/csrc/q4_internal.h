@@ -63,6 +63,7 @@ int timing_count();
 bool timing_active();
 
 // ---- tensor-core path (q4_mma.cu)
+int sm_count();   // SMs of the device (asked once; 148 without one)
 struct MmaLstmArgs {
   int32_t N, H, Kx_pad;
   const int32_t* acc_pre;   // optional precomputed input accumulators [row, 4H] in 4*cell+gate order

@@ -782,7 +782,7 @@ static cudaError_t quantize_t(const void* x, long long rows, int k, int k_pad, c
     e = cudaMemsetAsync(group_scale_out, 0, sizeof(float) * n_groups, s);
     if (e != cudaSuccess) return e;
     const long long splits = (in_group + 7) / 8;
-    const unsigned want = (unsigned)(4 * 148 / n_groups + 1);   // about four CTAs per SM over all groups
+    const unsigned want = (unsigned)(4 * sm_count() / n_groups + 1);   // about four CTAs per SM over all groups
     const dim3 grid((unsigned)n_groups, splits < want ? (unsigned)splits : want);
     k_absmax<FP16, VEC><<<grid, 256, 0, s>>>(x, rows, k, n_groups, (uint32_t*)group_scale_out);
     k_amax_to_scale<<<(n_groups + 255) / 256, 256, 0, s>>>((uint32_t*)group_scale_out, n_groups,

@@ -85,7 +85,7 @@ cudaError_t launch_unpack_multi(const UnpackJobs& jobs, cudaStream_t s, bool dep
   const long long total = (long long)jobs.n_rows_pad * (kmax >> 5);
   if (total > INT32_MAX) return cudaErrorInvalidValue;
   long long blocks = (total + 255) / 256;
-  const long long cap = (6 * 148 + jobs.n_jobs - 1) / jobs.n_jobs;   // about six CTAs per SM in all: one or two
+  const long long cap = (6 * sm_count() + jobs.n_jobs - 1) / jobs.n_jobs;   // about six CTAs per SM in all: one or two
                                                                      // pieces per thread at 1024 rows
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
@@ -640,7 +640,7 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
   if (warp == 5) tmem_dealloc(tmem, TCOLS);
 }
 
-static int g_sm_count() {
+int sm_count() {
   static int n = 0;
   if (n == 0) {
     int dev = 0;
@@ -679,7 +679,7 @@ static cudaError_t gemm_persistent_launch(const CUtensorMap& ta, const CUtensorM
   }
   const int tiles_m = (a.M + BM - 1) / BM, tiles_n = (a.J + BN - 1) / BN;
   const long long tiles = (long long)tiles_m * tiles_n * planes;
-  const int ctas = tiles < g_sm_count() ? (int)tiles : g_sm_count();
+  const int ctas = tiles < sm_count() ? (int)tiles : sm_count();
   return launch_ex(k_mma_gemm_persistent<BN>, dim3(ctas), dim3(192), gemm_smem<BN>(), s, dependent, 1, ta, tb, a, tiles_m,
                    tiles_n, planes, plane_out);
 }
@@ -691,7 +691,7 @@ static cudaError_t gemm_persistent_launch(const CUtensorMap& ta, const CUtensorM
 // direction and 9.5 us as 160 of width 64 in one launch (1903 rows: 2 x 28.9 -> 20.6 us, width 256 in both).
 static int gemm_tile_width(int M, int J, int planes, int narrowest) {
   for (int bn = 256; bn > narrowest; bn >>= 1)
-    if ((long long)((M + BM - 1) / BM) * ((J + bn - 1) / bn) * planes >= g_sm_count()) return bn;
+    if ((long long)((M + BM - 1) / BM) * ((J + bn - 1) / bn) * planes >= sm_count()) return bn;
   return narrowest;
 }
 
@@ -1514,7 +1514,7 @@ static cudaError_t lstm_launch(const MmaLstmArgs& a, const CUtensorMap& txa, con
 // 2.25 ms; with 32-wide tiles, and with 64 at two tiles per SM, the target LM's layers waited for the tiles of the
 // other networks instead (search of 16 utterances, label iteration 65 -> 70 us).
 static int lstm_tile_width(int row_tiles, int H) {
-  return row_tiles * ((4 * H + 63) / 64) <= 148 ? 64 : 128;
+  return row_tiles * ((4 * H + 63) / 64) <= sm_count() ? 64 : 128;
 }
 
 // Operands: xa int8 [rows_pad, Kx_pad] (ignored with acc_pre), xw int8 [4H, Kx_pad] interleaved,

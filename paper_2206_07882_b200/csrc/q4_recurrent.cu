@@ -1171,42 +1171,64 @@ size_t enc_recurrent_smem(int H, int BG) {
          (size_t)BG * (H / REC_CLUSTER) + 16;
 }
 
+bool enc_recurrent_supported(int H, int B, int dirs) {
+  (void)B;
+  (void)dirs;
+  if (H % 32 != 0 || H / REC_CLUSTER > 80) return false;
+  return enc_recurrent_smem(H, 8) <= REC_SMEM_MAX;
+}
+
 template <int BG>
 static cudaError_t rec_launch(const EncRecArgs& a, size_t smem, cudaStream_t s) {
-  static size_t configured = 0;
-  if (smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_enc_recurrent<BG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e = cudaFuncSetAttribute(k_enc_recurrent<BG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)REC_SMEM_MAX);
     if (e != cudaSuccess) return e;
-    configured = smem;
+    configured = true;
   }
   const cudaError_t e = launch_ex(k_enc_recurrent<BG>, dim3((unsigned)(a.dirs * a.n_groups * REC_CLUSTER)), dim3(REC_THREADS),
                                   smem, s, true, 1, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// How many 8-CTA clusters of this kernel can be resident at once on the current device
-// (15 on a 148-SM B200: clusters do not straddle GPCs); asked once.
-static int rec_max_clusters(int H) {
-  static int cached = 0;
-  if (cached > 0) return cached;
-  const size_t smem = enc_recurrent_smem(H, 8);
-  int n = 0;
-  if (cudaFuncSetAttribute(k_enc_recurrent<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(REC_CLUSTER * 16);
-    cfg.blockDim = dim3(REC_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = REC_CLUSTER;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, k_enc_recurrent<8>, &cfg) != cudaSuccess) n = 0;
+// How many clusters of `ctas` CTAs of a kernel can be resident at once on the current device; 0 if it cannot place
+// one, -1 if there is no answer (no device).
+static int resident_clusters(const void* kern, int ctas, int threads, size_t smem, size_t smem_max) {
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max) != cudaSuccess ||
+      (ctas > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+    cudaGetLastError();
+    return -1;
   }
-  cached = n > 0 ? n : 15;
-  return cached;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctas * 16);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+// The general kernel's clusters (15 of 640 cells on a 148-SM B200: clusters do not straddle GPCs); asked once a width.
+static int rec_max_clusters(int H) {
+  if (!enc_recurrent_supported(H, 0, 0)) return 15;   // no layer of this kernel
+  static int cached[8 * 80 / 32 + 1];
+  int& n = cached[H / 32];
+  if (n == 0) {
+    const int r = resident_clusters(reinterpret_cast<const void*>(&k_enc_recurrent<8>), REC_CLUSTER, REC_THREADS,
+                                    enc_recurrent_smem(H, 8), REC_SMEM_MAX);
+    n = r > 0 ? r : 15;
+  }
+  return n;
 }
 
 // The same question for the kernel whose clusters may take turns (its int8 variant, the one with the
@@ -1220,22 +1242,8 @@ static int rec_turns_max_clusters() {
   const size_t smem = (size_t)2 * 2 * REC_BG * H + (size_t)2 * REC_THREADS * sizeof(int4) + (size_t)3 * cpc * sizeof(float4) +
                       (size_t)4 * 2 * REC_BG * cpc + (size_t)2 * 2 * sizeof(uint64_t) + 32 +
                       (size_t)rec_turns_ksmem(true) * REC_THREADS * sizeof(uint4);
-  int n = 0;
-  if (cudaFuncSetAttribute(k_enc_recurrent_w4s<20, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(REC_CLUSTER * 16);
-    cfg.blockDim = dim3(REC4_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = REC_CLUSTER;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&n, k_enc_recurrent_w4s<20, true>, &cfg) != cudaSuccess) n = 0;
-  }
-  cached = n > 0 ? n : 15;
+  const int r = resident_clusters(reinterpret_cast<const void*>(&k_enc_recurrent_w4s<20, true>), REC_CLUSTER, REC4_THREADS, smem, smem);
+  cached = r > 0 ? r : 15;
   return cached;
 }
 
@@ -1264,13 +1272,6 @@ int enc_recurrent_sliced_set(int enabled) {
   const int prev = g_rec_sliced;
   g_rec_sliced = enabled ? 1 : 0;
   return prev;
-}
-
-bool enc_recurrent_supported(int H, int B, int dirs) {
-  (void)B;
-  (void)dirs;
-  if (H % 32 != 0 || H / REC_CLUSTER > 80) return false;
-  return enc_recurrent_smem(H, 8) <= REC_SMEM_MAX;
 }
 
 static size_t enc_recurrent_w4_smem(int H, int NU) {
@@ -1310,8 +1311,7 @@ static cudaError_t rec_w4_launch(const EncRecArgs& a, cudaStream_t s) {
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// A CTA of the kernel for few groups has an SM to itself.  Resident clusters: 7 of 16 CTAs, 11 of 10, 15 of 8 (a cluster
-// stays within a GPC, whose SMs are not a multiple of these).
+// A CTA of the kernel for few groups has an SM to itself.
 constexpr size_t REC_FEW_SMEM = 120 * 1024;
 
 template <int KS, int CL>
@@ -1328,6 +1328,30 @@ static cudaError_t rec_few_launch(const EncRecArgs& a, cudaStream_t s) {
                                   REC_FEW_SMEM, s, true, 1, a);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
+// How many clusters the kernel for few groups is used with: as many as are resident at once on the device (asked once;
+// none where a GPC cannot hold a cluster of that many CTAs: the other kernels take the layer then), at most `most`, the
+// number up to which it was measured to be the fastest.
+template <int KS, int CL, int most>
+static int rec_few_clusters() {
+  static int cached = -1;
+  if (cached < 0) {
+    const int r = resident_clusters(reinterpret_cast<const void*>(&k_enc_recurrent_few<KS, CL>), CL, 8 * 32 * KS / CL, REC_FEW_SMEM, REC_FEW_SMEM);
+    cached = r < 0 || r > most ? most : r;
+  }
+  return cached;
+}
+static int rec_few_clusters(int H, int ctas) {
+  switch (ctas == 10 ? 0 : H) {
+    case 0: return rec_few_clusters<20, 10, 11>();
+    case 64: return rec_few_clusters<2, 2, 15>();
+    case 128: return rec_few_clusters<4, 4, 15>();
+    case 256: return rec_few_clusters<8, 8, 15>();
+    case 320: return rec_few_clusters<10, 8, 7>();
+    case 512: return rec_few_clusters<16, 16, 7>();
+    case 640: return rec_few_clusters<20, 16, 7>();
+  }
+  return 0;   // widths the kernel is not built for
+}
 
 EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid_bits, bool hid_signed,
                               bool per_sequence_scale, bool dump, bool scratch) {
@@ -1337,8 +1361,7 @@ EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid
   p.groups = groups;
   p.max_clusters = rec_max_clusters(H);
   if (H == 640) p.max_clusters = p.max_clusters < rec_turns_max_clusters() ? p.max_clusters : rec_turns_max_clusters();
-  const bool few_h = H == 64 || H == 128 || H == 256 || H == 320 || H == 512 || H == 640;
-  if (few_h && hid_signed && !dump && (hid_bits == 4 || hid_bits == 8) && dirs * groups <= (H <= 256 ? 15 : 7)) {
+  if (hid_signed && !dump && (hid_bits == 4 || hid_bits == 8) && dirs * groups <= rec_few_clusters(H, 0)) {
     p.kernel = 3;
     p.ctas = H / 32 <= 8 ? H / 32 : H == 320 ? 8 : 16;
     p.groups_per_cluster = 1;
@@ -1356,7 +1379,7 @@ EncRecPlan enc_recurrent_plan(int T, int B, int dirs, int H, int w_bits, int hid
     const int lack = dirs * groups - p.max_clusters;
     const bool plain_only = w_bits == 8 || hid_bits == 8 || per_sequence_scale;
     // few enough groups for clusters of 10 CTAs of the kernel above (of what needs int8 fragments up to 8 a direction)
-    if (dirs * groups <= 11 && (!plain_only || groups <= 8)) {
+    if (dirs * groups <= rec_few_clusters(H, 10) && (!plain_only || groups <= 8)) {
       p.kernel = 3;
       p.ctas = 10;
       p.groups_per_cluster = 1;

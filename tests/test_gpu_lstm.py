@@ -173,6 +173,15 @@ def test_layer_clusters_of_ten(Bd, T, B, dirs, xb, hb, ob):
     layer_case(Bd, T, B, 32, 640, dirs, xb, hb, ob, seed=31)
 
 
+def test_recurrence_plan_on_this_device(Bd):
+    # the capacities asked of the device give a B200 the plan that the host assumes for one, whichever width comes first
+    plan = Bd.encoder_recurrence_plan
+    for H, most in ((320, 7), (128, 15), (64, 15), (640, 7), (512, 7), (256, 15)):
+        assert plan(9, 8 * most, 1, H)["kernel"] == 3 and (H == 640 or plan(9, 8 * most + 1, 1, H)["kernel"] == 0)
+    assert plan(9, 88, 1, 640)["kernel"] == 3 and plan(9, 89, 1, 640)["kernel"] == 1
+    assert plan(9, 89, 1, 640)["max_clusters"] == 15 <= plan(9, 500, 1, 96)["max_clusters"]
+
+
 def test_layer_clusters_taking_turns_at_a_surplus_group(Bd):
     # 57 sequences x 2 directions of 640 cells = 16 groups of 8 for the 15 clusters that fit: the seven
     # clusters of one direction take turns at its eighth group (9 of 64 steps each, one more on the
