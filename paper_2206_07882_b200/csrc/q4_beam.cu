@@ -534,7 +534,8 @@ static size_t sel_smem(const BeamSelArgs& a) {
 template <int MODE>
 static cudaError_t beam_select_launch(const BeamSelArgs& a, cudaStream_t s, bool dependent) {
   const size_t smem = sel_smem(a);
-  static size_t configured = 0;
+  static size_t configured_on[MAX_DEVICES];
+  size_t& configured = configured_on[device_slot()];
   if (smem > configured) {
     cudaError_t e = cudaFuncSetAttribute(k_beam_select<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -841,7 +842,8 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_tsd_select(const __grid_constant_
 template <int MODE>
 static cudaError_t tsd_select_launch(const BeamSelArgs& a, cudaStream_t s, bool dependent) {
   const size_t smem = sel_smem(a);
-  static size_t configured = 0;
+  static size_t configured_on[MAX_DEVICES];
+  size_t& configured = configured_on[device_slot()];
   if (smem > configured) {
     cudaError_t e = cudaFuncSetAttribute(k_tsd_select<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -62,6 +62,13 @@ constexpr int KC = 128;         // K elements staged per chunk
 constexpr int PITCH = KC + 16;  // shared-memory row pitch in bytes (16 B aligned, conflict-free)
 constexpr int NT = 256;         // threads per CTA of the tile kernels
 
+// A kernel's attributes belong to the device that is current when they are set: they are set at its first launch on each.
+constexpr int MAX_DEVICES = 64;
+inline int device_slot() {
+  int d = 0;
+  return cudaGetDevice(&d) == cudaSuccess && d >= 0 && d < MAX_DEVICES ? d : 0;
+}
+
 extern int64_t g_launches;      // kernels launched by this process
 extern int64_t g_quant_calls;   // activation-quantizer applications enqueued by this process
 

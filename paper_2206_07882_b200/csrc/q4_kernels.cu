@@ -766,7 +766,8 @@ static cudaError_t quantize_t(const void* x, long long rows, int k, int k_pad, c
       return cudaGetLastError();
     }
     if (rows >= n_groups && rows <= INT32_MAX && n_groups <= 65536 && smem <= QM_SMEM_MAX) {
-      static bool configured = false;
+      static bool configured_on[MAX_DEVICES];
+      bool& configured = configured_on[device_slot()];
       if (!configured) {
         e = cudaFuncSetAttribute(k_quantize_max<FP16, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)QM_SMEM_MAX);
         if (e != cudaSuccess) return e;

@@ -658,7 +658,8 @@ static size_t gemm_smem() {
 template <int BN>
 static cudaError_t gemm_launch(const CUtensorMap& ta, const CUtensorMap& tb, const MmaGemmArgs& a, cudaStream_t s,
                                bool dependent) {
-  static bool configured = false;
+  static bool configured_on[MAX_DEVICES];
+  bool& configured = configured_on[device_slot()];
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(k_mma_gemm<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem<BN>());
     if (e != cudaSuccess) return e;
@@ -670,7 +671,8 @@ static cudaError_t gemm_launch(const CUtensorMap& ta, const CUtensorMap& tb, con
 template <int BN>
 static cudaError_t gemm_persistent_launch(const CUtensorMap& ta, const CUtensorMap& tb, const MmaGemmArgs& a, int planes,
                                           long long plane_out, cudaStream_t s, bool dependent) {
-  static bool configured = false;
+  static bool configured_on[MAX_DEVICES];
+  bool& configured = configured_on[device_slot()];
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(k_mma_gemm_persistent<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)gemm_smem<BN>());
@@ -1144,7 +1146,8 @@ static cudaError_t lmhead_launch(const CUtensorMap& th, const CUtensorMap& tb, c
                                  cudaStream_t s, bool dependent) {
   static_assert(2 * NB * BK + BM * HEAD_BN1 <= HEAD_RING, "output-layer weights and outgoing codes share the ring's memory");
   const size_t smem = 2 * BM * BK + (size_t)HEAD_RING + 1024;
-  static bool configured = false;
+  static bool configured_on[MAX_DEVICES];
+  bool& configured = configured_on[device_slot()];
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(k_mma_lmhead<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -1490,7 +1493,8 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
 template <int BN>
 static cudaError_t lstm_launch(const MmaLstmArgs& a, const CUtensorMap& txa, const CUtensorMap& txw, const CUtensorMap& tha,
                                const CUtensorMap& thw, size_t smem, cudaStream_t s, bool dependent) {
-  static bool configured = false;
+  static bool configured_on[MAX_DEVICES];
+  bool& configured = configured_on[device_slot()];
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(k_mma_lstm<true, false, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, LSTM_SMEM_MAX);
     if (e == cudaSuccess)

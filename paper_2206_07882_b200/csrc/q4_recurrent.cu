@@ -1180,7 +1180,8 @@ bool enc_recurrent_supported(int H, int B, int dirs) {
 
 template <int BG>
 static cudaError_t rec_launch(const EncRecArgs& a, size_t smem, cudaStream_t s) {
-  static bool configured = false;
+  static bool configured_on[MAX_DEVICES];
+  bool& configured = configured_on[device_slot()];
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(k_enc_recurrent<BG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)REC_SMEM_MAX);
     if (e != cudaSuccess) return e;
@@ -1286,7 +1287,8 @@ static cudaError_t rec_w4s_launch(const EncRecArgs& a, cudaStream_t s) {
   const size_t smem = (size_t)2 * 2 * REC_BG * H + (size_t)2 * REC_THREADS * sizeof(int4) + (size_t)3 * cpc * sizeof(float4) +
                       (size_t)4 * 2 * REC_BG * cpc + (size_t)2 * 2 * sizeof(uint64_t) + 32 +
                       (size_t)rec_turns_ksmem(W8) * REC_THREADS * (W8 ? sizeof(uint4) : sizeof(uint2));
-  static bool configured = false;
+  static bool configured_on[MAX_DEVICES];
+  bool& configured = configured_on[device_slot()];
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(k_enc_recurrent_w4s<KS, W8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -1300,7 +1302,8 @@ static cudaError_t rec_w4s_launch(const EncRecArgs& a, cudaStream_t s) {
 template <int NU, int KS>
 static cudaError_t rec_w4_launch(const EncRecArgs& a, cudaStream_t s) {
   const size_t smem = enc_recurrent_w4_smem(32 * KS, NU);
-  static bool configured = false;
+  static bool configured_on[MAX_DEVICES];
+  bool& configured = configured_on[device_slot()];
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(k_enc_recurrent_w4<NU, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -1316,7 +1319,8 @@ constexpr size_t REC_FEW_SMEM = 120 * 1024;
 
 template <int KS, int CL>
 static cudaError_t rec_few_launch(const EncRecArgs& a, cudaStream_t s) {
-  static bool configured = false;
+  static bool configured_on[MAX_DEVICES];
+  bool& configured = configured_on[device_slot()];
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(k_enc_recurrent_few<KS, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)REC_FEW_SMEM);
     if (e == cudaSuccess && CL > 8)

@@ -237,7 +237,8 @@ cudaError_t launch_skinny_lstm(const SkinnyLstmArgs& a, cudaStream_t s, bool dep
   if (a.N <= 0) return cudaSuccess;
   const dim3 grid(a.H / 4), block(SK_THREADS);
   auto smem = [](int nt) { return (size_t)(SK_WARPS * 2 * 16 * 8 * nt + SK_WARPS * 16 + 12 * 32 * nt) * sizeof(int); };
-  static bool configured = false;
+  static bool configured_on[MAX_DEVICES];
+  bool& configured = configured_on[device_slot()];
   if (!configured) {
     cudaError_t ce = cudaFuncSetAttribute(k_skinny_lstm<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(4));
     if (ce != cudaSuccess) return ce;

@@ -150,3 +150,18 @@ def test_weight_mode_two_bit_storage(Bd):
     np.testing.assert_array_equal(dm2.scale.cpu().numpy(), amax.astype(np.float32))
     want2 = O.pack2(O.quantize_weights(w, amax.astype(np.float32), 2).astype(np.int16), 256)
     np.testing.assert_array_equal(dm2.q.cpu().numpy(), want2)
+
+
+@pytest.mark.skipif(torch.cuda.device_count() < 2, reason="needs two devices")
+def test_max_boundary_on_each_device_of_a_process(Bd):
+    # kernels that need an attribute set have it on every device that they are launched on
+    base = Bd.q4_act_symmetric(1.0, 8)
+    x = synth.Stream(15).normal("x", (640, 512)).astype(np.float32)      # 40 KB a CTA and more
+    results = []
+    for device in range(2):
+        with torch.cuda.device(device):
+            for groups in (1, 8):
+                codes, scales = Bd.quantize_pack_int4(torch.from_numpy(x).to(f"cuda:{device}"), base, mode=1, n_groups=groups)
+                results.append((groups, codes.cpu(), scales.cpu()))
+    for a, b in zip(results[:2], results[2:]):
+        assert torch.equal(a[1], b[1]) and torch.equal(a[2], b[2])
