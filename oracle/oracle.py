@@ -411,8 +411,9 @@ def encoder_forward(enc, features: np.ndarray, n_threads: int = 8, want_layers: 
     for l, dirs in enumerate(enc.layers):
         lw = dirs[0]
         hid_act = act_symmetric(lw.hid_alpha, lw.hid_bits)
-        nxt_bits = enc.layers[l + 1][0].w_ih.bits if l + 1 < len(enc.layers) else (
-            enc.proj.w.bits if enc.proj is not None else lw.hid_bits)
+        # codes as wide as the next layer's weights; 2-bit weights take 4-bit codes (Table 1)
+        nxt_bits = max(4, enc.layers[l + 1][0].w_ih.bits) if l + 1 < len(enc.layers) else (
+            max(4, enc.proj.w.bits) if enc.proj is not None else lw.hid_bits)
         out_act = act_symmetric(lw.hid_alpha, nxt_bits)
         L = Lstm(dirs)
         r = lstm_layer(L, xq, x_act, hid_act, out_act, x_scale_b=x_scale_b,

@@ -387,6 +387,20 @@ def test_layer_two_bit_weights(Bd):
         np.testing.assert_array_equal(got["c_n"].cpu().numpy(), ref["c_n"])
 
 
+@pytest.mark.parametrize("first,proj", [(4, 4), (8, 8), (4, 2)])
+def test_encoder_two_bit_weights(Bd, first, proj):
+    # 2-bit encoder weights (the first layer's and the projection's at their own widths): codes between the layers
+    # stay at 4 bits, or 8 where the next weights are 8 bits wide
+    w = synth.encoder(seed=27, T=24, B=6, F=64, H=64, L=3, D=64, first_layer_bits=first, w_bits=2, proj_bits=proj)
+    assert w["enc"].layers[1][0].w_ih.bits == 2
+    ref = O.encoder_forward(w["enc"], w["features"])
+    enc = Bd.Encoder(w["enc"])
+    assert [a.bits for a in enc.out_acts] == [4, 4, max(4, proj)]
+    got = enc.forward(torch.from_numpy(w["features"]).cuda())
+    assert Bd.q4_poll_status(enc.ws) == 0
+    np.testing.assert_array_equal(got["e"].cpu().numpy(), ref["e"])
+
+
 def test_outer_and_inner_quantizer_placement_counted_on_the_device(Bd):
     # Section 3.4 on the device: the library counts its activation-quantizer applications.  Outer
     # placement (quantize once at each cell output; the input once per frame): T + T L.  Inner
