@@ -46,6 +46,13 @@ int check_mat(const q4_mat* m, int rows, int k_pad_expected) {
   return Q4_OK;
 }
 
+// Rows that the tensor-core paths can address: a grid has 65535 row tiles, and the gather counts 32-code pieces in 32
+// bits (rows of k codes).  More go to the general kernels, which walk any number.
+inline bool mma_rows(long long rows, int k) {
+  const long long tiles = (rows + 127) / 128;
+  return tiles <= 65535 && tiles * 128 * (k / 32) <= INT32_MAX;
+}
+
 inline long long row_bytes(int k_pad, int bits) { return (long long)k_pad * bits / 8; }
 
 GemmArgs gemm_args(const void* x, long long x_stride, const int32_t* x_idx, const q4_act& xa, int M,
@@ -259,7 +266,7 @@ int q4_linear_forward(const void* xq, const q4_act* x_act, int32_t M, const q4_m
   if (!aligned16(xq) || !aligned16(out)) return Q4_ERR_ALIGN;
   {
     const int32_t wd[2] = {M, w->k_pad};
-    if (prepared && workspace && !dbg_acc && M >= 128 && aligned16(workspace) && aligned16(prepared) &&
+    if (prepared && workspace && !dbg_acc && M >= 128 && mma_rows(M, w->k_pad) && aligned16(workspace) && aligned16(prepared) &&
         workspace_bytes >= q4_workspace_bytes(Q4_WS_LINEAR, wd, 2)) {
       // tensor cores: int8 copy of the input rows, then the tiled GEMM on the prepared int8 weights
       cudaStream_t s = S(stream);
@@ -372,6 +379,7 @@ int qlstm_step(const void* xq, const q4_act* x_act, const int32_t* x_row_idx, co
   {
     const int32_t wd[3] = {N, w_ih->k_pad, H};
     if (prepared && workspace && hq_out && H % 128 == 0 && aligned16(workspace) && aligned16(prepared) &&
+        mma_rows(N, H > w_ih->k_pad ? H : w_ih->k_pad) &&
         (dbg_acc_ih == nullptr) == (dbg_acc_hh == nullptr) &&
         aligned16(c_in) && aligned16(c_out) && aligned16(h_f32_out) &&   // moved 16 bytes and more at a time
         workspace_bytes >= q4_workspace_bytes(Q4_WS_LSTM_STEP, wd, 3)) {
@@ -653,7 +661,7 @@ int qjoint_logprobs(const float* e, const int32_t* frame_idx, const void* pq, co
   ++g_quant_calls;   // tanh(e * p)
   const int32_t dims3[3] = {N, D, w_pred->k_pad};
   if (prepared_pred && prepared_out && z_act->is_signed && aligned16(prepared_pred) &&
-      aligned16(prepared_out) && workspace_bytes >= q4_workspace_bytes(Q4_WS_JOINT, dims3, 3)) {
+      aligned16(prepared_out) && mma_rows(N, w_pred->k_pad) && workspace_bytes >= q4_workspace_bytes(Q4_WS_JOINT, dims3, 3)) {
     // tensor cores for any number of rows (a 128-row tile of mostly empty rows included: 16 rows 15.7 us of device time in
     // three launches, 26.9 in the four of the kernels for unprepared weights): int8 copy of the hidden codes; projection GEMM whose epilogue forms
     // tanh(e * p) and quantizes it; output layer with the log-softmax in its epilogue (fused head kernel

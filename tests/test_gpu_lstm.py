@@ -606,6 +606,18 @@ def test_linear_on_the_tensor_cores_tile_widths(Bd, M, J, K):
     np.testing.assert_array_equal(got.cpu().numpy(), want)
 
 
+def test_linear_of_more_rows_than_a_grid_has_tiles_for(Bd):
+    # one row more than 65535 tiles of 128: the general kernel, the same sums
+    M, J, K = 65535 * 128 + 1, 4, 32
+    lin = Bd.DeviceLinear(synth._linear(synth.Stream(8), "lin", J, K)).prepare()
+    act = Bd.q4_act_symmetric(1.0, 4)
+    few = torch.randint(0, 256, (300, K // 2), dtype=torch.uint8, device="cuda")
+    xq = torch.zeros((M, K // 2), dtype=torch.uint8, device="cuda")
+    xq[:150], xq[-150:] = few[:150], few[150:]
+    got, want = Bd.q4_linear_forward(xq, act, lin), Bd.q4_linear_forward(few, act, lin)
+    assert torch.equal(got[:150], want[:150]) and torch.equal(got[-150:], want[150:])
+
+
 def test_bounded_wait_runs_out_and_the_stream_stays_usable(Bd):
     # The consumer of the tiled tensor-core GEMM waits for operand tiles a bounded number of polls.  With
     # the test hook the producer issues nothing (so nothing asynchronous is in flight): the wait runs
