@@ -127,9 +127,8 @@ __device__ __forceinline__ float label_score(double s_rho, float inc) { return (
 // A lower bound of the W-th best label proposal: the proposals are split into 16 disjoint groups (by lane
 // modulo 16); each group's best is a distinct proposal, so at least 16 >= W proposals reach the smallest of
 // the 16 group maxima.  An empty group gives -inf: everything valid passes.
-__device__ __forceinline__ float label_bound(const float (*gmax)[16], int W, int lane) {
+__device__ __forceinline__ float label_bound(const float (*gmax)[16], int lane) {   // rows of slots that are not there hold -inf
   float g = -INFINITY;
-  (void)W;   // rows of slots that are not there hold -inf
 #pragma unroll
   for (int w = 0; w < SEL_NT / 32; w += 2) g = fmaxf(g, gmax[w + (lane >> 4)][lane & 15]);
   g = fmaxf(g, __shfl_xor_sync(0xffffffffu, g, 16));
@@ -387,7 +386,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
       cand[(size_t)w2 * V + k] = NEG;
     }
   }
-  const float bound = fast ? label_bound(s_gmax, W, lane) : NEG;
+  const float bound = fast ? label_bound(s_gmax, lane) : NEG;
   __syncthreads();
 
   // ---- finished hypotheses: blank proposals that consume the last frame
@@ -694,7 +693,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_tsd_select(const __grid_constant_
       __syncwarp();
     }
   }
-  const float bound = fast ? label_bound(s_gmax, W, lane) : NEG;
+  const float bound = fast ? label_bound(s_gmax, lane) : NEG;
   __syncthreads();
 
   if (inner) {
