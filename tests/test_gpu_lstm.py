@@ -173,6 +173,17 @@ def test_layer_clusters_of_ten(Bd, T, B, dirs, xb, hb, ob):
     layer_case(Bd, T, B, 32, 640, dirs, xb, hb, ob, seed=31)
 
 
+# one kernel each for the numbers of groups beyond: clusters of 8 CTAs with packed weights and one, three and four groups a
+# cluster; with int8 fragments and one
+@pytest.mark.parametrize("T,B,dirs,xb,hb,ob,kernel,per_cluster", [(7, 45, 2, 4, 4, 4, 1, 1), (6, 98, 1, 4, 4, 8, 1, 1),
+                                                                  (3, 157, 2, 4, 4, 4, 1, 3), (3, 222, 2, 4, 4, 4, 1, 4),
+                                                                  (7, 45, 2, 8, 8, 4, 2, 1), (6, 50, 2, 4, 8, 8, 2, 1)])
+def test_layer_clusters_of_eight(Bd, T, B, dirs, xb, hb, ob, kernel, per_cluster):
+    p = Bd.encoder_recurrence_plan(T, B, dirs, 640, w_bits=hb, hid_bits=hb)
+    assert (p["kernel"], p["groups_per_cluster"], p["turns"]) == (kernel, per_cluster, [0, 0])
+    layer_case(Bd, T, B, 32, 640, dirs, xb, hb, ob, seed=37)
+
+
 def test_recurrence_plan_on_this_device(Bd):
     # the capacities asked of the device give a B200 the plan that the host assumes for one, whichever width comes first
     plan = Bd.encoder_recurrence_plan
@@ -218,9 +229,10 @@ def test_layer_time_slicing_equals_two_groups_per_cluster(Bd):
 
 
 @pytest.mark.parametrize("T,B,K,H", [(8, 5, 64, 32),
-                                     # 640 cells: int8 weights mostly in registers; 20 sequences = one group per
-                                     # cluster, 57 over 64 steps = the clusters of one direction take turns
-                                     (8, 20, 64, 640), (64, 57, 64, 640), (9, 30, 64, 640), (70, 2, 64, 128)])
+                                     # 640 cells: clusters of 16 CTAs, of 10, and of 8 with int8 weights mostly in
+                                     # registers (45 sequences one group per cluster, 57 over 64 steps the clusters of
+                                     # one direction take turns); 128 cells: clusters of 4
+                                     (8, 20, 64, 640), (64, 57, 64, 640), (9, 30, 64, 640), (9, 45, 64, 640), (70, 2, 64, 128)])
 def test_layer_per_sequence_input_scale(Bd, T, B, K, H):
     w = synth.single_layer(seed=5, T=T, B=B, K=K, H=H, bits=8, dirs=2)
     base = O.act_symmetric(1.0, 8)
