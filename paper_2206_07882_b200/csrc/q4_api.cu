@@ -1440,7 +1440,6 @@ static SearchGraph* plan_graph(SearchPlan* p, const SearchKey& key) {
       g.last_use = ++p->uses;
       return &g;
     }
-  const BesideCaptures guard;
   for (SearchGraph& g : p->graph)
     if ((!g.exec || cudaEventQuery(g.done) == cudaSuccess) && (!place || g.last_use < place->last_use)) place = &g;
   if (cudaPeekAtLastError() == cudaErrorNotReady) cudaGetLastError();   // an event that is not ready is no error
@@ -1527,6 +1526,7 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
     // the first two frames' steps always: the first step's networks start from the reset state, and the kernels set their
     // attributes at their first launch
     if (p && it == 2 * S1) {
+      const BesideCaptures guard;          // the first replay of a graph may allocate, too
       SearchGraph* g = plan_graph(p, key);
       const int first = it;
       if (g) {

@@ -648,7 +648,9 @@ def test_search_beside_a_capture_of_another_thread(Bd):
     dd = Bd.Decoder(dw, share_from=first)
     dd.alloc_state(3, 6, 120)
     x = torch.zeros(8, device="cuda")
-    side, failure = torch.cuda.Stream(), []
+    side, capturing, failure = torch.cuda.Stream(), torch.cuda.Stream(), []
+    while capturing in (side, *dd._aux_streams):         # torch hands its streams out in turn, more than once
+        capturing = torch.cuda.Stream()
 
     def search():
         try:
@@ -662,7 +664,7 @@ def test_search_beside_a_capture_of_another_thread(Bd):
 
     torch.cuda.synchronize()
     g = torch.cuda.CUDAGraph()
-    with torch.cuda.graph(g):
+    with torch.cuda.graph(g, stream=capturing):
         x.add_(1.0)
         worker = threading.Thread(target=search)
         worker.start()
