@@ -236,7 +236,7 @@ class Job:
         if self.kind == "predjoint":
             dw = synth.decoder(wl["seed"])
             self.pj = Bd.Decoder(dw)
-            # one-time int8 operands: from 128 rows on the library runs these calls on the tensor cores
+            # one-time int8 operands: with them the library runs these calls on the tensor cores
             self.pj.pred_lstm.prepare()
             self.pj.pred_proj.prepare()
             self.pj.joint_out.prepare()

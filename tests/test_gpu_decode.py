@@ -77,7 +77,7 @@ def pred_joint_gpu(Bd, dd, e_dev, frame_idx, tokens):
     """Teacher-forced prediction network + joint on the GPU: logp [N,S,V], hq codes [N,S,Hp]."""
     N, S = tokens.shape
     Hp, V = dd.pred_lstm.H, dd.V
-    # one-time int8 operands: from 128 rows on these calls run on the tensor-core kernels
+    # one-time int8 operands: these calls run on the tensor-core kernels (steps of up to 32 rows on the weight-streaming one)
     dd.pred_lstm.prepare()
     dd.pred_proj.prepare()
     dd.joint_out.prepare()

@@ -113,8 +113,14 @@ def test_quantize_steps_layers_and_linear_layers_stay_inside_their_buffers(guard
         x = torch.from_numpy(st.normal(f"x{bits}{K}", (rows, K)).astype(np.float32)).cuda()
         Bd.quantize_pack_int4(x, Bd.q4_act_symmetric(2.0, bits))
         Bd.quantize_pack_int4(x, Bd.q4_act_symmetric(1.0, bits), mode=1, n_groups=1)
-    # one step: DP4A kernel (ragged rows and widths), tensor-core kernel (prepared operands, ragged tile)
-    for N, K, H, prep in ((70, 200, 96, False), (5, 32, 32, False), (130, 256, 128, True), (300, 96, 256, True)):
+        Bd.quantize_pack_int4(x, Bd.q4_act_symmetric(1.0, bits), mode=1, n_groups=3)
+        Bd.quantize_pack_int4(x, Bd.q4_act_symmetric(1.0, bits), mode=1, n_groups=rows)
+    x = torch.from_numpy(st.normal("large", (1300, 1279)).astype(np.float32)).cuda()     # too large for a cluster
+    Bd.quantize_pack_int4(x, Bd.q4_act_symmetric(1.0, 8), mode=1, n_groups=1)
+    # one step: DP4A kernel (ragged rows and widths), weight-streaming kernel (up to 32 rows), tensor-core kernel
+    # (prepared operands, ragged tile, one row tile)
+    for N, K, H, prep in ((70, 200, 96, False), (5, 32, 32, False), (9, 128, 128, False), (31, 128, 256, True),
+                          (130, 256, 128, True), (300, 96, 256, True), (33, 96, 256, True), (1, 64, 128, True)):
         lw = synth._lstm(st, f"l{N}", K, H, 4, bias_std=0.2, hid_alpha=0.95, hid_bits=4)
         x_act, hid = O.act_symmetric(3.0, 4), O.act_symmetric(0.95, 4)
         xq = st.integers(f"xq{N}", (N, K), x_act.lo(), x_act.hi()).astype(np.int16)
@@ -123,11 +129,24 @@ def test_quantize_steps_layers_and_linear_layers_stay_inside_their_buffers(guard
         dl = Bd.DeviceLstm(lw)
         if prep:
             dl.prepare()
-        Bd.qlstm_step(pack_codes(xq, x_act, dl.w_ih.k_pad), to_act(x_act), pack_codes(hq, hid), c, dl, want_dbg=not prep)
-    # whole layers: step-by-step kernels, the general persistent kernel, the register-resident kernels
-    # (one group per cluster; clusters taking turns at 57 sequences x 2 directions; int8 weights)
-    for T, B, K, H, dirs, bits in ((9, 3, 48, 32, 2, 4), (20, 70, 240, 64, 2, 8), (12, 33, 128, 96, 1, 4),
-                                   (6, 20, 64, 640, 2, 4), (64, 57, 64, 640, 2, 4), (64, 57, 64, 640, 2, 8)):
+        Bd.qlstm_step(pack_codes(xq, x_act, dl.w_ih.k_pad), to_act(x_act), pack_codes(hq, hid), c, dl,
+                      want_dbg=not prep and N not in (9, 31))
+    # the joint network of few rows: unprepared and prepared, both forms of the output layer
+    for N, V, D, prep in ((5, 46, 64, False), (5, 46, 64, True), (33, 300, 256, True), (1, 46, 256, True)):
+        dd = Bd.Decoder(synth.decoder(seed=5, V=V, E=32, Hp=64, D=D, Hs=32, Ht=32))
+        if prep:
+            dd.pred_proj.prepare()
+            dd.joint_out.prepare()
+        pq = pack_codes(st.integers(f"pq{N}{V}", (N, 64), -7, 7).astype(np.int16), O.act_symmetric(1.0, 4))
+        e = torch.from_numpy(st.normal(f"je{N}{V}", (7, D)).astype(np.float32)).cuda()
+        fi = torch.from_numpy(st.integers(f"jf{N}{V}", (N,), 0, 6).astype(np.int32)).cuda()
+        Bd.qjoint_logprobs(e, fi, pq, Bd.q4_act_symmetric(1.0, 4), dd.pred_proj, dd.z_act, dd.joint_out)
+    # whole layers: step-by-step kernels, the general persistent kernel, the kernel for few groups on clusters of 4, 16
+    # and 10 CTAs, the register-resident kernels (one and two groups per cluster; clusters taking turns at 57 sequences x
+    # 2 directions; int8 weights)
+    for T, B, K, H, dirs, bits in ((9, 3, 48, 32, 2, 4), (20, 70, 240, 64, 2, 8), (12, 33, 128, 96, 1, 4), (6, 20, 64, 640, 2, 4),
+                                   (50, 3, 64, 128, 1, 4), (9, 20, 64, 640, 2, 4), (7, 30, 64, 640, 2, 8), (7, 45, 64, 640, 2, 4),
+                                   (7, 45, 64, 640, 2, 8), (6, 63, 64, 640, 2, 4), (64, 57, 64, 640, 2, 4), (64, 57, 64, 640, 2, 8)):
         w = synth.single_layer(seed=T + B, T=T, B=B, K=K, H=H, bits=bits, dirs=dirs)
         for lw in w["layers"]:
             lw.hid_bits = bits
@@ -151,8 +170,9 @@ def test_quantize_steps_layers_and_linear_layers_stay_inside_their_buffers(guard
 @pytest.mark.parametrize("tensor_cores", [True, False])
 def test_the_search_stays_inside_its_state_and_workspace(guarded, tensor_cores):
     Bd, g = guarded
-    # fused heads (V = 1024, D = 256) with 9 utterances x 16 slots = two ragged row tiles; odd sizes on the DP4A path
-    for V, D, utts in ((1024, 256, 9), (200, 64, 3)):
+    # fused heads (V = 1024, D = 256) with 9 utterances x 16 slots = two ragged row tiles; heads of separate kernels
+    # (D = 64); vocabularies whose rows are no multiple of 16 bytes, in heads of each width
+    for V, D, utts in ((1024, 256, 9), (200, 64, 3), (46, 256, 2), (301, 256, 3), (1101, 256, 2)):
         dw = synth.decoder(seed=77, V=V, E=32, Hp=128, D=D, Hs=128, Ht=128, tgt_layers=2, U_max=5, W=16)
         e = torch.from_numpy(synth.Stream(5).normal("e", (9, utts, D)).astype(np.float32)).cuda()
         dec = Bd.Decoder(dw, tensor_cores=tensor_cores)

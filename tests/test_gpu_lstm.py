@@ -117,8 +117,8 @@ def layer_case(Bd, T, B, K, H, dirs, xb=4, hb=4, ob=None, seed=0, x_clip=3.0, ma
         alt = Bd.qlstm_layer_forward(pack_codes(xq.reshape(T * B, K), x_act), to_act(x_act), T, B, layers,
                                      to_act(out), want_dbg=True, tensor_cores=False)
         assert torch.equal(alt["acc_ih"], got["acc_ih"]) and torch.equal(alt["yq"], got["yq"])
-    # the same call without the accumulator dumps (at 640 cells and 4 bits this takes the kernel that
-    # keeps the recurrent weights in registers)
+    # the same call without the accumulator dumps, which the general kernel alone makes: where the plan says so this
+    # takes one of the kernels that keep the recurrent weights in registers
     lean = Bd.qlstm_layer_forward(pack_codes(xq.reshape(T * B, K), x_act), to_act(x_act), T, B, layers,
                                   to_act(out), want_state=True)
     assert Bd.q4_poll_status(lean["workspace"]) == 0
@@ -488,10 +488,13 @@ def test_step_on_the_tensor_cores_with_prepared_weights(Bd, N, K, H, xb, hb, sig
     xq = st.integers("xq", (N, K), x_act.lo(), x_act.hi()).astype(np.int16)
     hq = st.integers("hq", (N, H), hid.lo() + 1, hid.hi()).astype(np.int16)
     c = st.normal("c", (N, H)).astype(np.float32)
-    n0 = Bd.launch_count()
     step_case(Bd, lw, x_act, hid, xq, hq, c, prepare=True)
-    # packing of the test operands aside: two gathers and one fused kernel (not the DP4A kernel alone)
-    assert Bd.launch_count() - n0 >= 3
+    # the gather and the fused kernel (the kernel for unprepared weights is one launch)
+    dl = Bd.DeviceLstm(lw).prepare()
+    operands = pack_codes(xq, x_act, dl.w_ih.k_pad), to_act(x_act), pack_codes(hq, hid), torch.from_numpy(c).cuda(), dl
+    n0 = Bd.launch_count()
+    Bd.qlstm_step(*operands, want_dbg=True)
+    assert Bd.launch_count() - n0 == 2
 
 
 @pytest.mark.parametrize("N", [20, 40, 130])
