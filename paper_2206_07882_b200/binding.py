@@ -128,6 +128,7 @@ def _stream():
 
 
 _SCRATCH_STREAMS = 16
+_capturing = torch.cuda.is_current_stream_capturing
 
 
 def _scratch(owner, need: int, device, stream: int) -> torch.Tensor:
@@ -135,7 +136,7 @@ def _scratch(owner, need: int, device, stream: int) -> torch.Tensor:
     streams must not share one.  It is allocated on the stream that uses it, so a buffer that is replaced or dropped
     is handed on in that stream's order.  A capture gets a buffer of its own from the graph's memory, which lives as
     long as the graph, whatever happens to the layer meanwhile."""
-    if torch.cuda.is_current_stream_capturing():
+    if _capturing():
         return torch.empty(need, dtype=torch.uint8, device=device)
     per = owner.stream_ws
     ws = per.get(stream)

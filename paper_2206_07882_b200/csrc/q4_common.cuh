@@ -16,21 +16,21 @@ namespace q4 {
 // has called it or exited.
 //
 // What a kernel may read before pdl_wait(): nothing that any kernel before it on the stream may be writing, the
-// caller's own kernels included.  Two exceptions read what a kernel of the same call further back wrote, in
-// chains whose every kernel between triggers only after its own wait, so that the writer has completed and its
-// writes are in the L2 when the reader starts:
+// caller's own kernels included.  The exceptions read what was written before the kernel before them, where that one
+// triggers only after its own wait, so that the writer has completed and its writes are in the L2 when the reader
+// starts:
 //   the count of rows with work (tile_without_work in q4_mma.cu);
 //   a layer's recurrence its prepared weights, constants and input scales (written before the input projection),
 //   and a second LSTM layer the operand tiles of its recurrent half (weights, and rows that the gather wrote).
 // They are read by the loads below, or by tile copies, which do not look into the L1.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ int32_t ld_acquire(const int32_t* p) {
+// loads that are coherent at device scope
+__device__ __forceinline__ int32_t ld_coherent(const int32_t* p) {
   int32_t v;
-  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p));
   return v;
 }
-// loads that are coherent at device scope
 __device__ __forceinline__ uint32_t ld_coherent(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p));

@@ -270,12 +270,13 @@ __device__ __forceinline__ void flag_timeout(int32_t* status) {
 //   The count is the one thing that is read before the kernel's wait.  The selection writes it; the first kernel of
 // a step's chains (the gather, the weight-streaming step or a kernel behind an event) triggers its successor only after its own wait
 // for the selection, and every later kernel of a chain starts after that.  So the count is in memory when any of these
-// kernels starts, and a load that acquires at the scope of the device cannot meet an older copy of it.
+// kernels starts, and a load that is coherent at device scope cannot meet an older copy of it.  (Nothing else is read on
+// its word, so it need not acquire: that would drop the SM's L1 under the kernels beside it.)
 //   A grid whose tiles all leave must not complete before its predecessor does, because its successor waits for this
 // grid only: one CTA of the first row tile, which leaves only if all do, waits before it leaves.
 __device__ __forceinline__ bool tile_without_work(const int32_t* n_active, int m0) {
   if (!n_active) return false;
-  if (m0 < ld_acquire(n_active)) return false;
+  if (m0 < ld_coherent(n_active)) return false;
   if (m0 == 0 && blockIdx.x == 0) {
     pdl_trigger();
     pdl_wait();
