@@ -3,11 +3,12 @@
 // operand, both K-major int8 in shared memory under the 128-byte swizzle.
 //   k_mma_gemm : D[128 x 32..256] tiles, epilogues: de-quantize+bias / re-quantize / joint element-wise;
 //   k_mma_gemm_persistent : the same main loop with the int32 sums stored as they are.
-//   k_mma_lstm : D_ih, D_hh[128 x 128] tiles (32 cells x 4 gates, gate-interleaved weight
-//                rows) with the whole LSTM cell update fused into the epilogue.
-// Warp roles per CTA: epilogue warps (one TMEM lane quarter each), one TMA producer thread,
-// one MMA issuer thread.  4-bit codes are unpacked to int8 once per call by k_unpack_rows /
-// k_prepare_w before they meet the tensor cores.
+//   k_mma_lstm : D_ih, D_hh[128 x 64 or 128] tiles (16 or 32 cells x 4 gates, gate-interleaved weight
+//                rows) with the whole LSTM cell update fused into the epilogue;
+//   k_mma_lmhead : bottleneck, re-quantization, output layer and log-softmax of a row tile on a cluster of CTAs.
+// Warp roles per CTA: epilogue warps (one TMEM lane quarter each), one producer warp, one MMA issuer warp (an
+// elected lane of each issues).  Codes are unpacked to int8 before they meet the tensor cores: rows of a call by
+// k_unpack_multi, a layer's input and weights by k_layer_prepare, weights once by k_prepare_w.
 #include <string.h>
 
 #include "q4_internal.h"
@@ -778,10 +779,9 @@ cudaError_t launch_mma_gemm_i32(const int8_t* x8, int M, const int8_t* w8, int J
 // of the blocks are exchanged through distributed shared memory as well; one cluster barrier later every
 // thread knows the row's log-sum-exp and stores log-probabilities: one global write, no separate log-softmax
 // pass.  With H = 0 there is no bottleneck: the 256-wide operand rows are read from memory (joint network).
-// Bound by the latency of this chain.  (With all 256 bottleneck columns in every CTA it was 5.0 us of bottleneck
-// sums + 2.8 us of re-quantization before the second MMA; codes stored to the peers 8 bytes at a time took
-// 5 us with 128 rows.  Frame-by-frame search of 5 utterances, 40 rows: 15.95 -> 14.4 ms, 64 utterances x 10 s
-// end to end 53.0 -> 51.6 ms.)
+// Bound by the latency of this chain.  (All 256 bottleneck columns in every CTA take 5.0 us of bottleneck sums and 2.8 us
+// of re-quantization before the second MMA; codes stored to the peers 8 bytes at a time 5 us with 128 rows.  Dealt out and
+// copied as blocks: frame-by-frame search of 5 utterances, 40 rows, 15.95 -> 14.4 ms.)
 constexpr int HEAD_D = 256;
 constexpr int HEAD_CTAS = 8;                 // = the portable cluster size
 constexpr int HEAD_BN1 = HEAD_D / HEAD_CTAS; // bottleneck columns per CTA

@@ -3,7 +3,7 @@
 // reading the weights once, so they are read as stored: packed 4-bit codes, 128-bit loads, no int8
 // copies, no staging through shared memory.
 //
-// One CTA owns the 16 weight rows of 4 cells (their i, f, g, o rows); its 16 warps split K in chunks
+// One CTA owns the 16 weight rows of 4 cells (their i, f, g, o rows); its 8 warps split K in chunks
 // of 128 codes (the input part, then the recurrent part); a warp fetches its next chunk while it
 // multiplies the present one.  Four CTAs fit an SM, so all CTAs of a layer (at most 512) are resident
 // together and the whole weight matrix is requested within the first microsecond.  A lane loads 16 bytes (32 codes) of two
