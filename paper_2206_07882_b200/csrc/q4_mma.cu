@@ -423,19 +423,17 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
         // joint network: z = tanh(e * p) with p the projected value just formed; quantized below.  A row without a
         // frame (negative index) has z = 0, as in k_joint_z
         const int er_idx = a.mul_idx[mi];
-        const float* er = a.mul_e + (long long)er_idx * a.J + j0;
-        float4 ev[8];
+        if (er_idx >= 0) {
+          const float* er = a.mul_e + (long long)er_idx * a.J + j0;
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-          ev[i] = er_idx >= 0 ? *reinterpret_cast<const float4*>(er + 4 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          v[4 * i] = tanh_fixed(__fmul_rn(ev[i].x, v[4 * i]));
-          v[4 * i + 1] = tanh_fixed(__fmul_rn(ev[i].y, v[4 * i + 1]));
-          v[4 * i + 2] = tanh_fixed(__fmul_rn(ev[i].z, v[4 * i + 2]));
-          v[4 * i + 3] = tanh_fixed(__fmul_rn(ev[i].w, v[4 * i + 3]));
-        }
-        if (er_idx < 0) {
+          for (int i = 0; i < 32; i += 4) {
+            const float4 ev = *reinterpret_cast<const float4*>(er + i);
+            v[i] = tanh_fixed(__fmul_rn(ev.x, v[i]));
+            v[i + 1] = tanh_fixed(__fmul_rn(ev.y, v[i + 1]));
+            v[i + 2] = tanh_fixed(__fmul_rn(ev.z, v[i + 2]));
+            v[i + 3] = tanh_fixed(__fmul_rn(ev.w, v[i + 3]));
+          }
+        } else {
 #pragma unroll
           for (int i = 0; i < 32; ++i) v[i] = 0.0f;
         }
