@@ -828,7 +828,9 @@ class GraphedStep:
     """Replays one whole pass (any callable that only enqueues library calls on the current
     stream) as a CUDA graph: the pass is run eagerly once (so that every kernel attribute is
     configured), captured once, then replayed.  The callable must read its input from the
-    static tensors it closes over; results are the tensors it returned during capture."""
+    static tensors it closes over; results are the tensors it returned during capture.  An Encoder's
+    workspace and a Decoder's state are the object's own: the graph holds until a larger call on the object
+    replaces them."""
 
     def __init__(self, fn):
         self.fn = fn
