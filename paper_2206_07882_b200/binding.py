@@ -124,28 +124,31 @@ def _raw_stream() -> int:
 
 
 def _stream():
-    return C.c_void_p(_raw_stream())
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 _SCRATCH_STREAMS = 16
 _capturing = torch.cuda.is_current_stream_capturing
 
 
-def _scratch(owner, need: int, device, stream: int) -> torch.Tensor:
-    """Workspace of a prepared layer's call on the current stream, one per stream: calls on one stream are ordered, calls on different
-    streams must not share one.  It is allocated on the stream that uses it, so a buffer that is replaced or dropped
-    is handed on in that stream's order.  A capture gets a buffer of its own from the graph's memory, which lives as
-    long as the graph, whatever happens to the layer meanwhile."""
-    if _capturing():
-        return torch.empty(need, dtype=torch.uint8, device=device)
+def _scratch(owner, rows: int, stream: int, call_id: int, dims: tuple, device) -> tuple:
+    """(workspace, rows it is good for, bytes) of a prepared layer's call on the current stream, one per stream: calls
+    on one stream are ordered, calls on different streams must not share one.  It is allocated on the stream that
+    uses it, so a buffer that is replaced or dropped is handed on in that stream's order.  A capture gets a buffer of
+    its own from the graph's memory, which lives as long as the graph, whatever happens to the layer meanwhile."""
     per = owner.stream_ws
-    ws = per.get(stream)
-    if ws is None or ws.numel() < need:
-        if ws is None and len(per) >= _SCRATCH_STREAMS:
+    entry = per.get(stream)
+    capturing = _capturing()
+    if capturing or entry is None or entry[1] < rows:
+        need = workspace_bytes(call_id, (rows,) + dims)
+        new = (torch.empty(need, dtype=torch.uint8, device=device), rows, need)
+        if capturing:
+            return new
+        if entry is None and len(per) >= _SCRATCH_STREAMS:
             del per[next(iter(per))]
-        ws = per[stream] = torch.empty(need, dtype=torch.uint8, device=device)
-    owner.ws = ws
-    return ws
+        entry = per[stream] = new
+    owner.ws = entry[0]
+    return entry
 
 
 def _chk(code: int, where: str):
@@ -390,15 +393,14 @@ def qlstm_step(xq: torch.Tensor, x_act: Act, hq_in: torch.Tensor, c_in: torch.Te
         r["acc_ih"] = torch.empty((N, 4 * H), dtype=torch.int32, device=dev)
         r["acc_hh"] = torch.empty((N, 4 * H), dtype=torch.int32, device=dev)
     wih, whh = layer.w_ih.c(), layer.w_hh.c()
-    ws, stream = None, _raw_stream()
+    ws, nbytes, stream = None, 0, _raw_stream()
     if layer.prepared is not None:      # tensor-core path
-        need = workspace_bytes(WS_LSTM_STEP, [N, layer.w_ih.k_pad, H])
-        ws = _scratch(layer, need, dev, stream)
+        ws, _, nbytes = _scratch(layer, N, stream, WS_LSTM_STEP, (layer.w_ih.k_pad, H), dev)
     _chk(lib().qlstm_step(_p(xq), C.byref(x_act), _p(x_row_idx), _p(hq_in), _p(c_in), C.c_int32(N),
                           C.byref(wih), C.byref(whh), _p(layer.bias), C.byref(layer.hid_act),
                           _p(r.get("hq")), _p(r["c"]), _p(r.get("h")), _p(r.get("acc_ih")),
                           _p(r.get("acc_hh")), _p(layer.prepared), _p(ws),
-                          C.c_size_t(ws.numel() if ws is not None else 0), C.c_void_p(stream)), "qlstm_step")
+                          C.c_size_t(nbytes), C.c_void_p(stream)), "qlstm_step")
     return r
 
 
@@ -436,13 +438,12 @@ def q4_linear_forward(xq: torch.Tensor, x_act: Act, lin: DeviceLinear, want_acc:
     out = torch.empty((M, lin.w.rows), dtype=torch.float32, device=xq.device)
     acc = torch.empty((M, lin.w.rows), dtype=torch.int32, device=xq.device) if want_acc else None
     w = lin.w.c()
-    ws, stream = None, _raw_stream()
+    ws, nbytes, stream = None, 0, _raw_stream()
     if getattr(lin, "prepared", None) is not None and not want_acc:
-        need = workspace_bytes(WS_LINEAR, [M, lin.w.k_pad])
-        ws = _scratch(lin, need, xq.device, stream)
+        ws, _, nbytes = _scratch(lin, M, stream, WS_LINEAR, (lin.w.k_pad,), xq.device)
     _chk(lib().q4_linear_forward(_p(xq), C.byref(x_act), C.c_int32(M), C.byref(w), _p(lin.bias),
                                  _p(out), _p(acc), _p(getattr(lin, "prepared", None)), _p(ws),
-                                 C.c_size_t(ws.numel() if ws is not None else 0), C.c_void_p(stream)), "q4_linear_forward")
+                                 C.c_size_t(nbytes), C.c_void_p(stream)), "q4_linear_forward")
     return (out, acc) if want_acc else out
 
 
