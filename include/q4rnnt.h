@@ -358,8 +358,12 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
  * CUDA graphs.  A graph belongs to the model, state, weights of Eq. 1 and workspace it was built for; frames, T and
  * u_max may change from call to call.  A call that finds no graph of its own builds one (host time of about a
  * millisecond; memory for the graph) in place of one whose replays have ended, and enqueues its steps one by one if
- * there is none: it waits for nothing.  One plan serves one search at a time.  Without a plan, in a stream capture,
- * while launches are timed and under q4_test_wait_expiry_set, the steps are enqueued one by one (same results).
+ * there is none: it waits for nothing.  One plan serves one search at a time.  In the tensor-core path with D = 256 the
+ * steps of an alignment-length synchronous search are the body of a loop in the graph (a conditional node), which ends
+ * when no utterance has labels left to propose; the iterations that are left then are carried out by two launches (same
+ * results, same history).  In a stream capture the loop becomes a node of the caller's graph.  Without a plan, in another
+ * search in a stream capture, below 96 steps, while launches are timed and under q4_test_wait_expiry_set, the steps are
+ * enqueued one by one (same results).
  * Graphs, and what they are captured on, are the plan's own: the streams lent with the state are used by single
  * steps only, and a plan may be made, used or destroyed while another thread captures a stream.  A plan uses the memory
  * of a search only in a search on it.  q4_search_plan_destroy waits for the replays on their way.
@@ -367,8 +371,8 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
 typedef void* q4_search_plan;
 int q4_search_plan_create(q4_search_plan* out);
 int q4_search_plan_destroy(q4_search_plan plan);
-/* What a plan has done so far (host counters, for tests and diagnostics): out[0] graphs built, out[1] replays
- * enqueued, out[2] attempts to build a graph that failed (the search then enqueued its steps one by one). */
+/* What a plan has done so far (host counters, for tests and diagnostics): out[0] graphs built, out[1] groups
+ * of 12 steps that replays were enqueued for, out[2] attempts to build a graph that failed (the search then enqueued its steps one by one). */
 int q4_search_plan_info(q4_search_plan plan, int64_t* out);
 int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, int32_t B, int32_t T, int32_t W,
                    int32_t u_max, float lambda_t, float lambda_s, float rho, int32_t time_synchronous,
@@ -399,7 +403,7 @@ size_t q4_workspace_bytes(int32_t call_id, const int32_t* dims, int32_t ndims);
 int q4_poll_status(const int32_t* device_status, q4_stream stream);
 
 /* Library version and the number of kernels launched so far by this process (a counter the
- * benchmark reads to report its launch count). */
+ * benchmark reads to report its launch count; a graph's loop counts as if it took all its turns). */
 int q4_version(void);
 int64_t q4_launch_count(void);
 /* Number of activation-quantizer applications enqueued so far (Section 3.4 counts them: T + T L

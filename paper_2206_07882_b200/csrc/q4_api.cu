@@ -915,10 +915,26 @@ static int check_model_lstm(const q4_lstm& L, const q4_act& x_act) {
   return check_lstm(&L.w_ih, &L.w_hh, &x_act, &L.hid_act, &H);
 }
 
-// One step; `call` non-null: e, T and u_max come from there, and its iteration number is added to `iter`.
+constexpr int PLAN_ITERS = 12;   // steps in a search's graph: even (the pending lists alternate), a multiple of the 1, 2, 3 or 4 calls per frame
+// Whether a search takes the tensor-core kernels: prepared weights, widths they cover and room for their operands.
+static bool search_uses_tensor_cores(const q4_model& m, const q4_beam_state& st, int B, int W, size_t workspace_bytes) {
+  const int Hp = m.pred_lstm.w_hh.k_pad, Hs = m.src.lstm[0].w_hh.k_pad, Ht = m.tgt.lstm[0].w_hh.k_pad;
+  const int Ep = m.pred_lstm.w_ih.k_pad;
+  const int32_t dims8[8] = {B, W, m.V, m.D, Ep, Hp, Hs, Ht};
+  return m.prepared != nullptr && m.src.n_layers == 1 && m.src.lstm[0].w_ih.k_pad == Ep && m.tgt.lstm[0].w_ih.k_pad == Ep &&
+         Hp % 128 == 0 && Hs % 128 == 0 && Ht % 128 == 0 &&
+         aligned16(st.pred_c) && aligned16(st.src_c) && aligned16(st.tgt_c[0]) && aligned16(st.tgt_c[1]) &&
+         workspace_bytes >= q4_workspace_bytes(Q4_WS_BEAM, dims8, 8);
+}
+// In the tensor-core path the first codes block of the workspace is free: there a search keeps when its utterances were frozen.
+static int32_t* search_frozen(void* workspace) { return reinterpret_cast<int32_t*>(static_cast<uint8_t*>(workspace) + 256); }
+
+// One step; `call` non-null: e, T and u_max come from there, and its iteration number is added to `iter`.  `frozen`: an
+// utterance without labels to propose is left to launch_search_tail; `loop`: this is the last step of a graph's loop.
 static int beam_step(const q4_model* model, q4_beam_state* state, const float* e, int32_t B, int32_t T, int32_t W,
                      int32_t iter, int32_t u_max, float lambda_t, float lambda_s, float rho, int32_t mode,
-                     void* workspace, size_t workspace_bytes, q4_stream stream, const SearchCall* call) {
+                     void* workspace, size_t workspace_bytes, q4_stream stream, SearchCall* call, int32_t* frozen,
+                     const cudaGraphConditionalHandle* loop) {
   if (!model || !e || !workspace) return Q4_ERR_NULL;
   if (mode < 0 || mode > 2) return Q4_ERR_UNSUPPORTED;
   if (B <= 0 || T <= 0 || W <= 0 || W > 16 || iter < 0 || u_max < 0) return Q4_ERR_DIM;
@@ -995,12 +1011,7 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
   // kernels (measured 3x on a single utterance), since the time goes to streaming the weights
   const int Hp = m.pred_lstm.w_hh.k_pad, Hs = m.src.lstm[0].w_hh.k_pad, Ht = m.tgt.lstm[0].w_hh.k_pad;
   const int Ep = m.pred_lstm.w_ih.k_pad;
-  const int32_t dims8[8] = {B, W, V, D, Ep, Hp, Hs, Ht};
-  const bool use_mma = m.prepared != nullptr && m.src.n_layers == 1 &&
-                       m.src.lstm[0].w_ih.k_pad == Ep && m.tgt.lstm[0].w_ih.k_pad == Ep &&
-                       Hp % 128 == 0 && Hs % 128 == 0 && Ht % 128 == 0 &&
-                       aligned16(st.pred_c) && aligned16(st.src_c) && aligned16(st.tgt_c[0]) && aligned16(st.tgt_c[1]) &&
-                       workspace_bytes >= q4_workspace_bytes(Q4_WS_BEAM, dims8, 8);
+  const bool use_mma = search_uses_tensor_cores(m, st, B, W, workspace_bytes);
   if (use_mma) {
     const size_t Np = ((size_t)N + 127) / 128 * 128;
     const int Hmax = Hp > Hs ? (Hp > Ht ? Hp : Ht) : (Hs > Ht ? Hs : Ht);
@@ -1150,14 +1161,15 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
     };
     auto linear_mma = [&](cudaStream_t s, bool dep, int tag_id, int wi, const q4_linear& L, const int8_t* x8,
                           float x_scale, int epi, void* out, long long ldo, const int32_t* out_idx,
-                          const q4_act* out_act, const int32_t* rows_active) -> int {
+                          const q4_act* out_act, const int32_t* rows_active, const int32_t* n_idle = nullptr) -> int {
       TagScope tag(tag_id);
       Q4_TRY(launch_mma_gemm(x8, L.w.k_pad, N, reinterpret_cast<const int8_t*>(pb + pp.lin[wi]), L.w.k_pad,
                              L.w.rows, L.w.k_pad, epi, out, ldo, out_idx, L.w.scale, L.bias, x_scale, out_act,
-                             st.status, rows_active, s, dep));
+                             st.status, rows_active, s, dep, nullptr, nullptr, n_idle, B));
       return Q4_OK;
     };
 
+    const int32_t* n_frozen = frozen ? &call->n_frozen : nullptr;   // all utterances frozen: the joint network has nothing to do
     const bool fused_head = D == 256 && V <= 2048;   // the fused head kernel: 256-wide bottleneck, one cluster per row tile
     // 1a. prediction network, then the joint network for every live slot (stream sp)
     if (nets) {
@@ -1168,7 +1180,8 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
     }
     {
       TagScope tag(TAG_JOINT);
-      Q4_TRY(launch_joint_z(e, nullptr, st.t, B, W, st.pred_p, st.row, N, D, m.z_act, nullptr, z8, live, sp, true, call));
+      Q4_TRY(launch_joint_z(e, nullptr, st.t, B, W, st.pred_p, st.row, N, D, m.z_act, nullptr, z8, live, sp, true, call,
+                            n_frozen ? B : 0));
     }
     // small vocabularies: logits, which the selection normalises in passing (one short kernel instead of a cluster's
     // exchange, and the order of sums of the kernels for few rows)
@@ -1188,10 +1201,12 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
       ja.lp = logits;
       ja.dst_row = live;
       ja.status = st.status;
+      ja.n_idle = n_frozen;
+      ja.all_idle = B;
       Q4_TRY(launch_mma_lmhead(ja, z8, D, nullptr, reinterpret_cast<const int8_t*>(pb + pp.lin[5]), sp, true));
     } else {
       Q4_CHECK(linear_mma(sp, true, TAG_JOINT, 5, m.joint_out, z8, m.z_act.scale, EPI_F32, logits, V, live, nullptr,
-                          nullptr));
+                          nullptr, n_frozen));
     }
     // 1b. source LM (stream ss) and target LM (stream stt)
     for (int which = 0; which < 2 && nets; ++which) {
@@ -1313,6 +1328,11 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
   BeamSelArgs sel;
   memset(&sel, 0, sizeof(sel));
   sel.call = call;
+  sel.frozen = frozen;
+  if (loop) {
+    sel.loop = *loop;
+    sel.loop_iters = PLAN_ITERS;
+  }
   sel.logits = logits;
   sel.src_lp = st.src_lp;
   sel.tgt_lp = st.tgt_lp;
@@ -1342,7 +1362,7 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
                         float lambda_s, float rho, int32_t mode, void* workspace,
                         size_t workspace_bytes, q4_stream stream) {
   return beam_step(model, state, e, B, T, W, iter, u_max, lambda_t, lambda_s, rho, mode, workspace, workspace_bytes, stream,
-                   nullptr);
+                   nullptr, nullptr, nullptr);
 }
 
 // ------------------------------------------------------------------------ whole search
@@ -1353,14 +1373,13 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
 // (W = 4) with the encoder before them: 8.9 -> 8.1 ms with 4-bit weights, 10.9 -> 9.6 with 8-bit ones (host time 11 -> 1 ms);
 // 5 utterances x 8 slots, 360 time-synchronous calls: 12.9 -> 11.9 ms.
 namespace {
-constexpr int PLAN_ITERS = 12;       // even (the pending lists alternate) and a multiple of the 1, 2, 3 or 4 calls per frame
 constexpr int PLAN_MIN_ITERS = 96;   // below, building the graph (1.0 ms of host time, once per kind of search and state) outweighs it
 struct SearchKey {                   // everything the graph was built from
   q4_model model;
   q4_beam_state state;
   void* workspace;
   size_t workspace_bytes;
-  int32_t B, W, tsd, dependent, exact;
+  int32_t B, W, tsd, dependent, exact, loop;
   float lambda_t, lambda_s, rho;
 };
 // One graph and the search it was built for.  PLAN_GRAPHS of them: a decoder that alternates between a few batch sizes,
@@ -1430,6 +1449,35 @@ int q4_search_plan_destroy(q4_search_plan plan) {
   return Q4_OK;
 }
 
+// PLAN_ITERS steps and the call's advance, captured on the plan's stream.  With a loop: the body of a graph's conditional
+// node, whose last selection asks for another turn.
+static int capture_steps(SearchPlan* p, SearchKey& key, const cudaGraphConditionalHandle* loop) {
+  SearchCall* call = static_cast<SearchCall*>(key.workspace);
+  // T and u_max (and the frames) only have to pass the argument checks here; the first frame's steps are never in the graph
+  for (int it = PLAN_ITERS; it < 2 * PLAN_ITERS; ++it)
+    Q4_CHECK(beam_step(&key.model, &key.state, static_cast<const float*>(key.workspace), key.B, 1 << 24, key.W, it, 0,
+                       key.lambda_t, key.lambda_s, key.rho, step_mode(key, it), key.workspace, key.workspace_bytes, p->stream,
+                       call, loop ? search_frozen(key.workspace) : nullptr, it == 2 * PLAN_ITERS - 1 ? loop : nullptr));
+  if (!loop) Q4_TRY(launch_search_advance(call, PLAN_ITERS, p->stream));
+  return Q4_OK;
+}
+// A conditional node in `g` behind `deps` that repeats the steps until every utterance is frozen (at least one turn).
+static int add_search_loop(SearchPlan* p, SearchKey& key, cudaGraph_t g, const cudaGraphNode_t* deps, size_t n_deps,
+                           cudaGraphNode_t* node) {
+  cudaGraphNodeParams np = {};
+  np.type = cudaGraphNodeTypeConditional;
+  np.conditional.type = cudaGraphCondTypeWhile;
+  np.conditional.size = 1;
+  if (cudaGraphConditionalHandleCreate(&np.conditional.handle, g, 1, cudaGraphCondAssignDefault) != cudaSuccess ||
+      cudaGraphAddNode(node, g, deps, n_deps, &np) != cudaSuccess ||
+      cudaStreamBeginCaptureToGraph(p->stream, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                    cudaStreamCaptureModeRelaxed) != cudaSuccess)
+    return Q4_ERR_CUDA;
+  int r = capture_steps(p, key, &np.conditional.handle);
+  if (cudaStreamEndCapture(p->stream, nullptr) != cudaSuccess && r == Q4_OK) r = Q4_ERR_CUDA;
+  return r;
+}
+
 // The graph of a search: the one that was built for the same arguments, else a new one in a free place or in
 // place of the one used longest ago whose last replay has ended.  Null (the search then enqueues its steps one by one)
 // if there is no such place, for the host does not wait for a replay here, or if the graph cannot be built.
@@ -1448,20 +1496,21 @@ static SearchGraph* plan_graph(SearchPlan* p, const SearchKey& key) {
   place->exec = nullptr;
   place->last_use = 0;
   memcpy(&place->key, &key, sizeof(key));   // padding included: keys are compared as bytes
-  SearchCall* call = static_cast<SearchCall*>(key.workspace);
   const int64_t l0 = g_launches, q0 = g_quant_calls;
-  int r = cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeRelaxed) == cudaSuccess ? Q4_OK : Q4_ERR_CUDA;
-  if (r == Q4_OK) {
-    // T and u_max (and the frames) only have to pass the argument checks here; the first frame's steps are never in the graph
-    for (int it = PLAN_ITERS; it < 2 * PLAN_ITERS && r == Q4_OK; ++it)
-      r = beam_step(&key.model, &place->key.state, static_cast<const float*>(key.workspace), key.B, 1 << 24, key.W, it, 0,
-                    key.lambda_t, key.lambda_s, key.rho, step_mode(key, it), key.workspace, key.workspace_bytes, p->stream, call);
-    if (r == Q4_OK && launch_search_advance(call, PLAN_ITERS, p->stream) != cudaSuccess) r = Q4_ERR_CUDA;
-    cudaGraph_t g = nullptr;
-    if (cudaStreamEndCapture(p->stream, &g) != cudaSuccess && r == Q4_OK) r = Q4_ERR_CUDA;
-    if (r == Q4_OK && cudaGraphInstantiate(&place->exec, g, 0) != cudaSuccess) r = Q4_ERR_CUDA;
-    if (g) cudaGraphDestroy(g);
+  cudaGraph_t g = nullptr;
+  int r;
+  if (key.loop) {
+    cudaGraphNode_t node;
+    r = cudaGraphCreate(&g, 0) == cudaSuccess ? add_search_loop(p, place->key, g, nullptr, 0, &node) : Q4_ERR_CUDA;
+  } else {
+    r = cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeRelaxed) == cudaSuccess ? Q4_OK : Q4_ERR_CUDA;
+    if (r == Q4_OK) {
+      r = capture_steps(p, place->key, nullptr);
+      if (cudaStreamEndCapture(p->stream, &g) != cudaSuccess && r == Q4_OK) r = Q4_ERR_CUDA;
+    }
   }
+  if (r == Q4_OK && cudaGraphInstantiate(&place->exec, g, 0) != cudaSuccess) r = Q4_ERR_CUDA;
+  if (g) cudaGraphDestroy(g);
   place->launches = g_launches - l0;
   place->quant_calls = g_quant_calls - q0;
   g_launches = l0;
@@ -1516,39 +1565,77 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
   const bool lent = st.aux_stream[0] && st.aux_stream[1] && st.aux_event[0] && st.aux_event[1] && st.aux_event[2];
   for (int i = 0; i < 2; ++i) key.state.aux_stream[i] = p && lent ? p->side[i] : nullptr;
   for (int i = 0; i < 3; ++i) key.state.aux_event[i] = p && lent ? p->side_event[i] : nullptr;
-  // step by step: in a stream that is being captured, while launches are timed or waits are made to run out (a graph
-  // would keep that), and in a short search
+  // An alignment-length synchronous search ends its steps when no utterance has labels left to propose; the iterations
+  // that are left then are carried out together.
+  key.loop = p && !key.tsd && !key.exact && search_tail_supported(model->V, model->D) &&
+             search_uses_tensor_cores(*model, *state, B, W, workspace_bytes);
+  // step by step: while launches are timed or waits are made to run out (a graph would keep that), in a short search, and
+  // without a loop in a stream that is being captured
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (p && (n_iters < PLAN_MIN_ITERS || timing_active() || test_wait_expiry_active() || cudaStreamIsCapturing(s, &cap) != cudaSuccess ||
-            cap != cudaStreamCaptureStatusNone))
+  if (p && (n_iters < PLAN_MIN_ITERS || timing_active() || test_wait_expiry_active() ||
+            cudaStreamIsCapturing(s, &cap) != cudaSuccess || (cap != cudaStreamCaptureStatusNone && !key.loop)))
     p = nullptr;
+  bool tail = false;
   for (int it = 0; it < n_iters;) {
     // the first two frames' steps always: the first step's networks start from the reset state, and the kernels set their
     // attributes at their first launch
     if (p && it == 2 * S1) {
       const BesideCaptures guard;          // the first replay of a graph may allocate, too
-      SearchGraph* g = plan_graph(p, key);
-      const int first = it;
-      if (g) {
-        Q4_TRY(launch_search_begin(static_cast<SearchCall*>(workspace), e, T, u_max, it - PLAN_ITERS, s));
-        for (; it + PLAN_ITERS <= n_iters; it += PLAN_ITERS) {
+      SearchCall* call = static_cast<SearchCall*>(workspace);
+      int32_t* frozen = key.loop ? search_frozen(workspace) : nullptr;
+      const int groups = (n_iters - it) / PLAN_ITERS;
+      const int turns = key.loop ? (n_iters - it + PLAN_ITERS - 1) / PLAN_ITERS : groups;
+      if (cap != cudaStreamCaptureStatusNone) {   // the loop becomes a node of the caller's graph
+        Q4_TRY(launch_search_begin(call, e, T, u_max, it - PLAN_ITERS, frozen, B, s));
+        const int64_t l0 = g_launches, q0 = g_quant_calls;
+        cudaGraph_t g;
+        const cudaGraphNode_t* deps;
+        size_t n_deps;
+        cudaGraphNode_t node;
+        Q4_TRY(cudaStreamGetCaptureInfo_v2(s, &cap, nullptr, &g, &deps, &n_deps));
+        Q4_CHECK(add_search_loop(p, key, g, deps, n_deps, &node));
+        Q4_TRY(cudaStreamUpdateCaptureDependencies(s, &node, 1, cudaStreamSetCaptureDependencies));
+        g_launches += (g_launches - l0) * (turns - 1);
+        g_quant_calls += (g_quant_calls - q0) * (turns - 1);
+        tail = true;
+      } else if (SearchGraph* g = plan_graph(p, key)) {
+        Q4_TRY(launch_search_begin(call, e, T, u_max, it - PLAN_ITERS, frozen, B, s));
+        for (int i = 0; i < (key.loop ? 1 : groups); ++i) {
           const cudaError_t le = cudaGraphLaunch(g->exec, s);
           if (le != cudaSuccess) {
             cudaEventRecord(g->done, s);   // of the replays before it
             return Q4_ERR_CUDA;
           }
-          g_launches += g->launches;
-          g_quant_calls += g->quant_calls;
-          ++p->replays;
         }
+        g_launches += g->launches * turns;
+        g_quant_calls += g->quant_calls * turns;
+        p->replays += groups;
         Q4_TRY(cudaEventRecord(g->done, s));
+        tail = key.loop != 0;
+        if (!tail) it += groups * PLAN_ITERS;
       }
+      if (tail) break;
       p = nullptr;                         // the rest step by step
-      if (it != first) continue;
+      if (it >= n_iters) break;
     }
     Q4_CHECK(beam_step(model, state, e, B, T, W, it, u_max, lambda_t, lambda_s, rho, step_mode(key, it), workspace,
-                       workspace_bytes, stream, nullptr));
+                       workspace_bytes, stream, nullptr, nullptr, nullptr));
     ++it;
+  }
+  if (tail) {
+    const q4_model& m = *model;
+    TailArgs a;
+    memset(&a, 0, sizeof(a));
+    a.call = static_cast<SearchCall*>(workspace);
+    a.frozen = search_frozen(workspace);
+    a.st = *state;
+    a.B = B;
+    a.W = W;
+    a.V = m.V;
+    a.z_act = m.z_act;
+    a.sc_out = m.joint_out.w.scale;
+    a.b_out = m.joint_out.bias;
+    Q4_TRY(launch_search_tail(a, T, static_cast<const int8_t*>(m.prepared) + plan_prepared(m).lin[5], s));
   }
   return Q4_OK;
 }

@@ -222,6 +222,18 @@ __device__ __forceinline__ void rank_list(const uint64_t* list, int ln, int W, i
 // entries of the short list; smaller vocabularies have as many proposals near the bound as large ones
 __host__ __device__ constexpr int sel_list_cap(int V) { return 16 * ((V + 31) / 32) > 512 ? 16 * ((V + 31) / 32) : 512; }
 
+// End of the last step of a graph's loop, by one thread of each utterance after all that it does: the last one
+// advances the call and asks for another turn.  (As a kernel of its own 2 us a turn.)  Every utterance is frozen by
+// iteration T + u_max, since no hypothesis lives beyond it, so the second condition never ends a loop; it bounds it.
+__device__ __forceinline__ void loop_step_end(const BeamSelArgs& a, int iter, int last) {
+  __threadfence();
+  if (atomicAdd(&a.call->arrived, 1) != a.B - 1) return;
+  __threadfence();
+  a.call->arrived = 0;
+  a.call->iter += a.loop_iters;   // (everyone has read it)
+  cudaGraphSetConditional(a.loop, ld_coherent(&a.call->n_frozen) < a.B && iter + 1 < last ? 1u : 0u);
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant__ BeamSelArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -284,6 +296,20 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
   }
   if (lane < 16) s_gmax[warp][lane] = NEG;
   const bool any_labels = __syncthreads_or(my_row >= 0 && my_u < u_max) != 0;
+  if (a.frozen && !any_labels) {   // this utterance's remaining iterations are carried out together (q4_tail.cu)
+    pdl_trigger();
+    if (warp == 0 && a.frozen[b] < 0) {
+      int left = lane < W && s_row[lane] >= 0 ? T - s_t[lane] : 0;
+      left = max(__reduce_max_sync(0xffffffffu, left), 0);
+      if (lane == 0) {
+        a.frozen[b] = iter;
+        a.frozen[a.B + b] = left;
+        atomicAdd(&a.call->n_frozen, 1);
+      }
+    }
+    if (a.loop_iters && tid == 0) loop_step_end(a, iter, T + u_max);
+    return;
+  }
 
   // ---- no slot of this utterance may emit a label (all at their label budget, or empty): the only
   // proposals are the blanks of the live slots, at most W of them, no two of which can describe the
@@ -517,6 +543,7 @@ __global__ void __launch_bounds__(SEL_NT, 1) k_beam_select(const __grid_constant
         st.bp_score[hist] = 0.0f;
       }
     }
+    if (a.loop_iters && lane == 0) loop_step_end(a, iter, T + u_max);
   }
 }
 
@@ -936,15 +963,21 @@ __global__ void k_beam_init(q4_beam_state st, int B, int W) {
   }
 }
 
-__global__ void k_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter) {
+__global__ void k_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter, int32_t* frozen, int B) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (frozen && i < B) frozen[i] = -1;
+  if (i != 0) return;
   call->e = e;
   call->T = T;
   call->u_max = u_max;
   call->iter = iter;
+  call->n_frozen = 0;
+  call->arrived = 0;
 }
 __global__ void k_search_advance(SearchCall* call, int iters) { call->iter += iters; }
-cudaError_t launch_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter, cudaStream_t s) {
-  k_search_begin<<<1, 1, 0, s>>>(call, e, T, u_max, iter);
+cudaError_t launch_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter, int32_t* frozen, int B,
+                                cudaStream_t s) {
+  k_search_begin<<<frozen ? (B + 127) / 128 : 1, 128, 0, s>>>(call, e, T, u_max, iter, frozen, B);
   ++g_launches;
   return cudaGetLastError();
 }
@@ -953,7 +986,6 @@ cudaError_t launch_search_advance(SearchCall* call, int iters, cudaStream_t s) {
   ++g_launches;
   return cudaGetLastError();
 }
-
 cudaError_t launch_beam_init(const q4_beam_state& st, int B, int W, int n_iters, cudaStream_t s) {
   (void)n_iters;
   k_beam_init<<<(B * W + 255) / 256, 256, 0, s>>>(st, B, W);

@@ -12,7 +12,7 @@ cudaError_t launch_logsoftmax(const float* in, float* out, int rows, int V, long
 cudaError_t launch_joint_z(const float* e, const int32_t* frame_idx, const int32_t* t_arr, int B,
                            int W, const float* p, const int32_t* p_idx, int N, int D,
                            const q4_act& za, uint8_t* zq, int8_t* z8, int32_t* live_out,
-                           cudaStream_t s, bool dependent = false, const struct SearchCall* call = nullptr);
+                           cudaStream_t s, bool dependent = false, const struct SearchCall* call = nullptr, int all_frozen = 0);
 cudaError_t launch_quantize(const void* x, bool fp16, long long rows, int k, int k_pad,
                             const q4_act& a, int mode, int n_groups, const float* scale_vec,
                             uint8_t* out, float* group_scale_out, cudaStream_t s);
@@ -24,11 +24,18 @@ struct SearchCall {
   const float* e;           // projected encoder frames
   int32_t T, u_max;
   int32_t iter;             // added to the launch's iteration number
+  int32_t n_frozen;         // utterances whose search has no labels left to propose (see q4_tail.cu)
+  int32_t arrived;          // utterances that have ended the last step of a loop's turn
 };
-cudaError_t launch_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter, cudaStream_t s);
+// frozen (nullable): [2 B] per utterance the iteration it was frozen at (set to -1 here) and the frames it had left
+cudaError_t launch_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter, int32_t* frozen, int B,
+                                cudaStream_t s);
 cudaError_t launch_search_advance(SearchCall* call, int iters, cudaStream_t s);
 struct BeamSelArgs {
-  const SearchCall* call;
+  SearchCall* call;
+  int32_t* frozen;          // [2 B], see launch_search_begin; null: every iteration is carried out here
+  cudaGraphConditionalHandle loop;   // last step of a graph's loop (loop_iters > 0 steps): decides on another turn
+  int32_t loop_iters;
   const float* logits;      // [B*W, V] joint logits (bias included), rows of empty slots ignored
   const float* src_lp;      // [R, V]
   const float* tgt_lp;      // [R, V]
@@ -42,6 +49,19 @@ struct BeamSelArgs {
 cudaError_t launch_beam_select(const BeamSelArgs& a, cudaStream_t s, bool dependent = false);
 cudaError_t launch_tsd_select(const BeamSelArgs& a, cudaStream_t s, bool dependent = false);
 cudaError_t launch_beam_init(const q4_beam_state& st, int B, int W, int n_iters, cudaStream_t s);
+// The iterations of a search that are left once no utterance proposes labels (q4_tail.cu).
+struct TailArgs {
+  const SearchCall* call;
+  const int32_t* frozen;    // [2 B]
+  q4_beam_state st;
+  int32_t B, W, V;
+  q4_act z_act;
+  const float* sc_out;      // [V] row scales of the joint network's output layer
+  const float* b_out;       // [V] or null
+};
+bool search_tail_supported(int V, int D);
+// wo8: int8 rows [V, 256] of the output layer; T: frames of the search
+cudaError_t launch_search_tail(const TailArgs& a, int T, const int8_t* wo8, cudaStream_t s);
 cudaError_t launch_traceback(const q4_beam_state& st, int B, int W, int n_iters, int u_max,
                              int32_t* tokens, int32_t* lens, float* scores, cudaStream_t s);
 
@@ -110,6 +130,8 @@ struct LmHeadArgs {
   float* lp;                  // [*, V] log-probabilities, row dst_row[n]
   const int32_t* dst_row;     // nullptr = n, negative = skip
   const int32_t* n_active;
+  const int32_t* n_idle;      // optional: nothing to do once *n_idle >= all_idle (read after the kernel's wait)
+  int32_t all_idle;
   int32_t* status;
   int32_t tile_rows, n_stages;   // set by the launcher
 };
@@ -143,7 +165,8 @@ cudaError_t launch_mma_gemm(const int8_t* x8, long long x_pitch, int M, const in
                             const int32_t* out_idx, const float* w_scale, const float* bias,
                             float x_scale, const q4_act* out_act, int32_t* status,
                             const int32_t* n_active, cudaStream_t s, bool dependent = false,
-                            const float* mul_e = nullptr, const int32_t* mul_idx = nullptr);
+                            const float* mul_e = nullptr, const int32_t* mul_idx = nullptr,
+                            const int32_t* n_idle = nullptr, int all_idle = 0);
 void test_wait_expiry_set(int skip_producer, uint32_t wait_limit);
 bool test_wait_expiry_active();
 cudaError_t launch_mma_gemm_i32(const int8_t* x8, int M, const int8_t* w8, int J, int K, int planes, int32_t* out,

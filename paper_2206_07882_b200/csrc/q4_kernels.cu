@@ -459,10 +459,14 @@ cudaError_t launch_logsoftmax(const float* in, float* out, int rows, int V, long
 __global__ void __launch_bounds__(256) k_joint_z(const float* e, const int32_t* frame_idx,
                                                  const int32_t* t_arr, int B, int W, const float* p,
                                                  const int32_t* p_idx, int N, int D, q4_act za,
-                                                 uint8_t* zq, int8_t* z8, int32_t* live_out, const SearchCall* call) {
+                                                 uint8_t* zq, int8_t* z8, int32_t* live_out, const SearchCall* call,
+                                                 int all_frozen) {
   pdl_trigger();
   pdl_wait();
-  if (call) e = call->e;
+  if (call) {
+    if (all_frozen && call->n_frozen >= all_frozen) return;   // nobody will read the codes
+    e = call->e;
+  }
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int half = D >> 1;
   if (i >= (long long)N * half) return;
@@ -491,12 +495,12 @@ __global__ void __launch_bounds__(256) k_joint_z(const float* e, const int32_t* 
 cudaError_t launch_joint_z(const float* e, const int32_t* frame_idx, const int32_t* t_arr, int B,
                            int W, const float* p, const int32_t* p_idx, int N, int D,
                            const q4_act& za, uint8_t* zq, int8_t* z8, int32_t* live_out,
-                           cudaStream_t s, bool dependent, const SearchCall* call) {
+                           cudaStream_t s, bool dependent, const SearchCall* call, int all_frozen) {
   if (N <= 0) return cudaSuccess;
   const long long total = (long long)N * (D / 2);
   timing_begin(s);
   cudaError_t le = launch_ex(k_joint_z, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, s, dependent, 1, e,
-                             frame_idx, t_arr, B, W, p, p_idx, N, D, za, zq, z8, live_out, call);
+                             frame_idx, t_arr, B, W, p, p_idx, N, D, za, zq, z8, live_out, call, all_frozen);
   timing_end(s);
   ++g_launches;
   return le != cudaSuccess ? le : cudaGetLastError();

@@ -297,6 +297,8 @@ struct MmaGemmArgs {
   q4_act out_act;
   int32_t* status;
   const int32_t* n_active;
+  const int32_t* n_idle;    // optional: nothing to do once *n_idle >= all_idle
+  int32_t all_idle;
   const float* mul_e;       // EPI_JOINTZ: the other factor, row mul_idx[m] of [*, J] fp32
   const int32_t* mul_idx;
   uint32_t wait_limit;      // polls before a wait gives up
@@ -347,7 +349,9 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
   tc_fence_after();
   const uint32_t tmem = tmem_base_s;
   pdl_wait();   // everything above overlaps the tail of the previous kernel of the stream
-  if (warp == 4) {
+  if (a.n_idle && ld_coherent(a.n_idle) >= a.all_idle) {   // the same for every thread of the grid
+    pdl_trigger();
+  } else if (warp == 4) {
     bool ok = true;
     int s = 0;
     uint32_t ph = 1;
@@ -703,7 +707,7 @@ cudaError_t launch_mma_gemm(const int8_t* x8, long long x_pitch, int M, const in
                             const int32_t* out_idx, const float* w_scale, const float* bias,
                             float x_scale, const q4_act* out_act, int32_t* status,
                             const int32_t* n_active, cudaStream_t s, bool dependent, const float* mul_e,
-                            const int32_t* mul_idx) {
+                            const int32_t* mul_idx, const int32_t* n_idle, int all_idle) {
   if (M <= 0 || J <= 0) return cudaSuccess;
   if (epi == EPI_JOINTZ && (!mul_e || !mul_idx || J % 32 != 0)) return cudaErrorInvalidValue;
   const int bn = gemm_tile_width(M, J, 1, 32);
@@ -727,6 +731,8 @@ cudaError_t launch_mma_gemm(const int8_t* x8, long long x_pitch, int M, const in
   a.n_active = n_active;
   a.mul_e = mul_e;
   a.mul_idx = mul_idx;
+  a.n_idle = n_idle;
+  a.all_idle = all_idle;
   a.wait_limit = g_wait_limit;
   a.skip_producer = g_skip_producer;
   timing_begin(s);
@@ -853,9 +859,12 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
   const uint32_t tmem = tmem_base_s;
   cl_barrier();   // every CTA of the cluster is running before anyone stores into a peer's shared memory
   pdl_wait();   // everything above (this barrier included) overlaps the tail of the previous kernel of the stream
+  const bool idle = a.n_idle && ld_coherent(a.n_idle) >= a.all_idle;   // the same for every thread of the grid
   bool codes_due = false;   // a wait has run out: the peers' codes may still be on their way here
 
-  if (warp == HEAD_EPI_WARPS) {
+  if (idle) {
+    pdl_trigger();
+  } else if (warp == HEAD_EPI_WARPS) {
     // ---- TMA producer: bottleneck operands through the ring, then my block of output-layer weights into
     // the ring's memory, which the bottleneck's MMAs have finished reading by then
     bool ok = true;
@@ -1127,7 +1136,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
     if (!ok && lane == 0) flag_timeout(a.status);
   }
   __syncwarp();
-  if (warp >= HEAD_EPI_WARPS) {   // the producer and issuer warps join the cluster barrier too
+  if (!idle && warp >= HEAD_EPI_WARPS) {   // the producer and issuer warps join the cluster barrier too
     pdl_trigger();
     cl_barrier();
     if (NB == 32) cl_barrier();

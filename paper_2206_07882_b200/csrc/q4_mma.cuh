@@ -90,6 +90,9 @@ __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
 }
 
+// int8 matrix [rows, k] with row pitch `pitch` bytes; box = 128 bytes of K x box_rows rows, 128-byte swizzle (q4_mma.cu).
+bool make_tmap_i8(CUtensorMap* m, const void* base, uint64_t k, uint64_t rows, uint64_t pitch, uint32_t box_rows);
+
 // ---- tensor memory ------------------------------------------------------------------
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst_smem)),

@@ -894,3 +894,42 @@ def test_grouped_search_equals_single_state_search(Bd):
         t3, l3, s3 = g()
         torch.cuda.synchronize()
         assert torch.equal(t1, t3) and torch.equal(s1, s3)
+
+
+@pytest.mark.parametrize("V,W,B,T,U,blank,bits", [
+    (46, 16, 3, 101, 7, 2.0, 4),      # vocabulary summed by a warp per row; utterances that spend their labels at different times
+    (256, 5, 2, 130, 30, 0.0, 8),
+    (257, 16, 2, 97, 20, 3.0, 4),     # blocks of 64 labels
+    (1024, 16, 5, 110, 12, 4.0, 4),   # blocks of 128
+    (1000, 1, 1, 300, 0, 0.0, 4),     # no label budget: everything is left to the end; a last block with few labels
+    (1030, 8, 2, 100, 90, -9.0, 8),   # blocks of 256; hardly any blank before the labels are spent
+    (300, 4, 2, 100, 60, 30.0, 4),    # blanks only: the beams end before any label budget is spent
+])
+def test_label_free_end_of_a_search_equals_its_steps(Bd, V, W, B, T, U, blank, bits):
+    # the iterations after the last label are carried out together: every beam of every iteration, the finished list and
+    # the state as the steps leave them, in a search of its own and in one captured by the caller
+    dw = synth.decoder(seed=91, V=V, E=32, Hp=128, D=256, Hs=128, Ht=128, tgt_layers=2, U_max=U, W=W, all_bits=bits)
+    dw.joint.out.bias[0] += np.float32(blank)
+    e = torch.from_numpy(synth.Stream(V + T).normal("e", (T, B, 256)).astype(np.float32)).cuda()
+    n = T + U
+    b = Bd.Decoder(dw)
+    b.alloc_state(B, W, n)
+    b.q4_beam_init()
+    for it in range(n):
+        b.dr_fusion_beam_step(e, T, it, U)
+    want = b.q4_traceback(n, U)
+    a = Bd.Decoder(dw)
+    captured = Bd.GraphedStep(lambda: a.decode(e, U))
+    state = ("bp_parent", "bp_token", "bp_score", "fin_n", "fin_score", "fin_iter", "fin_slot", "score", "t", "u", "hash",
+             "prev_hash", "last_tok", "row", "adv_src", "adv_dst", "adv_tok", "pend_n")
+    for run in (lambda: a.decode(e, U), captured, captured):
+        if a.state is not None:
+            for k in ("bp_parent", "bp_token", "bp_score"):
+                a.tensors[k].fill_(-7)
+        got = run()
+        assert a.tensors["status"].item() == 0
+        for x, y in zip(got, want):
+            assert torch.equal(x, y)
+        for k in state:
+            assert torch.equal(a.tensors[k], b.tensors[k]), k
+    assert a.search_plan_info()["built"] == 1
