@@ -789,7 +789,7 @@ cudaError_t launch_mma_gemm_i32(const int8_t* x8, int M, const int8_t* w8, int J
 constexpr int HEAD_D = 256;
 constexpr int HEAD_CTAS = 8;                 // = the portable cluster size
 constexpr int HEAD_BN1 = HEAD_D / HEAD_CTAS; // bottleneck columns per CTA
-constexpr int HEAD_MAX_STAGES = 8;
+constexpr int HEAD_MAX_STAGES = 16;
 constexpr int HEAD_RING = 80 * 1024;         // bytes of the operand ring; the output layer's weights, the outgoing codes, then
                                              // the log-probabilities on their way out use the same memory
 constexpr int HEAD_EPI_WARPS = 16;           // four warps per TMEM lane quarter
@@ -807,6 +807,13 @@ __device__ __forceinline__ void cl_store_f32(const float* local, uint32_t rank, 
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cl_map(smem_u32(local), rank)), "f"(v) : "memory");
 }
 
+// e^x as 2^(x log2 e) on the base-2 unit, results below the normal range as 0 (they are added to a sum of at least 1):
+// without the scaling that keeps them 4 instructions instead of 8
+__device__ __forceinline__ float exp_fast(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__fmul_rn(x, 1.4426950408889634f)));
+  return y;
+}
 template <int NB>
 __global__ void __cluster_dims__(HEAD_CTAS, 1, 1) __launch_bounds__(HEAD_THREADS, 1)
 k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ CUtensorMap tma_wb,
@@ -1009,9 +1016,19 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
     }
     // the block's maximum of every row, over the four column shares
     float (*red_m)[BM] = reinterpret_cast<float (*)[BM]>(ring), (*red_s)[BM] = red_m + 4;   // the weights have been read
+    // (entries beyond the vocabulary count as -inf; selected, not branched over: a branch around each exponential exposes its
+    // latency, 2950 clocks for 32 of them against 450)
+    if (busy) {
+      const int left = a.V - col0;
 #pragma unroll
-    for (int i = 0; i < CPT; ++i)
-      if (busy && col0 + i < a.V) my_m = fmaxf(my_m, v[i]);
+      for (int i = 0; i < CPT; ++i) {
+        if (i >= left) v[i] = -INFINITY;
+        my_m = fmaxf(my_m, v[i]);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < CPT; ++i) v[i] = 0.0f;
+    }
     if (NB == 32) {
       // Vocabularies of at most 256: the sums in the order of k_logsoftmax (one thread per entry, pairwise over
       // lanes, then over warps), so that the kernels for few rows and the tensor-core path give the same bits.
@@ -1028,7 +1045,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
 #pragma unroll
       for (int r = 0; r < HEAD_CTAS; ++r) m = fmaxf(m, part_m[r][rt]);
 #pragma unroll
-      for (int i = 0; i < CPT; ++i) ex[rt][CPT * cs + i] = busy && col0 + i < a.V ? expf(v[i] - m) : 0.0f;
+      for (int i = 0; i < CPT; ++i) ex[rt][CPT * cs + i] = busy ? expf(v[i] - m) : 0.0f;   // 0 beyond the vocabulary
       asm volatile("bar.sync 1, %0;" ::"n"(32 * HEAD_EPI_WARPS) : "memory");
       if (cs == 0) {
         float t[16];
@@ -1054,9 +1071,11 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
       // exponentials by the hardware base-2 unit: relative error near 1e-6, far inside what the
       // log-sum-exp of a thousand terms needs
       float my_s = 0.0f;
+      if (busy) {
+        const float top = my_m > -INFINITY ? my_m : 0.0f;
 #pragma unroll
-      for (int i = 0; i < CPT; ++i)
-        if (busy && col0 + i < a.V) my_s += __expf(v[i] - my_m);
+        for (int i = 0; i < CPT; ++i) my_s += exp_fast(v[i] - top);
+      }
       red_m[cs][rt] = my_m;
       red_s[cs][rt] = my_s;
       asm volatile("bar.sync 1, %0;" ::"n"(32 * HEAD_EPI_WARPS) : "memory");

@@ -217,11 +217,13 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_tail_blank(const __grid_const
         } else {
           float my_m = -INFINITY, my_s = 0.0f;
 #pragma unroll
-          for (int j = 0; j < CPT; ++j)
-            if (col0 + j < V) my_m = fmaxf(my_m, v[j]);
+          for (int j = 0; j < CPT; ++j) {
+            if (col0 + j >= V) v[j] = -INFINITY;
+            my_m = fmaxf(my_m, v[j]);
+          }
+          const float top = my_m > -INFINITY ? my_m : 0.0f;
 #pragma unroll
-          for (int j = 0; j < CPT; ++j)
-            if (col0 + j < V) my_s += __expf(v[j] - my_m);
+          for (int j = 0; j < CPT; ++j) my_s += __expf(v[j] - top);
           *reinterpret_cast<float2*>(red + ((i * 4 + cs) * TL_BM + rt) * 2) = make_float2(my_m, my_s);
           if (i == 0 && cs == 0) s_blank[rt] = v[0];
         }
