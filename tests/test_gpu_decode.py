@@ -933,3 +933,27 @@ def test_label_free_end_of_a_search_equals_its_steps(Bd, V, W, B, T, U, blank, b
         for k in state:
             assert torch.equal(a.tensors[k], b.tensors[k]), k
     assert a.search_plan_info()["built"] == 1
+
+
+@pytest.mark.parametrize("V,normalized", [(2, 1), (46, 1), (64, 1), (65, 1), (256, 1), (257, 1), (300, 0), (1023, 1), (1024, 0),
+                                          (1024, 1), (1025, 1)])
+@pytest.mark.parametrize("S", [None, 1])
+def test_selection_forms_agree_with_the_exact_search(Bd, V, normalized, S):
+    # every form of the selection kernels (labels per lane, rows of whole 16 bytes, logits or log-probabilities, more labels
+    # than registers hold) against the exact threshold search, with few and many slots
+    D = 256 if normalized else 128
+    dw = synth.decoder(seed=93, V=V, E=32, Hp=128, D=D, Hs=128, Ht=128, tgt_layers=1, U_max=6, W=16)
+    for B, W in ((2, 16), (3, 5), (9, 15)):
+        e = torch.from_numpy(synth.Stream(V + W).normal("e", (10, B, D)).astype(np.float32)).cuda()
+        runs = []
+        for exact in (False, True):
+            dd = Bd.Decoder(dw)
+            prev = Bd.beam_select_exact_set(exact)
+            try:
+                out = dd.decode(e, 6, W) if S is None else dd.decode_time_synchronous(e, S, 6, W)
+                torch.cuda.synchronize()
+            finally:
+                Bd.beam_select_exact_set(prev)
+            runs.append(list(out) + [dd.tensors[k] for k in ("bp_parent", "bp_token", "bp_score", "fin_n", "fin_score")])
+        for x, y in zip(*runs):
+            assert torch.equal(x, y)
