@@ -343,7 +343,8 @@ int q4_beam_init(q4_beam_state* state, int32_t B, int32_t W, int32_t n_iters, q4
  * bp_token = -1 - (call number within the frame of that proposal).
  * workspace: q4_workspace_bytes(Q4_WS_BEAM, {B, W, V, D}), or, to enable the tensor-core path
  * (needs model->prepared and LSTM widths that are multiples of 128),
- * q4_workspace_bytes(Q4_WS_BEAM, {B, W, V, D, E_pad, Hp, Hs, Ht}).  A bounded device wait that expires sets state->status to Q4_ERR_TIMEOUT.
+ * q4_workspace_bytes(Q4_WS_BEAM, {B, W, V, D, E_pad, Hp, Hs, Ht}).  With the state rows per utterance as a ninth entry
+ * (2 W where rows_per_utt is 0) q4_beam_search has room for its fastest kernels (up to 384 rows B W).  A bounded device wait that expires sets state->status to Q4_ERR_TIMEOUT.
  */
 int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float* e, int32_t B,
                         int32_t T, int32_t W, int32_t iter, int32_t u_max, float lambda_t,
@@ -394,7 +395,7 @@ int q4_feature_prologue(const float* mel, int32_t B, int32_t T100, int32_t M, vo
 
 #define Q4_WS_LSTM_LAYER 1 /* dims = {T, B, dirs, H} or {T, B, dirs, H, kx_pad} */
 #define Q4_WS_JOINT 2      /* dims = {N, D} or {N, D, Hp_pad} (tensor-core path) */
-#define Q4_WS_BEAM 3       /* dims = {B, W, V, D} or {B, W, V, D, E_pad, Hp, Hs, Ht} */
+#define Q4_WS_BEAM 3       /* dims = {B, W, V, D}, {B, W, V, D, E_pad, Hp, Hs, Ht} or the latter and the state rows per utterance */
 #define Q4_WS_LSTM_STEP 4  /* dims = {N, kx_pad, H} (tensor-core path of qlstm_step) */
 #define Q4_WS_LINEAR 5     /* dims = {M, k_pad} (tensor-core path of q4_linear_forward) */
 size_t q4_workspace_bytes(int32_t call_id, const int32_t* dims, int32_t ndims);

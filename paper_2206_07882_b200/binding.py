@@ -691,7 +691,7 @@ class Decoder:
         self.B, self.W, self.n_iters = B, W, n_iters
         dims = [B, W, self.V, self.D]
         if self.tensor_cores:
-            dims += [self.pred_lstm.w_ih.k_pad, Hp, Hs, Ht]
+            dims += [self.pred_lstm.w_ih.k_pad, Hp, Hs, Ht, RW]
         self.ws = torch.empty(workspace_bytes(WS_BEAM, dims), dtype=torch.uint8, device=dev)
 
     def q4_beam_init(self):

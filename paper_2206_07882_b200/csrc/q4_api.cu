@@ -46,6 +46,13 @@ int check_mat(const q4_mat* m, int rows, int k_pad_expected) {
   return Q4_OK;
 }
 
+// Hypothesis rows of a search that keeps the recurrent sums per state row (see search_keeps_sums).  They take 16 H bytes a
+// row and layer through memory instead of a gather and products in the step's longest chain, and the products
+// that make them take the SMs from the output heads and the selection when there are many: 160 frames, labels in
+// half of the iterations, ms with / without: 64 rows 4.06 / 5.05, 256 rows 4.31 / 4.87, 384 rows 8.38 / 8.89, 512 rows 9.94 / 9.86,
+// 1024 rows 12.0 / 9.6.
+constexpr int SUMS_MAX_ROWS = 384;
+
 // Rows that the tensor-core paths can address: a grid has 65535 row tiles, and the gather counts 32-code pieces in 32
 // bits (rows of k codes).  More go to the general kernels, which walk any number.
 inline bool mma_rows(long long rows, int k) {
@@ -212,6 +219,10 @@ size_t q4_workspace_bytes(int32_t call_id, const int32_t* dims, int32_t ndims) {
       (void)Hmax;
       n += align_up(Np * Hp) + align_up(Np * Hs) + 2 * align_up(Np * Ht); // new cell outputs, int8
       n += 3 * align_up(Np * D);                                         // bottleneck codes, z codes
+      if (ndims >= 9 && dims[8] > 0 && N <= SUMS_MAX_ROWS) {             // recurrent sums of every state row
+        const size_t R = (size_t)dims[0] * dims[8];
+        n += align_up(R * 4 * Hp * sizeof(float)) + align_up(R * 4 * Hs * sizeof(float)) + 2 * align_up(R * 4 * Ht * sizeof(float));
+      }
     }
     return n;
   }
@@ -731,8 +742,16 @@ struct PrepLstm {
 struct PrepPlan {
   PrepLstm lstm[4];   // prediction, source LM, target LM layer 1, target LM layer 2
   size_t lin[6];      // pred_proj, src.bott, src.out, tgt.bott, tgt.out, joint_out
+  size_t table[3];    // first layers: de-quantized input sums plus bias of every label (fp32 [V, 4H])
+  size_t emb8;        // int8 embedding rows, while the tables are made; 0: no tables
   size_t total;
 };
+// Tables of the first layers' input halves: 16 H bytes a label and network.
+constexpr int TABLE_MAX_V = 4096;
+bool search_tables(const q4_model& m) {
+  return m.V > 0 && m.V <= TABLE_MAX_V && m.src.n_layers == 1 && m.pred_lstm.w_hh.k_pad % 128 == 0 &&
+         m.src.lstm[0].w_hh.k_pad % 128 == 0 && m.tgt.lstm[0].w_hh.k_pad % 128 == 0;
+}
 const q4_lstm* model_lstm(const q4_model& m, int i) {
   switch (i) {
     case 0: return &m.pred_lstm;
@@ -775,6 +794,17 @@ PrepPlan plan_prepared(const q4_model& m) {
     p.lin[i] = o;
     o += align_up((size_t)L->w.rows * L->w.k_pad);
   }
+  if (search_tables(m)) {
+    size_t ep = 0;
+    for (int i = 0; i < 3; ++i) {
+      const q4_lstm* L = model_lstm(m, i);
+      p.table[i] = o;
+      o += align_up((size_t)m.V * L->w_ih.rows * sizeof(float));
+      if ((size_t)L->w_ih.k_pad > ep) ep = L->w_ih.k_pad;
+    }
+    p.emb8 = o;
+    o += align_up((size_t)m.V * ep);
+  }
   p.total = o;
   return p;
 }
@@ -813,6 +843,23 @@ int q4_prepare_model(q4_model* model, void* buffer, size_t bytes, q4_stream stre
     const q4_linear* L = model_linear(*model, i);
     Q4_CHECK(check_mat(&L->w, 0, 0));
     Q4_TRY(launch_prepare_w(L->w, 0, reinterpret_cast<int8_t*>(b + p.lin[i]), L->w.k_pad, 0, s));
+  }
+  for (int i = 0; i < 3 && p.emb8; ++i) {
+    const q4_lstm* L = model_lstm(*model, i);
+    const q4_act& act = i == 0 ? model->pred_emb_act : i == 1 ? model->src.emb_act : model->tgt.emb_act;
+    const void* emb = i == 0 ? model->pred_emb_q : i == 1 ? model->src.emb_q : model->tgt.emb_q;
+    if (!emb) return Q4_ERR_NULL;
+    Q4_CHECK(check_act(&act));
+    const int Ep = L->w_ih.k_pad, G = L->w_ih.rows;
+    int8_t* e8 = reinterpret_cast<int8_t*>(b + p.emb8);
+    UnpackJobs uj;
+    memset(&uj, 0, sizeof(uj));
+    uj.n_rows = uj.n_rows_pad = model->V;
+    add_unpack_job(uj, emb, row_bytes(Ep, act.bits), nullptr, act, Ep, e8);
+    Q4_TRY(launch_unpack_multi(uj, s, false));
+    Q4_TRY(launch_mma_gemm(e8, Ep, model->V, reinterpret_cast<const int8_t*>(b + p.lstm[i].xw), Ep, G, Ep, EPI_F32,
+                           b + p.table[i], G, nullptr, reinterpret_cast<const float*>(b + p.lstm[i].sc_ih),
+                           reinterpret_cast<const float*>(b + p.lstm[i].bias), 1.0f, nullptr, nullptr, nullptr, s, false));
   }
   model->prepared = buffer;
   return Q4_OK;
@@ -929,16 +976,35 @@ static bool search_uses_tensor_cores(const q4_model& m, const q4_beam_state& st,
 // In the tensor-core path the first codes block of the workspace is free: there a search keeps when its utterances were frozen.
 static int32_t* search_frozen(void* workspace) { return reinterpret_cast<int32_t*>(static_cast<uint8_t*>(workspace) + 256); }
 
-// One step; `call` non-null: e, T and u_max come from there, and its iteration number is added to `iter`.  `frozen`: an
-// utterance without labels to propose is left to launch_search_tail; `loop`: this is the last step of a graph's loop.
+// Whether a whole search takes the kernels that look the first layers' input halves up and keep the sums of the recurrent
+// halves per state row: tables with the prepared weights and room for the sums.
+static bool search_keeps_sums(const q4_model& m, const q4_beam_state& st, int B, int W, size_t workspace_bytes) {
+  const int RW = st.rows_per_utt > 0 ? st.rows_per_utt : 2 * W;
+  const int32_t dims9[9] = {B, W, m.V, m.D, m.pred_lstm.w_ih.k_pad, m.pred_lstm.w_hh.k_pad, m.src.lstm[0].w_hh.k_pad,
+                            m.tgt.lstm[0].w_hh.k_pad, RW};
+  return B * W <= SUMS_MAX_ROWS && m.prepared != nullptr && search_tables(m) && aligned16(st.pred_c) && aligned16(st.src_c) && aligned16(st.tgt_c[0]) &&
+         aligned16(st.tgt_c[1]) && workspace_bytes >= q4_workspace_bytes(Q4_WS_BEAM, dims9, 9);
+}
+
+// How a step is part of a search.
+struct StepMode {
+  SearchCall* call;                         // non-null: e, T and u_max come from there, its iteration number is added
+  int32_t* frozen;                          // non-null: an utterance without labels to propose is left to launch_search_tail
+  const cudaGraphConditionalHandle* loop;   // non-null: the last step of a graph's loop
+  bool sums;                                // see search_keeps_sums
+  cudaStream_t sums_stream;                 // non-null: a stream for the sums of the recurrent halves, with an event (else
+  cudaEvent_t sums_event;                   // they follow the source LM's head)
+};
+// One step.
 static int beam_step(const q4_model* model, q4_beam_state* state, const float* e, int32_t B, int32_t T, int32_t W,
                      int32_t iter, int32_t u_max, float lambda_t, float lambda_s, float rho, int32_t mode,
-                     void* workspace, size_t workspace_bytes, q4_stream stream, SearchCall* call, int32_t* frozen,
-                     const cudaGraphConditionalHandle* loop) {
+                     void* workspace, size_t workspace_bytes, q4_stream stream, const StepMode& how) {
   if (!model || !e || !workspace) return Q4_ERR_NULL;
   if (mode < 0 || mode > 2) return Q4_ERR_UNSUPPORTED;
   if (B <= 0 || T <= 0 || W <= 0 || W > 16 || iter < 0 || u_max < 0) return Q4_ERR_DIM;
   const q4_model& m = *model;
+  SearchCall* const call = how.call;
+  int32_t* const frozen = how.frozen;
   Q4_CHECK(check_state(state, m.tgt.n_layers));
   if (mode != 0) {   // time-synchronous search: candidate set, enough state rows, call number matches
     const q4_beam_state& ts = *state;
@@ -985,7 +1051,7 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
   // the first call of a frame of the time-synchronous search follows a frame close, which creates
   // no label extension: no network has anything to advance, only the joint runs
   const bool nets = !(mode != 0 && iter > 0 && iter % (state->tsd_smax + 1) == 0);
-  uint8_t* ws = static_cast<uint8_t*>(workspace) + 256;   // (the first 256 bytes: SearchCall of q4_beam_search)
+  uint8_t* ws = static_cast<uint8_t*>(workspace) + 256;   // (the first 256 bytes: SearchCall of q4_beam_search, at 128 a row count)
   uint8_t* zq = ws;
   ws += align_up((size_t)N * D);
   uint8_t* bq_src = ws;
@@ -1012,43 +1078,41 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
   const int Hp = m.pred_lstm.w_hh.k_pad, Hs = m.src.lstm[0].w_hh.k_pad, Ht = m.tgt.lstm[0].w_hh.k_pad;
   const int Ep = m.pred_lstm.w_ih.k_pad;
   const bool use_mma = search_uses_tensor_cores(m, st, B, W, workspace_bytes);
-  if (use_mma) {
+  if (use_mma || how.sums) {
     const size_t Np = ((size_t)N + 127) / 128 * 128;
-    const int Hmax = Hp > Hs ? (Hp > Ht ? Hp : Ht) : (Hs > Ht ? Hs : Ht);
-    (void)Hmax;
-    int8_t* xa8[3];   // embedding rows of the pending symbols: prediction, source LM, target LM
-    for (int i = 0; i < 3; ++i) {
-      xa8[i] = reinterpret_cast<int8_t*>(ws);
-      ws += align_up(Np * Ep);
+    auto take = [&](size_t bytes) {
+      uint8_t* p = ws;
+      ws += align_up(bytes);
+      return p;
+    };
+    const int hdim[4] = {Hp, Hs, Ht, Ht};   // prediction, source LM, target LM layers 1 and 2
+    int8_t* xa8[3] = {nullptr, nullptr, nullptr};            // embedding rows of the pending symbols
+    int8_t* ha8[4] = {nullptr, nullptr, nullptr, nullptr};   // previous cell outputs
+    if (!how.sums) {
+      for (int i = 0; i < 3; ++i) xa8[i] = reinterpret_cast<int8_t*>(take(Np * Ep));
+      for (int i = 0; i < 4; ++i) ha8[i] = reinterpret_cast<int8_t*>(take(Np * (size_t)hdim[i]));
     }
-    int8_t* ha8[4];   // previous cell outputs: prediction, source LM, target LM layers 1 and 2
-    const int hdim[4] = {Hp, Hs, Ht, Ht};
-    for (int i = 0; i < 4; ++i) {
-      ha8[i] = reinterpret_cast<int8_t*>(ws);
-      ws += align_up(Np * (size_t)hdim[i]);
-    }
-    int8_t* pred_h8 = reinterpret_cast<int8_t*>(ws);
-    ws += align_up(Np * Hp);
-    int8_t* src_h8 = reinterpret_cast<int8_t*>(ws);
-    ws += align_up(Np * Hs);
-    int8_t* tgt_h8[2];
-    tgt_h8[0] = reinterpret_cast<int8_t*>(ws);
-    ws += align_up(Np * Ht);
-    tgt_h8[1] = reinterpret_cast<int8_t*>(ws);
-    ws += align_up(Np * Ht);
+    int8_t* new_h8[4];                                       // new cell outputs
+    for (int i = 0; i < 4; ++i) new_h8[i] = reinterpret_cast<int8_t*>(take(Np * (size_t)hdim[i]));
+    int8_t* const pred_h8 = new_h8[0];
+    int8_t* const src_h8 = new_h8[1];
+    int8_t* const tgt_h8[2] = {new_h8[2], new_h8[3]};
     int8_t* bq8[2];
-    bq8[0] = reinterpret_cast<int8_t*>(ws);
-    ws += align_up(Np * D);
-    bq8[1] = reinterpret_cast<int8_t*>(ws);
-    ws += align_up(Np * D);
-    int8_t* z8 = reinterpret_cast<int8_t*>(ws);
+    for (int i = 0; i < 2; ++i) bq8[i] = reinterpret_cast<int8_t*>(take(Np * D));
+    int8_t* z8 = reinterpret_cast<int8_t*>(take(Np * D));
+    int32_t* const n_work = reinterpret_cast<int32_t*>(static_cast<uint8_t*>(workspace) + 128);
+    float* state_sums[4] = {nullptr, nullptr, nullptr, nullptr};
+    if (how.sums) {
+      const size_t R = (size_t)B * (st.rows_per_utt > 0 ? st.rows_per_utt : 2 * W);
+      for (int i = 0; i < 4; ++i) state_sums[i] = reinterpret_cast<float*>(take(R * 4 * (size_t)hdim[i] * sizeof(float)));
+    }
     const PrepPlan pp = plan_prepared(m);
     const uint8_t* pb = static_cast<const uint8_t*>(m.prepared);
 
     // at most 32 hypothesis rows (one utterance): the LSTM steps are bound by reading the weights once,
     // and a weight-streaming kernel reads them as stored (packed 4-bit), the state rows and embedding
     // rows too, so the gathers below are not needed
-    const bool skinny =
+    const bool skinny = !how.sums &&
         skinny_lstm_supported(N, Hp, Ep, m.pred_lstm.w_ih.bits, m.pred_lstm.w_hh.bits, m.pred_emb_act, m.pred_lstm.hid_act) &&
         skinny_lstm_supported(N, Hs, Ep, m.src.lstm[0].w_ih.bits, m.src.lstm[0].w_hh.bits, m.src.emb_act, m.src.lstm[0].hid_act) &&
         skinny_lstm_supported(N, Ht, Ep, m.tgt.lstm[0].w_ih.bits, m.tgt.lstm[0].w_hh.bits, m.tgt.emb_act, m.tgt.lstm[0].hid_act) &&
@@ -1056,7 +1120,7 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
                                                       m.tgt.lstm[0].hid_act, m.tgt.lstm[1].hid_act));
     // all gathers of the iteration in one launch: embedding rows by pending symbol, previous
     // cell-output codes by parent state row, unpacked to int8 operand rows
-    if (nets && !skinny) {
+    if (nets && !skinny && !how.sums) {
       UnpackJobs uj;
       memset(&uj, 0, sizeof(uj));
       add_unpack_job(uj, m.pred_emb_q, row_bytes(Ep, m.pred_emb_act.bits), cst.adv_tok, m.pred_emb_act, Ep, xa8[0]);
@@ -1074,6 +1138,51 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
       TagScope tag(TAG_MISC);
       Q4_TRY(launch_unpack_multi(uj, s, true));
     }
+    const q4_lstm* const first_layer[3] = {&m.pred_lstm, &m.src.lstm[0], &m.tgt.lstm[0]};
+    if (nets && how.sums) {   // the first layers of all networks
+      CellJobs cj;
+      memset(&cj, 0, sizeof(cj));
+      void* const hq[3] = {st.pred_hq, st.src_hq, st.tgt_hq[0]};
+      float* const c[3] = {st.pred_c, st.src_c, st.tgt_c[0]};
+      for (int i = 0; i < 3; ++i) {
+        CellJob& k = cj.job[i];
+        k.table = reinterpret_cast<const float*>(pb + pp.table[i]);
+        k.sums = state_sums[i];
+        k.sc_hh = reinterpret_cast<const float*>(pb + pp.lstm[i].sc_hh);
+        k.c = c[i];
+        k.hq = static_cast<uint8_t*>(hq[i]);
+        k.h8 = new_h8[i];
+        k.H = hdim[i];
+        k.hid_act = first_layer[i]->hid_act;
+      }
+      cj.n_jobs = 3;
+      cj.N = N;
+      cj.src_row = c_src;
+      cj.dst_row = c_dst;
+      cj.tok = c_tok;
+      cj.n_active = n_active;
+      cj.n_work = n_work;
+      TagScope tag(TAG_CELLS);
+      Q4_TRY(launch_search_cells(cj, s, true));
+    }
+    auto state_products = [&](cudaStream_t s, bool dep, int first, int count) -> int {
+      StateProductJobs sj;
+      memset(&sj, 0, sizeof(sj));
+      for (int i = 0; i < count; ++i) {
+        sj.job[i].h8 = new_h8[first + i];
+        sj.job[i].w8 = reinterpret_cast<const int8_t*>(pb + pp.lstm[first + i].hw);
+        sj.job[i].sums = state_sums[first + i];
+        sj.job[i].H = hdim[first + i];
+      }
+      sj.n_jobs = count;
+      sj.N = N;
+      sj.dst_row = c_dst;
+      sj.n_work = n_work;
+      sj.status = st.status;
+      TagScope tag(TAG_STATE);
+      Q4_TRY(launch_state_products(sj, s, dep));
+      return Q4_OK;
+    };
     // the three networks are independent until the selection: with two lent streams they run side
     // by side.  The call's own stream carries the longest chain, the target LM's (gather -> two layers -> head ->
     // selection as programmatic dependents without an event in between; a fork costs 2 to 4 us, a join 1 to 4).
@@ -1090,6 +1199,10 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
       Q4_TRY(cudaEventRecord(fork, s));
       Q4_TRY(cudaStreamWaitEvent(sp, fork, 0));
       Q4_TRY(cudaStreamWaitEvent(ss, fork, 0));
+      if (how.sums_stream) {
+        Q4_TRY(cudaStreamWaitEvent(how.sums_stream, fork, 0));
+        Q4_CHECK(state_products(how.sums_stream, false, 0, 3));
+      }
     }
     // one LSTM layer of one network for every pending slot
     // `dep`: the previous launch on the same stream is a kernel of this library, so this one may
@@ -1153,8 +1266,9 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
       a.status = st.status;
       a.n_active = n_active;
       a.premultiplied = 1;   // q4_prepare_model stored the products
-      a.h_first = dep ? h_first : 0;
+      a.h_first = dep && !how.sums ? h_first : 0;
       a.trigger_early = trigger_early;
+      a.hh_pre = how.sums ? state_sums[li] : nullptr;
       Q4_TRY(launch_mma_lstm(a, xa, Kx, reinterpret_cast<const int8_t*>(pb + pp.lstm[li].xw), Kx, ha, H,
                              reinterpret_cast<const int8_t*>(pb + pp.lstm[li].hw), H, s, dep));
       return Q4_OK;
@@ -1173,9 +1287,10 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
     const bool fused_head = D == 256 && V <= 2048;   // the fused head kernel: 256-wide bottleneck, one cluster per row tile
     // 1a. prediction network, then the joint network for every live slot (stream sp)
     if (nets) {
-      Q4_CHECK(lstm_mma(sp, !forked, TAG_PRED_LSTM, 0, m.pred_lstm, m.pred_emb_act, xa8[0], ha8[0], st.pred_hq,
-                        st.pred_c, pred_h8));
-      Q4_CHECK(linear_mma(sp, true, TAG_PRED_PROJ, 0, m.pred_proj, pred_h8, m.pred_lstm.hid_act.scale, EPI_F32,
+      if (!how.sums)
+        Q4_CHECK(lstm_mma(sp, !forked, TAG_PRED_LSTM, 0, m.pred_lstm, m.pred_emb_act, xa8[0], ha8[0], st.pred_hq,
+                          st.pred_c, pred_h8));
+      Q4_CHECK(linear_mma(sp, !how.sums || !forked, TAG_PRED_PROJ, 0, m.pred_proj, pred_h8, m.pred_lstm.hid_act.scale, EPI_F32,
                           st.pred_p, D, cst.adv_dst, nullptr, n_active));
     }
     {
@@ -1217,8 +1332,9 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
       float* c0 = which == 0 ? st.src_c : st.tgt_c[0];
       int8_t* h8_0 = which == 0 ? src_h8 : tgt_h8[0];
       float* lp = which == 0 ? st.src_lp : st.tgt_lp;
-      Q4_CHECK(lstm_mma(sl, which == 1 || !forked, which == 0 ? TAG_SRC_LSTM : TAG_TGT_L1, which == 0 ? 1 : 2, L0, lm.emb_act,
-                        xa8[which + 1], ha8[which + 1], hq0, c0, h8_0, 0, lm.n_layers == 2 ? 1 : 0));
+      if (!how.sums)
+        Q4_CHECK(lstm_mma(sl, which == 1 || !forked, which == 0 ? TAG_SRC_LSTM : TAG_TGT_L1, which == 0 ? 1 : 2, L0, lm.emb_act,
+                          xa8[which + 1], ha8[which + 1], hq0, c0, h8_0, 0, lm.n_layers == 2 ? 1 : 0));
       const int8_t* top8 = h8_0;
       const q4_lstm* last = &L0;
       if (lm.n_layers == 2) {
@@ -1229,7 +1345,9 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
                           tgt_h8[1], 1, 0));
         top8 = tgt_h8[1];
         last = &L1;
+        if (how.sums && forked) Q4_TRY(cudaEventRecord(reinterpret_cast<cudaEvent_t>(st.aux_event[0]), s));
       }
+      const bool head_dep = !how.sums || which == 1 || !forked;   // behind an event otherwise
       const int head_tag = which == 0 ? TAG_SRC_HEAD : TAG_TGT_HEAD;
       if (fused_head) {
         // bottleneck, re-quantization, output layer and log-softmax in one kernel
@@ -1251,21 +1369,29 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
         ha.n_active = n_active;
         ha.status = st.status;
         Q4_TRY(launch_mma_lmhead(ha, top8, ha.H, reinterpret_cast<const int8_t*>(pb + pp.lin[which == 0 ? 1 : 3]),
-                                 reinterpret_cast<const int8_t*>(pb + pp.lin[which == 0 ? 2 : 4]), sl, true));
+                                 reinterpret_cast<const int8_t*>(pb + pp.lin[which == 0 ? 2 : 4]), sl, head_dep));
       } else {
-        Q4_CHECK(linear_mma(sl, true, head_tag, which == 0 ? 1 : 3, lm.bott, top8, last->hid_act.scale, EPI_QUANT8,
+        Q4_CHECK(linear_mma(sl, head_dep, head_tag, which == 0 ? 1 : 3, lm.bott, top8, last->hid_act.scale, EPI_QUANT8,
                             bq8[which], D, nullptr, &lm.bott_act, n_active));
         Q4_CHECK(linear_mma(sl, true, head_tag, which == 0 ? 2 : 4, lm.out, bq8[which], lm.bott_act.scale, EPI_F32, lp,
                             V, cst.adv_dst, nullptr, n_active));
       }
     }
-    if (forked) {   // join: the call's stream waits for both side chains
-      cudaEvent_t j0 = reinterpret_cast<cudaEvent_t>(st.aux_event[1]);
-      cudaEvent_t j1 = reinterpret_cast<cudaEvent_t>(st.aux_event[2]);
-      Q4_TRY(cudaEventRecord(j0, sp));
-      Q4_TRY(cudaEventRecord(j1, ss));
-      Q4_TRY(cudaStreamWaitEvent(s, j0, 0));
-      Q4_TRY(cudaStreamWaitEvent(s, j1, 0));
+    if (forked) {
+      Q4_TRY(cudaEventRecord(reinterpret_cast<cudaEvent_t>(st.aux_event[1]), sp));
+      Q4_TRY(cudaEventRecord(reinterpret_cast<cudaEvent_t>(st.aux_event[2]), ss));
+    }
+    if (how.sums && nets) {   // sums for the next step, beside the target LM's head and the selection
+      cudaStream_t sx = forked && how.sums_stream ? how.sums_stream : ss;
+      if (sx == ss) Q4_CHECK(state_products(ss, true, 0, 3));
+      if (m.tgt.n_layers == 2) {
+        if (forked) Q4_TRY(cudaStreamWaitEvent(sx, reinterpret_cast<cudaEvent_t>(st.aux_event[0]), 0));
+        Q4_CHECK(state_products(sx, !forked, 3, 1));
+      }
+    }
+    if (forked) {   // join: the selection waits for both side chains (not for the sums)
+      Q4_TRY(cudaStreamWaitEvent(s, reinterpret_cast<cudaEvent_t>(st.aux_event[1]), 0));
+      Q4_TRY(cudaStreamWaitEvent(s, reinterpret_cast<cudaEvent_t>(st.aux_event[2]), 0));
     }
     if (!fused_head && nets) {  // log-softmax of both LMs' new rows in one launch
       TagScope tag(TAG_TGT_HEAD);
@@ -1329,8 +1455,8 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
   memset(&sel, 0, sizeof(sel));
   sel.call = call;
   sel.frozen = frozen;
-  if (loop) {
-    sel.loop = *loop;
+  if (how.loop) {
+    sel.loop = *how.loop;
     sel.loop_iters = PLAN_ITERS;
   }
   sel.logits = logits;
@@ -1351,9 +1477,15 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
   sel.mode = mode;
   TagScope tag_sel(TAG_SELECT);
   if (mode != 0)
-    Q4_TRY(launch_tsd_select(sel, s, use_mma));
+    Q4_TRY(launch_tsd_select(sel, s, use_mma || how.sums));
   else
-    Q4_TRY(launch_beam_select(sel, s, use_mma));
+    Q4_TRY(launch_beam_select(sel, s, use_mma || how.sums));
+  if (how.sums && nets && st.aux_stream[0] && st.aux_stream[1] && st.aux_event[0] && st.aux_event[1] && st.aux_event[2]) {
+    // the next step waits for the sums as well
+    cudaEvent_t done = how.sums_stream ? how.sums_event : reinterpret_cast<cudaEvent_t>(st.aux_event[2]);
+    Q4_TRY(cudaEventRecord(done, how.sums_stream ? how.sums_stream : reinterpret_cast<cudaStream_t>(st.aux_stream[1])));
+    Q4_TRY(cudaStreamWaitEvent(s, done, 0));
+  }
   return Q4_OK;
 }
 
@@ -1362,7 +1494,7 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
                         float lambda_s, float rho, int32_t mode, void* workspace,
                         size_t workspace_bytes, q4_stream stream) {
   return beam_step(model, state, e, B, T, W, iter, u_max, lambda_t, lambda_s, rho, mode, workspace, workspace_bytes, stream,
-                   nullptr, nullptr, nullptr);
+                   StepMode());
 }
 
 // ------------------------------------------------------------------------ whole search
@@ -1379,7 +1511,7 @@ struct SearchKey {                   // everything the graph was built from
   q4_beam_state state;
   void* workspace;
   size_t workspace_bytes;
-  int32_t B, W, tsd, dependent, exact, loop;
+  int32_t B, W, tsd, dependent, exact, loop, sums;
   float lambda_t, lambda_s, rho;
 };
 // One graph and the search it was built for.  PLAN_GRAPHS of them: a decoder that alternates between a few batch sizes,
@@ -1396,8 +1528,8 @@ struct SearchPlan {
   SearchGraph graph[PLAN_GRAPHS];
   int64_t built, replays, failed;    // graphs made, replays enqueued, attempts to make a graph that failed
   int64_t uses;
-  cudaStream_t stream, side[2];      // captured on: the graphs' chains, none of the caller's streams
-  cudaEvent_t side_event[3];
+  cudaStream_t stream, side[3];      // captured on: the graphs' chains, none of the caller's streams
+  cudaEvent_t side_event[4];
 };
 // While one of these lives, calls of this thread that a capture elsewhere in the process would take for unsafe (streams
 // and events made or destroyed, a graph instantiated, an event asked) leave that capture alone: none of them
@@ -1422,8 +1554,8 @@ int q4_search_plan_create(q4_search_plan* out) {
   bool ok = cudaStreamCreateWithFlags(&p->stream, cudaStreamNonBlocking) == cudaSuccess;
   for (int i = 0; i < PLAN_GRAPHS && ok; ++i)
     ok = cudaEventCreateWithFlags(&p->graph[i].done, cudaEventDisableTiming) == cudaSuccess;
-  for (int i = 0; i < 2 && ok; ++i) ok = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking) == cudaSuccess;
-  for (int i = 0; i < 3 && ok; ++i) ok = cudaEventCreateWithFlags(&p->side_event[i], cudaEventDisableTiming) == cudaSuccess;
+  for (int i = 0; i < 3 && ok; ++i) ok = cudaStreamCreateWithFlags(&p->side[i], cudaStreamNonBlocking) == cudaSuccess;
+  for (int i = 0; i < 4 && ok; ++i) ok = cudaEventCreateWithFlags(&p->side_event[i], cudaEventDisableTiming) == cudaSuccess;
   if (ok) return Q4_OK;
   q4_search_plan_destroy(p);
   *out = nullptr;
@@ -1441,9 +1573,9 @@ int q4_search_plan_destroy(q4_search_plan plan) {
     if (g.done) cudaEventDestroy(g.done);
   }
   if (p->stream) cudaStreamDestroy(p->stream);
-  for (int i = 0; i < 2; ++i)
-    if (p->side[i]) cudaStreamDestroy(p->side[i]);
   for (int i = 0; i < 3; ++i)
+    if (p->side[i]) cudaStreamDestroy(p->side[i]);
+  for (int i = 0; i < 4; ++i)
     if (p->side_event[i]) cudaEventDestroy(p->side_event[i]);
   free(p);
   return Q4_OK;
@@ -1454,10 +1586,13 @@ int q4_search_plan_destroy(q4_search_plan plan) {
 static int capture_steps(SearchPlan* p, SearchKey& key, const cudaGraphConditionalHandle* loop) {
   SearchCall* call = static_cast<SearchCall*>(key.workspace);
   // T and u_max (and the frames) only have to pass the argument checks here; the first frame's steps are never in the graph
-  for (int it = PLAN_ITERS; it < 2 * PLAN_ITERS; ++it)
+  for (int it = PLAN_ITERS; it < 2 * PLAN_ITERS; ++it) {
+    const StepMode how = {call, loop ? search_frozen(key.workspace) : nullptr, it == 2 * PLAN_ITERS - 1 ? loop : nullptr,
+                          key.sums != 0, key.sums && key.state.aux_stream[0] ? p->side[2] : nullptr, p->side_event[3]};
     Q4_CHECK(beam_step(&key.model, &key.state, static_cast<const float*>(key.workspace), key.B, 1 << 24, key.W, it, 0,
                        key.lambda_t, key.lambda_s, key.rho, step_mode(key, it), key.workspace, key.workspace_bytes, p->stream,
-                       call, loop ? search_frozen(key.workspace) : nullptr, it == 2 * PLAN_ITERS - 1 ? loop : nullptr));
+                       how));
+  }
   if (!loop) Q4_TRY(launch_search_advance(call, PLAN_ITERS, p->stream));
   return Q4_OK;
 }
@@ -1567,8 +1702,10 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
   for (int i = 0; i < 3; ++i) key.state.aux_event[i] = p && lent ? p->side_event[i] : nullptr;
   // An alignment-length synchronous search ends its steps when no utterance has labels left to propose; the iterations
   // that are left then are carried out together.
+  const bool sums = search_keeps_sums(*model, *state, B, W, workspace_bytes);
+  key.sums = sums;
   key.loop = p && !key.tsd && !key.exact && search_tail_supported(model->V, model->D) &&
-             search_uses_tensor_cores(*model, *state, B, W, workspace_bytes);
+             (sums || search_uses_tensor_cores(*model, *state, B, W, workspace_bytes));
   // step by step: while launches are timed or waits are made to run out (a graph would keep that), in a short search, and
   // without a loop in a stream that is being captured
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -1619,7 +1756,7 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
       if (it >= n_iters) break;
     }
     Q4_CHECK(beam_step(model, state, e, B, T, W, it, u_max, lambda_t, lambda_s, rho, step_mode(key, it), workspace,
-                       workspace_bytes, stream, nullptr, nullptr, nullptr));
+                       workspace_bytes, stream, StepMode{nullptr, nullptr, nullptr, sums, nullptr, nullptr}));
     ++it;
   }
   if (tail) {

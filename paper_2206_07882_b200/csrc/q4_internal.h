@@ -69,7 +69,7 @@ cudaError_t launch_traceback(const q4_beam_state& st, int B, int W, int n_iters,
 enum { TAG_NONE = 0, TAG_QUANT = 1, TAG_ENC_GEMM = 2, TAG_ENC_STEP = 3, TAG_LINEAR = 4,
        TAG_PRED_LSTM = 5, TAG_PRED_PROJ = 6, TAG_SRC_LSTM = 7, TAG_SRC_HEAD = 8, TAG_TGT_L1 = 9,
        TAG_TGT_L2 = 10, TAG_TGT_HEAD = 11, TAG_JOINT = 12, TAG_SELECT = 13, TAG_MISC = 14,
-       TAG_COUNT = 15 };
+       TAG_CELLS = 15, TAG_STATE = 16, TAG_COUNT = 17 };
 extern int g_tag;   // tag of the launches being issued
 struct TagScope {
   int prev;
@@ -115,6 +115,8 @@ struct MmaLstmArgs {
                             // the recurrent half of the K loop runs before waiting for that kernel
   int32_t trigger_early;    // 1: let the next kernel of the stream start beside this one
   int32_t tile_rows, n_stages;   // set by the launcher
+  const float* hh_pre;      // optional sums of the recurrent half, row src_row[n] of [*, 4H] in 4*cell+gate order (negative
+                            // row: zero); the recurrent operands are not read
   int32_t premultiplied;    // 1: sc_ih = x_scale * row scale and sc_hh = hidden scale * row scale already
 };
 struct LmHeadArgs {
@@ -191,6 +193,42 @@ cudaError_t launch_layer_prepare(LayerPrep a, cudaStream_t s, bool dependent);
 cudaError_t launch_mma_lstm(const MmaLstmArgs& a, const int8_t* xa, long long xa_pitch,
                             const int8_t* xw, long long xw_pitch, const int8_t* ha, long long ha_pitch,
                             const int8_t* hw, long long hw_pitch, cudaStream_t s, bool dependent = false);
+
+// ---- network advances of a whole search (q4_advance.cu)
+struct CellJob {
+  const float* table;       // [V, 4H] de-quantized input sums plus bias, columns in 4*cell+gate order
+  const float* sums;        // [*, 4H] sums of the recurrent half per state row, same order
+  const float* sc_hh;       // [4H] hidden scale * row scale, same order
+  float* c;                 // [*, H] cell states per state row
+  uint8_t* hq;              // packed codes per state row
+  int8_t* h8;               // [N, H] int8 codes per pending row
+  int32_t H;
+  q4_act hid_act;
+};
+struct CellJobs {
+  CellJob job[3];
+  int32_t n_jobs, N;
+  const int32_t* src_row;   // pending rows: state row extended (negative: zero state), state row written, label
+  const int32_t* dst_row;
+  const int32_t* tok;
+  const int32_t* n_active;
+  int32_t* n_work;          // receives the number of rows with work: the selection, which clears n_active, runs beside the products
+};
+cudaError_t launch_search_cells(const CellJobs& jobs, cudaStream_t s, bool dependent);
+struct StateProductJob {
+  const int8_t* h8;         // [N, H] int8 codes per pending row
+  const int8_t* w8;         // [4H, H] int8 recurrent weights, rows in 4*cell+gate order
+  float* sums;              // [*, 4H], row dst_row[n]
+  int32_t H;
+};
+struct StateProductJobs {
+  StateProductJob job[3];
+  int32_t n_jobs, N, tile_rows;   // tile_rows: set by the launcher
+  const int32_t* dst_row;
+  const int32_t* n_work;          // rows with work, as k_search_cells left it
+  int32_t* status;
+};
+cudaError_t launch_state_products(const StateProductJobs& jobs, cudaStream_t s, bool dependent);
 
 // ---- weight-streaming LSTM step for at most 32 rows (q4_skinny.cu)
 struct SkinnyLstmArgs {

@@ -957,3 +957,37 @@ def test_selection_forms_agree_with_the_exact_search(Bd, V, normalized, S):
             runs.append(list(out) + [dd.tensors[k] for k in ("bp_parent", "bp_token", "bp_score", "fin_n", "fin_score")])
         for x, y in zip(*runs):
             assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("B,W,S,layers,bits", [(3, 7, None, 2, 4), (8, 16, None, 2, 4), (9, 15, 1, 2, 4), (24, 16, None, 1, 8),
+                                               (25, 16, None, 2, 4), (2, 16, 3, 1, 4)])
+def test_search_that_keeps_sums_equals_its_steps(Bd, B, W, S, layers, bits):
+    # tables for the input halves and recurrent sums per state row against the step kernels: the edges of row tiles, the
+    # largest search that keeps them and one more, one or two target-LM layers
+    dw = synth.decoder(seed=95, V=300, E=32, Hp=256, D=256, Hs=128, Ht=384, tgt_layers=layers, U_max=12, W=W, all_bits=bits)
+    dw.joint.out.bias[0] += np.float32(2.0)
+    T = 30
+    e = torch.from_numpy(synth.Stream(B + W).normal("e", (T, B, 256)).astype(np.float32)).cuda()
+    n = T + 12 if S is None else T * (S + 1)
+    a, b = Bd.Decoder(dw), Bd.Decoder(dw)
+    got = a.decode(e, 12) if S is None else a.decode_time_synchronous(e, S, 12)
+    b.alloc_state(B, W, n, S)
+    b.q4_beam_init()
+    for it in range(n):
+        b.dr_fusion_beam_step(e, T, it, 12, mode=0 if S is None else 2 if it % (S + 1) == S else 1)
+    for x, y in zip(got, b.q4_traceback(n, 12)):
+        assert torch.equal(x, y)
+    assert a.tensors["status"].item() == 0
+    for k in ("bp_parent", "bp_token", "bp_score", "fin_n", "fin_score", "pred_c", "tgt_c0", "tgt_hq0", "pred_p"):
+        assert torch.equal(a.tensors[k], b.tensors[k]), k
+
+
+def test_search_with_embeddings_of_other_row_lengths(Bd):
+    # 2-bit weights of the prediction network pad its 10-wide embedding rows to 64 codes, the language models' to 32: the
+    # tables take each network's own, and the beams are the oracle's
+    dw = synth.decoder(seed=96, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=5, W=8, rnnt_w_bits=2)
+    e = synth.Stream(31).normal("e", (12, 3, 256)).astype(np.float32)
+    dd, tokens, lens, scores, ref = run_search(Bd, dw, e)
+    assert dd.pred_lstm.w_ih.k_pad != dd.src.lstm[0].w_ih.k_pad
+    frac, tr = compare_search(dd, tokens, lens, scores, ref, list(range(3)), 12, 5, 8, min_same=1.0)
+    assert tr == 1.0
