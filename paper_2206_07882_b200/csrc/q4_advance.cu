@@ -131,17 +131,16 @@ __global__ void __launch_bounds__(192, 2) k_state_products(const __grid_constant
   const int n_work = *jobs.n_work;
   if (m0 < n_work) {
     if (warp == 4) {
+      const uint32_t on = elect_one();
       bool ok = true;
       int s = 0;
       uint32_t ph = 1;
       for (int i = 0; i < nk && ok; ++i) {
-        ok = mbar_wait_warp(&empty[s], ph);   // passes at once for a stage that has never been filled
+        ok = i < SP_STAGES || mbar_wait_warp(&empty[s], ph);   // (a stage that has never been filled is free)
         if (!ok) break;
-        if (elect_one()) {
-          mbar_expect_tx(&full[s], STAGE);
-          tma_load_2d(smem + s * STAGE, ta, i * SP_BK, m0, &full[s]);
-          tma_load_2d(smem + s * STAGE + A_BYTES, tb, i * SP_BK, n0, &full[s]);
-        }
+        mbar_expect_tx(on, &full[s], STAGE);
+        tma_load_2d(on, smem + s * STAGE, ta, i * SP_BK, m0, &full[s]);
+        tma_load_2d(on, smem + s * STAGE + A_BYTES, tb, i * SP_BK, n0, &full[s]);
         if (++s == SP_STAGES) {
           s = 0;
           ph ^= 1;
@@ -150,26 +149,27 @@ __global__ void __launch_bounds__(192, 2) k_state_products(const __grid_constant
       if (!ok && lane == 0) atomicExch(jobs.status, Q4_ERR_TIMEOUT);
     } else if (warp == 5) {
       const uint32_t idesc = umma_idesc_i8(SP_BM, SP_BN);
-      bool ok = true;
+      const uint32_t on = elect_one();
+      bool ok = true, ready = mbar_test(&full[0], 0);
       int s = 0;
       uint32_t ph = 0;
       for (int i = 0; i < nk && ok; ++i) {
-        ok = mbar_wait_warp(&full[s], ph);
+        ok = mbar_wait_warp_tested(ready, &full[s], ph);
         if (!ok) break;
         tc_fence_after();
-        const uint64_t da = umma_desc_sw128(smem_u32(smem + s * STAGE));
-        const uint64_t db = umma_desc_sw128(smem_u32(smem + s * STAGE + A_BYTES));
-        if (elect_one()) {
-#pragma unroll
-          for (int kk = 0; kk < SP_BK / 32; ++kk) umma_i8(tmem, da + 2 * kk, db + 2 * kk, idesc, (i | kk) != 0);
-          umma_commit(&empty[s]);
-        }
+        const int st = s;
         if (++s == SP_STAGES) {
           s = 0;
           ph ^= 1;
         }
+        ready = mbar_test(&full[s], ph);
+        const uint64_t da = umma_desc_sw128(smem_u32(smem + st * STAGE));
+        const uint64_t db = umma_desc_sw128(smem_u32(smem + st * STAGE + A_BYTES));
+#pragma unroll
+        for (int kk = 0; kk < SP_BK / 32; ++kk) umma_i8(on, tmem, da + 2 * kk, db + 2 * kk, idesc, (i | kk) != 0);
+        umma_commit(on, &empty[st]);
       }
-      if (elect_one()) umma_commit(&acc_full);
+      umma_commit(on, &acc_full);
       if (!ok && lane == 0) atomicExch(jobs.status, Q4_ERR_TIMEOUT);
     } else {
       const int n = m0 + warp * 32 + lane;

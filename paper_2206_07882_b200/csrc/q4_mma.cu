@@ -352,17 +352,16 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
   if (a.n_idle && ld_coherent(a.n_idle) >= a.all_idle) {   // the same for every thread of the grid
     pdl_trigger();
   } else if (warp == 4) {
+    const uint32_t on = elect_one();
     bool ok = true;
     int s = 0;
     uint32_t ph = 1;
     for (int i = 0; i < nk && ok && !a.skip_producer; ++i) {
-      ok = mbar_wait_warp(&empty[s], ph, a.wait_limit);   // passes at once for a stage that has never been filled
+      ok = i < NS || mbar_wait_warp(&empty[s], ph, a.wait_limit);   // (a stage that has never been filled is free)
       if (!ok) break;
-      if (elect_one()) {
-        mbar_expect_tx(&full[s], STAGE);
-        tma_load_2d(smem + s * STAGE, &tma_a, i * BK, m0, &full[s]);
-        tma_load_2d(smem + s * STAGE + A_BYTES, &tma_b, i * BK, n0, &full[s]);
-      }
+      mbar_expect_tx(on, &full[s], STAGE);
+      tma_load_2d(on, smem + s * STAGE, &tma_a, i * BK, m0, &full[s]);
+      tma_load_2d(on, smem + s * STAGE + A_BYTES, &tma_b, i * BK, n0, &full[s]);
       if (++s == NS) {
         s = 0;
         ph ^= 1;
@@ -372,31 +371,32 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
     if (!ok && lane == 0) flag_timeout(a.status);
   } else if (warp == 5) {
     const uint32_t idesc = umma_idesc_i8(BM, GEMM_BN);
-    bool ok = true;
+    const uint32_t on = elect_one();
+    bool ok = true, ready = mbar_test(&full[0], 0);
     int s = 0;
     uint32_t ph = 0;
     for (int i = 0; i < nk && ok; ++i) {
-      ok = mbar_wait_warp(&full[s], ph, a.wait_limit);
+      ok = mbar_wait_warp_tested(ready, &full[s], ph, a.wait_limit);
       if (!ok) break;
       tc_fence_after();
-      const uint64_t da = umma_desc_sw128(smem_u32(smem + s * STAGE));
-      const uint64_t db = umma_desc_sw128(smem_u32(smem + s * STAGE + A_BYTES));
-      if (elect_one()) {
-#pragma unroll
-        for (int kk = 0; kk < BK / 32; ++kk) umma_i8(tmem, da + 2 * kk, db + 2 * kk, idesc, (i | kk) != 0);
-        umma_commit(&empty[s]);
-      }
+      const int st = s;
       if (++s == NS) {
         s = 0;
         ph ^= 1;
       }
+      ready = mbar_test(&full[s], ph);
+      const uint64_t da = umma_desc_sw128(smem_u32(smem + st * STAGE));
+      const uint64_t db = umma_desc_sw128(smem_u32(smem + st * STAGE + A_BYTES));
+#pragma unroll
+      for (int kk = 0; kk < BK / 32; ++kk) umma_i8(on, tmem, da + 2 * kk, db + 2 * kk, idesc, (i | kk) != 0);
+      umma_commit(on, &empty[st]);
     }
     if (!ok) {   // recorded before the epilogue is released, so that it stores nothing
       if (lane == 0) flag_timeout(a.status);
       __threadfence();
       __syncwarp();
     }
-    if (elect_one()) umma_commit(&acc_full);
+    umma_commit(on, &acc_full);
     pdl_trigger();
   } else if (warp < 4) {
     for (int c = tid; c < GEMM_BN; c += 128) {   // stage scale * row scale and bias while the MMAs run
@@ -528,20 +528,19 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
 
   if (warp == 4) {
     // ---- TMA producer: the ring position runs on across tiles
+    const uint32_t on = elect_one();
     bool ok = true;
-    int s = 0;
+    int s = 0, filled = 0;
     uint32_t ph = 1;
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
       const int m0 = (t / cols) * BM, ct = t % cols;
       const int w0 = (ct / tiles_n) * a.J + (ct % tiles_n) * GEMM_BN;   // first weight row of the tile
       for (int i = 0; i < nk; ++i) {
-        ok = mbar_wait_warp(&empty[s], ph);   // passes at once for a stage that has never been filled
+        ok = filled++ < PG_STAGES || mbar_wait_warp(&empty[s], ph);   // (a stage that has never been filled is free)
         if (!ok) break;
-        if (elect_one()) {
-          mbar_expect_tx(&full[s], STAGE);
-          tma_load_2d(smem + s * STAGE, &tma_a, i * BK, m0, &full[s]);
-          tma_load_2d(smem + s * STAGE + A_BYTES, &tma_b, i * BK, w0, &full[s]);
-        }
+        mbar_expect_tx(on, &full[s], STAGE);
+        tma_load_2d(on, smem + s * STAGE, &tma_a, i * BK, m0, &full[s]);
+        tma_load_2d(on, smem + s * STAGE + A_BYTES, &tma_b, i * BK, w0, &full[s]);
         if (++s == PG_STAGES) {
           s = 0;
           ph ^= 1;
@@ -553,7 +552,8 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
   } else if (warp == 5) {
     // ---- MMA issuer: tile `it` of this CTA accumulates into buffer it & 1
     const uint32_t idesc = umma_idesc_i8(BM, GEMM_BN);
-    bool ok = true;
+    const uint32_t on = elect_one();
+    bool ok = true, ready = mbar_test(&full[0], 0);
     int s = 0, it = 0;
     uint32_t ph = 0;
     for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++it) {
@@ -565,22 +565,22 @@ k_mma_gemm_persistent(const __grid_constant__ CUtensorMap tma_a, const __grid_co
       }
       const uint32_t d = tmem + (uint32_t)(buf * GEMM_BN);
       for (int i = 0; i < nk; ++i) {
-        ok = mbar_wait_warp(&full[s], ph);
+        ok = mbar_wait_warp_tested(ready, &full[s], ph);
         if (!ok) break;
         tc_fence_after();
-        const uint64_t da = umma_desc_sw128(smem_u32(smem + s * STAGE));
-        const uint64_t db = umma_desc_sw128(smem_u32(smem + s * STAGE + A_BYTES));
-        if (elect_one()) {
-#pragma unroll
-          for (int kk = 0; kk < BK / 32; ++kk) umma_i8(d, da + 2 * kk, db + 2 * kk, idesc, (i | kk) != 0);
-          umma_commit(&empty[s]);
-        }
+        const int st = s;
         if (++s == PG_STAGES) {
           s = 0;
           ph ^= 1;
         }
+        ready = mbar_test(&full[s], ph);
+        const uint64_t da = umma_desc_sw128(smem_u32(smem + st * STAGE));
+        const uint64_t db = umma_desc_sw128(smem_u32(smem + st * STAGE + A_BYTES));
+#pragma unroll
+        for (int kk = 0; kk < BK / 32; ++kk) umma_i8(on, d, da + 2 * kk, db + 2 * kk, idesc, (i | kk) != 0);
+        umma_commit(on, &empty[st]);
       }
-      if (ok && elect_one()) umma_commit(&acc_full[buf]);
+      if (ok) umma_commit(on, &acc_full[buf]);
     }
     pdl_trigger();
     if (!ok && lane == 0) flag_timeout(a.status);
@@ -874,28 +874,27 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
   } else if (warp == HEAD_EPI_WARPS) {
     // ---- TMA producer: bottleneck operands through the ring, then my block of output-layer weights into
     // the ring's memory, which the bottleneck's MMAs have finished reading by then
+    const uint32_t on = elect_one();
     bool ok = true;
     int s = 0;
     uint32_t ph = 1;
     for (int i = 0; i < nk1 && ok; ++i) {
-      ok = mbar_wait_warp(&empty[s], ph);
+      ok = i < NS || mbar_wait_warp(&empty[s], ph);   // (a stage that has never been filled is free)
       if (!ok) break;
-      if (elect_one()) {
-        mbar_expect_tx(&full[s], STAGE);
-        tma_load_2d(ring + s * STAGE, &tma_h, i * BK, m0, &full[s]);
-        tma_load_2d(ring + s * STAGE + A_BYTES, &tma_wb, i * BK, nb * HEAD_BN1, &full[s]);
-      }
+      mbar_expect_tx(on, &full[s], STAGE);
+      tma_load_2d(on, ring + s * STAGE, &tma_h, i * BK, m0, &full[s]);
+      tma_load_2d(on, ring + s * STAGE + A_BYTES, &tma_wb, i * BK, nb * HEAD_BN1, &full[s]);
       if (++s == NS) {
         s = 0;
         ph ^= 1;
       }
     }
     if (ok && nk1 > 0) ok = mbar_wait_warp(&acc1_full, 0);
-    if (ok && elect_one()) {
-      mbar_expect_tx(&w_full, nk1 > 0 ? 2 * B2_BYTES : 2 * (B2_BYTES + A_BYTES));
+    if (ok) {
+      mbar_expect_tx(on, &w_full, nk1 > 0 ? 2 * B2_BYTES : 2 * (B2_BYTES + A_BYTES));
       for (int kc = 0; kc < 2; ++kc) {
-        if (nk1 == 0) tma_load_2d(ops + kc * BM * BK, &tma_h, kc * BK, m0, &w_full);
-        tma_load_2d(ring + kc * B2_BYTES, &tma_wo, kc * BK, nb * NB, &w_full);
+        if (nk1 == 0) tma_load_2d(on, ops + kc * BM * BK, &tma_h, kc * BK, m0, &w_full);
+        tma_load_2d(on, ring + kc * B2_BYTES, &tma_wo, kc * BK, nb * NB, &w_full);
       }
     }
     pdl_trigger();
@@ -903,40 +902,39 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
   } else if (warp == HEAD_EPI_WARPS + 1) {
     // ---- MMA issuer
     const uint32_t idesc1 = umma_idesc_i8(BM, HEAD_BN1), idesc2 = umma_idesc_i8(BM, NB);
-    bool ok = true;
+    const uint32_t on = elect_one();
+    bool ok = true, ready = mbar_test(&full[0], 0);
     int s = 0;
     uint32_t ph = 0;
     for (int i = 0; i < nk1 && ok; ++i) {
-      ok = mbar_wait_warp(&full[s], ph);
+      ok = mbar_wait_warp_tested(ready, &full[s], ph);
       if (!ok) break;
       tc_fence_after();
-      const uint64_t da = umma_desc_sw128(smem_u32(ring + s * STAGE));
-      const uint64_t db = umma_desc_sw128(smem_u32(ring + s * STAGE + A_BYTES));
-      if (elect_one()) {
-#pragma unroll
-        for (int kk = 0; kk < BK / 32; ++kk) umma_i8(tmem, da + 2 * kk, db + 2 * kk, idesc1, (i | kk) != 0);
-        umma_commit(&empty[s]);
-      }
+      const int st = s;
       if (++s == NS) {
         s = 0;
         ph ^= 1;
       }
+      ready = mbar_test(&full[s], ph);
+      const uint64_t da = umma_desc_sw128(smem_u32(ring + st * STAGE));
+      const uint64_t db = umma_desc_sw128(smem_u32(ring + st * STAGE + A_BYTES));
+#pragma unroll
+      for (int kk = 0; kk < BK / 32; ++kk) umma_i8(on, tmem, da + 2 * kk, db + 2 * kk, idesc1, (i | kk) != 0);
+      umma_commit(on, &empty[st]);
     }
-    if (elect_one()) umma_commit(&acc1_full);
+    umma_commit(on, &acc1_full);
     if (ok) ok = mbar_wait_warp(&w_full, 0);
     if (ok && nk1 > 0) ok = mbar_wait_warp(&ops_ready, 0);
     codes_due = !ok && nk1 > 0;
     tc_fence_after();
-    if (elect_one()) {
 #pragma unroll
-      for (int j = 0; j < HEAD_D / 32; ++j) {
-        const uint64_t da = nk1 > 0 ? umma_desc_sw32(smem_u32(ops + j * BM * HEAD_BN1))
-                                    : umma_desc_sw128(smem_u32(ops + (j >> 2) * BM * BK)) + 2 * (j & 3);
-        const uint64_t db = umma_desc_sw128(smem_u32(ring + (j >> 2) * B2_BYTES)) + 2 * (j & 3);
-        if (ok) umma_i8(tmem + NB, da, db, idesc2, j != 0);
-      }
-      umma_commit(&acc2_full);
+    for (int j = 0; j < HEAD_D / 32; ++j) {
+      const uint64_t da = nk1 > 0 ? umma_desc_sw32(smem_u32(ops + j * BM * HEAD_BN1))
+                                  : umma_desc_sw128(smem_u32(ops + (j >> 2) * BM * BK)) + 2 * (j & 3);
+      const uint64_t db = umma_desc_sw128(smem_u32(ring + (j >> 2) * B2_BYTES)) + 2 * (j & 3);
+      umma_i8(ok ? on : 0u, tmem + NB, da, db, idesc2, j != 0);
     }
+    umma_commit(on, &acc2_full);
     pdl_trigger();
     if (!ok && lane == 0) flag_timeout(a.status);
   } else {
@@ -1277,23 +1275,22 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
   const int x_first = h_first ? nkh : 0, hh_first = h_first ? 0 : nkx;   // first chunk of each part
 
   if (warp == LSTM_EPI_WARPS) {
+    const uint32_t on = elect_one();
     bool ok = true;
     int s = 0;
     uint32_t ph = 1;
     for (int i = 0; i < nk && ok; ++i) {
-      ok = mbar_wait_warp(&empty[s], ph);   // passes at once for a stage that has never been filled
+      ok = i < NS || mbar_wait_warp(&empty[s], ph);   // (a stage that has never been filled is free)
       if (!ok) break;
       const bool xpart = h_first ? i >= nkh : i < nkx;
       if (h_first && i == x_first) pdl_wait();
-      if (elect_one()) {
-        mbar_expect_tx(&full[s], STAGE);
-        if (xpart) {
-          tma_load_2d(smem + s * STAGE, &tma_xa, (i - x_first) * BK, m0, &full[s]);
-          tma_load_2d(smem + s * STAGE + A_BYTES, &tma_xw, (i - x_first) * BK, n0, &full[s]);
-        } else {
-          tma_load_2d(smem + s * STAGE, &tma_ha, (i - hh_first) * BK, m0, &full[s]);
-          tma_load_2d(smem + s * STAGE + A_BYTES, &tma_hw, (i - hh_first) * BK, n0, &full[s]);
-        }
+      mbar_expect_tx(on, &full[s], STAGE);
+      if (xpart) {
+        tma_load_2d(on, smem + s * STAGE, &tma_xa, (i - x_first) * BK, m0, &full[s]);
+        tma_load_2d(on, smem + s * STAGE + A_BYTES, &tma_xw, (i - x_first) * BK, n0, &full[s]);
+      } else {
+        tma_load_2d(on, smem + s * STAGE, &tma_ha, (i - hh_first) * BK, m0, &full[s]);
+        tma_load_2d(on, smem + s * STAGE + A_BYTES, &tma_hw, (i - hh_first) * BK, n0, &full[s]);
       }
       if (++s == NS) {
         s = 0;
@@ -1304,29 +1301,30 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
     if (!ok && lane == 0) flag_timeout(a.status);
   } else if (warp == LSTM_EPI_WARPS + 1) {
     const uint32_t idesc = umma_idesc_i8(BM, LSTM_BN);
-    bool ok = true;
+    const uint32_t on = elect_one();
+    bool ok = true, ready = mbar_test(&full[0], 0);
     int s = 0;
     uint32_t ph = 0;
     for (int i = 0; i < nk && ok; ++i) {
-      ok = mbar_wait_warp(&full[s], ph);
+      ok = mbar_wait_warp_tested(ready, &full[s], ph);
       if (!ok) break;
       tc_fence_after();
-      const uint64_t da = umma_desc_sw128(smem_u32(smem + s * STAGE));
-      const uint64_t db = umma_desc_sw128(smem_u32(smem + s * STAGE + A_BYTES));
-      const bool xpart = h_first ? i >= nkh : i < nkx;
-      const uint32_t d = tmem + (xpart ? 0 : LSTM_BN);
-      const int first = xpart ? x_first : hh_first;
-      if (elect_one()) {
-#pragma unroll
-        for (int kk = 0; kk < BK / 32; ++kk) umma_i8(d, da + 2 * kk, db + 2 * kk, idesc, (i != first) || kk != 0);
-        umma_commit(&empty[s]);
-      }
+      const int st = s;
       if (++s == NS) {
         s = 0;
         ph ^= 1;
       }
+      ready = mbar_test(&full[s], ph);
+      const uint64_t da = umma_desc_sw128(smem_u32(smem + st * STAGE));
+      const uint64_t db = umma_desc_sw128(smem_u32(smem + st * STAGE + A_BYTES));
+      const bool xpart = h_first ? i >= nkh : i < nkx;
+      const uint32_t d = tmem + (xpart ? 0 : LSTM_BN);
+      const int first = xpart ? x_first : hh_first;
+#pragma unroll
+      for (int kk = 0; kk < BK / 32; ++kk) umma_i8(on, d, da + 2 * kk, db + 2 * kk, idesc, (i != first) || kk != 0);
+      umma_commit(on, &empty[st]);
     }
-    if (elect_one()) umma_commit(&acc_full);
+    umma_commit(on, &acc_full);
     pdl_trigger();
     if (!ok && lane == 0) flag_timeout(a.status);
   } else if (warp < LSTM_EPI_WARPS) {

@@ -39,6 +39,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// The same without being suspended until the phase ends (or a time limit): a look ahead
+__device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 // Bounded wait: gives up after `limit` polls and returns false (the caller flags the error
 // and stops waiting for anything else).
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t limit = (1u << 22)) {
@@ -49,32 +61,45 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
   return false;
 }
 
-// One lane of a converged warp.  The loops that issue copies and MMAs are walked by a whole warp with
-// warp-uniform values, and one elected lane issues: the instructions take their operands from uniform
-// registers, and from a loop that a single lane of a divergent branch walks every operand is moved there at
-// each issue.  Measured: an int8 MMA 128 x N x 32 takes 86 clocks from a divergent branch for any N <= 128,
-// 71 (N = 32) to 77 (N = 128) this way; a K chunk (wait, four MMAs, commit) of the LM head 0.31 -> 0.22 us.
-__device__ __forceinline__ bool elect_one() {
+// One lane of a converged warp.  The loops that issue copies and MMAs are walked by a whole warp with warp-uniform values;
+// the instructions themselves are predicated on the elected lane (the forms below with `on` as first argument), not branched
+// over: they take descriptors and coordinates from uniform registers, and inside a branch of one lane that arithmetic is done
+// in ordinary ones and moved for each instruction.  The next stage's barrier is tested before a chunk's MMAs are issued, so
+// that the latency of the answer passes beside them (mbar_test: mbarrier.try_wait would hold the warp while that stage is still
+// on its way, 13 to 20 % of a search).  Clocks per K chunk (wait, four int8 MMAs 128 x N x 32, commit; operands
+// in place, all SMs), N = 32 / 64 / 128: 308 / 318 / 334 with a branch and without the test, 168 / 192 / 256 this way; the
+// tensor cores take 160 / 192 / 256.
+__device__ __forceinline__ uint32_t elect_one() {
   uint32_t p;
   asm volatile(
       "{\n\t.reg .pred P;\n\t.reg .b32 R;\n\t"
       "elect.sync R|P, 0xffffffff;\n\t"
       "selp.b32 %0, 1, 0, P;\n\t}"
       : "=r"(p));
-  return p != 0;
+  return p;
+}
+__device__ __forceinline__ void mbar_expect_tx(uint32_t on, uint64_t* bar, uint32_t bytes) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t"
+      "@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(smem_u32(bar)), "r"(bytes), "r"(on)
+      : "memory");
 }
 __device__ __forceinline__ int uniform_warp() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, uint32_t limit = (1u << 22)) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, limit)) != 0;
 }
+// the same where the barrier has been tested already
+__device__ __forceinline__ bool mbar_wait_warp_tested(bool ready, uint64_t* bar, uint32_t parity, uint32_t limit = (1u << 22)) {
+  return __all_sync(0xffffffffu, ready) != 0 || mbar_wait_warp(bar, parity, limit);
+}
 
 // 2-D tiled TMA load into shared memory, completion counted on an mbarrier.  x is the
 // innermost (contiguous) coordinate and must be a multiple of 16 bytes.
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y,
-                                            uint64_t* bar) {
+__device__ __forceinline__ void tma_load_2d(uint32_t on, void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y)
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n\t}"
+      ::"r"(smem_u32(dst)), "l"(map), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(on)
       : "memory");
 }
 // `bytes` (a multiple of 16) from this CTA's shared memory into the shared memory of a CTA of the cluster by
@@ -135,20 +160,23 @@ __device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t smem_addr) {
 __device__ __forceinline__ uint32_t umma_idesc_i8(int M, int N) {
   return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-// D[tmem] (+)= A[smem] * B[smem]^T, 128 x N x 32 int8, issued by one thread.
-__device__ __forceinline__ void umma_i8(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+// D[tmem] (+)= A[smem] * B[smem]^T, 128 x N x 32 int8, by the lane whose `on` is not 0.
+__device__ __forceinline__ void umma_i8(uint32_t on, uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                         uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "@q tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(on)
       : "memory");
 }
-// Arrive on an mbarrier when all MMAs issued so far by this thread have completed.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
+// Arrive on an mbarrier when all MMAs issued so far by that lane have completed.
+__device__ __forceinline__ void umma_commit(uint32_t on, uint64_t* bar) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(smem_u32(bar)), "r"(on)
+      : "memory");
 }
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp receives lane (base+i).
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, int (&r)[32]) {

@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_tail_blank(const __grid_const
   bool ok = true;
 
   if (warp == TL_WARPS) {
+    const uint32_t on = elect_one();
     int s = 0;
     uint32_t ph = 1, issued = 0;
     for (int g = blockIdx.x; g < n_tiles && ok; g += gridDim.x) {
@@ -95,11 +96,9 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_tail_blank(const __grid_const
       for (int i = 0; i < n_blk; ++i) {
         ok = mbar_wait_warp(&empty[s], ph);   // passes at once for a stage that has never been filled
         if (!ok) break;
-        if (elect_one()) {
-          mbar_expect_tx(&full[s], Z::STAGE);
+        mbar_expect_tx(on, &full[s], Z::STAGE);
 #pragma unroll
-          for (int kc = 0; kc < 2; ++kc) tma_load_2d(ring + s * Z::STAGE + kc * NB * 128, &tma_wo, kc * 128, i * NB, &full[s]);
-        }
+        for (int kc = 0; kc < 2; ++kc) tma_load_2d(on, ring + s * Z::STAGE + kc * NB * 128, &tma_wo, kc * 128, i * NB, &full[s]);
         ++issued;
         if (++s == Z::NS) {
           s = 0;
@@ -112,7 +111,7 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_tail_blank(const __grid_const
       for (uint32_t j = issued - n; j != issued; ++j) mbar_wait_warp(&full[j % Z::NS], (j / Z::NS) & 1);
     }
   } else if (warp == TL_WARPS + 1) {
-    const uint32_t idesc = umma_idesc_i8(TL_BM, NB);
+    const uint32_t idesc = umma_idesc_i8(TL_BM, NB), on = elect_one();
     int s = 0, blk = 0, tile = 0;
     uint32_t ph = 0;
     for (int g = blockIdx.x; g < n_tiles && ok; g += gridDim.x) {
@@ -127,16 +126,14 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_tail_blank(const __grid_const
         if (ok) ok = mbar_wait_warp(&full[s], ph);
         if (!ok) break;
         tc_fence_after();
-        if (elect_one()) {
 #pragma unroll
-          for (int j = 0; j < TL_D / 32; ++j) {
-            const uint64_t da = umma_desc_sw128(smem_u32(ops + (j >> 2) * TL_BM * 128)) + 2 * (j & 3);
-            const uint64_t db = umma_desc_sw128(smem_u32(ring + s * Z::STAGE + (j >> 2) * NB * 128)) + 2 * (j & 3);
-            umma_i8(tmem + buf * NB, da, db, idesc, j != 0);
-          }
-          umma_commit(&empty[s]);
-          umma_commit(&acc_full[buf]);
+        for (int j = 0; j < TL_D / 32; ++j) {
+          const uint64_t da = umma_desc_sw128(smem_u32(ops + (j >> 2) * TL_BM * 128)) + 2 * (j & 3);
+          const uint64_t db = umma_desc_sw128(smem_u32(ring + s * Z::STAGE + (j >> 2) * NB * 128)) + 2 * (j & 3);
+          umma_i8(on, tmem + buf * NB, da, db, idesc, j != 0);
         }
+        umma_commit(on, &empty[s]);
+        umma_commit(on, &acc_full[buf]);
         if (++s == Z::NS) {
           s = 0;
           ph ^= 1;
