@@ -1080,9 +1080,9 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
       if (cs == 0) {   // this CTA's (max, sum) of the row goes to every CTA of the cluster
         const float m = fmaxf(fmaxf(red_m[0][rt], red_m[1][rt]), fmaxf(red_m[2][rt], red_m[3][rt]));
         float ssum = 0.0f;
+        const float top = m > -INFINITY ? m : 0.0f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (red_s[i][rt] > 0.0f) ssum += red_s[i][rt] * __expf(red_m[i][rt] - m);
+        for (int i = 0; i < 4; ++i) ssum += red_s[i][rt] * exp_fast(red_m[i][rt] - top);   // 0 for a share without entries
 #pragma unroll
         for (int r = 0; r < HEAD_CTAS; ++r) {
           cl_store_f32(&part_m[nb][rt], (uint32_t)r, m);
@@ -1101,9 +1101,9 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
 #pragma unroll
       for (int r = 0; r < HEAD_CTAS; ++r) m = fmaxf(m, pm[r]);
       float ssum = 0.0f;
+      const float top = m > -INFINITY ? m : 0.0f;
 #pragma unroll
-      for (int r = 0; r < HEAD_CTAS; ++r)
-        if (ps[r] > 0.0f) ssum += ps[r] * __expf(pm[r] - m);
+      for (int r = 0; r < HEAD_CTAS; ++r) ssum += ps[r] * exp_fast(pm[r] - top);
       lse = m + logf(ssum);
     }
     // A thread's log-probabilities belong to one row and the rows of a warp's lanes are V floats
