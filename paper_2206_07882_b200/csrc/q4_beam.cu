@@ -940,48 +940,6 @@ cudaError_t launch_tsd_select(const BeamSelArgs& a, cudaStream_t s, bool depende
   return le != cudaSuccess ? le : cudaGetLastError();
 }
 
-// Trace-back of the time-synchronous search: a frame-closing call points at the call of the same
-// frame whose blank created the entry; an inner call points at its parent slot of the call before.
-__global__ void k_traceback_tsd(q4_beam_state st, int B, int W, int n_iters, int u_max, int32_t* tokens,
-                                int32_t* lens, float* scores) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b >= B) return;
-  const int S1 = st.tsd_smax + 1;
-  int j = -1, s = -1;
-  float sc = 0.0f;
-  if (st.fin_n[b] > 0) {
-    sc = st.fin_score[b * W];
-    j = st.fin_iter[b * W] - 1;
-    s = st.fin_slot[b * W];
-  } else if (n_iters > 0 && st.row[b * W] >= 0) {
-    sc = st.score[b * W];
-    j = n_iters - 1;
-    s = 0;
-  }
-  int32_t* out = tokens + (size_t)b * u_max;
-  int len = 0;
-  while (j >= 0 && s >= 0) {
-    const size_t h = ((size_t)j * B + b) * W + s;
-    const int k = st.bp_token[h];
-    const int par = st.bp_parent[h];
-    if (j % S1 == S1 - 1) {         // frame close: jump to the set the blank was proposed from
-      j = j - (S1 - 1) + (-1 - k) - 1;
-    } else {
-      if (k > 0 && len < u_max) out[len++] = k;
-      --j;
-    }
-    s = par;
-  }
-  for (int i = 0; i < len / 2; ++i) {
-    const int32_t tmp = out[i];
-    out[i] = out[len - 1 - i];
-    out[len - 1 - i] = tmp;
-  }
-  for (int i = len; i < u_max; ++i) out[i] = 0;
-  lens[b] = len;
-  scores[b] = sc;
-}
-
 __global__ void k_beam_init(q4_beam_state st, int B, int W) {
   const int o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o == 0) st.status[0] = 0;
@@ -1045,17 +1003,21 @@ cudaError_t launch_beam_init(const q4_beam_state& st, int B, int W, int n_iters,
   return cudaGetLastError();
 }
 
-// One warp per utterance.  The walk from the winning slot back to the root is a chain of
-// dependent look-ups; to keep it off the memory latency, the warp first copies the back-pointer
-// rows of 32 consecutive iterations into shared memory (one iteration per lane, all W slots),
-// then lane 0 follows the chain there.
-constexpr int TB_WARPS = 4;
-__global__ void __launch_bounds__(32 * TB_WARPS) k_traceback(q4_beam_state st, int B, int W, int n_iters, int u_max,
-                                                             int32_t* tokens, int32_t* lens, float* scores) {
-  __shared__ int s_par[TB_WARPS][32][MAXW], s_tok[TB_WARPS][32][MAXW];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b = blockIdx.x * TB_WARPS + warp;
-  if (b >= B) return;
+// One CTA per utterance.  The walk from the winning slot back to the root is a chain of dependent look-ups; to keep it off
+// the memory latency, the back-pointers of TB_ITERS consecutive iterations are copied into shared memory (one iteration per
+// thread, the next block's while the present one is walked), then thread 0 follows the chain there, 40 clocks an iteration.
+// 750 iterations: 168 us with 32 iterations per round trip, the strings written as they are found.
+//   TSD: a frame-closing call of the time-synchronous search points at the call of the same frame whose blank created the
+// entry; an inner call points at its parent slot of the call before.
+constexpr int TB_ITERS = 128;
+template <bool TSD>
+__global__ void __launch_bounds__(TB_ITERS) k_traceback(q4_beam_state st, int B, int W, int n_iters, int u_max, int32_t* tokens,
+                                                        int32_t* lens, float* scores) {
+  __shared__ int s_par[TB_ITERS][MAXW + 1], s_tok[TB_ITERS][MAXW + 1];
+  __shared__ int s_out[TB_ITERS];            // labels of the block, last one first
+  __shared__ int s_n, s_slot, s_iter;
+  const int S1 = TSD ? st.tsd_smax + 1 : 1;
+  const int tid = threadIdx.x, b = blockIdx.x;
   int j, s;
   float sc;
   if (st.fin_n[b] > 0) {
@@ -1073,34 +1035,59 @@ __global__ void __launch_bounds__(32 * TB_WARPS) k_traceback(q4_beam_state st, i
   }
   int32_t* out = tokens + (size_t)b * u_max;
   int len = 0;
-  while (j >= 0 && s >= 0) {   // uniform across the warp
-    const int jl = j - lane;
-    if (jl >= 0) {
-      const size_t h = ((size_t)jl * B + b) * W;
-      for (int i = 0; i < W; ++i) {
-        s_par[warp][lane][i] = st.bp_parent[h + i];
-        s_tok[warp][lane][i] = st.bp_token[h + i];
+  int par[MAXW], tok[MAXW];
+  auto fetch = [&](int top) {
+    const int it = top - tid;
+    const size_t h = ((size_t)max(it, 0) * B + b) * W;
+#pragma unroll
+    for (int i = 0; i < MAXW; ++i)
+      if (i < W && it >= 0) {
+        par[i] = st.bp_parent[h + i];
+        tok[i] = st.bp_token[h + i];
       }
-    }
-    __syncwarp();
-    if (lane == 0) {
-      for (int l = 0; l < 32 && j >= 0 && s >= 0; ++l, --j) {
-        const int k = s_tok[warp][l][s];
-        if (k > 0 && len < u_max) out[len++] = k;
-        s = s_par[warp][l][s];
+  };
+  if (j >= 0) fetch(j);
+  for (int top = j; j >= 0 && s >= 0; top -= TB_ITERS) {   // uniform across the block; iterations [top - TB_ITERS + 1, top]
+#pragma unroll
+    for (int i = 0; i < MAXW; ++i)
+      if (i < W) {
+        s_par[tid][i] = par[i];
+        s_tok[tid][i] = tok[i];
       }
+    __syncthreads();
+    if (top >= TB_ITERS) fetch(top - TB_ITERS);
+    if (tid == 0) {
+      int n = 0;
+      while (j > top - TB_ITERS && j >= 0 && s >= 0) {
+        const int k = s_tok[top - j][s], p = s_par[top - j][s];
+        if (TSD && j % S1 == S1 - 1) {   // frame close: to the set the blank was proposed from
+          j = j - (S1 - 1) + (-1 - k) - 1;
+        } else {
+          if (k > 0) s_out[n++] = k;
+          --j;
+        }
+        s = p;
+      }
+      s_n = n;
+      s_slot = s;
+      s_iter = j;
     }
-    j = __shfl_sync(0xffffffffu, j, 0);
-    s = __shfl_sync(0xffffffffu, s, 0);
-    __syncwarp();
+    __syncthreads();
+    const int n = min(s_n, u_max - len);
+    if (tid < n) out[len + tid] = s_out[tid];
+    len += n;
+    s = s_slot;
+    j = s_iter;
+    __syncthreads();
   }
-  if (lane == 0) {
-    for (int i = 0; i < len / 2; ++i) {
-      const int32_t tmp = out[i];
-      out[i] = out[len - 1 - i];
-      out[len - 1 - i] = tmp;
-    }
-    for (int i = len; i < u_max; ++i) out[i] = 0;
+  // the string was found from its end (no more than u_max labels, the last ones of the walk dropped)
+  for (int i = tid; i < len / 2; i += TB_ITERS) {
+    const int32_t a = out[i];
+    out[i] = out[len - 1 - i];
+    out[len - 1 - i] = a;
+  }
+  for (int i = len + tid; i < u_max; i += TB_ITERS) out[i] = 0;
+  if (tid == 0) {
     lens[b] = len;
     scores[b] = sc;
   }
@@ -1109,9 +1096,9 @@ __global__ void __launch_bounds__(32 * TB_WARPS) k_traceback(q4_beam_state st, i
 cudaError_t launch_traceback(const q4_beam_state& st, int B, int W, int n_iters, int u_max,
                              int32_t* tokens, int32_t* lens, float* scores, cudaStream_t s) {
   if (st.nb_score)   // the state of a time-synchronous search
-    k_traceback_tsd<<<(B + 63) / 64, 64, 0, s>>>(st, B, W, n_iters, u_max, tokens, lens, scores);
+    k_traceback<true><<<B, TB_ITERS, 0, s>>>(st, B, W, n_iters, u_max, tokens, lens, scores);
   else
-    k_traceback<<<(B + TB_WARPS - 1) / TB_WARPS, 32 * TB_WARPS, 0, s>>>(st, B, W, n_iters, u_max, tokens, lens, scores);
+    k_traceback<false><<<B, TB_ITERS, 0, s>>>(st, B, W, n_iters, u_max, tokens, lens, scores);
   ++g_launches;
   return cudaGetLastError();
 }
