@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(192, 2) k_state_products(const __grid_constant
       }
       if (!ok && lane == 0) atomicExch(jobs.status, Q4_ERR_TIMEOUT);
     } else if (warp == 5) {
-      const uint32_t idesc = umma_idesc_i8(SP_BM, SP_BN);
+      const uint32_t idesc = umma_idesc_i8(umma_rows(jobs.tile_rows), SP_BN);
       const uint32_t on = elect_one();
       bool ok = true, ready = mbar_test(&full[0], 0);
       int s = 0;
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(192, 2) k_state_products(const __grid_constant
       umma_commit(on, &acc_full);
       if (!ok && lane == 0) atomicExch(jobs.status, Q4_ERR_TIMEOUT);
     } else {
-      const int n = m0 + warp * 32 + lane;
+      const int n = m0 + umma_lane_row(umma_rows(jobs.tile_rows), warp, lane);
       const int dst = n < n_work ? jobs.dst_row[n] : -1;
       const bool ok = mbar_wait_warp(&acc_full, 0);
       tc_fence_after();

@@ -328,6 +328,7 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
   const int tid = threadIdx.x, warp = uniform_warp(), lane = tid & 31;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * GEMM_BN;   // row tiles slowest: tiles with work are dispatched first
   const int nk = (a.K + BK - 1) / BK;
+  const int mm = umma_rows(a.M);
   if (tile_without_work(a.n_active, m0)) return;
 
   if (tid == 0) {
@@ -370,7 +371,7 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
     pdl_trigger();
     if (!ok && lane == 0) flag_timeout(a.status);
   } else if (warp == 5) {
-    const uint32_t idesc = umma_idesc_i8(BM, GEMM_BN);
+    const uint32_t idesc = umma_idesc_i8(mm, GEMM_BN);
     const uint32_t on = elect_one();
     bool ok = true, ready = mbar_test(&full[0], 0);
     int s = 0;
@@ -410,7 +411,7 @@ k_mma_gemm(const __grid_constant__ CUtensorMap tma_a, const __grid_constant__ CU
     tc_fence_after();
     pdl_trigger();   // the main loop is over: the next kernel may set itself up
     if (!ok && lane == 0) flag_timeout(a.status);
-    const int mi = m0 + warp * 32 + lane;
+    const int mi = m0 + umma_lane_row(mm, warp, lane);
     int m = -1;
     if (mi < a.M && !(a.n_active && mi >= *a.n_active)) m = a.out_idx ? a.out_idx[mi] : mi;
     const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
@@ -839,6 +840,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
   const int m0 = blockIdx.y * BM;
   const int nb = blockIdx.x;                    // my blocks of columns = my cluster rank
   const int nk1 = (a.H + BK - 1) / BK;
+  const int mm = umma_rows(a.tile_rows);
   if (tile_without_work(a.n_active, m0)) return;   // the whole cluster leaves
 
   if (tid == 0) {
@@ -901,7 +903,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
     if (!ok && lane == 0) flag_timeout(a.status);
   } else if (warp == HEAD_EPI_WARPS + 1) {
     // ---- MMA issuer
-    const uint32_t idesc1 = umma_idesc_i8(BM, HEAD_BN1), idesc2 = umma_idesc_i8(BM, NB);
+    const uint32_t idesc1 = umma_idesc_i8(mm, HEAD_BN1), idesc2 = umma_idesc_i8(mm, NB);
     const uint32_t on = elect_one();
     bool ok = true, ready = mbar_test(&full[0], 0);
     int s = 0;
@@ -940,7 +942,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
   } else {
     // ---- epilogue: warp = (lane quarter q, column share cs)
     const int q = warp & 3, cs = warp >> 2;
-    const int rt = q * 32 + lane;
+    const int rt = umma_lane_row(mm, q, lane);
     const int n = m0 + rt;
     int dst = -1;
     if (n < a.N && !(a.n_active && n >= *a.n_active)) dst = a.dst_row ? a.dst_row[n] : n;
@@ -1241,6 +1243,7 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
   const int nkx = a.acc_pre ? 0 : (a.Kx_pad + BK - 1) / BK;
   const int nkh = HH_MEM ? 0 : (a.H + BK - 1) / BK;
   const int nk = nkx + nkh;
+  const int mm = umma_rows(a.tile_rows);
   if (tile_without_work(a.n_active, m0)) return;
 
   if (tid == 0) {
@@ -1300,7 +1303,7 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
     pdl_trigger();
     if (!ok && lane == 0) flag_timeout(a.status);
   } else if (warp == LSTM_EPI_WARPS + 1) {
-    const uint32_t idesc = umma_idesc_i8(BM, LSTM_BN);
+    const uint32_t idesc = umma_idesc_i8(mm, LSTM_BN);
     const uint32_t on = elect_one();
     bool ok = true, ready = mbar_test(&full[0], 0);
     int s = 0;
@@ -1330,7 +1333,7 @@ k_mma_lstm(const __grid_constant__ CUtensorMap tma_xa, const __grid_constant__ C
   } else if (warp < LSTM_EPI_WARPS) {
     if (h_first) pdl_wait();   // the row lists and cell states below are read after it, beside the input half
     const int q = warp & 3, hf = warp >> 2;
-    const int rt = q * 32 + lane;            // row within the tile
+    const int rt = umma_lane_row(mm, q, lane);   // row within the tile
     const int n = m0 + rt;                   // row of this launch
     int src = -1, dst = -1;
     if (n < a.N && !(a.n_active && n >= *a.n_active)) {

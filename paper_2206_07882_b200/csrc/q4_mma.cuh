@@ -156,11 +156,20 @@ __device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t smem_addr) {
   d |= (uint64_t)6 << 61;                               // layout: 32-byte swizzle
   return d;
 }
+// Tiles of at most 16 rows are multiplied as 64-row tiles: an MMA of 32, 64 or 128 weight rows takes 24 / 32 / 64 clocks
+// instead of 40 / 48 / 64 (measured; the rows' way into the tensor cores bounds the narrow ones).  Row r is lane
+// 32 (r / 16) + r % 16 of tensor memory there; the other lanes hold nothing and stand for the rows from 64 on.  With more rows
+// than the 16 of a lane quarter the epilogue works on half-filled warps: 160 frames of one utterance at beam 16 3.72 ->
+// 3.60 ms, beam 1 1.89 -> 1.85, but 8 x 8 rows 3.86 -> 3.90.
+__host__ __device__ constexpr int umma_rows(int tile_rows) { return tile_rows <= 16 ? 64 : 128; }
+__device__ __forceinline__ int umma_lane_row(int m, int quarter, int lane) {   // row of a warp's lane, m = umma_rows()
+  return m == 128 ? 32 * quarter + lane : lane < 16 ? 16 * quarter + lane : 48 + 16 * quarter + lane;
+}
 // Instruction descriptor: signed 8-bit A and B, both K-major, int32 accumulate, M x N tile.
 __device__ __forceinline__ uint32_t umma_idesc_i8(int M, int N) {
   return (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-// D[tmem] (+)= A[smem] * B[smem]^T, 128 x N x 32 int8, by the lane whose `on` is not 0.
+// D[tmem] (+)= A[smem] * B[smem]^T, M x N x 32 int8 (M, N: see umma_idesc_i8), by the lane whose `on` is not 0.
 __device__ __forceinline__ void umma_i8(uint32_t on, uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                         uint32_t accumulate) {
   asm volatile(
