@@ -241,8 +241,9 @@ typedef struct {
 /* Optional one-time weight preparation for the tensor-core search path (weights are
  * quantized once, activations at every step: Section 3.2).  Writes int8, gate-interleaved
  * copies of the step weights into `buffer` (device, q4_prepared_bytes(model) bytes, owned by
- * the caller, must outlive the model's use) and sets model->prepared.  With prepared == NULL
- * the search uses the DP4A kernels on the packed weights. */
+ * the caller, must outlive the model's use) and sets model->prepared.  Up to 4096 labels it holds the input halves of the first
+ * LSTM layers as well, one fp32 row per label and network (16 H bytes), made from the embedding tables, which must be set
+ * before the call and not change after it.  With prepared == NULL the search uses the DP4A kernels on the packed weights. */
 size_t q4_prepared_bytes(const q4_model* model);
 int q4_prepare_model(q4_model* model, void* buffer, size_t bytes, q4_stream stream);
 

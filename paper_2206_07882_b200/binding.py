@@ -721,6 +721,11 @@ class Decoder:
                                   C.c_float(dw.rho), C.c_int32(1 if time_synchronous else 0), _p(self.ws),
                                   C.c_size_t(self.ws.numel()), plan, _stream()), "q4_beam_search")
 
+    def search_steps_taken(self) -> int:
+        """Steps that the last looped search on this state ran before its label-free end (waits for the device)."""
+        iteration = int(self.ws[16:20].view(torch.int32).item())     # of the call block, a group of 12 steps behind
+        return iteration + 12
+
     def search_plan_info(self) -> dict:
         """Graphs built, replays enqueued and failed builds of the decoder's search plan."""
         out = (C.c_int64 * 3)()

@@ -977,8 +977,10 @@ static bool search_uses_tensor_cores(const q4_model& m, const q4_beam_state& st,
 static int32_t* search_frozen(void* workspace) { return reinterpret_cast<int32_t*>(static_cast<uint8_t*>(workspace) + 256); }
 
 // Whether a whole search takes the kernels that look the first layers' input halves up and keep the sums of the recurrent
-// halves per state row: tables with the prepared weights and room for the sums.
-static bool search_keeps_sums(const q4_model& m, const q4_beam_state& st, int B, int W, size_t workspace_bytes) {
+// halves per state row: tables with the prepared weights and room for the sums, both read 32 bytes at a time.
+static bool search_keeps_sums(const q4_model& m, const q4_beam_state& st, int B, int W, const void* workspace,
+                              size_t workspace_bytes) {
+  if ((reinterpret_cast<uintptr_t>(workspace) | reinterpret_cast<uintptr_t>(m.prepared)) & 31u) return false;
   const int RW = st.rows_per_utt > 0 ? st.rows_per_utt : 2 * W;
   const int32_t dims9[9] = {B, W, m.V, m.D, m.pred_lstm.w_ih.k_pad, m.pred_lstm.w_hh.k_pad, m.src.lstm[0].w_hh.k_pad,
                             m.tgt.lstm[0].w_hh.k_pad, RW};
@@ -1709,9 +1711,9 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
   for (int i = 0; i < 3; ++i) key.state.aux_event[i] = p && lent ? p->side_event[i] : nullptr;
   // An alignment-length synchronous search ends its steps when no utterance has labels left to propose; the iterations
   // that are left then are carried out together.
-  const bool sums = search_keeps_sums(*model, *state, B, W, workspace_bytes);
+  const bool sums = search_keeps_sums(*model, *state, B, W, workspace, workspace_bytes);
   key.sums = sums;
-  key.loop = p && !key.tsd && !key.exact && search_tail_supported(model->V, model->D) &&
+  key.loop = p && !key.tsd && !key.exact && search_tail_supported(model->V, model->D) && aligned16(state->pred_p) &&
              (sums || search_uses_tensor_cores(*model, *state, B, W, workspace_bytes));
   // step by step: while launches are timed or waits are made to run out (a graph would keep that), in a short search, and
   // without a loop in a stream that is being captured

@@ -991,3 +991,37 @@ def test_search_with_embeddings_of_other_row_lengths(Bd):
     assert dd.pred_lstm.w_ih.k_pad != dd.src.lstm[0].w_ih.k_pad
     frac, tr = compare_search(dd, tokens, lens, scores, ref, list(range(3)), 12, 5, 8, min_same=1.0)
     assert tr == 1.0
+
+
+@pytest.mark.parametrize("what", ["workspace", "prepared", "pred_p"])
+def test_search_with_buffers_at_smaller_alignments(Bd, what):
+    # a workspace or prepared weights at a 16-byte boundary, projected prediction rows at an 8-byte one: kernels that move more
+    # at a time are not taken, the beams are the same
+    import ctypes as C
+    dw = synth.decoder(seed=97, V=300, E=32, Hp=128, D=256, Hs=128, Ht=128, tgt_layers=2, U_max=9, W=6)
+    dw.joint.out.bias[0] += np.float32(3.0)
+    e = torch.from_numpy(synth.Stream(33).normal("e", (100, 3, 256)).astype(np.float32)).cuda()
+    a, b = Bd.Decoder(dw), Bd.Decoder(dw)
+    want = b.decode(e)
+    a.alloc_state(3, 6, 109)
+    shift = 8 if what == "pred_p" else 16
+
+    def moved(t):
+        big = torch.zeros(t.numel() * t.element_size() + 32, dtype=torch.uint8, device="cuda")
+        return big[shift:shift + t.numel() * t.element_size()].view(t.dtype).view(t.shape)
+
+    if what == "workspace":
+        a.ws = moved(a.ws)
+    elif what == "prepared":
+        a.prepared = moved(a.prepared)
+        assert Bd.lib().q4_prepare_model(C.byref(a.model), C.c_void_p(a.prepared.data_ptr()), C.c_size_t(a.prepared.numel()), None) == 0
+        torch.cuda.synchronize()
+    else:
+        a.tensors["pred_p"] = moved(a.tensors["pred_p"])
+        a.state.pred_p = a.tensors["pred_p"].data_ptr()
+    got = a.decode(e)
+    for x, y in zip(got, want):
+        assert torch.equal(x, y)
+    assert a.tensors["status"].item() == 0
+    for k in ("bp_parent", "bp_token", "bp_score"):
+        assert torch.equal(a.tensors[k][:109], b.tensors[k][:109]), k
