@@ -982,10 +982,9 @@ k_enc_recurrent_few(const EncRecArgs a) {
   extern __shared__ __align__(16) uint8_t rec_smem[];
   constexpr int BG = REC_BG, H = 32 * KS, G = 4 * H;
   constexpr int cpc = H / CL;               // cells per CTA
-  constexpr int NTHR = 8 * cpc, CW = NTHR / 32;
+  constexpr int NTHR = 8 * cpc;
   constexpr int UB = BG * H, MB = BG * cpc; // bytes of the group's hidden codes, of this CTA's part
-  constexpr int PIECES = MB / 16;           // of this CTA's codes
-  static_assert(cpc % 8 == 0 && PIECES * CL <= NTHR, "units of 8 cells; a thread sends at most one piece");
+  static_assert(cpc % 8 == 0 && 4 * CL <= 64 && cpc / 8 < 16, "two warps a unit of 8 cells, a barrier each; a thread sends at most one piece");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = cluster_rank();
   const int cid = blockIdx.x / CL;
@@ -1044,6 +1043,24 @@ k_enc_recurrent_few(const EncRecArgs a) {
   const int ylo = act_lo(a.out_act), yhi = act_hi(a.out_act);
   const bool y4 = a.out_act.bits == 4;
   const int at = (cl >> 3) * 64 + n * 8 + (cl & 7);      // my code within the CTA's part
+  const int unit = warp >> 1, tstep = d == 0 ? 1 : -1;
+  auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + unit) : "memory"); };
+  // one sequence's output codes of this unit of 8 cells, by the first 8 lanes of a warp
+  auto store_y = [&](int buf, int t) {
+    const int by = grp * BG + lane, c0 = (int)rank * cpc + unit * 8;
+    if (lane >= 8 || by >= B) return;
+    const uint2 v = *reinterpret_cast<const uint2*>(stage_y + buf * MB + unit * 64 + lane * 8);
+    uint8_t* y = D.yq + ((size_t)t * B + by) * a.yq_ld;
+    if (y4) {
+      auto pk = [](uint32_t x) -> uint32_t {   // bytes (c, c+1) -> one byte: low nibble c, high nibble c+1
+        const uint32_t m = (x & 0x000F000Fu) | ((x >> 4) & 0x00F000F0u);
+        return (m & 0xFFu) | ((m >> 8) & 0xFF00u);
+      };
+      *reinterpret_cast<uint32_t*>(y + (c0 >> 1)) = pk(v.x) | (pk(v.y) << 16);
+    } else {
+      *reinterpret_cast<uint2*>(y + c0) = v;
+    }
+  };
   float c_state = 0.0f;
   int q = 0;
   // input accumulators of my item, fetched one step ahead
@@ -1102,46 +1119,35 @@ k_enc_recurrent_few(const EncRecArgs a) {
       hh[2] = e ? r1 : m1;
       hh[3] = e ? m1 : r1;
     }
-    int q2 = 0;
+    float hval = 0.0f;
     if (live) {
       const float pi = __fmaf_rn((float)hh[0], s_hh.x, __fmaf_rn((float)pre.x, s_ih.x, bb.x));
       const float pf = __fmaf_rn((float)hh[1], s_hh.y, __fmaf_rn((float)pre.y, s_ih.y, bb.y));
       const float pg = __fmaf_rn((float)hh[2], s_hh.z, __fmaf_rn((float)pre.z, s_ih.z, bb.z));
       const float po = __fmaf_rn((float)hh[3], s_hh.w, __fmaf_rn((float)pre.w, s_ih.w, bb.w));
-      float hval;
       cell_fixed_p(pi, pf, pg, po, c_state, c_state, hval);
       q = quantize1(hval, a.hid_act.inv_scale, a.hid_act.zero_point, hlo, hhi);
-      q2 = quantize1(hval, a.out_act.inv_scale, a.out_act.zero_point, ylo, yhi);
     }
-    // staged by step parity; every thread then sends one 16-byte piece of this CTA's codes to one CTA.  The pieces of a
-    // destination belong to consecutive lanes: their stores travel together.
+    // staged by step parity; the two warps of a unit then send its 16-byte pieces, a destination's on consecutive lanes.
+    // Only they wait for one another.
     stage[cur * MB + at] = (int8_t)q;
+    pair_sync();
+    if ((tid & 63) < 4 * CL) {
+      const uint32_t r = (uint32_t)(tid & 63) >> 2;
+      const int off = unit * 64 + (tid & 3) * 16;
+      st_async_v4(map_to_rank(hb_addr + (uint32_t)(nxt * UB + (int)rank * MB + off), r),
+                  *reinterpret_cast<const uint4*>(stage + cur * MB + off), map_to_rank(full_addr + (uint32_t)(nxt * 8), r));
+    }
+    // the output codes of the step before, complete since the barrier above; this step's are made while its recurrent
+    // codes travel
+    if (step > 0 && (warp & 1) == cur) store_y(nxt, t - tstep);
+    int q2 = 0;
+    if (live) q2 = quantize1(hval, a.out_act.inv_scale, a.out_act.zero_point, ylo, yhi);
     stage_y[cur * MB + at] = (int8_t)q2;
-    __syncthreads();
-    if (tid < PIECES * CL) {
-      const uint32_t r = (uint32_t)(tid / PIECES);
-      const int ch = tid % PIECES;
-      st_async_v4(map_to_rank(hb_addr + (uint32_t)(nxt * UB + (int)rank * MB + ch * 16), r),
-                  *reinterpret_cast<const uint4*>(stage + cur * MB + ch * 16), map_to_rank(full_addr + (uint32_t)(nxt * 8), r));
-    }
-    // one warp, a different one every step, writes this CTA's share of the layer output
-    if (warp == step % CW) {
-      for (int i = lane; i < MB / 8; i += 32) {
-        const int bl = i & 7, by = grp * BG + bl, c0 = (int)rank * cpc + (i & ~7);
-        if (by >= B) continue;
-        const uint2 v = *reinterpret_cast<const uint2*>(stage_y + cur * MB + i * 8);
-        uint8_t* y = D.yq + ((size_t)t * B + by) * a.yq_ld;
-        if (y4) {
-          auto pk = [](uint32_t x) -> uint32_t {   // bytes (c, c+1) -> one byte: low nibble c, high nibble c+1
-            const uint32_t m = (x & 0x000F000Fu) | ((x >> 4) & 0x00F000F0u);
-            return (m & 0xFFu) | ((m >> 8) & 0xFF00u);
-          };
-          *reinterpret_cast<uint32_t*>(y + (c0 >> 1)) = pk(v.x) | (pk(v.y) << 16);
-        } else {
-          *reinterpret_cast<uint2*>(y + c0) = v;
-        }
-      }
-    }
+  }
+  if (T > 0) {
+    pair_sync();
+    if ((warp & 1) == 0) store_y((T - 1) & 1, d == 0 ? T - 1 : 0);
   }
   pdl_trigger();
   // the codes sent in the last step are still on their way: nobody leaves before they have landed (bounded)
