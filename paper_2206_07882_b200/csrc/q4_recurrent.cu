@@ -983,12 +983,8 @@ k_enc_recurrent_few(const EncRecArgs a) {
   constexpr int BG = REC_BG, H = 32 * KS, G = 4 * H;
   constexpr int cpc = H / CL;               // cells per CTA
   constexpr int NTHR = 8 * cpc;
-  // With four warps on every scheduler half of them multiply first and update their cells while the others multiply (32
-  // utterances x 500 frames 6.05 -> 5.93 ms).  Of two or three warps the two halves' chains of MMAs would add up
-  // (11 x 173 1.40 -> 1.38 ms, but one utterance 1.06 -> 1.08).
-  constexpr bool halves = NTHR == 512;
   constexpr int UB = BG * H, MB = BG * cpc; // bytes of the group's hidden codes, of this CTA's part
-  static_assert(cpc % 8 == 0 && 4 * CL <= 64 && cpc / 8 < 15, "two warps a unit of 8 cells, a barrier each; a thread sends at most one piece");
+  static_assert(cpc % 8 == 0 && 4 * CL <= 64 && cpc / 8 < 16, "two warps a unit of 8 cells, a barrier each; a thread sends at most one piece");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = cluster_rank();
   const int cid = blockIdx.x / CL;
@@ -1104,14 +1100,12 @@ k_enc_recurrent_few(const EncRecArgs a) {
     for (int c = 0; c < 2; ++c)
 #pragma unroll
       for (int r = 0; r < 4; ++r) acc[c][r] = 0;
-    if (halves && warp >= NTHR / 64) asm volatile("bar.sync 15, %0;" ::"n"(NTHR) : "memory");
     const int8_t* hrow = hb + cur * UB + t4 * 64 + g * 8;
 #pragma unroll
     for (int s = 0; s < KS; ++s) {
       const uint2 v = *reinterpret_cast<const uint2*>(hrow + 256 * s);
       mma_s8(acc[s & 1], w[4 * s], w[4 * s + 1], w[4 * s + 2], w[4 * s + 3], v.x, v.y);
     }
-    if (halves && warp < NTHR / 64) asm volatile("bar.arrive 15, %0;" ::"n"(NTHR) : "memory");
     // the four gates of my item: two of them come from lane ^ 4
     int hh[4];
     {
