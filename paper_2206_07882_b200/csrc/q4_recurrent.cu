@@ -965,8 +965,10 @@ __device__ __forceinline__ void st_async_v4(uint32_t addr, uint4 v, uint32_t bar
 // 16, 11 of 10) that is the better split.  Narrower layers take clusters of 32 or 40 cells per CTA.  The codes travel as
 // 16-byte st.async stores, a destination's on consecutive lanes: an exchange alone takes 840 cycles among 16 CTAs, against
 // 1270 as one bulk copy per destination (the engine takes them one by one) and 1300 with a lane's destinations
-// interleaved.  Whole encoders of 6 layers: 11 utterances x 173 frames 2.27 -> 1.50 ms (16 CTAs; 1.62 with bulk
-// copies), 32 x 500 6.65 -> 6.06 ms (10 CTAs); one layer of 128 cells, 50 steps with its projection: 92 -> 44 us (4 CTAs; 76
+// interleaved.  The two warps of 8 cells wait for one another only and send their unit at once; the output codes are made
+// while it travels (a block barrier, output codes first and one warp storing them: 1.505 and 6.07 ms below).  Whole encoders
+// of 6 layers: 11 utterances x 173 frames 2.27 -> 1.39 ms (16 CTAs; 1.62 with bulk copies and a block barrier), 32 x 500
+// 6.65 -> 6.04 ms (10 CTAs: clusters of 11 and more have room for 7, not 8); one layer of 128 cells, 50 steps with its projection: 92 -> 44 us (4 CTAs; 76
 // on one CTA without any exchange, whose 32 warps are bound by issue slots).
 //
 // A CTA owns cpc = H / CL cells, a warp 4 of them: its 16 weight rows stay in registers as the int8 A fragments
