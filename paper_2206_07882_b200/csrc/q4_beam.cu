@@ -228,8 +228,11 @@ __device__ __forceinline__ int list_rank(const uint64_t* list, int ln, uint64_t 
   for (int j = 0; j < ln; ++j) rank += list[j] > mine;
   return rank;
 }
-// entries of the short list; smaller vocabularies have as many proposals near the bound as large ones
-__host__ __device__ constexpr int sel_list_cap(int V) { return 16 * ((V + 31) / 32) > 512 ? 16 * ((V + 31) / 32) : 512; }
+// Entries of the short list: what the exact threshold can leave (W heads, each with a strided share of its slot's labels);
+// smaller vocabularies have as many proposals near the bound as large ones.  By W, so that the list and its entries (12
+// bytes) leave room for every W x V that a step takes (200 KB of increments): with 16 shares for every W a beam of 8 took
+// 6016 labels, a beam of 1 22848 instead of 51200.
+__host__ __device__ constexpr int sel_list_cap(int W, int V) { return W * ((V + 31) / 32) > 512 ? W * ((V + 31) / 32) : 512; }
 
 // End of the last step of a graph's loop, by one thread of each utterance after all that it does: the last one
 // advances the call and asks for another turn.  (As a kernel of its own 2 us a turn.)  Every utterance is frozen by
@@ -331,7 +334,7 @@ template <int MODE, int NE>
 __global__ void __launch_bounds__(SEL_THREADS, 1) k_beam_select(const __grid_constant__ BeamSelArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int W = a.W, V = a.V;
-  const int cap = sel_list_cap(V);
+  const int cap = sel_list_cap(W, V);
   uint64_t* list = reinterpret_cast<uint64_t*>(smem_raw);                   // keys of the proposals that pass the bound
   uint32_t* entry = reinterpret_cast<uint32_t*>(list + cap);
   float* cand = reinterpret_cast<float*>(entry + cap);                      // [W * V] increments of the labels
@@ -607,7 +610,7 @@ static int sel_form(const BeamSelArgs& a) {
   return wide && a.normalized ? SEL_WIDE : SEL_1024;
 }
 static size_t sel_smem(const BeamSelArgs& a) {
-  return (size_t)sel_list_cap(a.V) * (sizeof(uint64_t) + sizeof(uint32_t)) + (size_t)a.W * a.V * sizeof(float);
+  return (size_t)sel_list_cap(a.W, a.V) * (sizeof(uint64_t) + sizeof(uint32_t)) + (size_t)a.W * a.V * sizeof(float);
 }
 static cudaError_t sel_launch(void (*kern)(const BeamSelArgs), size_t (&configured_on)[MAX_DEVICES], const BeamSelArgs& a,
                               cudaStream_t s, bool dependent) {
@@ -646,7 +649,7 @@ template <int MODE, int NE>
 __global__ void __launch_bounds__(SEL_THREADS, 1) k_tsd_select(const __grid_constant__ BeamSelArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int W = a.W, V = a.V;
-  const int cap = sel_list_cap(V);
+  const int cap = sel_list_cap(W, V);
   uint64_t* list = reinterpret_cast<uint64_t*>(smem_raw);                   // keys of the proposals that pass the bound
   uint32_t* entry = reinterpret_cast<uint32_t*>(list + cap);
   float* cand = reinterpret_cast<float*>(entry + cap);                      // [W * V] increments of the labels

@@ -292,6 +292,25 @@ def test_tensor_core_search_odd_vocabulary(Bd, V, D):
     assert tr == 1.0
 
 
+@pytest.mark.parametrize("W,V", [(1, 28940), (2, 19296), (4, 11579), (8, 6400), (12, 4266), (16, 3200), (1, 51200)])
+@pytest.mark.parametrize("S,H", [(None, 128), (1, 32)])
+def test_search_of_the_largest_vocabularies(Bd, W, V, S, H):
+    # the widest vocabularies that the selection's shared memory held once, and the last one that the argument check
+    # (200 KB for W x V) lets pass: every beam of every iteration as the oracle's
+    dw = synth.decoder(seed=65, V=V, E=32, Hp=H, D=32, Hs=H, Ht=H, tgt_layers=1, U_max=4, W=W)
+    e = synth.Stream(W + V).normal("e", (5, 2, 32)).astype(np.float32)
+    if S is None:
+        dd, tokens, lens, scores, ref = run_search(Bd, dw, e)
+        frac, tr = compare_search(dd, tokens, lens, scores, ref, [0, 1], 5, 4, W, min_same=1.0)
+    else:
+        dd, tokens, lens, scores, ref = run_tsd(Bd, dw, e, S)
+        tr = compare_tsd(dd, tokens, lens, scores, ref, [0, 1], 5, S, W)
+    assert tr == 1.0
+    dw = synth.decoder(seed=65, V=200 * 256 // W + 1, E=32, Hp=32, D=32, Hs=32, Ht=32, tgt_layers=1, U_max=4, W=W)
+    with pytest.raises(Bd.Q4Error):
+        Bd.Decoder(dw).decode(torch.from_numpy(e).cuda())
+
+
 def test_search_without_frames(Bd):
     # no frames and, in the alignment-length search, no label budget: no steps, every utterance's string is empty
     dw = synth.decoder(seed=64, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=5, W=8)
