@@ -236,16 +236,23 @@ typedef struct {
   q4_linear joint_out; /* D -> V */
   q4_lm src, tgt;
   void* prepared; /* NULL, or the buffer filled by q4_prepare_model (tensor-core operands) */
+  void* tables;   /* NULL, or the buffer filled by q4_prepare_tables; read with prepared set only */
 } q4_model;
 
 /* Optional one-time weight preparation for the tensor-core search path (weights are
  * quantized once, activations at every step: Section 3.2).  Writes int8, gate-interleaved
  * copies of the step weights into `buffer` (device, q4_prepared_bytes(model) bytes, owned by
- * the caller, must outlive the model's use) and sets model->prepared.  Up to 4096 labels it holds the input halves of the first
- * LSTM layers as well, one fp32 row per label and network (16 H bytes), made from the embedding tables, which must be set
- * before the call and not change after it.  With prepared == NULL the search uses the DP4A kernels on the packed weights. */
+ * the caller, must outlive the model's use), sets model->prepared and clears model->tables.  The embedding tables are not read.
+ * With prepared == NULL the search uses the DP4A kernels on the packed weights. */
 size_t q4_prepared_bytes(const q4_model* model);
 int q4_prepare_model(q4_model* model, void* buffer, size_t bytes, q4_stream stream);
+/* Optional, after q4_prepare_model: the input halves of the first LSTM layers for every label (one fp32 row per label and
+ * network, 16 H bytes), which whole searches of few rows look up instead of multiplying embedding rows.  `buffer`: device,
+ * 32-byte aligned, q4_table_bytes(model, rows) bytes, owned by the caller; sets model->tables.  q4_table_bytes is 0 where a
+ * search of `rows` = B W rows takes no tables (above 384 rows or 4096 labels, widths that are no multiples of 128).  The tables
+ * are made from the embedding tables as they are at the call: when those change, call it again, or set tables to NULL. */
+size_t q4_table_bytes(const q4_model* model, int32_t rows);
+int q4_prepare_tables(q4_model* model, void* buffer, size_t bytes, q4_stream stream);
 
 /*
  * Caller-owned search state for B utterances x W beam slots.  R = B * 2W "state rows" hold

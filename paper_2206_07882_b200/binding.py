@@ -56,7 +56,7 @@ class ModelS(C.Structure):
     _fields_ = [("V", C.c_int32), ("E", C.c_int32), ("D", C.c_int32), ("pred_emb_q", C.c_void_p),
                 ("pred_emb_act", Act), ("pred_lstm", LstmS), ("pred_proj", LinearS),
                 ("z_act", Act), ("joint_out", LinearS), ("src", LmS), ("tgt", LmS),
-                ("prepared", C.c_void_p)]
+                ("prepared", C.c_void_p), ("tables", C.c_void_p)]
 
 
 class BeamStateS(C.Structure):
@@ -81,7 +81,7 @@ class BeamStateS(C.Structure):
 EXPORTS = ["q4_act_symmetric", "q4_act_asymmetric", "quantize_pack_int4", "qlstm_layer_forward",
            "qlstm_step", "q4_linear_forward", "qjoint_logprobs", "q4_beam_init",
            "dr_fusion_beam_step", "q4_beam_search", "q4_search_plan_create", "q4_search_plan_destroy", "q4_search_plan_info", "q4_traceback", "q4_feature_prologue", "q4_workspace_bytes",
-           "q4_poll_status", "q4_version", "q4_launch_count", "q4_dependent_launch_set", "q4_beam_select_exact_set", "q4_timing_set", "q4_timing_count", "q4_prepared_bytes", "q4_prepare_model", "qjoint_logprobs_static", "q4_quantizer_calls", "q4_prepared_lstm_bytes", "q4_prepare_lstm",
+           "q4_poll_status", "q4_version", "q4_launch_count", "q4_dependent_launch_set", "q4_beam_select_exact_set", "q4_timing_set", "q4_timing_count", "q4_prepared_bytes", "q4_prepare_model", "q4_table_bytes", "q4_prepare_tables", "qjoint_logprobs_static", "q4_quantizer_calls", "q4_prepared_lstm_bytes", "q4_prepare_lstm",
            "q4_prepared_linear_bytes", "q4_prepare_linear", "q4_test_wait_expiry_set", "q4_encoder_time_slicing_set", "q4_encoder_recurrence_plan"]
 
 _lib = None
@@ -98,6 +98,7 @@ def lib() -> C.CDLL:
         _lib.q4_workspace_bytes.restype = C.c_size_t
         _lib.q4_launch_count.restype = C.c_int64
         _lib.q4_prepared_bytes.restype = C.c_size_t
+        _lib.q4_table_bytes.restype = C.c_size_t
         _lib.q4_quantizer_calls.restype = C.c_int64
         _lib.q4_prepared_lstm_bytes.restype = C.c_size_t
         _lib.q4_prepared_linear_bytes.restype = C.c_size_t
@@ -593,7 +594,7 @@ class Decoder:
         if share_from is not None:
             # a second search state over the same device weights (read-only, prepared operands included)
             for name in ("V", "E", "D", "pred_emb_act", "pred_emb_q", "pred_lstm", "pred_proj", "z_act", "joint_out",
-                         "src", "tgt", "model", "prepared"):
+                         "src", "tgt", "model", "prepared", "tables"):
                 setattr(self, name, getattr(share_from, name))
             return
         self.V, self.E = dw.pred.emb.shape
@@ -612,19 +613,30 @@ class Decoder:
         m.pred_lstm, m.pred_proj = self.pred_lstm.c(), self.pred_proj.c()
         m.z_act, m.joint_out = self.z_act, self.joint_out.c()
         m.src, m.tgt = self.src.c(), self.tgt.c()
-        m.prepared = None
+        m.prepared = m.tables = None
         self.prepared = None
+        self.tables = []        # the buffer of q4_prepare_tables, shared with the decoders that share the weights
         if tensor_cores:
             self.q4_prepare_model()
         self.state = None
         self.S_max = None
 
     def q4_prepare_model(self):
-        """One-time int8 / gate-interleaved copies of the step weights for the tensor cores."""
+        """One-time int8 / gate-interleaved copies of the step weights for the tensor cores, and the tables made from
+        them if there are any.  To be called again when weights or embedding codes have been changed in place."""
         n = int(lib().q4_prepared_bytes(C.byref(self.model)))
         self.prepared = torch.empty(n, dtype=torch.uint8, device=self.device)
         _chk(lib().q4_prepare_model(C.byref(self.model), _p(self.prepared), C.c_size_t(n), _stream()),
              "q4_prepare_model")
+        if self.tables:
+            self.q4_prepare_tables(self.tables[0].numel())
+
+    def q4_prepare_tables(self, n: int):
+        """The first layers' input halves of every label, for searches of few rows (n: q4_table_bytes)."""
+        if not self.tables:
+            self.tables.append(torch.empty(n, dtype=torch.uint8, device=self.device))
+        _chk(lib().q4_prepare_tables(C.byref(self.model), _p(self.tables[0]), C.c_size_t(n), _stream()),
+             "q4_prepare_tables")
 
     def step_weight_bytes(self) -> int:
         return (self.pred_lstm.nbytes() + self.pred_proj.nbytes() + self.joint_out.nbytes() +
@@ -693,6 +705,10 @@ class Decoder:
         if self.tensor_cores:
             dims += [self.pred_lstm.w_ih.k_pad, Hp, Hs, Ht, RW]
         self.ws = torch.empty(workspace_bytes(WS_BEAM, dims), dtype=torch.uint8, device=dev)
+        n = int(lib().q4_table_bytes(C.byref(self.model), C.c_int32(N))) if self.tensor_cores else 0
+        if n and not self.tables and not torch.cuda.is_current_stream_capturing():
+            self.q4_prepare_tables(n)
+            torch.cuda.current_stream().synchronize()     # decoders that share the weights may run on other streams
 
     def q4_beam_init(self):
         _chk(lib().q4_beam_init(C.byref(self.state), C.c_int32(self.B), C.c_int32(self.W),

@@ -742,13 +742,17 @@ struct PrepLstm {
 struct PrepPlan {
   PrepLstm lstm[4];   // prediction, source LM, target LM layer 1, target LM layer 2
   size_t lin[6];      // pred_proj, src.bott, src.out, tgt.bott, tgt.out, joint_out
-  size_t table[3];    // first layers: de-quantized input sums plus bias of every label (fp32 [V, 4H])
-  size_t emb8;        // int8 embedding rows, while the tables are made; 0: no tables
   size_t total;
 };
-// Tables of the first layers' input halves: 16 H bytes a label and network.
+struct TablePlan {
+  size_t table[3];    // first layers: de-quantized input sums plus bias of every label (fp32 [V, 4H])
+  size_t emb8;        // int8 embedding rows, while the tables are made
+  size_t total;
+};
+// Tables of the first layers' input halves: 16 H bytes a label and network, so a bound on memory (268 MB with 1024, 1024 and
+// 2048 cells); a look-up costs the same at any V.
 constexpr int TABLE_MAX_V = 4096;
-bool search_tables(const q4_model& m) {
+bool tables_supported(const q4_model& m) {
   return m.V > 0 && m.V <= TABLE_MAX_V && m.src.n_layers == 1 && m.pred_lstm.w_hh.k_pad % 128 == 0 &&
          m.src.lstm[0].w_hh.k_pad % 128 == 0 && m.tgt.lstm[0].w_hh.k_pad % 128 == 0;
 }
@@ -794,18 +798,20 @@ PrepPlan plan_prepared(const q4_model& m) {
     p.lin[i] = o;
     o += align_up((size_t)L->w.rows * L->w.k_pad);
   }
-  if (search_tables(m)) {
-    size_t ep = 0;
-    for (int i = 0; i < 3; ++i) {
-      const q4_lstm* L = model_lstm(m, i);
-      p.table[i] = o;
-      o += align_up((size_t)m.V * L->w_ih.rows * sizeof(float));
-      if ((size_t)L->w_ih.k_pad > ep) ep = L->w_ih.k_pad;
-    }
-    p.emb8 = o;
-    o += align_up((size_t)m.V * ep);
-  }
   p.total = o;
+  return p;
+}
+TablePlan plan_tables(const q4_model& m) {
+  TablePlan p;
+  size_t o = 0, ep = 0;
+  for (int i = 0; i < 3; ++i) {
+    const q4_lstm* L = model_lstm(m, i);
+    p.table[i] = o;
+    o += align_up((size_t)m.V * L->w_ih.rows * sizeof(float));
+    if ((size_t)L->w_ih.k_pad > ep) ep = L->w_ih.k_pad;
+  }
+  p.emb8 = o;
+  p.total = o + align_up((size_t)m.V * ep);
   return p;
 }
 }  // namespace
@@ -844,24 +850,44 @@ int q4_prepare_model(q4_model* model, void* buffer, size_t bytes, q4_stream stre
     Q4_CHECK(check_mat(&L->w, 0, 0));
     Q4_TRY(launch_prepare_w(L->w, 0, reinterpret_cast<int8_t*>(b + p.lin[i]), L->w.k_pad, 0, s));
   }
-  for (int i = 0; i < 3 && p.emb8; ++i) {
+  model->prepared = buffer;
+  model->tables = nullptr;   // they belong to the preparation before
+  return Q4_OK;
+}
+
+size_t q4_table_bytes(const q4_model* model, int32_t rows) {
+  if (!model || rows <= 0 || rows > SUMS_MAX_ROWS || !tables_supported(*model)) return 0;
+  return plan_tables(*model).total;
+}
+int q4_prepare_tables(q4_model* model, void* buffer, size_t bytes, q4_stream stream) {
+  if (!model || !buffer || !model->prepared) return Q4_ERR_NULL;
+  if (!tables_supported(*model)) return Q4_ERR_UNSUPPORTED;
+  if (reinterpret_cast<uintptr_t>(buffer) & 31u) return Q4_ERR_ALIGN;
+  const TablePlan t = plan_tables(*model);
+  if (bytes < t.total) return Q4_ERR_WORKSPACE;
+  const PrepPlan p = plan_prepared(*model);
+  const uint8_t* w = static_cast<const uint8_t*>(model->prepared);
+  uint8_t* b = static_cast<uint8_t*>(buffer);
+  cudaStream_t s = S(stream);
+  TagScope tag(TAG_MISC);
+  for (int i = 0; i < 3; ++i) {
     const q4_lstm* L = model_lstm(*model, i);
     const q4_act& act = i == 0 ? model->pred_emb_act : i == 1 ? model->src.emb_act : model->tgt.emb_act;
     const void* emb = i == 0 ? model->pred_emb_q : i == 1 ? model->src.emb_q : model->tgt.emb_q;
     if (!emb) return Q4_ERR_NULL;
     Q4_CHECK(check_act(&act));
     const int Ep = L->w_ih.k_pad, G = L->w_ih.rows;
-    int8_t* e8 = reinterpret_cast<int8_t*>(b + p.emb8);
+    int8_t* e8 = reinterpret_cast<int8_t*>(b + t.emb8);
     UnpackJobs uj;
     memset(&uj, 0, sizeof(uj));
     uj.n_rows = uj.n_rows_pad = model->V;
     add_unpack_job(uj, emb, row_bytes(Ep, act.bits), nullptr, act, Ep, e8);
     Q4_TRY(launch_unpack_multi(uj, s, false));
-    Q4_TRY(launch_mma_gemm(e8, Ep, model->V, reinterpret_cast<const int8_t*>(b + p.lstm[i].xw), Ep, G, Ep, EPI_F32,
-                           b + p.table[i], G, nullptr, reinterpret_cast<const float*>(b + p.lstm[i].sc_ih),
-                           reinterpret_cast<const float*>(b + p.lstm[i].bias), 1.0f, nullptr, nullptr, nullptr, s, false));
+    Q4_TRY(launch_mma_gemm(e8, Ep, model->V, reinterpret_cast<const int8_t*>(w + p.lstm[i].xw), Ep, G, Ep, EPI_F32,
+                           b + t.table[i], G, nullptr, reinterpret_cast<const float*>(w + p.lstm[i].sc_ih),
+                           reinterpret_cast<const float*>(w + p.lstm[i].bias), 1.0f, nullptr, nullptr, nullptr, s, false));
   }
-  model->prepared = buffer;
+  model->tables = buffer;
   return Q4_OK;
 }
 
@@ -977,15 +1003,16 @@ static bool search_uses_tensor_cores(const q4_model& m, const q4_beam_state& st,
 static int32_t* search_frozen(void* workspace) { return reinterpret_cast<int32_t*>(static_cast<uint8_t*>(workspace) + 256); }
 
 // Whether a whole search takes the kernels that look the first layers' input halves up and keep the sums of the recurrent
-// halves per state row: tables with the prepared weights and room for the sums, both read 32 bytes at a time.
+// halves per state row: prepared weights, tables and room for the sums, the last two read 32 bytes at a time.
 static bool search_keeps_sums(const q4_model& m, const q4_beam_state& st, int B, int W, const void* workspace,
                               size_t workspace_bytes) {
-  if ((reinterpret_cast<uintptr_t>(workspace) | reinterpret_cast<uintptr_t>(m.prepared)) & 31u) return false;
+  if (!m.prepared || !m.tables || !tables_supported(m) || !aligned16(m.prepared)) return false;
+  if ((reinterpret_cast<uintptr_t>(workspace) | reinterpret_cast<uintptr_t>(m.tables)) & 31u) return false;
   const int RW = st.rows_per_utt > 0 ? st.rows_per_utt : 2 * W;
   const int32_t dims9[9] = {B, W, m.V, m.D, m.pred_lstm.w_ih.k_pad, m.pred_lstm.w_hh.k_pad, m.src.lstm[0].w_hh.k_pad,
                             m.tgt.lstm[0].w_hh.k_pad, RW};
-  return B * W <= SUMS_MAX_ROWS && m.prepared != nullptr && search_tables(m) && aligned16(st.pred_c) && aligned16(st.src_c) && aligned16(st.tgt_c[0]) &&
-         aligned16(st.tgt_c[1]) && workspace_bytes >= q4_workspace_bytes(Q4_WS_BEAM, dims9, 9);
+  return B * W <= SUMS_MAX_ROWS && aligned16(st.pred_c) && aligned16(st.src_c) && aligned16(st.tgt_c[0]) && aligned16(st.tgt_c[1]) &&
+         workspace_bytes >= q4_workspace_bytes(Q4_WS_BEAM, dims9, 9);
 }
 
 // How a step is part of a search.
@@ -1144,11 +1171,12 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
     if (nets && how.sums) {   // the first layers of all networks
       CellJobs cj;
       memset(&cj, 0, sizeof(cj));
+      const TablePlan tp = plan_tables(m);
       void* const hq[3] = {st.pred_hq, st.src_hq, st.tgt_hq[0]};
       float* const c[3] = {st.pred_c, st.src_c, st.tgt_c[0]};
       for (int i = 0; i < 3; ++i) {
         CellJob& k = cj.job[i];
-        k.table = reinterpret_cast<const float*>(pb + pp.table[i]);
+        k.table = reinterpret_cast<const float*>(static_cast<const uint8_t*>(m.tables) + tp.table[i]);
         k.sums = state_sums[i];
         k.sc_hh = reinterpret_cast<const float*>(pb + pp.lstm[i].sc_hh);
         k.c = c[i];

@@ -1044,3 +1044,70 @@ def test_search_with_buffers_at_smaller_alignments(Bd, what):
     assert a.tensors["status"].item() == 0
     for k in ("bp_parent", "bp_token", "bp_score"):
         assert torch.equal(a.tensors[k][:109], b.tensors[k][:109]), k
+
+
+def test_embeddings_after_the_preparation_of_the_weights(Bd):
+    # q4_prepare_model reads no embedding tables: it takes a model without them, and a search follows what they hold when it
+    # runs, unless tables have been made from them, which are made again with the weights
+    import copy
+    import ctypes as C
+    dw = synth.decoder(seed=96, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=5, W=8)
+    other = copy.deepcopy(dw)
+    for part in (other.pred, other.src, other.tgt):
+        part.emb = -part.emb
+    e = torch.from_numpy(synth.Stream(31).normal("e", (12, 3, 256)).astype(np.float32)).cuda()
+    a, b = Bd.Decoder(dw), Bd.Decoder(other)
+    want = [t.clone() for t in b.decode(e)] + [b.tensors["bp_score"]]
+    before = [t.clone() for t in a.decode(e)] + [a.tensors["bp_score"].clone()]
+    assert not torch.equal(before[-1], want[-1])
+
+    def check(d):
+        for x, y in zip([*d.decode(e), d.tensors["bp_score"]], want):
+            assert torch.equal(x, y)
+
+    for x, y in ((a.pred_emb_q, b.pred_emb_q), (a.src.emb_q, b.src.emb_q), (a.tgt.emb_q, b.tgt.emb_q)):
+        x.copy_(y)
+    a.model.tables = None
+    check(a)
+    m = Bd.Decoder(dw)
+    tables = m.model.pred_emb_q, m.model.src.emb_q, m.model.tgt.emb_q
+    m.model.pred_emb_q = m.model.src.emb_q = m.model.tgt.emb_q = None
+    m.q4_prepare_model()
+    m.model.pred_emb_q, m.model.src.emb_q, m.model.tgt.emb_q = tables
+    for x, y in ((m.pred_emb_q, b.pred_emb_q), (m.src.emb_q, b.src.emb_q), (m.tgt.emb_q, b.tgt.emb_q)):
+        x.copy_(y)
+    check(m)
+    assert m.model.tables and not Bd.lib().q4_table_bytes(C.byref(m.model), C.c_int32(385))
+    for x in (m.pred_emb_q, m.src.emb_q, m.tgt.emb_q):       # other codes, tables of them, then the codes of before
+        x.fill_(0x11)
+    m.q4_prepare_model()
+    assert not torch.equal(m.decode(e)[2], want[2])
+    for x, y in zip((m.pred_emb_q, m.src.emb_q, m.tgt.emb_q), (b.pred_emb_q, b.src.emb_q, b.tgt.emb_q)):
+        x.copy_(y)
+    m.q4_prepare_model()
+    check(m)
+
+
+def test_search_with_prepared_weights_at_a_16_byte_boundary_and_tables(Bd):
+    # tables have a buffer of their own: weights at a 16-byte boundary serve the kernels that look labels up
+    import ctypes as C
+    dw = synth.decoder(seed=97, V=300, E=32, Hp=128, D=256, Hs=128, Ht=128, tgt_layers=2, U_max=9, W=6)
+    dw.joint.out.bias[0] += np.float32(3.0)
+    e = torch.from_numpy(synth.Stream(33).normal("e", (100, 3, 256)).astype(np.float32)).cuda()
+    a, b = Bd.Decoder(dw), Bd.Decoder(dw)
+    want = b.decode(e)
+    a.alloc_state(3, 6, 109)
+    big = torch.zeros(a.prepared.numel() + 32, dtype=torch.uint8, device="cuda")
+    a.prepared = big[16:16 + a.prepared.numel()]
+    n = a.tables[0].numel()
+    lib, m = Bd.lib(), C.byref(a.model)
+    at = lambda t, o=0: C.c_void_p(t.data_ptr() + o)
+    assert lib.q4_prepare_model(m, at(a.prepared), C.c_size_t(a.prepared.numel()), None) == 0 and not a.model.tables
+    assert lib.q4_prepare_tables(m, at(a.tables[0], 16), C.c_size_t(n), None) != 0            # not at a 32-byte boundary
+    assert lib.q4_prepare_tables(m, at(a.tables[0]), C.c_size_t(n - 1), None) != 0
+    assert lib.q4_prepare_tables(m, at(a.tables[0]), C.c_size_t(n), None) == 0 and a.model.tables
+    torch.cuda.synchronize()
+    for x, y in zip(a.decode(e), want):
+        assert torch.equal(x, y)
+    for k in ("bp_parent", "bp_token", "bp_score", "pred_c", "tgt_c0"):
+        assert torch.equal(a.tensors[k], b.tensors[k]), k
