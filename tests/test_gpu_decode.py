@@ -978,6 +978,26 @@ def test_selection_forms_agree_with_the_exact_search(Bd, V, normalized, S):
             assert torch.equal(x, y)
 
 
+@pytest.mark.parametrize("V", [260, 516, 1000, 1024])
+@pytest.mark.parametrize("S,D,tensor_cores", [(None, 64, True), (1, 64, True), (None, 256, False), (None, 256, True)])
+def test_selection_of_rows_at_smaller_alignments(Bd, V, S, D, tensor_cores):
+    # logits and log-probabilities, in the form that reads rows 16 bytes at a time and, with a language model's rows at a
+    # 4-byte boundary, in the one that reads single elements: the same bits
+    dw = synth.decoder(seed=94, V=V, E=32, Hp=128, D=D, Hs=128, Ht=128, tgt_layers=1, U_max=6, W=16)
+    for B, W in ((1, 16), (3, 5)):
+        e = torch.from_numpy(synth.Stream(V + W).normal("e", (10, B, D)).astype(np.float32)).cuda()
+        runs = []
+        for shift in (0, 1):
+            dd = Bd.Decoder(dw, tensor_cores=tensor_cores)
+            dd.alloc_state(B, W, 16 if S is None else 20, S)
+            rows = torch.zeros(dd.tensors["src_lp"].numel() + 4, device="cuda")
+            dd.state.src_lp = rows[shift:].data_ptr()
+            out = dd.decode(e, 6, W) if S is None else dd.decode_time_synchronous(e, S, 6, W)
+            runs.append(list(out) + [dd.tensors[k] for k in ("bp_parent", "bp_token", "bp_score", "fin_n", "fin_score", "status")])
+        for x, y in zip(*runs):
+            assert torch.equal(x, y)
+
+
 @pytest.mark.parametrize("B,W,S,layers,bits", [(3, 7, None, 2, 4), (8, 16, None, 2, 4), (9, 15, 1, 2, 4), (24, 16, None, 1, 8),
                                                (25, 16, None, 2, 4), (2, 16, 3, 1, 4)])
 def test_search_that_keeps_sums_equals_its_steps(Bd, B, W, S, layers, bits):
