@@ -370,9 +370,10 @@ int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float
  * there is none: it waits for nothing.  One plan serves one search at a time.  In the tensor-core path with D = 256 the
  * steps of an alignment-length synchronous search are the body of a loop in the graph (a conditional node), which ends
  * when no utterance has labels left to propose; the iterations that are left then are carried out by two launches (same
- * results, same history).  In a stream capture the loop becomes a node of the caller's graph.  Without a plan, in another
- * search in a stream capture, below 96 steps, while launches are timed and under q4_test_wait_expiry_set, the steps are
- * enqueued one by one (same results).
+ * results, same history).  In a stream capture the loop becomes a node of the caller's graph (if it cannot, the steps are
+ * captured one by one): CUDA refuses a graph with such a node as a child graph and in cudaGraphClone; a caller who needs
+ * either captures without a plan.  Without a plan, in another search in a stream capture, below 96 steps, while launches
+ * are timed and under q4_test_wait_expiry_set, the steps are enqueued one by one (same results).
  * Graphs, and what they are captured on, are the plan's own: the streams lent with the state are used by single
  * steps only, and a plan may be made, used or destroyed while another thread captures a stream.  A plan uses the memory
  * of a search only in a search on it.  q4_search_plan_destroy waits for the replays on their way.
@@ -381,8 +382,11 @@ typedef void* q4_search_plan;
 int q4_search_plan_create(q4_search_plan* out);
 int q4_search_plan_destroy(q4_search_plan plan);
 /* What a plan has done so far (host counters, for tests and diagnostics): out[0] graphs built, out[1] groups
- * of 12 steps that replays were enqueued for, out[2] attempts to build a graph that failed (the search then enqueued its steps one by one). */
+ * of 12 steps that replays were enqueued for, out[2] attempts to build a graph, or a loop in the caller's, that failed (the search then enqueued its steps one by one). */
 int q4_search_plan_info(q4_search_plan plan, int64_t* out);
+/* Test hook: from now on every loop that a search with this plan builds fails, before its node is added (where = 1) or before
+ * the node is filled (2); 0 restores normal operation.  Graphs built before are not touched. */
+int q4_test_search_loop_failure_set(q4_search_plan plan, int32_t where);
 int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, int32_t B, int32_t T, int32_t W,
                    int32_t u_max, float lambda_t, float lambda_s, float rho, int32_t time_synchronous,
                    void* workspace, size_t workspace_bytes, q4_search_plan plan, q4_stream stream);

@@ -82,7 +82,7 @@ EXPORTS = ["q4_act_symmetric", "q4_act_asymmetric", "quantize_pack_int4", "qlstm
            "qlstm_step", "q4_linear_forward", "qjoint_logprobs", "q4_beam_init",
            "dr_fusion_beam_step", "q4_beam_search", "q4_search_plan_create", "q4_search_plan_destroy", "q4_search_plan_info", "q4_traceback", "q4_feature_prologue", "q4_workspace_bytes",
            "q4_poll_status", "q4_version", "q4_launch_count", "q4_dependent_launch_set", "q4_beam_select_exact_set", "q4_timing_set", "q4_timing_count", "q4_prepared_bytes", "q4_prepare_model", "q4_table_bytes", "q4_prepare_tables", "qjoint_logprobs_static", "q4_quantizer_calls", "q4_prepared_lstm_bytes", "q4_prepare_lstm",
-           "q4_prepared_linear_bytes", "q4_prepare_linear", "q4_test_wait_expiry_set", "q4_encoder_time_slicing_set", "q4_encoder_recurrence_plan"]
+           "q4_prepared_linear_bytes", "q4_prepare_linear", "q4_test_wait_expiry_set", "q4_test_search_loop_failure_set", "q4_encoder_time_slicing_set", "q4_encoder_recurrence_plan"]
 
 _lib = None
 

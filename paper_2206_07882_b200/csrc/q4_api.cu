@@ -1556,7 +1556,8 @@ struct SearchGraph {
 };
 struct SearchPlan {
   SearchGraph graph[PLAN_GRAPHS];
-  int64_t built, replays, failed;    // graphs made, replays enqueued, attempts to make a graph that failed
+  int64_t built, replays, failed;    // graphs made, replays enqueued, attempts to make a graph or a loop that failed
+  int32_t test_failure;              // see q4_test_search_loop_failure_set
   int64_t uses;
   // Captured on: the graphs' chains, none of the caller's streams.  side[2] or side[3] take the recurrent sums: up to 128 rows
   // with a lower priority than the rest, so that the joint network's chain, which is the longest there, does not queue
@@ -1633,19 +1634,23 @@ static int capture_steps(SearchPlan* p, SearchKey& key, const cudaGraphCondition
   if (!loop) Q4_TRY(launch_search_advance(call, PLAN_ITERS, p->stream));
   return Q4_OK;
 }
-// A conditional node in `g` behind `deps` that repeats the steps until every utterance is frozen (at least one turn).
-static int add_search_loop(SearchPlan* p, SearchKey& key, cudaGraph_t g, const cudaGraphNode_t* deps, size_t n_deps,
-                           cudaGraphNode_t* node) {
+// A conditional node in `g`, behind nothing, that repeats the steps until every utterance is frozen while *handle is not 0;
+// `first`: its value when the graph is launched.  A node that could not be filled stays in the graph (nodes cannot be
+// taken out of a graph that is being captured), so there `first` is 0 and launch_search_begin sets the value.
+static int add_search_loop(SearchPlan* p, SearchKey& key, cudaGraph_t g, unsigned first, cudaGraphNode_t* node,
+                           cudaGraphConditionalHandle* handle) {
   cudaGraphNodeParams np = {};
   np.type = cudaGraphNodeTypeConditional;
   np.conditional.type = cudaGraphCondTypeWhile;
   np.conditional.size = 1;
-  if (cudaGraphConditionalHandleCreate(&np.conditional.handle, g, 1, cudaGraphCondAssignDefault) != cudaSuccess ||
-      cudaGraphAddNode(node, g, deps, n_deps, &np) != cudaSuccess ||
+  if (p->test_failure == 1 ||
+      cudaGraphConditionalHandleCreate(&np.conditional.handle, g, first, cudaGraphCondAssignDefault) != cudaSuccess ||
+      cudaGraphAddNode(node, g, nullptr, 0, &np) != cudaSuccess || p->test_failure == 2 ||
       cudaStreamBeginCaptureToGraph(p->stream, np.conditional.phGraph_out[0], nullptr, nullptr, 0,
                                     cudaStreamCaptureModeRelaxed) != cudaSuccess)
     return Q4_ERR_CUDA;
-  int r = capture_steps(p, key, &np.conditional.handle);
+  *handle = np.conditional.handle;
+  int r = capture_steps(p, key, handle);
   if (cudaStreamEndCapture(p->stream, nullptr) != cudaSuccess && r == Q4_OK) r = Q4_ERR_CUDA;
   return r;
 }
@@ -1673,7 +1678,8 @@ static SearchGraph* plan_graph(SearchPlan* p, const SearchKey& key) {
   int r;
   if (key.loop) {
     cudaGraphNode_t node;
-    r = cudaGraphCreate(&g, 0) == cudaSuccess ? add_search_loop(p, place->key, g, nullptr, 0, &node) : Q4_ERR_CUDA;
+    cudaGraphConditionalHandle handle;
+    r = cudaGraphCreate(&g, 0) == cudaSuccess ? add_search_loop(p, place->key, g, 1, &node, &handle) : Q4_ERR_CUDA;
   } else {
     r = cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeRelaxed) == cudaSuccess ? Q4_OK : Q4_ERR_CUDA;
     if (r == Q4_OK) {
@@ -1697,6 +1703,12 @@ static SearchGraph* plan_graph(SearchPlan* p, const SearchKey& key) {
   return place;
 }
 
+int q4_test_search_loop_failure_set(q4_search_plan plan, int32_t where) {
+  if (!plan) return Q4_ERR_NULL;
+  if (where < 0 || where > 2) return Q4_ERR_UNSUPPORTED;
+  static_cast<SearchPlan*>(plan)->test_failure = where;
+  return Q4_OK;
+}
 int q4_search_plan_info(q4_search_plan plan, int64_t* out) {
   if (!plan || !out) return Q4_ERR_NULL;
   const SearchPlan* p = static_cast<const SearchPlan*>(plan);
@@ -1759,19 +1771,30 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
       int32_t* frozen = key.loop ? search_frozen(workspace) : nullptr;
       const int groups = (n_iters - it) / PLAN_ITERS;
       const int turns = key.loop ? (n_iters - it + PLAN_ITERS - 1) / PLAN_ITERS : groups;
-      if (cap != cudaStreamCaptureStatusNone) {   // the loop becomes a node of the caller's graph
-        Q4_TRY(launch_search_begin(call, e, T, u_max, it - PLAN_ITERS, frozen, B, s));
+      if (cap != cudaStreamCaptureStatusNone) {   // the loop becomes a node of the caller's graph, if it can be one
         const int64_t l0 = g_launches, q0 = g_quant_calls;
         cudaGraph_t g;
         const cudaGraphNode_t* deps;
         size_t n_deps;
         cudaGraphNode_t node;
+        cudaGraphConditionalHandle handle;
         Q4_TRY(cudaStreamGetCaptureInfo_v2(s, &cap, nullptr, &g, &deps, &n_deps));
-        Q4_CHECK(add_search_loop(p, key, g, deps, n_deps, &node));
-        Q4_TRY(cudaStreamUpdateCaptureDependencies(s, &node, 1, cudaStreamSetCaptureDependencies));
-        g_launches += (g_launches - l0) * (turns - 1);
-        g_quant_calls += (g_quant_calls - q0) * (turns - 1);
-        tail = true;
+        if (add_search_loop(p, key, g, 0, &node, &handle) == Q4_OK) {
+          g_launches += (g_launches - l0) * (turns - 1);
+          g_quant_calls += (g_quant_calls - q0) * (turns - 1);
+          Q4_TRY(launch_search_begin(call, e, T, u_max, it - PLAN_ITERS, frozen, B, s, &handle));
+          Q4_TRY(cudaStreamGetCaptureInfo_v2(s, &cap, nullptr, &g, &deps, &n_deps));
+          if (n_deps != 1) return Q4_ERR_CUDA;   // the launch above
+          const cudaGraphNode_t begin = deps[0];
+          Q4_TRY(cudaGraphAddDependencies(g, &begin, &node, 1));
+          Q4_TRY(cudaStreamUpdateCaptureDependencies(s, &node, 1, cudaStreamSetCaptureDependencies));
+          tail = true;
+        } else {
+          g_launches = l0;
+          g_quant_calls = q0;
+          ++p->failed;
+          cudaGetLastError();
+        }
       } else if (SearchGraph* g = plan_graph(p, key)) {
         Q4_TRY(launch_search_begin(call, e, T, u_max, it - PLAN_ITERS, frozen, B, s));
         for (int i = 0; i < (key.loop ? 1 : groups); ++i) {

@@ -986,10 +986,12 @@ __global__ void k_beam_init(q4_beam_state st, int B, int W) {
   }
 }
 
-__global__ void k_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter, int32_t* frozen, int B) {
+__global__ void k_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter, int32_t* frozen, int B, int has_loop,
+                               cudaGraphConditionalHandle loop) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (frozen && i < B) frozen[i] = -1;
   if (i != 0) return;
+  if (has_loop) cudaGraphSetConditional(loop, 1);
   call->e = e;
   call->T = T;
   call->u_max = u_max;
@@ -999,8 +1001,9 @@ __global__ void k_search_begin(SearchCall* call, const float* e, int T, int u_ma
 }
 __global__ void k_search_advance(SearchCall* call, int iters) { call->iter += iters; }
 cudaError_t launch_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter, int32_t* frozen, int B,
-                                cudaStream_t s) {
-  k_search_begin<<<frozen ? (B + 127) / 128 : 1, 128, 0, s>>>(call, e, T, u_max, iter, frozen, B);
+                                cudaStream_t s, const cudaGraphConditionalHandle* loop) {
+  k_search_begin<<<frozen ? (B + 127) / 128 : 1, 128, 0, s>>>(call, e, T, u_max, iter, frozen, B, loop != nullptr,
+                                                              loop ? *loop : cudaGraphConditionalHandle());
   ++g_launches;
   return cudaGetLastError();
 }

@@ -27,9 +27,10 @@ struct SearchCall {
   int32_t n_frozen;         // utterances whose search has no labels left to propose (see q4_tail.cu)
   int32_t arrived;          // utterances that have ended the last step of a loop's turn
 };
-// frozen (nullable): [2 B] per utterance the iteration it was frozen at (set to -1 here) and the frames it had left
+// frozen (nullable): [2 B] per utterance the iteration it was frozen at (set to -1 here) and the frames it had left;
+// loop (nullable): a loop behind it in the same graph, which takes its first turn
 cudaError_t launch_search_begin(SearchCall* call, const float* e, int T, int u_max, int iter, int32_t* frozen, int B,
-                                cudaStream_t s);
+                                cudaStream_t s, const cudaGraphConditionalHandle* loop = nullptr);
 cudaError_t launch_search_advance(SearchCall* call, int iters, cudaStream_t s);
 struct BeamSelArgs {
   SearchCall* call;

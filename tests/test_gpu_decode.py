@@ -656,6 +656,34 @@ def test_search_plan_keeps_no_test_hook(Bd):
     assert dd.tensors["status"].item() == 0
 
 
+@pytest.mark.parametrize("where", [1, 2])
+def test_search_whose_loop_cannot_be_built(Bd, where):
+    # the loop's node is refused, or cannot be filled: the steps are enqueued, or captured by the caller, one by one
+    import ctypes as C
+    dw = synth.decoder(seed=67, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=9, W=6)
+    e = torch.from_numpy(synth.Stream(26).normal("e", (111, 3, 256)).astype(np.float32)).cuda()
+    plain = Bd.Decoder(dw, concurrent=False)
+    want = [t.clone() for t in plain.decode(e)]
+    dd = Bd.Decoder(dw)
+    dd.alloc_state(3, 6, 120)
+    dd.decode(e[:30], 5)                                                   # short: makes the plan, builds nothing
+    fail = lambda x: Bd.lib().q4_test_search_loop_failure_set(dd._plan.handle, C.c_int32(x))
+    captured = Bd.GraphedStep(lambda: dd.decode(e))
+    assert fail(3) != 0 and fail(where) == 0
+    for run in (lambda: dd.decode(e), captured, captured):                 # (the second makes an eager pass and a captured one)
+        dd.tensors["bp_score"].fill_(-7)
+        for x, y in zip(run(), want):
+            assert torch.equal(x, y)
+        assert dd.tensors["status"].item() == 0 and torch.equal(dd.tensors["bp_score"], plain.tensors["bp_score"])
+    assert dd.search_plan_info() == dict(built=0, replays=0, failed=3)
+    assert fail(0) == 0
+    looped = Bd.GraphedStep(lambda: dd.decode(e))
+    for run in (looped, looped):
+        for x, y in zip(run(), want):
+            assert torch.equal(x, y)
+    assert dd.search_plan_info() == dict(built=1, replays=9, failed=3)
+
+
 def test_search_beside_a_capture_of_another_thread(Bd):
     # a search that creates its plan and builds its graph on one thread leaves a capture that another thread has open
     # (in the strictest mode, torch's default) as it is
