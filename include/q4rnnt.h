@@ -249,7 +249,8 @@ int q4_prepare_model(q4_model* model, void* buffer, size_t bytes, q4_stream stre
 /* Optional, after q4_prepare_model: the input halves of the first LSTM layers for every label (one fp32 row per label and
  * network, 16 H bytes), which whole searches of few rows look up instead of multiplying embedding rows.  `buffer`: device,
  * 32-byte aligned, q4_table_bytes(model, rows) bytes, owned by the caller; sets model->tables.  q4_table_bytes is 0 where a
- * search of `rows` = B W rows takes no tables (above 384 rows or 4096 labels, widths that are no multiples of 128).  The tables
+ * search of `rows` = B W rows takes no tables (above 384 rows, or 256 unless D = 256 and V <= 2048; above
+ * 4096 labels; widths that are no multiples of 128).  The tables
  * are made from the embedding tables as they are at the call: when those change, call it again, or set tables to NULL. */
 size_t q4_table_bytes(const q4_model* model, int32_t rows);
 int q4_prepare_tables(q4_model* model, void* buffer, size_t bytes, q4_stream stream);
@@ -352,7 +353,7 @@ int q4_beam_init(q4_beam_state* state, int32_t B, int32_t W, int32_t n_iters, q4
  * workspace: q4_workspace_bytes(Q4_WS_BEAM, {B, W, V, D}), or, to enable the tensor-core path
  * (needs model->prepared and LSTM widths that are multiples of 128),
  * q4_workspace_bytes(Q4_WS_BEAM, {B, W, V, D, E_pad, Hp, Hs, Ht}).  With the state rows per utterance as a ninth entry
- * (2 W where rows_per_utt is 0) q4_beam_search has room for its fastest kernels (up to 384 rows B W).  A bounded device wait that expires sets state->status to Q4_ERR_TIMEOUT.
+ * (2 W where rows_per_utt is 0) q4_beam_search has room for its fastest kernels (see q4_prepare_tables).  A bounded device wait that expires sets state->status to Q4_ERR_TIMEOUT.
  */
 int dr_fusion_beam_step(const q4_model* model, q4_beam_state* state, const float* e, int32_t B,
                         int32_t T, int32_t W, int32_t iter, int32_t u_max, float lambda_t,

@@ -46,12 +46,17 @@ int check_mat(const q4_mat* m, int rows, int k_pad_expected) {
   return Q4_OK;
 }
 
-// Hypothesis rows of a search that keeps the recurrent sums per state row (see search_keeps_sums).  They take 16 H bytes a
+// Hypothesis rows up to which a search keeps the recurrent sums per state row (see search_keeps_sums).  They take 16 H bytes a
 // row and layer through memory instead of a gather and products in the step's longest chain, and the products
-// that make them take the SMs from the output heads and the selection when there are many: 160 frames, labels in
-// half of the iterations, ms with / without: 64 rows 4.06 / 5.05, 256 rows 4.31 / 4.87, 384 rows 8.38 / 8.89, 512 rows 9.94 / 9.86,
-// 1024 rows 12.0 / 9.6.
-constexpr int SUMS_MAX_ROWS = 384;
+// that make them take the SMs from the output heads and the selection when there are many: with 1024, 1024 and 2048 cells,
+// 160 frames, labels in half of the iterations, ms with / without: 64 rows 4.06 / 5.05, 256 rows 4.31 / 4.87, 384 rows
+// 8.38 / 8.89, 512 rows 9.94 / 9.86, 1024 rows 12.0 / 9.6.  Without the fused output heads (D = 256, up to 2048 labels) the
+// heads are launches of their own with tiles for every SM, and the line lies lower: 100 frames, D = 128, 252 rows 4.89 /
+// 4.87 with labels all the way and 7.30 / 7.63 in half of the iterations, 384 rows 6.01 / 5.31 and 8.64 / 9.06; 4096 labels,
+// 384 rows 10.7 / 9.9 and 12.1 / 11.5.
+constexpr int SUMS_MAX_ROWS = 384, SUMS_MAX_ROWS_PLAIN = 256;
+constexpr bool fused_heads(int V, int D) { return D == 256 && V <= 2048; }   // 256-wide bottleneck, one cluster per row tile
+constexpr int sums_max_rows(int V, int D) { return fused_heads(V, D) ? SUMS_MAX_ROWS : SUMS_MAX_ROWS_PLAIN; }
 
 // Rows that the tensor-core paths can address: a grid has 65535 row tiles, and the gather counts 32-code pieces in 32
 // bits (rows of k codes).  More go to the general kernels, which walk any number.
@@ -219,7 +224,7 @@ size_t q4_workspace_bytes(int32_t call_id, const int32_t* dims, int32_t ndims) {
       (void)Hmax;
       n += align_up(Np * Hp) + align_up(Np * Hs) + 2 * align_up(Np * Ht); // new cell outputs, int8
       n += 3 * align_up(Np * D);                                         // bottleneck codes, z codes
-      if (ndims >= 9 && dims[8] > 0 && N <= SUMS_MAX_ROWS) {             // recurrent sums of every state row
+      if (ndims >= 9 && dims[8] > 0 && N <= (size_t)sums_max_rows((int)V, (int)D)) {   // recurrent sums of every state row
         const size_t R = (size_t)dims[0] * dims[8];
         n += align_up(R * 4 * Hp * sizeof(float)) + align_up(R * 4 * Hs * sizeof(float)) + 2 * align_up(R * 4 * Ht * sizeof(float));
       }
@@ -856,7 +861,7 @@ int q4_prepare_model(q4_model* model, void* buffer, size_t bytes, q4_stream stre
 }
 
 size_t q4_table_bytes(const q4_model* model, int32_t rows) {
-  if (!model || rows <= 0 || rows > SUMS_MAX_ROWS || !tables_supported(*model)) return 0;
+  if (!model || rows <= 0 || rows > sums_max_rows(model->V, model->D) || !tables_supported(*model)) return 0;
   return plan_tables(*model).total;
 }
 int q4_prepare_tables(q4_model* model, void* buffer, size_t bytes, q4_stream stream) {
@@ -1011,7 +1016,7 @@ static bool search_keeps_sums(const q4_model& m, const q4_beam_state& st, int B,
   const int RW = st.rows_per_utt > 0 ? st.rows_per_utt : 2 * W;
   const int32_t dims9[9] = {B, W, m.V, m.D, m.pred_lstm.w_ih.k_pad, m.pred_lstm.w_hh.k_pad, m.src.lstm[0].w_hh.k_pad,
                             m.tgt.lstm[0].w_hh.k_pad, RW};
-  return B * W <= SUMS_MAX_ROWS && aligned16(st.pred_c) && aligned16(st.src_c) && aligned16(st.tgt_c[0]) && aligned16(st.tgt_c[1]) &&
+  return B * W <= sums_max_rows(m.V, m.D) && aligned16(st.pred_c) && aligned16(st.src_c) && aligned16(st.tgt_c[0]) && aligned16(st.tgt_c[1]) &&
          workspace_bytes >= q4_workspace_bytes(Q4_WS_BEAM, dims9, 9);
 }
 
@@ -1314,7 +1319,7 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
     };
 
     const int32_t* n_frozen = frozen ? &call->n_frozen : nullptr;   // all utterances frozen: the joint network has nothing to do
-    const bool fused_head = D == 256 && V <= 2048;   // the fused head kernel: 256-wide bottleneck, one cluster per row tile
+    const bool fused_head = fused_heads(V, D);
     // 1a. prediction network, then the joint network for every live slot (stream sp)
     if (nets) {
       if (!how.sums)

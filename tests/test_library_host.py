@@ -157,3 +157,18 @@ def test_encoder_recurrence_plan_lays_groups_on_clusters():
                                                C.c_int32(4), C.c_int32(0), (C.c_int32 * 17)()) == -2
     assert Bd.lib().q4_encoder_recurrence_plan(C.c_int32(5), C.c_int32(4), C.c_int32(2), C.c_int32(640), C.c_int32(4),
                                                C.c_int32(4), C.c_int32(0), None) == -1
+
+
+@pytest.mark.parametrize("V,D,most", [(1024, 256, 384), (2048, 256, 384), (2049, 256, 256), (46, 128, 256)])
+def test_rows_of_searches_that_look_labels_up(Bd, V, D, most):
+    # the largest search that keeps recurrent sums, with and without the fused output heads: tables and room for the sums
+    m = Bd.ModelS()
+    m.V, m.E, m.D, m.src.n_layers, m.tgt.n_layers = V, 32, D, 1, 2
+    for l in (m.pred_lstm, m.src.lstm[0], m.tgt.lstm[0], m.tgt.lstm[1]):
+        l.w_ih.rows = l.w_hh.rows = 512
+        l.w_ih.k_pad, l.w_hh.k_pad = 32, 128
+    dims = [V, D, 32, 128, 128, 128]
+    for rows, want in ((1, True), (most, True), (most + 1, False)):
+        assert bool(Bd.lib().q4_table_bytes(C.byref(m), C.c_int32(rows))) == want
+        with_sums = Bd.workspace_bytes(Bd.WS_BEAM, [rows, 1] + dims + [2])
+        assert (with_sums > Bd.workspace_bytes(Bd.WS_BEAM, [rows, 1] + dims)) == want
