@@ -424,7 +424,8 @@ int64_t q4_launch_count(void);
  * per sequence with the quantizer at the cell outputs, 2 T L with quantizers at the cell inputs):
  * +1 per quantize_pack_int4 call on activations (modes 0 and 1), +1 per qlstm_step with hq_out,
  * +T*dirs per qlstm_layer_forward (twice that when out_act differs from hid_act), +1 per joint
- * call, and the corresponding sum per beam step.  A call covers all rows it is given (a batch of
+ * call, and the corresponding sum per beam step (a whole search counts all of its steps, also those that
+ * are carried out together).  A call covers all rows it is given (a batch of
  * sequences counts once).  reset != 0 sets the counter back to zero after reading it. */
 int64_t q4_quantizer_calls(int32_t reset);
 

@@ -1786,7 +1786,7 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
         Q4_TRY(cudaStreamGetCaptureInfo_v2(s, &cap, nullptr, &g, &deps, &n_deps));
         if (add_search_loop(p, key, g, 0, &node, &handle) == Q4_OK) {
           g_launches += (g_launches - l0) * (turns - 1);
-          g_quant_calls += (g_quant_calls - q0) * (turns - 1);
+          g_quant_calls = q0 + (g_quant_calls - q0) / PLAN_ITERS * (n_iters - it);   // every step's, whoever carries it out
           Q4_TRY(launch_search_begin(call, e, T, u_max, it - PLAN_ITERS, frozen, B, s, &handle));
           Q4_TRY(cudaStreamGetCaptureInfo_v2(s, &cap, nullptr, &g, &deps, &n_deps));
           if (n_deps != 1) return Q4_ERR_CUDA;   // the launch above
@@ -1810,7 +1810,7 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
           }
         }
         g_launches += g->launches * turns;
-        g_quant_calls += g->quant_calls * turns;
+        g_quant_calls += key.loop ? g->quant_calls / PLAN_ITERS * (n_iters - it) : g->quant_calls * groups;
         p->replays += groups;
         Q4_TRY(cudaEventRecord(g->done, s));
         tail = key.loop != 0;

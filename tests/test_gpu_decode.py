@@ -982,6 +982,24 @@ def test_label_free_end_of_a_search_equals_its_steps(Bd, V, W, B, T, U, blank, b
     assert a.search_plan_info()["built"] == 1
 
 
+@pytest.mark.parametrize("T,U,S", [(111, 9, None), (100, 12, None), (30, 5, None), (60, 4, 1)])
+def test_search_counts_the_quantizers_of_all_its_steps(Bd, T, U, S):
+    # prediction, source and two target layers, two bottlenecks and tanh(e p) a step: in a looped, captured, replayed or plain
+    # search, whether its steps are a multiple of a graph's or not
+    dw = synth.decoder(seed=67, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=U, W=6)
+    e = torch.from_numpy(synth.Stream(27).normal("e", (T, 3, 256)).astype(np.float32)).cuda()
+    n = T + U if S is None else T * (S + 1)
+    for concurrent in (True, False):
+        dd = Bd.Decoder(dw, concurrent=concurrent)
+        run = (lambda: dd.decode(e)) if S is None else (lambda: dd.decode_time_synchronous(e, S))
+        run()
+        Bd.quantizer_calls(reset=True)
+        run()
+        assert Bd.quantizer_calls(reset=True) == 7 * n
+        Bd.GraphedStep(run)()                                  # an eager pass and a captured one
+        assert Bd.quantizer_calls(reset=True) == 14 * n
+
+
 @pytest.mark.parametrize("V,normalized", [(2, 1), (46, 1), (64, 1), (65, 1), (256, 1), (257, 1), (300, 0), (1023, 1), (1024, 0),
                                           (1024, 1), (1025, 1)])
 @pytest.mark.parametrize("S", [None, 1])
