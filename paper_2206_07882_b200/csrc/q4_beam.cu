@@ -107,9 +107,9 @@ __device__ __forceinline__ void copy_row(float* dst, const float* src, int V, in
   }
 }
 // where a warp reads its slot's joint row: the copy on its way to shared memory (waits for it), else the row itself
-template <int MODE>
-__device__ __forceinline__ const float* copied_row(const float* copy, const float* row) {
-  if (MODE != 2) return row;
+template <bool COPIED>
+__device__ __forceinline__ const float* logits_row(const float* copy, const float* row) {
+  if (!COPIED) return row;
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncwarp();
   return copy;
@@ -338,7 +338,7 @@ __device__ __forceinline__ void list_free_rows(uint64_t free_mask, int* rows, in
   __syncwarp();
 }
 
-template <int MODE, int NE>
+template <int MODE, int NE, bool LOGITS = false>
 __global__ void __launch_bounds__(SEL_THREADS, 1) k_beam_select(const __grid_constant__ BeamSelArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int W = a.W, V = a.V;
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) k_beam_select(const __grid_con
   }
   float lse = 0.0f;
   if (my_row >= 0) {
-    if (!normalized) lse = row_lse<MODE>(v, copied_row<MODE>(cand + (size_t)warp * V, x), V, lane);
+    if (!normalized) lse = row_lse<MODE>(v, logits_row<LOGITS>(cand + (size_t)warp * V, x), V, lane);
     if (lane == 0) {
       s_slot.lse[warp] = lse;
       s_slot.blank[warp] = (float)((double)my_score + (double)((MODE == 1 ? v[0] : x0) - lse));
@@ -609,15 +609,16 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) k_beam_select(const __grid_con
 // Which form of the kernels takes a vocabulary: registers hold up to 1024 labels of a slot, and rows are read 16 bytes at
 // a time where those of all three tables can be.  A selection with joint rows that are not normalised, summed 32 elements
 // apart in the shared copy / in registers that were read 4 bytes at a time: 8 x 16 slots of 1024 labels 13.9 / 17.9 us,
-// 24 x 16 of 512 12.9 / 15.8, 64 x 16 of 1000 14.2 / 16.4.
-enum { SEL_ANY, SEL_64, SEL_256, SEL_1024, SEL_WIDE };
+// 24 x 16 of 512 12.9 / 15.8, 64 x 16 of 1000 14.2 / 16.4.  A kernel of its own: without LOGITS the sums in the
+// kernel of the normalised rows cost a search of 16 x 16 slots 0.8 %.
+enum { SEL_ANY, SEL_64, SEL_256, SEL_1024, SEL_WIDE, SEL_WIDE_LOGITS };
 static int sel_form(const BeamSelArgs& a) {
   if (a.V > 1024) return SEL_ANY;
   if (a.V <= 64) return SEL_64;
   if (a.V <= 256) return SEL_256;
   const bool wide = a.V % 4 == 0 && ((reinterpret_cast<uintptr_t>(a.logits) | reinterpret_cast<uintptr_t>(a.src_lp) |
                                       reinterpret_cast<uintptr_t>(a.tgt_lp)) & 15) == 0;
-  return wide ? SEL_WIDE : SEL_1024;
+  return !wide ? SEL_1024 : a.normalized ? SEL_WIDE : SEL_WIDE_LOGITS;
 }
 static size_t sel_smem(const BeamSelArgs& a) {
   return (size_t)sel_list_cap(a.W, a.V) * (sizeof(uint64_t) + sizeof(uint32_t)) + (size_t)a.W * a.V * sizeof(float);
@@ -634,9 +635,9 @@ static cudaError_t sel_launch(void (*kern)(const BeamSelArgs), size_t (&configur
   return launch_ex(kern, dim3(a.B), dim3(SEL_THREADS), smem, s, dependent, 1, a);
 }
 cudaError_t launch_beam_select(const BeamSelArgs& a, cudaStream_t s, bool dependent) {
-  static size_t configured[5][MAX_DEVICES];
-  static void (*const kern[5])(const BeamSelArgs) = {k_beam_select<0, 1>, k_beam_select<1, 2>, k_beam_select<1, 8>,
-                                                     k_beam_select<1, 32>, k_beam_select<2, 32>};
+  static size_t configured[6][MAX_DEVICES];
+  static void (*const kern[6])(const BeamSelArgs) = {k_beam_select<0, 1>, k_beam_select<1, 2>, k_beam_select<1, 8>,
+                                                     k_beam_select<1, 32>, k_beam_select<2, 32>, k_beam_select<2, 32, true>};
   const int form = sel_form(a);
   timing_begin(s);
   const cudaError_t le = sel_launch(kern[form], configured[form], a, s, dependent);
@@ -655,7 +656,7 @@ cudaError_t launch_beam_select(const BeamSelArgs& a, cudaStream_t s, bool depend
 // extensions of the alignment-length synchronous search.  In the frame-closing call (mode 2) no
 // label is proposed and the W best candidates (score, insertion order) open frame t + 1.
 constexpr int TSD_MAXC = 64;
-template <int MODE, int NE>
+template <int MODE, int NE, bool LOGITS = false>
 __global__ void __launch_bounds__(SEL_THREADS, 1) k_tsd_select(const __grid_constant__ BeamSelArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int W = a.W, V = a.V;
@@ -749,7 +750,7 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) k_tsd_select(const __grid_cons
   }
   float lse = 0.0f;
   if (my_row >= 0) {
-    if (!a.normalized) lse = row_lse<MODE>(v, copied_row<MODE>(cand + (size_t)warp * V, x), V, lane);
+    if (!a.normalized) lse = row_lse<MODE>(v, logits_row<LOGITS>(cand + (size_t)warp * V, x), V, lane);
     if (lane == 0) s_slot.lse[warp] = lse;
     if (lane == 0) s_slot.blank[warp] = (float)((double)my_score + (double)((MODE == 1 ? v[0] : x0) - lse));
   }
@@ -942,9 +943,9 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) k_tsd_select(const __grid_cons
 }
 
 cudaError_t launch_tsd_select(const BeamSelArgs& a, cudaStream_t s, bool dependent) {
-  static size_t configured[5][MAX_DEVICES];
-  static void (*const kern[5])(const BeamSelArgs) = {k_tsd_select<0, 1>, k_tsd_select<1, 2>, k_tsd_select<1, 8>,
-                                                     k_tsd_select<1, 32>, k_tsd_select<2, 32>};
+  static size_t configured[6][MAX_DEVICES];
+  static void (*const kern[6])(const BeamSelArgs) = {k_tsd_select<0, 1>, k_tsd_select<1, 2>, k_tsd_select<1, 8>,
+                                                     k_tsd_select<1, 32>, k_tsd_select<2, 32>, k_tsd_select<2, 32, true>};
   const int form = sel_form(a);
   timing_begin(s);
   const cudaError_t le = sel_launch(kern[form], configured[form], a, s, dependent);
