@@ -463,7 +463,9 @@ int q4_encoder_recurrence_plan(int32_t T, int32_t B, int32_t dirs, int32_t H, in
  * projections) launches with a producer that issues no copy at all, so that the consumer's wait
  * runs out after wait_limit polls (0 = the normal limit); nothing asynchronous is in flight, every
  * thread of the kernel still reaches its final barrier, tensor memory is freed, nothing is stored
- * and the status word reads Q4_ERR_TIMEOUT.  (0, 0) restores normal operation.  Process-wide. */
+ * and the status word reads Q4_ERR_TIMEOUT.  skip_producer = 2 has another effect: the kernel that forms a
+ * search's recurrent sums gives up its waits after wait_limit polls (0: at once) with its copies and products on their
+ * way, and stays until they are done.  (0, 0) restores normal operation; without skip_producer wait_limit has no effect.  Process-wide. */
 int q4_test_wait_expiry_set(int32_t skip_producer, uint32_t wait_limit);
 
 /* Threads: the library keeps a few process-wide host variables (launch and quantizer counters, the

@@ -133,10 +133,10 @@ __global__ void __launch_bounds__(192, 2) k_state_products(const __grid_constant
     if (warp == 4) {
       const uint32_t on = elect_one();
       bool ok = true;
-      int s = 0;
+      int s = 0, i = 0;
       uint32_t ph = 1;
-      for (int i = 0; i < nk && ok; ++i) {
-        ok = i < SP_STAGES || mbar_wait_warp(&empty[s], ph);   // (a stage that has never been filled is free)
+      for (; i < nk; ++i) {
+        ok = i < SP_STAGES || mbar_wait_warp(&empty[s], ph, jobs.wait_limit);   // (a stage that has never been filled is free)
         if (!ok) break;
         mbar_expect_tx(on, &full[s], STAGE);
         tma_load_2d(on, smem + s * STAGE, ta, i * SP_BK, m0, &full[s]);
@@ -146,7 +146,10 @@ __global__ void __launch_bounds__(192, 2) k_state_products(const __grid_constant
           ph ^= 1;
         }
       }
-      if (!ok && lane == 0) atomicExch(jobs.status, Q4_ERR_TIMEOUT);
+      if (!ok) {
+        if (lane == 0) atomicExch(jobs.status, Q4_ERR_TIMEOUT);
+        ring_landed(full, SP_STAGES, i);
+      }
     } else if (warp == 5) {
       const uint32_t idesc = umma_idesc_i8(umma_rows(jobs.tile_rows), SP_BN);
       const uint32_t on = elect_one();
@@ -154,7 +157,7 @@ __global__ void __launch_bounds__(192, 2) k_state_products(const __grid_constant
       int s = 0;
       uint32_t ph = 0;
       for (int i = 0; i < nk && ok; ++i) {
-        ok = mbar_wait_warp_tested(ready, &full[s], ph);
+        ok = mbar_wait_warp_tested(ready, &full[s], ph, jobs.wait_limit);
         if (!ok) break;
         tc_fence_after();
         const int st = s;
@@ -170,13 +173,19 @@ __global__ void __launch_bounds__(192, 2) k_state_products(const __grid_constant
         umma_commit(on, &empty[st]);
       }
       umma_commit(on, &acc_full);
-      if (!ok && lane == 0) atomicExch(jobs.status, Q4_ERR_TIMEOUT);
+      if (!ok) {
+        if (lane == 0) atomicExch(jobs.status, Q4_ERR_TIMEOUT);
+        ring_landed(full, SP_STAGES, nk);
+      }
     } else {
       const int n = m0 + umma_lane_row(umma_rows(jobs.tile_rows), warp, lane);
       const int dst = n < n_work ? jobs.dst_row[n] : -1;
-      const bool ok = mbar_wait_warp(&acc_full, 0);
+      const bool ok = mbar_wait_warp(&acc_full, 0, jobs.wait_limit);
       tc_fence_after();
-      if (!ok && lane == 0) atomicExch(jobs.status, Q4_ERR_TIMEOUT);
+      if (!ok) {   // tensor memory is not freed before the products that have been issued are done
+        if (lane == 0) atomicExch(jobs.status, Q4_ERR_TIMEOUT);
+        mbar_wait_warp(&acc_full, 0);
+      }
       float* const out = jobs.job[p].sums + (long long)dst * 4 * K + n0;
       const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
@@ -200,6 +209,7 @@ __global__ void __launch_bounds__(192, 2) k_state_products(const __grid_constant
 cudaError_t launch_state_products(const StateProductJobs& args, cudaStream_t s, bool dependent) {
   StateProductJobs a = args;
   const int rows_pad = (a.N + SP_BM - 1) / SP_BM * SP_BM;
+  a.wait_limit = test_ring_wait_limit();
   a.tile_rows = a.N < SP_BM ? (a.N + 7) / 8 * 8 : SP_BM;   // a single row tile fetches no rows beyond the launch's
   StateMaps maps;
   memset(&maps, 0, sizeof(maps));

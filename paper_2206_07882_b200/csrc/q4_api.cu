@@ -120,7 +120,7 @@ int q4_beam_select_exact_set(int32_t enabled) {
   return prev;
 }
 int q4_test_wait_expiry_set(int32_t skip_producer, uint32_t wait_limit) {
-  test_wait_expiry_set(skip_producer ? 1 : 0, wait_limit);
+  test_wait_expiry_set(skip_producer == 2 ? 2 : skip_producer ? 1 : 0, wait_limit);
   return Q4_OK;
 }
 int q4_encoder_time_slicing_set(int32_t enabled) { return enc_recurrent_sliced_set(enabled ? 1 : 0); }

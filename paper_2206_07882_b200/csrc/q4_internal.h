@@ -172,6 +172,7 @@ cudaError_t launch_mma_gemm(const int8_t* x8, long long x_pitch, int M, const in
                             const int32_t* n_idle = nullptr, int all_idle = 0);
 void test_wait_expiry_set(int skip_producer, uint32_t wait_limit);
 bool test_wait_expiry_active();
+uint32_t test_ring_wait_limit();   // polls before a wait of k_state_products gives up
 cudaError_t launch_mma_gemm_i32(const int8_t* x8, int M, const int8_t* w8, int J, int K, int planes, int32_t* out,
                                 int32_t* status, cudaStream_t s, bool dependent = false);
 // One launch for what a layer call prepares (k_layer_prepare).
@@ -228,6 +229,7 @@ struct StateProductJobs {
   const int32_t* dst_row;
   const int32_t* n_work;          // rows with work, as k_search_cells left it
   int32_t* status;
+  uint32_t wait_limit;            // polls before a wait gives up; set by the launcher
 };
 cudaError_t launch_state_products(const StateProductJobs& jobs, cudaStream_t s, bool dependent);
 

@@ -306,13 +306,17 @@ struct MmaGemmArgs {
 };
 
 // Test hook (q4_test_wait_expiry_set): the next launches of k_mma_gemm get this limit and flag.
-static uint32_t g_wait_limit = 1u << 22;
+constexpr uint32_t WAIT_LIMIT = 1u << 22;   // polls
+static uint32_t g_wait_limit = WAIT_LIMIT, g_ring_wait_limit = WAIT_LIMIT;
 static int g_skip_producer = 0;
-void test_wait_expiry_set(int skip_producer, uint32_t wait_limit) {
-  g_skip_producer = skip_producer;
-  g_wait_limit = wait_limit ? wait_limit : (1u << 22);
+// mode 1: no copies, short waits in k_mma_gemm; 2: short waits in k_state_products
+void test_wait_expiry_set(int mode, uint32_t wait_limit) {
+  g_skip_producer = mode == 1;
+  g_wait_limit = mode == 1 && wait_limit ? wait_limit : WAIT_LIMIT;
+  g_ring_wait_limit = mode == 2 ? wait_limit : WAIT_LIMIT;
 }
-bool test_wait_expiry_active() { return g_skip_producer != 0 || g_wait_limit != (1u << 22); }
+bool test_wait_expiry_active() { return g_skip_producer != 0 || g_ring_wait_limit != WAIT_LIMIT; }
+uint32_t test_ring_wait_limit() { return g_ring_wait_limit; }
 
 template <int GEMM_BN>
 __global__ void __launch_bounds__(192, 1)

@@ -93,6 +93,14 @@ __device__ __forceinline__ bool mbar_wait_warp_tested(bool ready, uint64_t* bar,
   return __all_sync(0xffffffffu, ready) != 0 || mbar_wait_warp(bar, parity, limit);
 }
 
+// After a wait that has run out: nobody leaves while copies are on their way into the block's memory (bounded).  The last of
+// the `issued` copies into a ring of `stages`; by a producer that gave up, for those it has issued, and by a consumer that gave
+// up, for all of them (if the producer has not issued them all, it waits for its own).
+__device__ __forceinline__ void ring_landed(uint64_t* full, int stages, int issued) {
+  for (int j = max(issued - stages, 0); j < issued; ++j)
+    if (!mbar_wait_warp(&full[j % stages], (uint32_t)(j / stages) & 1u)) break;
+}
+
 // 2-D tiled TMA load into shared memory, completion counted on an mbarrier.  x is the
 // innermost (contiguous) coordinate and must be a multiple of 16 bytes.
 __device__ __forceinline__ void tma_load_2d(uint32_t on, void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {

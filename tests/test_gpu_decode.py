@@ -684,6 +684,29 @@ def test_search_whose_loop_cannot_be_built(Bd, where):
     assert dd.search_plan_info() == dict(built=1, replays=9, failed=3)
 
 
+@pytest.mark.parametrize("W,H", [(6, 256), (16, 1024)])
+def test_products_stay_until_their_copies_have_landed(Bd, W, H):
+    # Waits of the recurrent sums' kernel give up at once, or after one poll, while its copies are on their way, fewer and more
+    # of them than its ring holds: a search has the right scores or reads Q4_ERR_TIMEOUT, and the next one is right.
+    import ctypes as C
+    dw = synth.decoder(seed=67, V=64, E=32, Hp=H, D=256, Hs=H, Ht=H, tgt_layers=2, U_max=9, W=W)
+    e = torch.from_numpy(synth.Stream(29).normal("e", (20, 3, 256)).astype(np.float32)).cuda()
+    dd = Bd.Decoder(dw)
+    want = [t.clone() for t in dd.decode(e)] + [dd.tensors["bp_score"].clone()]
+    for limit in (0, 0, 1, 0):
+        assert Bd.lib().q4_test_wait_expiry_set(C.c_int32(2), C.c_uint32(limit)) == 0
+        try:
+            got = dd.decode(e)
+            torch.cuda.synchronize()
+        finally:
+            Bd.lib().q4_test_wait_expiry_set(C.c_int32(0), C.c_uint32(0))
+        status = dd.tensors["status"].item()
+        assert status == -8 or (limit and status == 0 and torch.equal(dd.tensors["bp_score"], want[3]))   # Q4_ERR_TIMEOUT
+        for x, y in zip([*dd.decode(e), dd.tensors["bp_score"]], want):
+            assert torch.equal(x, y)
+        assert dd.tensors["status"].item() == 0
+
+
 def test_search_beside_a_capture_of_another_thread(Bd):
     # a search that creates its plan and builds its graph on one thread leaves a capture that another thread has open
     # (in the strictest mode, torch's default) as it is
