@@ -812,13 +812,6 @@ __device__ __forceinline__ void cl_store_f32(const float* local, uint32_t rank, 
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cl_map(smem_u32(local), rank)), "f"(v) : "memory");
 }
 
-// e^x as 2^(x log2 e) on the base-2 unit, results below the normal range as 0 (they are added to a sum of at least 1):
-// without the scaling that keeps them 4 instructions instead of 8
-__device__ __forceinline__ float exp_fast(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__fmul_rn(x, 1.4426950408889634f)));
-  return y;
-}
 template <int NB>
 __global__ void __cluster_dims__(HEAD_CTAS, 1, 1) __launch_bounds__(HEAD_THREADS, 1)
 k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ CUtensorMap tma_wb,
@@ -1074,21 +1067,15 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
     } else {
       // exponentials by the hardware base-2 unit: relative error near 1e-6, far inside what the
       // log-sum-exp of a thousand terms needs
-      float my_s = 0.0f;
-      if (busy) {
-        const float top = my_m > -INFINITY ? my_m : 0.0f;
-#pragma unroll
-        for (int i = 0; i < CPT; ++i) my_s += exp_fast(v[i] - top);
-      }
+      const float my_s = busy ? exp_sum(v, my_m) : 0.0f;
       red_m[cs][rt] = my_m;
       red_s[cs][rt] = my_s;
       asm volatile("bar.sync 1, %0;" ::"n"(32 * HEAD_EPI_WARPS) : "memory");
       if (cs == 0) {   // this CTA's (max, sum) of the row goes to every CTA of the cluster
-        const float m = fmaxf(fmaxf(red_m[0][rt], red_m[1][rt]), fmaxf(red_m[2][rt], red_m[3][rt]));
-        float ssum = 0.0f;
-        const float top = m > -INFINITY ? m : 0.0f;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) ssum += red_s[i][rt] * exp_fast(red_m[i][rt] - top);   // 0 for a share without entries
+        const float ms[4] = {red_m[0][rt], red_m[1][rt], red_m[2][rt], red_m[3][rt]};
+        const float ss[4] = {red_s[0][rt], red_s[1][rt], red_s[2][rt], red_s[3][rt]};
+        const float m = fmaxf(fmaxf(ms[0], ms[1]), fmaxf(ms[2], ms[3]));
+        const float ssum = exp_sum(ms, ss, m);
 #pragma unroll
         for (int r = 0; r < HEAD_CTAS; ++r) {
           cl_store_f32(&part_m[nb][rt], (uint32_t)r, m);
@@ -1106,11 +1093,7 @@ k_mma_lmhead(const __grid_constant__ CUtensorMap tma_h, const __grid_constant__ 
       float m = -INFINITY;
 #pragma unroll
       for (int r = 0; r < HEAD_CTAS; ++r) m = fmaxf(m, pm[r]);
-      float ssum = 0.0f;
-      const float top = m > -INFINITY ? m : 0.0f;
-#pragma unroll
-      for (int r = 0; r < HEAD_CTAS; ++r) ssum += ps[r] * exp_fast(pm[r] - top);
-      lse = m + logf(ssum);
+      lse = m + logf(exp_sum(pm, ps, m));
     }
     // A thread's log-probabilities belong to one row and the rows of a warp's lanes are V floats
     // apart, so storing them directly touches 32 lines per instruction.  A full 128-column block goes

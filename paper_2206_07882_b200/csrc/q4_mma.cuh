@@ -63,8 +63,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32
 
 // One lane of a converged warp.  The loops that issue copies and MMAs are walked by a whole warp with warp-uniform values;
 // the instructions themselves are predicated on the elected lane (the forms below with `on` as first argument), not branched
-// over: they take descriptors and coordinates from uniform registers, and inside a branch of one lane that arithmetic is done
-// in ordinary ones and moved for each instruction.  The next stage's barrier is tested before a chunk's MMAs are issued, so
+// over.  The next stage's barrier is tested before a chunk's MMAs are issued, so
 // that the latency of the answer passes beside them (mbar_test: mbarrier.try_wait would hold the warp while that stage is still
 // on its way, 13 to 20 % of a search).  Clocks per K chunk (wait, four int8 MMAs 128 x N x 32, commit; operands
 // in place, all SMs), N = 32 / 64 / 128: 308 / 318 / 334 with a branch and without the test, 168 / 192 / 256 this way; the
@@ -125,6 +124,36 @@ __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
 
 // int8 matrix [rows, k] with row pitch `pitch` bytes; box = 128 bytes of K x box_rows rows, 128-byte swizzle (q4_mma.cu).
 bool make_tmap_i8(CUtensorMap* m, const void* base, uint64_t k, uint64_t rows, uint64_t pitch, uint32_t box_rows);
+
+// ---- sums of exponentials -------------------------------------------------------------
+// The output heads and the label-free end of a search sum a row's exponentials in shares, by these two functions, so that a
+// blank's log-probability is the same bits in both.
+// e^x = 2^(x log2 e) on the base-2 unit (ex2.approx: relative error 2^-22); .ftz: a result below 2^-126 is 0.  For terms of a
+// sum that has a term e^0 = 1 only: 2^11 entries of less than 2^-126 are 2^-115 of it, its rounding is 2^-24.
+__device__ __forceinline__ float exp_of_sum(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__fmul_rn(x, 1.4426950408889634f)));
+  return y;
+}
+// A share's sum relative to its maximum m; entries that do not count are -inf (m = -inf: a share without entries).
+// No branch for one: 32 exponentials with a branch each took 2950 clocks of a head, 1690 this way.
+template <int N>
+__device__ __forceinline__ float exp_sum(const float (&v)[N], float m) {
+  const float top = m > -INFINITY ? m : 0.0f;
+  float sum = 0.0f;
+#pragma unroll
+  for (int i = 0; i < N; ++i) sum += exp_of_sum(v[i] - top);
+  return sum;
+}
+// Shares (maximum, sum) relative to the maximum m of all; a share without entries adds 0.
+template <int N>
+__device__ __forceinline__ float exp_sum(const float (&part_m)[N], const float (&part_s)[N], float m) {
+  const float top = m > -INFINITY ? m : 0.0f;
+  float sum = 0.0f;
+#pragma unroll
+  for (int i = 0; i < N; ++i) sum += part_s[i] * exp_of_sum(part_m[i] - top);
+  return sum;
+}
 
 // ---- tensor memory ------------------------------------------------------------------
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {

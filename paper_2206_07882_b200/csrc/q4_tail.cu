@@ -4,8 +4,8 @@
 // (it "freezes" the utterance), the steps end when all utterances are frozen, and two launches do the rest:
 //   k_tail_blank : log P(blank) of every frozen slot at every frame that is left, as one batch of joint-network rows;
 //   k_tail_walk  : the remaining iterations of each utterance, one warp each: scores, order, finished list, history.
-// The arithmetic is the step kernels' own, operation for operation (tanh(e p) and its codes, sums over the vocabulary in
-// the same order), so beams and scores are the same bits.  A step costs 12 us (one utterance) to 25 us (64 x 16 slots) of
+// The arithmetic is the step kernels' own (tanh(e p) and its codes; sums over the vocabulary in the same order, with the
+// heads' functions), so beams and scores are the same bits.  A step costs 12 us (one utterance) to 25 us (64 x 16 slots) of
 // dependent launches when nothing is labelled, a joint-network row here about 1 ns.
 #include <string.h>
 
@@ -212,16 +212,13 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_tail_blank(const __grid_const
 #pragma unroll
           for (int j = 0; j < CPT; ++j) red[rt * TL_PITCH + col0 + j] = v[j];   // columns beyond V are not read
         } else {
-          float my_m = -INFINITY, my_s = 0.0f;
+          float my_m = -INFINITY;
 #pragma unroll
           for (int j = 0; j < CPT; ++j) {
             if (col0 + j >= V) v[j] = -INFINITY;
             my_m = fmaxf(my_m, v[j]);
           }
-          const float top = my_m > -INFINITY ? my_m : 0.0f;
-#pragma unroll
-          for (int j = 0; j < CPT; ++j) my_s += __expf(v[j] - top);
-          *reinterpret_cast<float2*>(red + ((i * 4 + cs) * TL_BM + rt) * 2) = make_float2(my_m, my_s);
+          *reinterpret_cast<float2*>(red + ((i * 4 + cs) * TL_BM + rt) * 2) = make_float2(my_m, exp_sum(v, my_m));
           if (i == 0 && cs == 0) s_blank[rt] = v[0];
         }
       }
@@ -250,26 +247,25 @@ __global__ void __launch_bounds__(TL_THREADS, 1) k_tail_blank(const __grid_const
           if (lane == 0) put(r, x[0] - (m + logf(sum)));
         }
       } else if (cs == 0) {
-        float pm[TL_BLOCKS], ps[TL_BLOCKS], m = -INFINITY, ssum = 0.0f;
+        float pm[TL_BLOCKS], ps[TL_BLOCKS], m = -INFINITY;
 #pragma unroll
         for (int i = 0; i < TL_BLOCKS; ++i) {
           pm[i] = -INFINITY;
           ps[i] = 0.0f;
           if (i < n_blk) {
-            float2 x[4];
+            float xm[4], xs[4];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) x[c] = *reinterpret_cast<const float2*>(red + ((i * 4 + c) * TL_BM + rt) * 2);
-            pm[i] = fmaxf(fmaxf(x[0].x, x[1].x), fmaxf(x[2].x, x[3].x));
-#pragma unroll
-            for (int c = 0; c < 4; ++c)
-              if (x[c].y > 0.0f) ps[i] += x[c].y * __expf(x[c].x - pm[i]);
+            for (int c = 0; c < 4; ++c) {
+              const float2 x = *reinterpret_cast<const float2*>(red + ((i * 4 + c) * TL_BM + rt) * 2);
+              xm[c] = x.x;
+              xs[c] = x.y;
+            }
+            pm[i] = fmaxf(fmaxf(xm[0], xm[1]), fmaxf(xm[2], xm[3]));
+            ps[i] = exp_sum(xm, xs, pm[i]);
           }
           m = fmaxf(m, pm[i]);
         }
-#pragma unroll
-        for (int i = 0; i < TL_BLOCKS; ++i)
-          if (ps[i] > 0.0f) ssum += ps[i] * __expf(pm[i] - m);
-        put(rt, s_blank[rt] - (m + logf(ssum)));
+        put(rt, s_blank[rt] - (m + logf(exp_sum(pm, ps, m))));
       }
     }
   }
