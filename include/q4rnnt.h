@@ -385,6 +385,9 @@ int q4_search_plan_destroy(q4_search_plan plan);
 /* What a plan has done so far (host counters, for tests and diagnostics): out[0] graphs built, out[1] groups
  * of 12 steps that replays were enqueued for, out[2] attempts to build a graph, or a loop in the caller's, that failed (the search then enqueued its steps one by one). */
 int q4_search_plan_info(q4_search_plan plan, int64_t* out);
+/* Steps of the last search enqueued with this plan (`workspace`: the search's; of a captured one its last replay): all of
+ * them, or those before its label-free end.  Synchronises `stream`. */
+int q4_search_steps_taken(q4_search_plan plan, const void* workspace, q4_stream stream, int32_t* steps);
 /* Test hook: from now on every loop that a search with this plan builds fails, before its node is added (where = 1) or before
  * the node is filled (2); 0 restores normal operation.  Graphs built before are not touched. */
 int q4_test_search_loop_failure_set(q4_search_plan plan, int32_t where);

@@ -80,7 +80,7 @@ class BeamStateS(C.Structure):
 
 EXPORTS = ["q4_act_symmetric", "q4_act_asymmetric", "quantize_pack_int4", "qlstm_layer_forward",
            "qlstm_step", "q4_linear_forward", "qjoint_logprobs", "q4_beam_init",
-           "dr_fusion_beam_step", "q4_beam_search", "q4_search_plan_create", "q4_search_plan_destroy", "q4_search_plan_info", "q4_traceback", "q4_feature_prologue", "q4_workspace_bytes",
+           "dr_fusion_beam_step", "q4_beam_search", "q4_search_plan_create", "q4_search_plan_destroy", "q4_search_plan_info", "q4_search_steps_taken", "q4_traceback", "q4_feature_prologue", "q4_workspace_bytes",
            "q4_poll_status", "q4_version", "q4_launch_count", "q4_dependent_launch_set", "q4_beam_select_exact_set", "q4_timing_set", "q4_timing_count", "q4_prepared_bytes", "q4_prepare_model", "q4_table_bytes", "q4_prepare_tables", "qjoint_logprobs_static", "q4_quantizer_calls", "q4_prepared_lstm_bytes", "q4_prepare_lstm",
            "q4_prepared_linear_bytes", "q4_prepare_linear", "q4_test_wait_expiry_set", "q4_test_search_loop_failure_set", "q4_encoder_time_slicing_set", "q4_encoder_recurrence_plan"]
 
@@ -731,6 +731,7 @@ class Decoder:
             _chk(lib().q4_search_plan_create(C.byref(plan)), "q4_search_plan_create")
             self._plan = _SearchPlan(plan)
         plan = self._plan.handle if self._plan is not None and self.state.aux_stream[0] else None
+        self._steps = T * (self.S_max + 1) if time_synchronous else T + u_max
         dw = self.dw
         _chk(lib().q4_beam_search(C.byref(self.model), C.byref(self.state), _p(e), C.c_int32(self.B), C.c_int32(T),
                                   C.c_int32(self.W), C.c_int32(u_max), C.c_float(dw.lambda_t), C.c_float(dw.lambda_s),
@@ -738,9 +739,12 @@ class Decoder:
                                   C.c_size_t(self.ws.numel()), plan, _stream()), "q4_beam_search")
 
     def search_steps_taken(self) -> int:
-        """Steps that the last looped search on this state ran before its label-free end (waits for the device)."""
-        iteration = int(self.ws[16:20].view(torch.int32).item())     # of the call block, a group of 12 steps behind
-        return iteration + 12
+        """Steps of the last search on this state, without those of a label-free end (waits for the device)."""
+        if self._plan is None:
+            return self._steps
+        n = C.c_int32()
+        _chk(lib().q4_search_steps_taken(self._plan.handle, _p(self.ws), _stream(), C.byref(n)), "q4_search_steps_taken")
+        return n.value
 
     def search_plan_info(self) -> dict:
         """Graphs built, replays enqueued and failed builds of the decoder's search plan."""

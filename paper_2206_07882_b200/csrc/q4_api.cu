@@ -1563,6 +1563,7 @@ struct SearchPlan {
   SearchGraph graph[PLAN_GRAPHS];
   int64_t built, replays, failed;    // graphs made, replays enqueued, attempts to make a graph or a loop that failed
   int32_t test_failure;              // see q4_test_search_loop_failure_set
+  int32_t last_iters, last_looped;   // steps of the last search; whether a loop ended them
   int64_t uses;
   // Captured on: the graphs' chains, none of the caller's streams.  side[2] or side[3] take the recurrent sums: up to 128 rows
   // with a lower priority than the rest, so that the joint network's chain, which is the longest there, does not queue
@@ -1714,6 +1715,18 @@ int q4_test_search_loop_failure_set(q4_search_plan plan, int32_t where) {
   static_cast<SearchPlan*>(plan)->test_failure = where;
   return Q4_OK;
 }
+int q4_search_steps_taken(q4_search_plan plan, const void* workspace, q4_stream stream, int32_t* steps) {
+  if (!plan || !workspace || !steps) return Q4_ERR_NULL;
+  const SearchPlan* p = static_cast<const SearchPlan*>(plan);
+  *steps = p->last_iters;
+  if (!p->last_looped) return Q4_OK;
+  SearchCall call;
+  Q4_TRY(cudaMemcpyAsync(&call, workspace, sizeof(call), cudaMemcpyDeviceToHost, S(stream)));
+  Q4_TRY(cudaStreamSynchronize(S(stream)));
+  const int taken = call.iter + PLAN_ITERS;   // (the call's number is that of the turn's first step, less PLAN_ITERS)
+  if (taken < *steps) *steps = taken;
+  return Q4_OK;
+}
 int q4_search_plan_info(q4_search_plan plan, int64_t* out) {
   if (!plan || !out) return Q4_ERR_NULL;
   const SearchPlan* p = static_cast<const SearchPlan*>(plan);
@@ -1767,6 +1780,7 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
             cudaStreamIsCapturing(s, &cap) != cudaSuccess || (cap != cudaStreamCaptureStatusNone && !key.loop)))
     p = nullptr;
   bool tail = false;
+  SearchPlan* const plan_of_call = static_cast<SearchPlan*>(plan);
   for (int it = 0; it < n_iters;) {
     // the first two frames' steps always: the first step's networks start from the reset state, and the kernels set their
     // attributes at their first launch
@@ -1823,6 +1837,10 @@ int q4_beam_search(const q4_model* model, q4_beam_state* state, const float* e, 
     Q4_CHECK(beam_step(model, state, e, B, T, W, it, u_max, lambda_t, lambda_s, rho, step_mode(key, it), workspace,
                        workspace_bytes, stream, StepMode{nullptr, nullptr, nullptr, sums, nullptr, nullptr}));
     ++it;
+  }
+  if (plan_of_call) {
+    plan_of_call->last_iters = n_iters;
+    plan_of_call->last_looped = tail;
   }
   if (tail) {
     const q4_model& m = *model;

@@ -1023,6 +1023,25 @@ def test_search_counts_the_quantizers_of_all_its_steps(Bd, T, U, S):
         assert Bd.quantizer_calls(reset=True) == 14 * n
 
 
+def test_steps_that_a_search_has_taken(Bd):
+    # without labels a loop takes one turn of 12 steps behind the first two; a search that is not looped takes all of its own,
+    # whatever ran on the state before
+    dw = synth.decoder(seed=67, V=46, E=10, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=9, W=6)
+    e = torch.from_numpy(synth.Stream(28).normal("e", (110, 3, 256)).astype(np.float32)).cuda()
+    dd = Bd.Decoder(dw)
+    dd.alloc_state(3, 6, 220)
+    captured = Bd.GraphedStep(lambda: dd.decode(e, 0))
+    for run, low, high in ((lambda: dd.decode(e, 0), 14, 14), (lambda: dd.decode(e[:50], 5), 55, 55), (captured, 14, 14),
+                           (lambda: dd.decode(e, 9), 14, 119)):
+        run()
+        assert low <= dd.search_steps_taken() <= high
+    plain = Bd.Decoder(dw, concurrent=False)
+    plain.decode(e, 9)
+    assert plain.search_steps_taken() == 119
+    dd.decode_time_synchronous(e, 1, 9)
+    assert dd.search_steps_taken() == 220
+
+
 @pytest.mark.parametrize("V,normalized", [(2, 1), (46, 1), (64, 1), (65, 1), (256, 1), (257, 1), (300, 0), (1023, 1), (1024, 0),
                                           (1024, 1), (1025, 1)])
 @pytest.mark.parametrize("S", [None, 1])
