@@ -929,15 +929,27 @@ def test_search_all_eight_bit(Bd, dims):
     assert tr == 1.0
 
 
+@pytest.mark.parametrize("single_steps", [True, False])
 @pytest.mark.parametrize("B,W", [(1, 5), (1, 16), (2, 16), (3, 7)])
-def test_search_few_rows_weight_streaming_kernels(Bd, B, W):
-    # at most 32 hypothesis rows and widths that are multiples of 128: the LSTM steps run on the
+def test_search_few_rows_weight_streaming_kernels(Bd, B, W, single_steps):
+    # at most 32 hypothesis rows and widths that are multiples of 128: the LSTM steps of single steps run on the
     # weight-streaming kernel that reads packed 4-bit weights, state rows and embedding rows as stored
-    # (signed prediction-network input, unsigned LM input with its zero point); every beam of every
-    # iteration as the oracle's
+    # (signed prediction-network input, unsigned LM input with its zero point), those of a whole search on the kernels that
+    # look labels up and keep sums; every beam of every iteration as the oracle's
     dw = synth.decoder(seed=99, V=128, E=128, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=6, W=W)
     e = synth.Stream(17).normal("e", (9, B, 256)).astype(np.float32)
-    dd, tokens, lens, scores, ref = run_search(Bd, dw, e)
+    if single_steps:
+        dd = Bd.Decoder(dw)
+        dd.alloc_state(B, W, 15)
+        dd.q4_beam_init()
+        e_dev = torch.from_numpy(e).cuda()
+        for it in range(15):
+            dd.dr_fusion_beam_step(e_dev, 9, it, 6)
+        tokens, lens, scores = (t.cpu().numpy() for t in dd.q4_traceback(15, 6))
+        assert dd.tensors["status"].item() == 0
+        ref = O.alsd(O.Decoder(dw), e)
+    else:
+        dd, tokens, lens, scores, ref = run_search(Bd, dw, e)
     frac, tr = compare_search(dd, tokens, lens, scores, ref, list(range(B)), 9, 6, W, min_same=1.0)
     assert tr == 1.0
 
@@ -1107,6 +1119,36 @@ def test_search_that_keeps_sums_equals_its_steps(Bd, B, W, S, layers, bits):
     assert a.tensors["status"].item() == 0
     for k in ("bp_parent", "bp_token", "bp_score", "fin_n", "fin_score", "pred_c", "tgt_c0", "tgt_hq0", "pred_p"):
         assert torch.equal(a.tensors[k], b.tensors[k]), k
+
+
+@pytest.mark.parametrize("B,W,S", [(9, 15, None), (16, 16, None), (24, 16, None), (17, 8, 1), (24, 16, 2)])
+def test_replayed_search_that_keeps_sums_equals_its_steps(Bd, B, W, S):
+    # the same from a graph (a loop, or groups of steps), where the products of one, two and three row tiles have a stream of
+    # their own beside the heads and the selection: the decoder's graph twice, and one captured by the caller twice
+    dw = synth.decoder(seed=92, V=300, E=32, Hp=256, D=256, Hs=128, Ht=384, tgt_layers=2, U_max=25, W=W)
+    dw.joint.out.bias[0] += np.float32(3.0)
+    T, U = (101, 25) if S is None else (50, 25)
+    e = torch.from_numpy(synth.Stream(B * W).normal("e", (T, B, 256)).astype(np.float32)).cuda()
+    n = T + U if S is None else T * (S + 1)
+    a, b = Bd.Decoder(dw), Bd.Decoder(dw)
+    b.alloc_state(B, W, n, S)
+    b.q4_beam_init()
+    for it in range(n):
+        b.dr_fusion_beam_step(e, T, it, U, mode=0 if S is None else 2 if it % (S + 1) == S else 1)
+    want = b.q4_traceback(n, U)
+    decode = (lambda: a.decode(e, U)) if S is None else (lambda: a.decode_time_synchronous(e, S, U))
+    captured = Bd.GraphedStep(decode)
+    keys = ["bp_parent", "bp_token", "bp_score", "fin_n", "fin_score", "fin_iter", "fin_slot", "score", "row", "status", "pred_c",
+            "src_c", "tgt_c0", "tgt_c1", "pred_hq", "src_hq", "tgt_hq0", "tgt_hq1", "pred_p", "src_lp", "tgt_lp"]
+    for run in (decode, decode, captured, captured):
+        if a.state is not None:
+            for k in keys[:3] + keys[10:14]:
+                a.tensors[k].fill_(0)
+        for x, y in zip(run(), want):
+            assert torch.equal(x, y)
+        for k in keys:
+            assert torch.equal(a.tensors[k], b.tensors[k]), k
+    assert a.search_plan_info()["built"] == 1 and a.model.tables
 
 
 def test_search_with_embeddings_of_other_row_lengths(Bd):

@@ -178,10 +178,15 @@ def test_the_search_stays_inside_its_state_and_workspace(guarded, tensor_cores):
         dec = Bd.Decoder(dw, tensor_cores=tensor_cores)
         dec.decode(e)
         dec.decode_time_synchronous(e, 2)
-    # one utterance: the weight-streaming step kernel
-    dw = synth.decoder(seed=78, V=1024, E=32, Hp=256, D=256, Hs=256, Ht=256, tgt_layers=2, U_max=5, W=16)
+    # one utterance: a whole search, and single steps on the weight-streaming step kernel
+    dw = synth.decoder(seed=78, V=1024, E=128, Hp=256, D=256, Hs=256, Ht=256, tgt_layers=2, U_max=5, W=16)
     e = torch.from_numpy(synth.Stream(6).normal("e", (9, 1, 256)).astype(np.float32)).cuda()
-    Bd.Decoder(dw, tensor_cores=tensor_cores).decode(e)
+    dec = Bd.Decoder(dw, tensor_cores=tensor_cores)
+    dec.decode(e)
+    dec.q4_beam_init()
+    for it in range(14):
+        dec.dr_fusion_beam_step(e, 9, it, 5)
+    dec.q4_traceback(14, 5)
     assert g.check() > 20
 
 
