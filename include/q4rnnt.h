@@ -482,7 +482,8 @@ int q4_test_wait_expiry_set(int32_t skip_producer, uint32_t wait_limit);
  * pairs were used.  tag_mask 0 switches timing off (the default).  Tags: 1 quantize, 2
  * encoder input GEMM, 3 encoder recurrent step, 4 linear, 5 prediction LSTM, 6 prediction
  * projection, 7 source-LM LSTM, 8 source-LM head, 9 target-LM layer 1, 10 target-LM layer 2,
- * 11 target-LM head, 12 joint, 13 beam selection, 14 other. */
+ * 11 target-LM head, 12 joint, 13 beam selection, 14 other, 15 first layers of a search that looks
+ * labels up, 16 its recurrent sums. */
 int q4_timing_set(uint32_t tag_mask, void** start_events, void** stop_events, int32_t* tags_out,
                   int32_t capacity);
 int q4_timing_count(void);

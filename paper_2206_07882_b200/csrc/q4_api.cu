@@ -755,7 +755,8 @@ struct TablePlan {
   size_t total;
 };
 // Tables of the first layers' input halves: 16 H bytes a label and network, so a bound on memory (268 MB with 1024, 1024 and
-// 2048 cells); a look-up costs the same at any V.
+// 2048 cells); a look-up costs the same at any V.  100 frames, ms with / without: 1024 labels, 12 rows 1.41 / 1.92,
+// 4096 labels, 12 rows 6.76 / 7.10 and 96 rows 7.38 / 7.54.
 constexpr int TABLE_MAX_V = 4096;
 bool tables_supported(const q4_model& m) {
   return m.V > 0 && m.V <= TABLE_MAX_V && m.src.n_layers == 1 && m.pred_lstm.w_hh.k_pad % 128 == 0 &&
@@ -1096,13 +1097,14 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
   ws += align_up((size_t)N * V * sizeof(float));
   int32_t* live = reinterpret_cast<int32_t*>(ws);
   ws += align_up((size_t)N * sizeof(int32_t));
-  // pending advances of this iteration, compacted by the previous selection (or the reset)
+  // pending advances of this iteration as the previous selection (or the reset) listed them: up to 128 rows every slot at its
+  // own place (those without an advance -1), beyond only the slots that have one
   const int par = iter & 1;
   int32_t* c_src = st.pend_src + (size_t)par * N;
   int32_t* c_dst = st.pend_dst + (size_t)par * N;
   int32_t* c_tok = st.pend_tok + (size_t)par * N;
   const int32_t* n_active = st.pend_n + par;
-  q4_beam_state cst = st;   // same state, pending advances in compacted order
+  q4_beam_state cst = st;   // same state, pending advances in the order of the list
   cst.adv_src = c_src;
   cst.adv_dst = c_dst;
   cst.adv_tok = c_tok;
@@ -1219,8 +1221,11 @@ static int beam_step(const q4_model* model, q4_beam_state* state, const float* e
       return Q4_OK;
     };
     // the three networks are independent until the selection: with two lent streams they run side
-    // by side.  The call's own stream carries the longest chain, the target LM's (gather -> two layers -> head ->
-    // selection as programmatic dependents without an event in between; a fork costs 2 to 4 us, a join 1 to 4).
+    // by side.  The call's own stream carries the target LM's chain (gather -> two layers -> head ->
+    // selection as programmatic dependents without an event in between; a fork costs 2 to 4 us, a join 1 to 4), which is
+    // the longest of a step that multiplies its first layers: with 1024 rows its launches, each alone, take 114 us, the
+    // prediction and joint networks' 109.  In a search that keeps sums the joint network's is longer from 16 rows on: 40 and
+    // 33 us with 16 rows, 42 and 34 with 40, 47 and 45 with 128, 48 and 43 with 256.
     // Against the prediction/joint chain there, 150 iterations with labels in most: 16 slots 4.62 -> 4.38 ms, 16 x 16
     // slots 6.64 -> 6.36, time-synchronous 4 x 8 slots 12.8 -> 12.1; with labels in a third: 3.61 -> 3.59, 5.15 ->
     // 5.22, 12.9 -> 12.1
@@ -1566,8 +1571,9 @@ struct SearchPlan {
   int32_t last_iters, last_looped;   // steps of the last search; whether a loop ended them
   int64_t uses;
   // Captured on: the graphs' chains, none of the caller's streams.  side[2] or side[3] take the recurrent sums: up to 128 rows
-  // with a lower priority than the rest, so that the joint network's chain, which is the longest there, does not queue
-  // behind them (8 rows 3.83 -> 3.55 ms); with more rows the next step would wait for them (384 rows 5.1 -> 6.0).
+  // with a lower priority than the rest, so that the launches of the joint network's chain do not queue
+  // behind them (8 rows 3.83 -> 3.55 ms); with more rows the next step would wait for them (384 rows 5.1 -> 6.0).  Networks of
+  // 1024, 1024 and 2048 cells: 192 tiles of products a row tile, for 148 SMs.
   cudaStream_t stream, side[4];
   cudaEvent_t side_event[4];
 };

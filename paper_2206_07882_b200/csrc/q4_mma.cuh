@@ -196,7 +196,8 @@ __device__ __forceinline__ uint64_t umma_desc_sw32(uint32_t smem_addr) {
 // Tiles of at most 16 rows are multiplied as 64-row tiles: an MMA of 32, 64 or 128 weight rows takes 24 / 32 / 64 clocks
 // instead of 40 / 48 / 64 (measured; the rows' way into the tensor cores bounds the narrow ones).  Row r is lane
 // 32 (r / 16) + r % 16 of tensor memory there; the other lanes hold nothing and stand for the rows from 64 on.  With more rows
-// than the 16 of a lane quarter the epilogue works on half-filled warps: 160 frames of one utterance at beam 16 3.72 ->
+// than the 16 of a lane quarter the epilogue works on half-filled warps.  Networks of 1024, 1024 and 2048 cells,
+// 160 frames of one utterance at beam 16 3.72 ->
 // 3.60 ms, beam 1 1.89 -> 1.85, but 8 x 8 rows 3.86 -> 3.90.
 __host__ __device__ constexpr int umma_rows(int tile_rows) { return tile_rows <= 16 ? 64 : 128; }
 __device__ __forceinline__ int umma_lane_row(int m, int quarter, int lane) {   // row of a warp's lane, m = umma_rows()
