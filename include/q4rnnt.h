@@ -438,7 +438,7 @@ int64_t q4_quantizer_calls(int32_t reset);
  * on it.  Not an operation of the paper. */
 int q4_dependent_launch_set(int32_t enabled);
 
-/* The beam selection first bounds the W-th best proposal from below by the smallest of 16
+/* The beam selection first bounds the W-th best proposal from below by the W-th best of 32
  * group maxima and ranks the few proposals above that bound; if they overflow its short list
  * it falls back to an exact bit-by-bit threshold search.  enabled != 0 makes every selection
  * take the exact search (for tests; both give the same beam).  Returns the previous setting. */

@@ -581,7 +581,7 @@ class _SearchPlan:
 
 class Decoder:
     """Device copy of prediction network, joint network and both fusion LMs, the search
-    state, and the iteration loop (one library call per search iteration)."""
+    state, and the searches (one library call for a whole search, or one per iteration)."""
 
     def __init__(self, dw, device="cuda", tensor_cores: bool = True, concurrent: bool = True, share_from=None):
         self.dw = dw
