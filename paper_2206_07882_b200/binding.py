@@ -615,7 +615,7 @@ class Decoder:
         m.src, m.tgt = self.src.c(), self.tgt.c()
         m.prepared = m.tables = None
         self.prepared = None
-        self.tables = []        # the buffer of q4_prepare_tables, shared with the decoders that share the weights
+        self.tables = []        # buffer of q4_prepare_tables and its event, shared with the decoders that share the weights
         if tensor_cores:
             self.q4_prepare_model()
         self.state = None
@@ -634,9 +634,10 @@ class Decoder:
     def q4_prepare_tables(self, n: int):
         """The first layers' input halves of every label, for searches of few rows (n: q4_table_bytes)."""
         if not self.tables:
-            self.tables.append(torch.empty(n, dtype=torch.uint8, device=self.device))
+            self.tables += [torch.empty(n, dtype=torch.uint8, device=self.device), torch.cuda.Event()]
         _chk(lib().q4_prepare_tables(C.byref(self.model), _p(self.tables[0]), C.c_size_t(n), _stream()),
              "q4_prepare_tables")
+        self.tables[1].record()
 
     def step_weight_bytes(self) -> int:
         return (self.pred_lstm.nbytes() + self.pred_proj.nbytes() + self.joint_out.nbytes() +
@@ -706,9 +707,10 @@ class Decoder:
             dims += [self.pred_lstm.w_ih.k_pad, Hp, Hs, Ht, RW]
         self.ws = torch.empty(workspace_bytes(WS_BEAM, dims), dtype=torch.uint8, device=dev)
         n = int(lib().q4_table_bytes(C.byref(self.model), C.c_int32(N))) if self.tensor_cores else 0
-        if n and not self.tables and not torch.cuda.is_current_stream_capturing():
-            self.q4_prepare_tables(n)
-            torch.cuda.current_stream().synchronize()     # decoders that share the weights may run on other streams
+        if n and not torch.cuda.is_current_stream_capturing():
+            if not self.tables:
+                self.q4_prepare_tables(n)
+            torch.cuda.current_stream().wait_event(self.tables[1])     # made by another decoder, on another stream perhaps
 
     def q4_beam_init(self):
         _chk(lib().q4_beam_init(C.byref(self.state), C.c_int32(self.B), C.c_int32(self.W),

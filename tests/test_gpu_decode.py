@@ -1238,6 +1238,26 @@ def test_embeddings_after_the_preparation_of_the_weights(Bd):
     check(m)
 
 
+def test_tables_made_on_another_stream(Bd):
+    # a decoder that shares the weights takes the tables that the first one is still making, late on its own stream
+    dw = synth.decoder(seed=96, V=300, E=32, Hp=128, D=256, Hs=128, Ht=256, tgt_layers=2, U_max=5, W=8)
+    e = torch.from_numpy(synth.Stream(34).normal("e", (12, 3, 256)).astype(np.float32)).cuda()
+    want = [t.clone() for t in Bd.Decoder(dw).decode(e)]
+    first = Bd.Decoder(dw)
+    second = Bd.Decoder(dw, share_from=first)
+    torch.cuda.synchronize()
+    late, side = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(late):
+        torch.cuda._sleep(200_000_000)                         # a tenth of a second
+        first.alloc_state(3, 8, 17)
+    with torch.cuda.stream(side):
+        got = second.decode(e)
+    torch.cuda.synchronize()
+    assert first.model.tables and second.tables is first.tables
+    for x, y in zip(got, want):
+        assert torch.equal(x, y)
+
+
 def test_search_with_prepared_weights_at_a_16_byte_boundary_and_tables(Bd):
     # tables have a buffer of their own: weights at a 16-byte boundary serve the kernels that look labels up
     import ctypes as C
